@@ -29,6 +29,13 @@
  *  - Errors: arguments are checked before anything is launched; a call that returns an
  *    error before launching leaves the outputs untouched.  CUDA errors map to
  *    MACH_ERR_CUDA.  No C++ exception crosses this boundary.
+ *  - Workspaces: ensembles that no kernel reads directly in their storage type and frame
+ *    count are rewritten into whole frame tiles on every run (grids of at least 6 or 16
+ *    voxels per sample; mach_plan_info.variant then names the tiles, e.g. "+x32+x8").  Each
+ *    run takes its workspace, 8 bytes per sample and padded frame, in stream order from a
+ *    memory pool that the plan owns (at most a sixteenth of the device memory per run; one
+ *    workspace is kept between runs and released with the plan).  Runs on a capturing
+ *    stream, or without memory for the workspace, allocate nothing and beamform directly.
  *  - Threads: a plan is read-only after creation.  Calls that share a plan may run on
  *    different streams concurrently, except when mach_plan_info.frame_tiles > 1 and
  *    Power Doppler is requested (those calls share the plan's partial-sum scratch and

@@ -74,10 +74,9 @@ struct SlotMeta {
 // completes on the slot's "full" barrier.  Returns false when a wait gave up (the error
 // word is then set); r counts the slots issued.
 template <int NBUF>
-__device__ __forceinline__ bool produce_windows(const DasParams& p, int64_t tile, int lane, unsigned char* ring,
-                                                size_t slot_bytes, int sample_bytes, SlotMeta* meta, uint64_t* full,
-                                                uint64_t* empty, int& r) {
-  const unsigned char* iq = static_cast<const unsigned char*>(p.iq);
+__device__ __forceinline__ bool produce_windows(const DasParams& p, const unsigned char* iq, int64_t tile, int lane,
+                                                unsigned char* ring, size_t slot_bytes, int sample_bytes,
+                                                SlotMeta* meta, uint64_t* full, uint64_t* empty, int& r) {
   const size_t row_bytes = static_cast<size_t>(p.F) * sample_bytes;
   const size_t slab = static_cast<size_t>(p.S) * row_bytes;
   const float4 blo = p.tbox[2 * tile], bhi = p.tbox[2 * tile + 1];
@@ -243,7 +242,8 @@ __global__ void __launch_bounds__((NWC + 1) * 32) __maxnreg__(MAXR) k_das_staged
       }
     }
     if constexpr (!TABLE)
-      ok = produce_windows<NBUF>(p, tile, lane, smem, L.slot_bytes, kBytes, meta, full, empty, r);
+      ok = produce_windows<NBUF>(p, static_cast<const unsigned char*>(p.iq), tile, lane, smem, L.slot_bytes, kBytes,
+                                 meta, full, empty, r);
     if (lane == 0) finish_producer<NBUF, PB>(p, ok, r, meta, full, empty);
     return;
   }

@@ -188,6 +188,122 @@ cudaError_t convert_as(const float2* src, int order, void* dst, int64_t N, int64
   return cudaGetLastError();
 }
 
+// ---- repacking for the exact-frame kernels ------------------------------------------------
+// One item = 4 consecutive frames of one sample: read in the source's storage type, widened
+// to float32, written as 4 real and 4 imaginary parts of a split row (tiles of split_frames).
+// VEC: frames one load may take (4, 2 or 1, by F's divisibility: rows start on 16-, 8- or
+// 4-byte boundaries for the 16-bit types, 16 or 8 for complex64).
+template <int DT, int VEC>
+__device__ __forceinline__ void load_quad(const void* src, int64_t n, int f, int F, float4& re, float4& im) {
+  if constexpr (DT == MACH_IQ_C64_SPLIT) {
+    const float* row = static_cast<const float*>(src) + 2 * n * F + f;
+    if (f < F) {
+      re = __ldg(reinterpret_cast<const float4*>(row));
+      im = __ldg(reinterpret_cast<const float4*>(row + F));
+    }
+  } else if constexpr (DT == MACH_IQ_C64) {
+    const float2* row = static_cast<const float2*>(src) + n * F + f;
+    if constexpr (VEC >= 2) {
+      if (f < F) {
+        const float4 a = __ldg(reinterpret_cast<const float4*>(row));
+        re.x = a.x; im.x = a.y; re.y = a.z; im.y = a.w;
+      }
+      if (f + 2 < F) {
+        const float4 b = __ldg(reinterpret_cast<const float4*>(row + 2));
+        re.z = b.x; im.z = b.y; re.w = b.z; im.w = b.w;
+      }
+    } else {
+      float2 a[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) a[e] = f + e < F ? __ldg(row + e) : make_float2(0.f, 0.f);
+      re = make_float4(a[0].x, a[1].x, a[2].x, a[3].x);
+      im = make_float4(a[0].y, a[1].y, a[2].y, a[3].y);
+    }
+  } else {
+    uint32_t h[4] = {0u, 0u, 0u, 0u};
+    const uint32_t* row = static_cast<const uint32_t*>(src) + n * F + f;
+    if constexpr (VEC == 4) {
+      if (f < F) {
+        const uint4 a = __ldg(reinterpret_cast<const uint4*>(row));
+        h[0] = a.x; h[1] = a.y; h[2] = a.z; h[3] = a.w;
+      }
+    } else if constexpr (VEC == 2) {
+#pragma unroll
+      for (int e = 0; e < 4; e += 2)
+        if (f + e < F) {
+          const uint2 a = __ldg(reinterpret_cast<const uint2*>(row + e));
+          h[e] = a.x; h[e + 1] = a.y;
+        }
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (f + e < F) h[e] = __ldg(row + e);
+    }
+    float2 a[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      if constexpr (DT == MACH_IQ_F16X2) a[e] = __half22float2(*reinterpret_cast<const __half2*>(&h[e]));
+      else a[e] = make_float2(__uint_as_float(h[e] << 16), __uint_as_float(h[e] & 0xffff0000u));
+    }
+    re = make_float4(a[0].x, a[1].x, a[2].x, a[3].x);
+    im = make_float4(a[0].y, a[1].y, a[2].y, a[3].y);
+  }
+}
+
+constexpr int kRepackItems = 4;   // items in flight per thread
+
+template <int DT, int VEC>
+__global__ void __launch_bounds__(256) k_iq_repack(const void* __restrict__ src, float* __restrict__ dst, int64_t N,
+                                                   int F, int full, int tail, int rows_per_block) {
+  const int quads = (32 * full + tail) / 4;
+  const int64_t n0 = static_cast<int64_t>(blockIdx.x) * rows_per_block;
+  const int items = static_cast<int>(min(static_cast<int64_t>(rows_per_block), N - n0)) * quads;
+  for (int base = threadIdx.x; base < items; base += 256 * kRepackItems) {
+    float4 re[kRepackItems], im[kRepackItems];
+#pragma unroll
+    for (int k = 0; k < kRepackItems; ++k) {
+      const int i = base + 256 * k;
+      re[k] = im[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (i < items) load_quad<DT, VEC>(src, n0 + i / quads, 4 * (i % quads), F, re[k], im[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < kRepackItems; ++k) {
+      const int i = base + 256 * k;
+      if (i >= items) break;
+      const int64_t n = n0 + i / quads;
+      const int f = 4 * (i % quads);
+      const int ft = f < 32 * full ? 32 : tail;              // frames of the item's tile
+      float* row = dst + (f < 32 * full ? (f / 32) * N * 64 : full * N * 64) + n * (2 * ft);
+      const int at = f < 32 * full ? f % 32 : f - 32 * full;
+      *reinterpret_cast<float4*>(row + at) = re[k];
+      *reinterpret_cast<float4*>(row + ft + at) = im[k];
+    }
+  }
+}
+
+cudaError_t launch_iq_repack(const void* src, int src_dtype, float* dst, int64_t N, int F, cudaStream_t s) {
+  const FrameSplit fs = split_frames(F);
+  const int quads = fs.padded() / 4;
+  const int rows = std::max(1, 256 * kRepackItems * 2 / quads);
+  const unsigned grid = static_cast<unsigned>((N + rows - 1) / rows);
+  const int vec = F % 4 == 0 ? 4 : (F % 2 == 0 ? 2 : 1);
+  auto go = [&](auto* kernel) {
+    kernel<<<grid, 256, 0, s>>>(src, dst, N, F, fs.full, fs.tail, rows);
+    return cudaGetLastError();
+  };
+  switch (src_dtype) {
+    case MACH_IQ_C64: return vec >= 2 ? go(k_iq_repack<MACH_IQ_C64, 2>) : go(k_iq_repack<MACH_IQ_C64, 1>);
+    case MACH_IQ_C64_SPLIT: return go(k_iq_repack<MACH_IQ_C64_SPLIT, 4>);
+    case MACH_IQ_F16X2:
+      return vec == 4 ? go(k_iq_repack<MACH_IQ_F16X2, 4>)
+                      : vec == 2 ? go(k_iq_repack<MACH_IQ_F16X2, 2>) : go(k_iq_repack<MACH_IQ_F16X2, 1>);
+    case MACH_IQ_BF16X2:
+      return vec == 4 ? go(k_iq_repack<MACH_IQ_BF16X2, 4>)
+                      : vec == 2 ? go(k_iq_repack<MACH_IQ_BF16X2, 2>) : go(k_iq_repack<MACH_IQ_BF16X2, 1>);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
 cudaError_t launch_iq_convert(const float2* src, int src_order, void* dst, int dst_dtype, int64_t T, int64_t C,
                               int64_t S, int64_t F, cudaStream_t s) {
   const int64_t N = T * C * S;

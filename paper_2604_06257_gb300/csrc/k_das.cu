@@ -279,6 +279,9 @@ const VariantShape kShapes[] = {
     {"staged_c64p_x64_v4_t8x8",    4, 16,   8,   64,  kWarps, false, true,  8, 8, 3, 16, true, 8, 8},
     {"staged_c64p_x16_f4v2w7_t8x14", 4, 4, 16,   16,  7,      false, true,  8, 8, 3, 28, true, 8, 14},
     {"staged_c64p_x8_f4v1w7_t8x14", 4,  2,  16,    8,  7,      false, true,  8, 8, 3, 28, true, 8, 14},
+    {"staged_c64p_x16_f8v1w7",     8,  2,  16,   16,  7,      false, true,  8, 8, 3, 28, true},
+    {"staged_c64p_x16_f8v1w4",     8,  2,  16,   16,  4,      false, true,  8, 8, 3, 16, true, 8, 8},
+    {"staged_c64p_x8_f8v1w4",      8,  1,  32,    8,  4,      false, true,  8, 8, 3, 32, true, 8, 16},
 };
 static_assert(sizeof(kShapes) / sizeof(kShapes[0]) == V_COUNT, "one shape row per variant");
 
@@ -322,12 +325,14 @@ cudaError_t launch_das(const DasParams& p, Variant v, cudaStream_t s) {
     default: return cudaErrorInvalidValue;
   }
   if (e != cudaSuccess) return e;
-  if (p.frame_tiles > 1 && p.pd) {
-    const int64_t blocks = (p.V + 255) / 256;
-    k_pd_reduce<<<static_cast<unsigned>(blocks), 256, 0, s>>>(p.pd_part, p.pd, p.V, p.frame_tiles);
-    e = cudaGetLastError();
-  }
+  if (p.frame_tiles > 1 && p.pd) e = launch_pd_reduce(p.pd_part, p.pd, p.V, p.frame_tiles, s);
   return e;
+}
+
+cudaError_t launch_pd_reduce(const float* part, float* pd, int64_t V, int tiles, cudaStream_t s) {
+  const int64_t blocks = (V + 255) / 256;
+  k_pd_reduce<<<static_cast<unsigned>(blocks), 256, 0, s>>>(part, pd, V, tiles);
+  return cudaGetLastError();
 }
 
 }  // namespace mach

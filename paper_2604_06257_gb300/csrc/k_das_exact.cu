@@ -89,9 +89,21 @@ __device__ __forceinline__ void mac4(float2* acc, const float4 cw, const float4 
 // lane group g starts at frame 4 (jl + FL (c ^ swz)), swz = g & 1 when FL = 4 and a lane
 // holds two chunks: the two lane groups of a quarter warp then read opposite halves of
 // their rows first, which keeps every 128-bit load free of bank conflicts.
+// Rows of 8 and 16 frames leave several lane groups on the same banks (their real parts
+// span 32 or 64 bytes), so every other group reads the imaginary parts first: it keeps its
+// sums with real and imaginary parts exchanged and gets its weights with the imaginary
+// parts negated (half_swap), which is the same FMA sequence.  With 8 frames per lane in
+// rows of 16 the chunks alternate over pairs of groups, so a quarter warp's four groups read
+// four different 32-byte pieces.
+// Measured (256 x 256 px, 128 elements | 64^3 voxels, 1024 elements, 3 transmits): 16 frames,
+// 4 x 2 per lane 101 -> 93 us | 4562 -> 4163 us; at 8 frames per lane 81 | 3840 us.
 template <int FL, int FPL>
 __device__ __forceinline__ int chunk_swizzle(int g) {
-  return (FL == 4 && FPL == 8) ? (g & 1) : 0;
+  return FPL == 8 ? (FL == 4 ? (g & 1) : FL <= 2 ? ((g >> 1) & 1) : 0) : 0;
+}
+template <int FT>
+__device__ __forceinline__ int half_swap(int g) {
+  return FT <= 16 ? (g & 1) : 0;
 }
 
 // Accumulators of one lane: VPG voxel slots x FPL frames, as packed pairs.
@@ -100,17 +112,25 @@ struct Acc {
   float2 a[VPG][FPL];
 };
 
+// IQ of the block's frame tile (PART: one of several in p.iq, see k_das_exact).
+template <bool PART>
+__device__ __forceinline__ const unsigned char* tile_iq(const DasParams& p) {
+  const unsigned char* iq = static_cast<const unsigned char*>(p.iq);
+  if constexpr (PART) iq += blockIdx.y * p.iq_tile_bytes;
+  return iq;
+}
+
 // The terms of one pair when some kept term falls outside the staged window (not
 // expected: the windows carry a margin): such terms read their taps from global memory.
 // Out of line, with the accumulators passed and returned by value, so that neither its
 // registers nor an address of the accumulators burden the hot loop.
-template <int FT, int FPL, int VPG, int G>
+template <int FT, int FPL, int VPG, int G, bool PART>
 __device__ __noinline__ Acc<VPG, FPL> outside_pair(const DasParams& p, Acc<VPG, FPL> acc, const SlotMeta m,
                                                    const unsigned char* wsrc, uint32_t cw_at, uint32_t of_at, int jl,
-                                                   int swz) {
+                                                   int order) {
   constexpr int RB = FT * 8, IMO = FT * 4, FL = FT / FPL;
-  const unsigned char* gsrc =
-      static_cast<const unsigned char*>(p.iq) + ((static_cast<size_t>(m.t) * p.C + m.c) * p.S + m.lo) * RB + jl * 16;
+  const int swz = FT <= 16 ? order & 1 : order, hs = FT <= 16 ? order >> 1 : 0;   // chunk and half orders
+  const unsigned char* gsrc = tile_iq<PART>(p) + ((static_cast<size_t>(m.t) * p.C + m.c) * p.S + m.lo) * RB + jl * 16;
 #pragma unroll
   for (int k = 0; k < VPG; ++k) {
     const float4 cw = lds128(cw_at + k * G * 16);
@@ -119,9 +139,10 @@ __device__ __noinline__ Acc<VPG, FPL> outside_pair(const DasParams& p, Acc<VPG, 
     const unsigned char* src = (rrow >= 0 && rrow + 1 < m.rows ? wsrc : gsrc) + off;
 #pragma unroll
     for (int c = 0; c < FPL / 4; ++c) {
-      const unsigned char* x = src + (c ^ swz) * FL * 16;
-      mac4(&acc.a[k][4 * c], cw, *reinterpret_cast<const float4*>(x), *reinterpret_cast<const float4*>(x + IMO),
-           *reinterpret_cast<const float4*>(x + RB), *reinterpret_cast<const float4*>(x + RB + IMO));
+      const unsigned char* x = src + (c ^ swz) * FL * 16 + hs * IMO;
+      const unsigned char* z = src + (c ^ swz) * FL * 16 + (1 - hs) * IMO;
+      mac4(&acc.a[k][4 * c], cw, *reinterpret_cast<const float4*>(x), *reinterpret_cast<const float4*>(z),
+           *reinterpret_cast<const float4*>(x + RB), *reinterpret_cast<const float4*>(z + RB));
     }
   }
   return acc;
@@ -134,7 +155,12 @@ __device__ __noinline__ Acc<VPG, FPL> outside_pair(const DasParams& p, Acc<VPG, 
 // releases each ring slot right after its last read instead of at the end of the round.
 constexpr int kSleep = 1, kEarly = 2;
 
-template <int FT, int FPL, int VPG, int NWC, int NBUF, int MAXR, int FLAGS>
+//
+// PART: the launch covers frames p.f_first ... of an ensemble of p.f_total frames that the
+// frame tiles need not fill: blockIdx.y is the frame tile, its rows (zero beyond the last
+// frame) start p.iq_tile_bytes after the previous tile's, frames past the last one are not
+// written, and Power Doppler leaves as one partial sum per tile when there are several.
+template <int FT, int FPL, int VPG, int NWC, int NBUF, int MAXR, int FLAGS, bool PART = false>
 __global__ void __launch_bounds__((NWC + 1) * 32) __maxnreg__(MAXR) k_das_exact(const DasParams p) {
   constexpr int FL = FT / FPL;
   constexpr int G = 32 / FL;
@@ -170,7 +196,7 @@ __global__ void __launch_bounds__((NWC + 1) * 32) __maxnreg__(MAXR) k_das_exact(
 
   if (warp == NWC) {   // producer
     int r = 0;
-    const bool ok = produce_windows<NBUF>(p, tile, lane, smem, L.slot_bytes, 8, meta, full, empty, r);
+    const bool ok = produce_windows<NBUF>(p, tile_iq<PART>(p), tile, lane, smem, L.slot_bytes, 8, meta, full, empty, r);
     if (lane == 0) finish_producer<NBUF, PB>(p, ok, r, meta, full, empty);
     return;
   }
@@ -185,6 +211,8 @@ __global__ void __launch_bounds__((NWC + 1) * 32) __maxnreg__(MAXR) k_das_exact(
   const int sub = lane / WV;
   const int q = lane % WV;
   const int swz = chunk_swizzle<FL, FPL>(g);
+  const int hs = half_swap<FT>(g);
+  const float im_sign = half_swap<FT>(q / VPG) ? -1.0f : 1.0f;   // of the group that reads this lane's terms
   float* txc = txc_all + warp * (p.T * 32);
   const int64_t v_term = tile_voxel_blocked(p, tile, warp * WV + q);
   const float4 vpos = v_term >= 0 ? p.vox[v_term] : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -193,7 +221,8 @@ __global__ void __launch_bounds__((NWC + 1) * 32) __maxnreg__(MAXR) k_das_exact(
   const uint32_t coef_w = s0 + static_cast<uint32_t>(L.coef_off()) + warp * 32 * 16;
   const uint32_t offs_w = s0 + static_cast<uint32_t>(L.offs_off()) + warp * 32 * 4;
   const uint32_t slot_bytes = static_cast<uint32_t>(L.slot_bytes);
-  const uint32_t lane_tap = s0 + jl * 16 + swz * FL * 16;   // chunk 0; chunk 1 at +/- FL * 16
+  const uint32_t lane_tap = s0 + jl * 16 + swz * FL * 16 + hs * IMO;   // chunk 0; chunk 1 at +/- FL * 16
+  const uint32_t im_at = hs ? -IMO : IMO;                              // the other parts, from there
   if (tx_cached) {
     for (int t = 0; t < p.T; ++t) txc[t * 32 + lane] = v_term >= 0 ? p.tx[static_cast<size_t>(t) * p.V + v_term] : 0.f;
   }
@@ -236,7 +265,12 @@ __global__ void __launch_bounds__((NWC + 1) * 32) __maxnreg__(MAXR) k_das_exact(
     const bool active = i0 >= 0;
     const int row = active ? i0 - mm.lo : 0;
     const bool outside = active && (row < 0 || row + 1 >= mm.rows);
-    sts128(coef_w + store_at * 16, tap_weights(rec));
+    float4 tw = tap_weights(rec);
+    if constexpr (FT <= 16) {   // exact
+      tw.y *= im_sign;
+      tw.w *= im_sign;
+    }
+    sts128(coef_w + store_at * 16, tw);
     sts32(offs_w + store_at * 4, row * RB);
     const unsigned act = __ballot_sync(0xffffffffu, active);
     const unsigned outm = __ballot_sync(0xffffffffu, outside);
@@ -269,12 +303,17 @@ __global__ void __launch_bounds__((NWC + 1) * 32) __maxnreg__(MAXR) k_das_exact(
           for (int c = 0; c < FPL / 4; ++c) {
             // chunk c lies (c ^ swz - swz) FL * 16 bytes from chunk 0's lane address
             const uint32_t b = a + ((c ^ swz) - swz) * FL * 16;
-            mac4(&acc.a[k][4 * c], cw, lds128(b), lds128(b + IMO), lds128(b + RB), lds128(b + RB + IMO));
+            if constexpr (FT <= 16) {
+              const uint32_t z = b + im_at;
+              mac4(&acc.a[k][4 * c], cw, lds128(b), lds128(z), lds128(b + RB), lds128(z + RB));
+            } else {
+              mac4(&acc.a[k][4 * c], cw, lds128(b), lds128(b + IMO), lds128(b + RB), lds128(b + RB + IMO));
+            }
           }
         }
       } else {
-        acc = outside_pair<FT, FPL, VPG, G>(p, acc, meta[slot], smem + slot * slot_bytes + jl * 16, cw_at, of_at,
-                                            jl, swz);
+        acc = outside_pair<FT, FPL, VPG, G, PART>(p, acc, meta[slot], smem + slot * slot_bytes + jl * 16, cw_at, of_at,
+                                            jl, FT <= 16 ? swz | hs << 1 : swz);
       }
       if constexpr ((FLAGS & kEarly) != 0) {   // every lane has read the slot: release it
         __syncwarp();
@@ -293,6 +332,14 @@ __global__ void __launch_bounds__((NWC + 1) * 32) __maxnreg__(MAXR) k_das_exact(
   for (int k = 0; k < VPG; ++k) {
     const int64_t v = tile_voxel_blocked(p, tile, warp * WV + g * VPG + k);
     float pw = 0.f;
+    if (hs) {   // sums kept with real and imaginary parts exchanged
+#pragma unroll
+      for (int e = 0; e < FPL; e += 2) {
+        const float2 t = acc.a[k][e];
+        acc.a[k][e] = acc.a[k][e + 1];
+        acc.a[k][e + 1] = t;
+      }
+    }
 #pragma unroll
     for (int c = 0; c < FPL / 4; ++c) {
 #pragma unroll
@@ -301,7 +348,23 @@ __global__ void __launch_bounds__((NWC + 1) * 32) __maxnreg__(MAXR) k_das_exact(
         pw = fmaf(a.x, a.x, fmaf(a.y, a.y, pw));
       }
       if (v >= 0 && p.y) {
-        float2* dst = p.y + v * p.ystride + 4 * (jl + FL * (c ^ swz));
+        const int f0 = 4 * (jl + FL * (c ^ swz));
+        if constexpr (PART) {
+          const int f = p.f_first + static_cast<int>(blockIdx.y) * FT + f0;
+          float2* dst = p.y + v * p.ystride + f;
+#pragma unroll
+          for (int e = 0; e < 4; e += 2) {
+            const float2 a = acc_frame<C64Planar, 4>(&acc.a[k][4 * c], e), b = acc_frame<C64Planar, 4>(&acc.a[k][4 * c], e + 1);
+            if (p.ystride % 2 == 0) {   // even rows: pairs of frames on the 16-byte grid
+              if (f + e < p.f_total) *reinterpret_cast<float4*>(dst + e) = make_float4(a.x, a.y, b.x, b.y);
+            } else {
+              if (f + e < p.f_total) dst[e] = a;
+              if (f + e + 1 < p.f_total) dst[e + 1] = b;
+            }
+          }
+          continue;
+        }
+        float2* dst = p.y + v * p.ystride + f0;
         const float2 a0 = acc_frame<C64Planar, 4>(&acc.a[k][4 * c], 0), a1 = acc_frame<C64Planar, 4>(&acc.a[k][4 * c], 1);
         const float2 a2 = acc_frame<C64Planar, 4>(&acc.a[k][4 * c], 2), a3 = acc_frame<C64Planar, 4>(&acc.a[k][4 * c], 3);
         *reinterpret_cast<float4*>(dst) = make_float4(a0.x, a0.y, a1.x, a1.y);
@@ -310,7 +373,12 @@ __global__ void __launch_bounds__((NWC + 1) * 32) __maxnreg__(MAXR) k_das_exact(
     }
 #pragma unroll
     for (int o = FL / 2; o > 0; o >>= 1) pw += __shfl_xor_sync(0xffffffffu, pw, o);
-    if (jl == 0 && v >= 0 && p.pd) p.pd[v] = pw;
+    if (jl == 0 && v >= 0 && p.pd) {
+      if (PART && p.frame_tiles > 1)
+        p.pd_part[static_cast<int64_t>(p.f_tile + static_cast<int>(blockIdx.y)) * p.V + v] = pw;
+      else
+        p.pd[v] = pw;
+    }
   }
 }
 
@@ -353,8 +421,34 @@ cudaError_t launch_das_exact(const DasParams& p, Variant v, cudaStream_t s) {
     case V_SX64_F8V2: return go_staged(k_das_exact<64, 8, 2, 8, 8, 72, 0>, 8, p, sm, s);
     case V_SX16_F4V2W7: case V_SX16_F4V2W7_T8X14:
       return go_staged(k_das_exact<16, 4, 2, 7, 8, 64, kEarly>, 7, p, sm, s);
+    case V_SX16_F8V1W7: return go_staged(k_das_exact<16, 8, 1, 7, 8, 64, kEarly>, 7, p, sm, s);
+    case V_SX16_F8V1W4: return go_staged(k_das_exact<16, 8, 1, 4, 8, 64, kEarly>, 4, p, sm, s);
+    case V_SX8_F8V1W4: return go_staged(k_das_exact<8, 8, 1, 4, 8, 64, kEarly>, 4, p, sm, s);
     case V_SX16_F4V1W7: return go_staged(k_das_exact<16, 4, 1, 7, 8, 64, kEarly>, 7, p, sm, s);
     case V_SX8_F4V1W7: case V_SX8_F4V1W7_T8X14: return go_staged(k_das_exact<8, 4, 1, 7, 8, 64, kEarly>, 7, p, sm, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+// The kernels of a repacked ensemble (see mach_internal.h): the exact-frame shapes above, one
+// launch per run of equal frame tiles.
+cudaError_t launch_das_parts(const DasParams& p, Variant v, int tiles, cudaStream_t s) {
+  DasParams q = p;
+  const size_t sm = exact_smem_bytes(v, p.rows_cap, p.T);
+  auto go = [&](auto* kernel, int nwc) -> cudaError_t {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sm));
+    if (e != cudaSuccess) return e;
+    const int64_t blocks = static_cast<int64_t>(p.tiles_x) * p.tiles_y * p.tiles_z;
+    kernel<<<dim3(static_cast<unsigned>(blocks), static_cast<unsigned>(tiles)), (nwc + 1) * 32, sm, s>>>(q);
+    return cudaGetLastError();
+  };
+  switch (v) {
+    case V_SX32_F8V1W7T14E: case V_SX32_F8V1W7_T8X7E: return go(k_das_exact<32, 8, 1, 7, 8, 64, kEarly, true>, 7);
+    case V_SX16_F8V1W7: return go(k_das_exact<16, 8, 1, 7, 8, 64, kEarly, true>, 7);
+    case V_SX16_F8V1W4: return go(k_das_exact<16, 8, 1, 4, 8, 64, kEarly, true>, 4);
+    case V_SX16_F4V1W7: return go(k_das_exact<16, 4, 1, 7, 8, 64, kEarly, true>, 7);
+    case V_SX8_F8V1W4: return go(k_das_exact<8, 8, 1, 4, 8, 64, kEarly, true>, 4);
+    case V_SX8_F4V1W7: return go(k_das_exact<8, 4, 1, 7, 8, 64, kEarly, true>, 7);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -76,6 +76,9 @@ enum Variant : int32_t {
   V_SX64_C64P_T8X8,     // as V_SX64_C64P with one-plane 8 x 8 x 1 tiles on 3D grids
   V_SX16_F4V2W7_T8X14,  // as V_SX16_F4V2W7 with one-plane 8 x 14 x 1 tiles on 3D grids
   V_SX8_F4V1W7_T8X14,   // as V_SX8_F4V1W7 with one-plane 8 x 14 x 1 tiles on 3D grids
+  V_SX16_F8V1W7,        // F = 16 exactly: 8 frames x 1 voxel per lane, 7 consumer warps
+  V_SX16_F8V1W4,        // as V_SX16_F8V1W7 with 4 consumer warps: 16 x 4 tiles, 8 x 8 x 1 on 3D grids
+  V_SX8_F8V1W4,         // F = 8 exactly: 8 frames x 1 voxel per lane, 4 consumer warps, 8 x 16 x 1 tiles on 3D grids
   V_COUNT
 };
 
@@ -137,7 +140,31 @@ struct DasParams {
   const int64_t* tile_pairs;  // [tiles + 1] index of each tile's first pair (pairs in copy order)
   const int4* pair_desc;      // [pairs] (transmit, element, first row, rows) of each copied window
   const float4* term_rec;     // [pairs][voxel slots of a block] term records, in consumer order
+  // repacked ensembles only (F is then the frame tile, frame_tiles the tiles of all launches)
+  int f_first, f_total;       // first frame of the launch, frames of the ensemble
+  int f_tile;                 // frame tiles of the launches before this one
+  size_t iq_tile_bytes;       // repacked bytes of one frame tile
 };
+
+// Repacked ensembles.  The exact-frame kernels read split complex64 rows of 8, 16 or 32
+// frames; any other ensemble (complex64, 16-bit pairs, other frame counts) is rewritten into
+// such rows first: consecutive frames in tiles of 32, the rest in one tile of 8, 16 or 32,
+// zero beyond the last frame.  Every tile is a full [T][C][S] array of its own.
+struct FrameSplit {
+  int full;          // tiles of 32 frames
+  int tail;          // frames of the last tile: 8 or 16 (0: none)
+  int tiles() const { return full + (tail ? 1 : 0); }
+  int padded() const { return 32 * full + tail; }
+};
+inline FrameSplit split_frames(int F) {
+  const int rest = F % 32;
+  FrameSplit f{F / 32, rest == 0 ? 0 : rest <= 8 ? 8 : 16};
+  if (rest > 16) {
+    ++f.full;
+    f.tail = 0;
+  }
+  return f;
+}
 
 // Tables built once per plan (kernel K1).
 struct TableParams {
@@ -167,6 +194,11 @@ size_t staged_smem_bytes(Variant v, int rows_cap, int F, int T, bool table);
 cudaError_t launch_das_staged(const DasParams& p, Variant v, cudaStream_t s);
 // Staged variants whose frame count is a compile-time constant (k_das_exact.cu).
 size_t exact_smem_bytes(Variant v, int rows_cap, int T);
+// Rows of N = T C S samples in any storage type into the tiles of split_frames(F) at dst.
+cudaError_t launch_iq_repack(const void* src, int src_dtype, float* dst, int64_t N, int F, cudaStream_t s);
+// Exact-frame kernel over `tiles` repacked frame tiles of variant_shape(v).frame_tile frames.
+cudaError_t launch_das_parts(const DasParams& p, Variant v, int tiles, cudaStream_t s);
+cudaError_t launch_pd_reduce(const float* part, float* pd, int64_t V, int tiles, cudaStream_t s);
 cudaError_t launch_das_exact(const DasParams& p, Variant v, cudaStream_t s);
 // Plan-time term table (k_das_table.cu): which staged variants have a table form, the
 // per-(tile, element) windows of every transmit (rows 0 = pair not used) and their

@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <cstdio>
 #include <cstring>
 #include <new>
 #include <vector>
@@ -34,6 +35,21 @@ struct mach_plan_s {
   int4* d_pair_desc = nullptr;
   float4* d_term_rec = nullptr;
   int64_t table_bytes = 0;
+  // repacked route (see repack_plan): the exact-frame launches over repacked frame tiles, and
+  // the pool that each run takes its workspace from
+  struct Part {
+    Variant v = V_COUNT;
+    int tiles = 0;              // frame tiles of the launch
+    DasParams base{};
+    size_t at = 0;              // byte offset of its first tile in the workspace
+    float4* d_tbox = nullptr;
+    float2* d_txr = nullptr;
+  };
+  Part parts[2];
+  int n_parts = 0;
+  size_t ws_bytes = 0;          // workspace of one run: repacked IQ, partial Power Doppler sums
+  size_t pd_at = 0;
+  cudaMemPool_t pool = nullptr;
 };
 
 namespace {
@@ -177,6 +193,7 @@ Variant unstaged(Variant v) {
     case V_SX64_C64P_T16: case V_SX64_C64P_T16E: case V_SX64_C64P_T8X8:
       return V_F64_C64P;
     case V_SX16_F4V2W7: case V_SX16_F4V1W7: case V_SX8_F4V1W7: case V_SX16_F4V2W7_T8X14: case V_SX8_F4V1W7_T8X14:
+    case V_SX16_F8V1W7: case V_SX16_F8V1W4: case V_SX8_F8V1W4:
       return V_F32_C64P;
     case V_ST64_B16_V4: return V_F64_B16;
     default: return v;
@@ -221,6 +238,7 @@ Variant generic_staged(Variant v) {
     case V_SX64_C64P_T16E: case V_SX64_C64P_T8X8:
       return V_ST64_C64P_V4;
     case V_SX16_F4V2W7: case V_SX16_F4V1W7: case V_SX8_F4V1W7: case V_SX16_F4V2W7_T8X14: case V_SX8_F4V1W7_T8X14:
+    case V_SX16_F8V1W7:
       return V_F32_C64P;
     default: return v;
   }
@@ -268,6 +286,11 @@ void release(mach_plan_s* p) {
   cudaFree(p->d_tile_pairs);
   cudaFree(p->d_pair_desc);
   cudaFree(p->d_term_rec);
+  for (auto& q : p->parts) {
+    cudaFree(q.d_tbox);
+    cudaFree(q.d_txr);
+  }
+  if (p->pool) cudaMemPoolDestroy(p->pool);
   delete p;
 }
 
@@ -410,6 +433,112 @@ static mach_status build_term_table(mach_plan_s* p, DasParams& b, cudaStream_t s
   b.term_rec = p->d_term_rec;
   p->table_bytes = static_cast<int64_t>(bytes);
   p->table = true;
+  return done(MACH_OK);
+}
+
+// Repacked route: ensembles that no exact-frame kernel reads directly are rewritten into
+// split complex64 rows of whole frame tiles on every run (k_iq_repack) and beamformed by the
+// exact-frame kernels.
+// What it buys (251 x 251 px, 128 elements, 2048 samples, V / S = 31, cold L2; direct kernel
+// -> repacking and exact-frame kernels, us): complex64 5 frames 304 -> 71, 8: 214 -> 71,
+// 16: 214 -> 86, 25: 314 -> 122, 32: 154 -> 123, 40: 273 -> 192, 64: 378 -> 234,
+// 200: 1193 -> 731; float16 25: 322 -> 124, 32: 162 -> 125, 64: 257 -> 235.  The odd counts
+// gain most: the direct kernels read them one frame at a time.
+// The repacking costs one pass over the IQ whatever the grid, the gain grows with the voxels
+// that read each sample, V / S; hence the bounds below.  A workspace above a sixteenth of
+// the device's memory, a capturing stream, or a failed workspace allocation takes the direct
+// kernel.
+static mach_status repack_plan(mach_plan_s* p, const DasParams& b, bool list, cudaStream_t s,
+                               size_t total_mem) {
+  const VariantShape& direct = variant_shape(p->variant);
+  if (direct.exact_frames || direct.channel_lanes) return MACH_OK;
+  const int64_t N = static_cast<int64_t>(b.T) * b.C * b.S;
+  if (b.V < static_cast<int64_t>(direct.staged ? 16 : 6) * b.S || N > (int64_t{1} << 36)) return MACH_OK;
+  const FrameSplit fs = split_frames(b.F);
+  const size_t iq_bytes = static_cast<size_t>(N) * 8 * fs.padded();
+  const size_t pd_bytes = fs.tiles() > 1 ? sizeof(float) * static_cast<size_t>(b.V) * fs.tiles() : 0;
+  if (iq_bytes + pd_bytes > total_mem / 16) return MACH_OK;
+  if (fs.full > 65535) return MACH_OK;   // grid y limit
+  const bool grid3d = !list && b.ny > 1;
+  struct Want { Variant v; int tiles; } want[2];
+  int n = 0;
+  if (fs.full) want[n++] = {grid3d ? V_SX32_F8V1W7_T8X7E : V_SX32_F8V1W7T14E, fs.full};
+  // Tails, time of the exact-frame kernel alone (256 x 256 px, 128 elements, 1 transmit |
+  // 201 x 233 px, 192 elements, 3 transmits | 64^3 voxels, 1024 elements, 3 transmits):
+  //   16 frames: 8 per lane, 7 warps 81 | 144 | 3840 us, 4 warps 83 | 130 | 3621 us;
+  //              4 per lane, 7 warps 91 | 124 | 5345 us
+  //    8 frames: 4 per lane, 7 warps 64 | 115 | 2947 us; 8 per lane, 4 warps 91 | 138 | 2672 us
+  if (fs.tail == 8) want[n++] = {grid3d ? V_SX8_F8V1W4 : V_SX8_F4V1W7, 1};
+  if (fs.tail == 16) want[n++] = {grid3d ? V_SX16_F8V1W4 : b.T == 1 ? V_SX16_F8V1W7 : V_SX16_F4V1W7, 1};
+  int* d_stats = nullptr;
+  int64_t scratch = 0, bytes = 0;
+  // every way out but the last one leaves the plan on its direct kernel
+  auto done = [&](mach_status e) {
+    cudaFree(d_stats);
+    if (p->n_parts == 0)
+      for (auto& q : p->parts) {
+        cudaFree(q.d_tbox);
+        cudaFree(q.d_txr);
+        q.d_tbox = nullptr;
+        q.d_txr = nullptr;
+      }
+    return e;
+  };
+  if (dev_alloc(reinterpret_cast<void**>(&d_stats), 2 * sizeof(int), &scratch) != MACH_OK) return done(MACH_OK);
+  for (int k = 0; k < n; ++k) {
+    mach_plan_s::Part& q = p->parts[k];
+    const VariantShape& sh = variant_shape(want[k].v);
+    DasParams t = b;
+    if (configure_tiles(t, want[k].v, list, b.V, sh.frame_tile) != MACH_OK) return done(MACH_OK);
+    const int64_t tiles = static_cast<int64_t>(t.tiles_x) * t.tiles_y * t.tiles_z;
+    if (dev_alloc(reinterpret_cast<void**>(&q.d_tbox), sizeof(float4) * 2 * tiles, &bytes) != MACH_OK ||
+        dev_alloc(reinterpret_cast<void**>(&q.d_txr), sizeof(float2) * b.T * tiles, &bytes) != MACH_OK)
+      return done(MACH_OK);
+    t.F = sh.frame_tile;
+    t.frame_tiles = fs.tiles();
+    t.tbox = q.d_tbox;
+    t.txr = q.d_txr;
+    int stats[2] = {0, 0};
+    if (launch_tile_bounds(t, q.d_tbox, q.d_txr, d_stats, s) != cudaSuccess ||
+        cudaMemcpyAsync(stats, d_stats, sizeof(stats), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        cudaStreamSynchronize(s) != cudaSuccess)
+      return done(MACH_ERR_CUDA);
+    t.rows_cap = std::max(2, stats[0]);
+    if (exact_smem_bytes(want[k].v, t.rows_cap, b.T) > kStagedSmemCap) return done(MACH_OK);
+    t.f_first = k == 0 ? 0 : 32 * fs.full;
+    t.f_total = b.F;
+    t.f_tile = k == 0 ? 0 : fs.full;
+    t.iq_tile_bytes = static_cast<size_t>(N) * 8 * sh.frame_tile;
+    q.v = want[k].v;
+    q.tiles = want[k].tiles;
+    q.base = t;
+    q.at = k == 0 ? 0 : static_cast<size_t>(N) * 8 * 32 * fs.full;
+  }
+  // a pool of the plan's own: each run takes its workspace in stream order, so that calls on
+  // several streams never share one; one workspace is kept between runs, the others go back
+  cudaMemPoolProps props{};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = p->device;
+  if (cudaMemPoolCreate(&p->pool, &props) != cudaSuccess) {
+    cudaGetLastError();
+    p->pool = nullptr;
+    return done(MACH_OK);
+  }
+  p->pd_at = iq_bytes;
+  p->ws_bytes = iq_bytes + pd_bytes;
+  uint64_t keep = (p->ws_bytes >> 25 << 25) + (64u << 20);   // the pool maps memory in blocks
+  if (cudaMemPoolSetAttribute(p->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) cudaGetLastError();
+  void* first = nullptr;   // mapped now rather than in the first run
+  if (cudaMallocFromPoolAsync(&first, p->ws_bytes, p->pool, s) != cudaSuccess ||
+      cudaFreeAsync(first, s) != cudaSuccess) {
+    cudaGetLastError();
+    cudaMemPoolDestroy(p->pool);
+    p->pool = nullptr;
+    return done(MACH_OK);
+  }
+  p->device_bytes += bytes;
+  p->n_parts = n;
   return done(MACH_OK);
 }
 
@@ -639,6 +768,7 @@ mach_status mach_das_plan(const mach_das_desc* d, void* stream, mach_plan* out) 
     if (!variant_shape(var).staged || !table_supported(var)) return fail(MACH_ERR_UNSUPPORTED);
     if ((st = build_term_table(p, b, s)) != MACH_OK) return fail(st);
   }
+  if (!forced && !d->term_table && (st = repack_plan(p, b, list, s, total_b)) != MACH_OK) return fail(st);
   if (cudaStreamSynchronize(s) != cudaSuccess) return fail(MACH_ERR_CUDA);
   cudaFree(d_raw);
   cudaFree(d_u);
@@ -657,12 +787,48 @@ mach_status mach_plan_destroy(mach_plan p) {
   return MACH_OK;
 }
 
+// One run over the repacked ensemble; false (nothing launched) when the stream is being
+// captured, where a run makes no allocation, or when there is no memory for the workspace.
+static bool run_repacked(mach_plan p, const void* iq, float* pd, void* y, cudaStream_t s, cudaError_t* err) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  if (cap != cudaStreamCaptureStatusNone) return false;
+  char* ws = nullptr;
+  if (cudaMallocFromPoolAsync(reinterpret_cast<void**>(&ws), p->ws_bytes, p->pool, s) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  const DasParams& b = p->base;
+  const int64_t N = static_cast<int64_t>(b.T) * b.C * b.S;
+  cudaError_t e = launch_iq_repack(iq, p->d.iq_dtype, reinterpret_cast<float*>(ws), N, b.F, s);
+  float* part = reinterpret_cast<float*>(ws + p->pd_at);
+  for (int k = 0; k < p->n_parts && e == cudaSuccess; ++k) {
+    DasParams q = p->parts[k].base;
+    q.iq = ws + p->parts[k].at;
+    q.y = static_cast<float2*>(y);
+    q.pd = pd;
+    q.pd_part = part;
+    e = launch_das_parts(q, p->parts[k].v, p->parts[k].tiles, s);
+  }
+  const int tiles = p->parts[0].base.frame_tiles;
+  if (e == cudaSuccess && pd && tiles > 1) e = launch_pd_reduce(part, pd, b.V, tiles, s);
+  const cudaError_t f = cudaFreeAsync(ws, s);
+  *err = e != cudaSuccess ? e : f;
+  return true;
+}
+
 static mach_status run(mach_plan p, const void* iq, float* pd, void* y, void* stream) {
   if (!p || !iq || (!pd && !y)) return MACH_ERR_INVALID_ARG;
   // vector loads and bulk copies need 16-byte aligned IQ; outputs are float2 / float4
   if ((reinterpret_cast<uintptr_t>(iq) & 15u) || (reinterpret_cast<uintptr_t>(y) & 15u) ||
       (reinterpret_cast<uintptr_t>(pd) & 3u))
     return MACH_ERR_INVALID_ARG;
+  cudaError_t re = cudaSuccess;
+  if (p->n_parts && run_repacked(p, iq, pd, y, static_cast<cudaStream_t>(stream), &re))
+    return re == cudaSuccess ? MACH_OK : MACH_ERR_CUDA;
   DasParams q = p->base;
   q.iq = iq;
   q.y = static_cast<float2*>(y);
@@ -715,6 +881,11 @@ mach_status mach_plan_get_info(mach_plan p, mach_plan_info* info) {
   std::memset(info, 0, sizeof(*info));
   const VariantShape& s = variant_shape(p->variant);
   std::strncpy(info->variant, s.name, sizeof(info->variant) - 1);
+  if (p->n_parts) {   // the frame tiles that runs repack the ensemble into
+    const size_t n = std::strlen(info->variant);
+    std::snprintf(info->variant + n, sizeof(info->variant) - n, p->n_parts == 2 ? "+x%d+x%d" : "+x%d",
+                  p->parts[0].base.F, p->parts[1].base.F);
+  }
   info->frames_per_lane = s.frames_per_lane;
   info->lanes_per_voxel = s.lanes_per_voxel;
   info->voxels_per_cta = s.voxels_per_warp * s.warps;

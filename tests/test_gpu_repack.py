@@ -1,0 +1,85 @@
+"""Ensembles that are rewritten into whole frame tiles before beamforming: every storage type,
+frame counts around the edges of the tiles (8, 16 and 32 frames and their sums), 2D and 3D,
+one and several transmits, against the FP64 oracle and the direct kernel."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import synth
+import paper_2604_06257_gb300 as m
+from metrics import nrmse_db
+
+pytestmark = pytest.mark.gpu
+
+CASES = [(F, dt) for F in (5, 8, 9, 16, 17, 25, 31, 32, 33, 40, 41, 49, 64, 65, 100)
+         for dt in ("c64", "f16x2", "bf16x2", "c64split")
+         if dt != "c64split" or (F % 4 == 0 and F not in (8, 16, 32, 64))]
+
+
+def dense(F, dt, ndim=2, T=1):
+    """Few samples and many voxels, so that repacking pays."""
+    name = "doppler2d" if ndim == 2 else "volume3d"
+    acq = synth.make_acquisition(name, "small")
+    dims = (53, 1, 67) if ndim == 2 else (17, 13, 19)
+    ang = np.zeros((T, 2))
+    ang[:, 0] = np.linspace(-0.1, 0.1, T) if T > 1 else 0.0
+    # a shallow grid under the middle of the array, so that 200 samples reach its floor
+    mid = len(acq.elem_pos) // 2
+    origin = (-dims[0] * 5e-5, 0.0 if ndim == 2 else -dims[1] * 5e-5, 1e-3)
+    return acq.replace(grid_dims=dims, grid_origin=origin, grid_step=(1e-4, 0.0 if ndim == 2 else 1e-4, 1e-5),
+                       elem_pos=acq.elem_pos[mid - 12:mid + 12], tx_angles=ang, n_samples=200, n_frames=F, iq_dtype=dt)
+
+
+def stored(acq, seed):
+    iq = synth.random_iq(acq.replace(iq_dtype="c64"), seed, device="cuda")
+    x = synth.iqmod.to_c64split(iq) if acq.iq_dtype == "c64split" else synth.iqmod.to_storage(iq, acq.iq_dtype)
+    ref = iq.cpu() if acq.iq_dtype in ("c64", "c64split") else synth.iqmod.from_storage(x.cpu())
+    return x, ref
+
+
+@pytest.mark.parametrize("F,dt", CASES)
+def test_repacked_frames_match_oracle(F, dt):
+    for ndim, T in ((2, 1), (2, 3), (3, 2)):
+        acq = dense(F, dt, ndim, T)
+        if acq.n_vox < 16 * acq.n_samples:
+            pytest.fail("grid too small for the repacked route")
+        x, ref = stored(acq, F + T)
+        with m.Plan(**m.plan_kwargs(acq)) as p:
+            assert "+x" in p.info()["variant"], p.info()
+            pd, y = p.power_doppler(x, want_y=True)
+            y_only = p.run(x)
+            pd_only, _ = p.power_doppler(x)
+            torch.cuda.synchronize()
+            assert p.device_status() == m.MACH_OK
+            # a captured run allocates nothing: it takes the direct kernel
+            g = torch.cuda.CUDAGraph()
+            yg = torch.zeros_like(y)
+            with torch.cuda.graph(g):
+                m.mach_das_run(p.handle, x, yg)
+            g.replay()
+            torch.cuda.synchronize()
+        assert torch.equal(y, y_only) and torch.equal(pd, pd_only)
+        idx = np.arange(0, acq.n_vox, 7)
+        y_ref, pd_ref = oracle.das(acq, ref, idx)
+        assert nrmse_db(y.cpu().numpy()[idx], y_ref) <= -100, (ndim, T)
+        assert nrmse_db(pd.cpu().numpy()[idx].astype(np.float64), pd_ref) <= -100, (ndim, T)
+        assert nrmse_db(yg.cpu().numpy(), y.cpu().numpy()) <= -110, (ndim, T)
+
+
+def test_repacked_runs_share_a_plan_across_streams():
+    """Concurrent calls on one plan take separate workspaces."""
+    acq = dense(25, "f16x2", 2, 3)
+    xs = [stored(acq, s)[0] for s in range(6)]
+    with m.Plan(**m.plan_kwargs(acq)) as p:
+        want = [p.run(x) for x in xs]
+        torch.cuda.synchronize()
+        streams = [torch.cuda.Stream() for _ in xs]
+        got = [torch.zeros_like(w) for w in want]
+        torch.cuda.synchronize()
+        for _ in range(4):
+            for s, x, y in zip(streams, xs, got):
+                m.mach_das_run(p.handle, x, y, stream=s)
+        torch.cuda.synchronize()
+    for a, b in zip(got, want):
+        assert torch.equal(a, b)
