@@ -272,7 +272,11 @@ typedef struct mach_batch_s *mach_batch;
 /* Plan a batch of n instances (each described as for mach_das_plan, all with the same
  * iq_dtype, not the split layout, n_frames <= 64): builds every instance's tables and one
  * work list of (instance, voxel tile) items, sorted by decreasing estimated cost, for
- * one persistent launch.  shapes: NULL or n entries.  Synchronises `stream`.
+ * one persistent launch.  shapes: NULL or n entries.  With NULL, instances of more than 4
+ * frames whose own plan would repack them (see Workspaces above) are repacked and beamformed
+ * by one exact-frame launch per tile shape instead; the batch owns their workspace (at most a
+ * sixteenth of the device memory in all, none if that cannot be had) and mach_batch_get_info
+ * still reports the lane mapping they would take otherwise.  Synchronises `stream`.
  * Errors: INVALID_ARG, UNSUPPORTED, OOM, CUDA. */
 mach_status mach_batch_plan(const mach_das_desc *descs, int32_t n, const mach_tile_shape *shapes,
                             void *stream, mach_batch *out);
@@ -283,9 +287,9 @@ mach_status mach_batch_plan(const mach_das_desc *descs, int32_t n, const mach_ti
 mach_status mach_batch_bind(mach_batch b, const void *const *iq_devs, void *const *y_devs,
                             float *const *pd_devs, void *stream);
 
-/* Beamform every instance of the batch in one launch on `stream` (stream-ordered; no
+/* Beamform every instance of the batch on `stream` (stream-ordered; no
  * host synchronisation, so it can be captured in a CUDA graph).  Runs on the same batch
- * must be ordered on one stream (they share the work counter). */
+ * must be ordered on one stream (they share the work counter and the workspace). */
 mach_status mach_batch_run(mach_batch b, void *stream);
 
 typedef struct {

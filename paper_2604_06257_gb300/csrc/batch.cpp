@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <cstdint>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <vector>
 
@@ -28,6 +29,23 @@ struct mach_batch_s {
   std::vector<void*> bounds;             // per staged instance: tile boxes and transmit-delay ranges
   int64_t points = 0;
   bool bound = false;
+  // repacked instances: what each needs before the shared launches, and the launches (one
+  // per exact-frame shape and kMultiMax entries)
+  struct Repacked {
+    int inst, dtype, F, tiles;
+    int64_t N, V;
+    size_t at;                           // its bytes in the workspace below
+    size_t pd_at;
+  };
+  struct Multi {
+    Variant v;
+    MultiArgs args;
+    int2* d_items;
+    int n_items;
+  };
+  std::vector<Repacked> repacked;
+  std::vector<std::unique_ptr<Multi>> multi;
+  char* ws = nullptr;
 };
 
 namespace {
@@ -36,6 +54,8 @@ void release(mach_batch_s* b) {
   if (!b) return;
   for (mach_plan p : b->plans) mach_plan_destroy(p);
   for (void* q : b->bounds) cudaFree(q);
+  for (auto& m : b->multi) cudaFree(m->d_items);
+  cudaFree(b->ws);
   cudaFree(b->d_insts);
   cudaFree(b->d_items);
   cudaFree(b->d_counter);
@@ -92,6 +112,60 @@ void staged_tile(int n, int nx, int ny, int nz, bool list, int tile[3]) {
   }
 }
 
+// The launches over the repacked instances' frame tiles: instances grouped by exact-frame
+// shape, each group's (frame tile, voxel tile) items longest first; the workspace for all of
+// them, which runs share in stream order as they do the work counter.
+mach_status plan_repacked(mach_batch_s* b, cudaStream_t s) {
+  struct Item { int entry, ftile; int64_t tile; double cost; };
+  struct Group { std::vector<Item> items; mach_batch_s::Multi* m = nullptr; };
+  std::vector<Group> groups;
+  for (const auto& q : b->repacked) {
+    const RepackPart* parts = nullptr;
+    size_t ws_i = 0, pd_i = 0;
+    const int np = plan_repack(b->plans[q.inst], &parts, &ws_i, &pd_i);
+    for (int k = 0; k < np; ++k) {
+      // 2D and 3D shapes of 32 frames are one kernel
+      const Variant v = parts[k].v == V_SX32_F8V1W7_T8X7E ? V_SX32_F8V1W7T14E : parts[k].v;
+      Group* g = nullptr;
+      for (auto& c : groups)
+        if (c.m->v == v && c.m->args.n < kMultiMax) g = &c;
+      if (!g) {
+        b->multi.emplace_back(new mach_batch_s::Multi{});
+        groups.emplace_back();
+        g = &groups.back();
+        g->m = b->multi.back().get();
+        g->m->v = v;
+      }
+      const int entry = g->m->args.n++;
+      g->m->args.inst[entry] = q.inst;
+      DasParams& p = g->m->args.p[entry];
+      p = parts[k].base;
+      p.iq = b->ws + q.at + parts[k].at;
+      p.pd_part = reinterpret_cast<float*>(b->ws + q.at + q.pd_at);
+      const int64_t tiles = static_cast<int64_t>(p.tiles_x) * p.tiles_y * p.tiles_z;
+      const double cost = static_cast<double>(p.C) * p.T * p.tile_x * p.tile_y * p.tile_z;
+      for (int64_t t = tiles - 1; t >= 0; --t)
+        for (int f = 0; f < parts[k].tiles; ++f) g->items.push_back({entry, f, t, cost});
+    }
+  }
+  for (auto& g : groups) {
+    if (g.items.size() > static_cast<size_t>(INT32_MAX)) return MACH_ERR_UNSUPPORTED;
+    std::stable_sort(g.items.begin(), g.items.end(), [](const Item& a, const Item& c) { return a.cost > c.cost; });
+    std::vector<int2> h(g.items.size());
+    for (size_t k = 0; k < h.size(); ++k)
+      h[k] = make_int2(g.items[k].entry | g.items[k].ftile << 16, static_cast<int>(g.items[k].tile));
+    g.m->n_items = static_cast<int>(h.size());
+    if (cudaMalloc(&g.m->d_items, sizeof(int2) * h.size()) != cudaSuccess) {
+      cudaGetLastError();
+      return MACH_ERR_OOM;
+    }
+    if (cudaMemcpyAsync(g.m->d_items, h.data(), sizeof(int2) * h.size(), cudaMemcpyHostToDevice, s) != cudaSuccess ||
+        cudaStreamSynchronize(s) != cudaSuccess)
+      return MACH_ERR_CUDA;
+  }
+  return MACH_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -137,13 +211,31 @@ mach_status mach_batch_plan(const mach_das_desc* descs, int32_t n, const mach_ti
   b->plans.assign(n, nullptr);
   b->host_insts.resize(n);
   b->shapes.resize(n);
+  size_t free_mem = 0, total_mem = 0, ws_total = 0;
+  if (cudaMemGetInfo(&free_mem, &total_mem) != cudaSuccess) {
+    cudaGetLastError();
+    release(b);
+    return MACH_ERR_CUDA;
+  }
   struct Item { int inst; int64_t tile; double cost; };
   std::vector<Item> items;
+  std::vector<char> is_repacked(n, 0);
   for (int i = 0; i < n; ++i) {
-    mach_status st = mach_das_plan(&descs[i], stream, &b->plans[i]);
+    mach_status st = make_batch_plan(&descs[i], stream, &b->plans[i]);
     if (st != MACH_OK) {
       release(b);
       return st;
+    }
+    // default shapes only: an instance that its plan would repack joins the launches over
+    // repacked tiles
+    const RepackPart* parts = nullptr;
+    size_t ws_i = 0, pd_i = 0;
+    if (!shapes && plan_repack(b->plans[i], &parts, &ws_i, &pd_i) && ws_total + ws_i <= total_mem / 16) {
+      is_repacked[i] = 1;
+      const DasParams& q = *plan_params(b->plans[i]);
+      b->repacked.push_back({i, dt, q.F, parts[0].base.frame_tiles, static_cast<int64_t>(q.T) * q.C * q.S, q.V,
+                             ws_total, pd_i});
+      ws_total += (ws_i + 255) / 256 * 256;
     }
     mach_tile_shape sh = shapes ? shapes[i] : default_shape(descs[i].n_frames);
     const DasParams base = *plan_params(b->plans[i]);
@@ -242,6 +334,20 @@ mach_status mach_batch_plan(const mach_das_desc* descs, int32_t n, const mach_ti
     for (int64_t t = tiles - 1; t >= 0; --t) items.push_back({i, t, cost});
     b->points += static_cast<int64_t>(p.V) * p.C * p.T * p.F;
   }
+  if (!b->repacked.empty()) {
+    if (cudaMalloc(&b->ws, ws_total) == cudaSuccess) {
+      if (const mach_status st = plan_repacked(b, s); st != MACH_OK) {
+        release(b);
+        return st;
+      }
+      items.erase(std::remove_if(items.begin(), items.end(), [&](const Item& t) { return is_repacked[t.inst]; }),
+                  items.end());
+    } else {   // no memory for the workspace: every instance on its lane mapping
+      cudaGetLastError();
+      b->ws = nullptr;
+      b->repacked.clear();
+    }
+  }
   if (items.size() > static_cast<size_t>(INT32_MAX)) {
     release(b);
     return MACH_ERR_UNSUPPORTED;
@@ -251,14 +357,15 @@ mach_status mach_batch_plan(const mach_das_desc* descs, int32_t n, const mach_ti
   for (size_t k = 0; k < items.size(); ++k) hitems[k] = make_int2(items[k].inst, static_cast<int>(items[k].tile));
   b->n_items = static_cast<int>(items.size());
   if (cudaMalloc(&b->d_insts, sizeof(BatchInstance) * n) != cudaSuccess ||
-      cudaMalloc(&b->d_items, sizeof(int2) * hitems.size()) != cudaSuccess ||
+      cudaMalloc(&b->d_items, sizeof(int2) * std::max<size_t>(1, hitems.size())) != cudaSuccess ||
       cudaMalloc(&b->d_counter, 2 * sizeof(int)) != cudaSuccess) {
     cudaGetLastError();
     release(b);
     return MACH_ERR_OOM;
   }
-  if (cudaMemcpyAsync(b->d_items, hitems.data(), sizeof(int2) * hitems.size(), cudaMemcpyHostToDevice, s) !=
-          cudaSuccess ||
+  for (auto& m : b->multi) m->args.insts = b->d_insts;
+  if ((!hitems.empty() && cudaMemcpyAsync(b->d_items, hitems.data(), sizeof(int2) * hitems.size(),
+                                          cudaMemcpyHostToDevice, s) != cudaSuccess) ||
       cudaMemsetAsync(b->d_counter, 0, 2 * sizeof(int), s) != cudaSuccess ||
       cudaMemcpyAsync(b->d_insts, b->host_insts.data(), sizeof(BatchInstance) * n, cudaMemcpyHostToDevice, s) !=
           cudaSuccess ||
@@ -302,16 +409,33 @@ mach_status mach_batch_bind(mach_batch b, const void* const* iq_devs, void* cons
 
 mach_status mach_batch_run(mach_batch b, void* stream) {
   if (!b || !b->bound) return MACH_ERR_INVALID_ARG;
-  return launch_batch(b->iq_dtype, b->d_insts, b->d_items, b->n_items, b->d_counter, b->grid, b->slot_bytes,
-                      static_cast<cudaStream_t>(stream)) == cudaSuccess
-             ? MACH_OK
-             : MACH_ERR_CUDA;
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  cudaError_t e = cudaSuccess;
+  // the repacked tiles first: their launches hold the longest blocks
+  for (const auto& q : b->repacked) {
+    if (e != cudaSuccess) break;
+    e = launch_iq_repack(nullptr, &b->d_insts[q.inst].p.iq, q.dtype, reinterpret_cast<float*>(b->ws + q.at), q.N, q.F, s);
+  }
+  for (const auto& m : b->multi) {
+    if (e != cudaSuccess) break;
+    e = launch_das_multi(m->args, m->v, m->d_items, m->n_items, s);
+  }
+  for (const auto& q : b->repacked) {
+    if (e != cudaSuccess) break;
+    if (q.tiles > 1)
+      e = launch_pd_reduce(reinterpret_cast<const float*>(b->ws + q.at + q.pd_at), nullptr, &b->d_insts[q.inst].p.pd, q.V,
+                           q.tiles, s);
+  }
+  if (e == cudaSuccess && b->n_items)
+    e = launch_batch(b->iq_dtype, b->d_insts, b->d_items, b->n_items, b->d_counter, b->grid, b->slot_bytes, s);
+  return e == cudaSuccess ? MACH_OK : MACH_ERR_CUDA;
 }
 
 mach_status mach_batch_get_info(mach_batch b, mach_batch_info* info, mach_tile_shape* shapes_or_null) {
   if (!b || !info) return MACH_ERR_INVALID_ARG;
   info->instances = b->n;
   info->items = b->n_items;
+  for (const auto& m : b->multi) info->items += m->n_items;
   info->blocks = b->grid;
   info->blocks_per_sm = b->per_sm;
   info->points = b->points;

@@ -1,5 +1,7 @@
 // k_batch.cu -- ragged batches: many DAS instances in one persistent launch.
 //
+// This kernel takes the instances that are not repacked into whole frame tiles (F <= 4,
+// explicit shapes, grids of few voxels per sample); the others run in k_das_exact_multi.
 // A batch holds instances of different sizes (2D and 3D grids, element, transmit and
 // frame counts).  Their voxel tiles form one work list, sorted by decreasing estimated
 // cost; a persistent grid (as many blocks as fit on the GPU) pulls (instance, tile) items

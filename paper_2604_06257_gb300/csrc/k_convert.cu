@@ -253,9 +253,12 @@ __device__ __forceinline__ void load_quad(const void* src, int64_t n, int f, int
 constexpr int kRepackItems = 4;   // items in flight per thread
 
 template <int DT, int VEC>
-__global__ void __launch_bounds__(256) k_iq_repack(const void* __restrict__ src, float* __restrict__ dst, int64_t N,
-                                                   int F, int full, int tail, int rows_per_block) {
+__global__ void __launch_bounds__(256) k_iq_repack(const void* __restrict__ src,
+                                                   const void* const* __restrict__ src_slot,
+                                                   float* __restrict__ dst, int64_t N, int F, int full,
+                                                   int tail, int rows_per_block) {
   const int quads = (32 * full + tail) / 4;
+  if (src_slot) src = *src_slot;
   const int64_t n0 = static_cast<int64_t>(blockIdx.x) * rows_per_block;
   const int items = static_cast<int>(min(static_cast<int64_t>(rows_per_block), N - n0)) * quads;
   for (int base = threadIdx.x; base < items; base += 256 * kRepackItems) {
@@ -281,14 +284,15 @@ __global__ void __launch_bounds__(256) k_iq_repack(const void* __restrict__ src,
   }
 }
 
-cudaError_t launch_iq_repack(const void* src, int src_dtype, float* dst, int64_t N, int F, cudaStream_t s) {
+cudaError_t launch_iq_repack(const void* src, const void* const* src_slot, int src_dtype, float* dst, int64_t N, int F,
+                             cudaStream_t s) {
   const FrameSplit fs = split_frames(F);
   const int quads = fs.padded() / 4;
   const int rows = std::max(1, 256 * kRepackItems * 2 / quads);
   const unsigned grid = static_cast<unsigned>((N + rows - 1) / rows);
   const int vec = F % 4 == 0 ? 4 : (F % 2 == 0 ? 2 : 1);
   auto go = [&](auto* kernel) {
-    kernel<<<grid, 256, 0, s>>>(src, dst, N, F, fs.full, fs.tail, rows);
+    kernel<<<grid, 256, 0, s>>>(src, src_slot, dst, N, F, fs.full, fs.tail, rows);
     return cudaGetLastError();
   };
   switch (src_dtype) {

@@ -204,9 +204,10 @@ __global__ void __launch_bounds__(NWARP * 32) k_das_channels(const DasParams p) 
 }
 
 __global__ void __launch_bounds__(256) k_pd_reduce(const float* __restrict__ part, float* __restrict__ pd,
-                                                   int64_t V, int tiles) {
+                                                   float* const* __restrict__ pd_slot, int64_t V, int tiles) {
   const int64_t v = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (v >= V) return;
+  if (pd_slot) pd = *pd_slot;
+  if (v >= V || !pd) return;
   float s = 0.f;
   for (int t = 0; t < tiles; ++t) s += part[static_cast<int64_t>(t) * V + v];
   pd[v] = s;
@@ -325,13 +326,14 @@ cudaError_t launch_das(const DasParams& p, Variant v, cudaStream_t s) {
     default: return cudaErrorInvalidValue;
   }
   if (e != cudaSuccess) return e;
-  if (p.frame_tiles > 1 && p.pd) e = launch_pd_reduce(p.pd_part, p.pd, p.V, p.frame_tiles, s);
+  if (p.frame_tiles > 1 && p.pd) e = launch_pd_reduce(p.pd_part, p.pd, nullptr, p.V, p.frame_tiles, s);
   return e;
 }
 
-cudaError_t launch_pd_reduce(const float* part, float* pd, int64_t V, int tiles, cudaStream_t s) {
+cudaError_t launch_pd_reduce(const float* part, float* pd, float* const* pd_slot, int64_t V, int tiles,
+                             cudaStream_t s) {
   const int64_t blocks = (V + 255) / 256;
-  k_pd_reduce<<<static_cast<unsigned>(blocks), 256, 0, s>>>(part, pd, V, tiles);
+  k_pd_reduce<<<static_cast<unsigned>(blocks), 256, 0, s>>>(part, pd, pd_slot, V, tiles);
   return cudaGetLastError();
 }
 

@@ -16,6 +16,8 @@
 //    16-byte weight record and a 4-byte offset and adds one integer per term;
 //  * all shared-memory traffic of the inner loop uses 32-bit shared addresses.
 #include <cuda_runtime.h>
+
+#include <algorithm>
 #include <cstdint>
 
 #include "das_staged.cuh"
@@ -112,11 +114,11 @@ struct Acc {
   float2 a[VPG][FPL];
 };
 
-// IQ of the block's frame tile (PART: one of several in p.iq, see k_das_exact).
+// IQ of the block's frame tile (PART: one of several in p.iq, see das_exact_block).
 template <bool PART>
-__device__ __forceinline__ const unsigned char* tile_iq(const DasParams& p) {
+__device__ __forceinline__ const unsigned char* tile_iq(const DasParams& p, unsigned ftile) {
   const unsigned char* iq = static_cast<const unsigned char*>(p.iq);
-  if constexpr (PART) iq += blockIdx.y * p.iq_tile_bytes;
+  if constexpr (PART) iq += ftile * p.iq_tile_bytes;
   return iq;
 }
 
@@ -127,10 +129,11 @@ __device__ __forceinline__ const unsigned char* tile_iq(const DasParams& p) {
 template <int FT, int FPL, int VPG, int G, bool PART>
 __device__ __noinline__ Acc<VPG, FPL> outside_pair(const DasParams& p, Acc<VPG, FPL> acc, const SlotMeta m,
                                                    const unsigned char* wsrc, uint32_t cw_at, uint32_t of_at, int jl,
-                                                   int order) {
+                                                   unsigned order) {
   constexpr int RB = FT * 8, IMO = FT * 4, FL = FT / FPL;
-  const int swz = FT <= 16 ? order & 1 : order, hs = FT <= 16 ? order >> 1 : 0;   // chunk and half orders
-  const unsigned char* gsrc = tile_iq<PART>(p) + ((static_cast<size_t>(m.t) * p.C + m.c) * p.S + m.lo) * RB + jl * 16;
+  // chunk and half orders, the frame tile above them
+  const int swz = FT <= 16 || PART ? order & 1 : order, hs = FT <= 16 ? (order >> 1) & 1 : 0;
+  const unsigned char* gsrc = tile_iq<PART>(p, order >> 2) + ((static_cast<size_t>(m.t) * p.C + m.c) * p.S + m.lo) * RB + jl * 16;
 #pragma unroll
   for (int k = 0; k < VPG; ++k) {
     const float4 cw = lds128(cw_at + k * G * 16);
@@ -157,11 +160,15 @@ constexpr int kSleep = 1, kEarly = 2;
 
 //
 // PART: the launch covers frames p.f_first ... of an ensemble of p.f_total frames that the
-// frame tiles need not fill: blockIdx.y is the frame tile, its rows (zero beyond the last
+// frame tiles need not fill: a tile's rows (zero beyond the last
 // frame) start p.iq_tile_bytes after the previous tile's, frames past the last one are not
 // written, and Power Doppler leaves as one partial sum per tile when there are several.
-template <int FT, int FPL, int VPG, int NWC, int NBUF, int MAXR, int FLAGS, bool PART = false>
-__global__ void __launch_bounds__((NWC + 1) * 32) __maxnreg__(MAXR) k_das_exact(const DasParams p) {
+//
+// das_exact_block is one block's work.  W says what that is: voxel tile, frame tile and
+// outputs, read where they are needed (a value kept across the hot loop costs registers that
+// the 64 of a thread do not have: 1 % of a 94 x 94 x 178 volume, 6 % of a 25-frame run).
+template <int FT, int FPL, int VPG, int NWC, int NBUF, int FLAGS, bool PART, class W>
+__device__ __forceinline__ void das_exact_block(const DasParams& p, const W& w) {
   constexpr int FL = FT / FPL;
   constexpr int G = 32 / FL;
   constexpr int WV = G * VPG;
@@ -181,9 +188,7 @@ __global__ void __launch_bounds__((NWC + 1) * 32) __maxnreg__(MAXR) k_das_exact(
 
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
-  // the last tiles (deepest rows of the grid, the widest apertures: the most pairs) start
-  // first, so that the light shallow tiles fill the tail of the launch
-  const int64_t tile = static_cast<int64_t>(gridDim.x) - 1 - blockIdx.x;
+  const int64_t tile = w.tile();
 
   if (threadIdx.x == 0) {
     for (int b = 0; b < NBUF; ++b) {
@@ -196,7 +201,7 @@ __global__ void __launch_bounds__((NWC + 1) * 32) __maxnreg__(MAXR) k_das_exact(
 
   if (warp == NWC) {   // producer
     int r = 0;
-    const bool ok = produce_windows<NBUF>(p, tile_iq<PART>(p), tile, lane, smem, L.slot_bytes, 8, meta, full, empty, r);
+    const bool ok = produce_windows<NBUF>(p, tile_iq<PART>(p, w.ftile()), tile, lane, smem, L.slot_bytes, 8, meta, full, empty, r);
     if (lane == 0) finish_producer<NBUF, PB>(p, ok, r, meta, full, empty);
     return;
   }
@@ -313,7 +318,7 @@ __global__ void __launch_bounds__((NWC + 1) * 32) __maxnreg__(MAXR) k_das_exact(
         }
       } else {
         acc = outside_pair<FT, FPL, VPG, G, PART>(p, acc, meta[slot], smem + slot * slot_bytes + jl * 16, cw_at, of_at,
-                                            jl, FT <= 16 ? swz | hs << 1 : swz);
+                                            jl, FT <= 16 || PART ? swz | hs << 1 | w.ftile() << 2 : swz);
       }
       if constexpr ((FLAGS & kEarly) != 0) {   // every lane has read the slot: release it
         __syncwarp();
@@ -347,11 +352,11 @@ __global__ void __launch_bounds__((NWC + 1) * 32) __maxnreg__(MAXR) k_das_exact(
         const float2 a = acc_frame<C64Planar, 4>(&acc.a[k][4 * c], e);
         pw = fmaf(a.x, a.x, fmaf(a.y, a.y, pw));
       }
-      if (v >= 0 && p.y) {
+      if (v >= 0 && w.y()) {
         const int f0 = 4 * (jl + FL * (c ^ swz));
         if constexpr (PART) {
-          const int f = p.f_first + static_cast<int>(blockIdx.y) * FT + f0;
-          float2* dst = p.y + v * p.ystride + f;
+          const int f = p.f_first + static_cast<int>(w.ftile()) * FT + f0;
+          float2* dst = w.y() + v * p.ystride + f;
 #pragma unroll
           for (int e = 0; e < 4; e += 2) {
             const float2 a = acc_frame<C64Planar, 4>(&acc.a[k][4 * c], e), b = acc_frame<C64Planar, 4>(&acc.a[k][4 * c], e + 1);
@@ -364,7 +369,7 @@ __global__ void __launch_bounds__((NWC + 1) * 32) __maxnreg__(MAXR) k_das_exact(
           }
           continue;
         }
-        float2* dst = p.y + v * p.ystride + f0;
+        float2* dst = w.y() + v * p.ystride + f0;
         const float2 a0 = acc_frame<C64Planar, 4>(&acc.a[k][4 * c], 0), a1 = acc_frame<C64Planar, 4>(&acc.a[k][4 * c], 1);
         const float2 a2 = acc_frame<C64Planar, 4>(&acc.a[k][4 * c], 2), a3 = acc_frame<C64Planar, 4>(&acc.a[k][4 * c], 3);
         *reinterpret_cast<float4*>(dst) = make_float4(a0.x, a0.y, a1.x, a1.y);
@@ -373,13 +378,51 @@ __global__ void __launch_bounds__((NWC + 1) * 32) __maxnreg__(MAXR) k_das_exact(
     }
 #pragma unroll
     for (int o = FL / 2; o > 0; o >>= 1) pw += __shfl_xor_sync(0xffffffffu, pw, o);
-    if (jl == 0 && v >= 0 && p.pd) {
+    if (jl == 0 && v >= 0 && w.pd()) {
       if (PART && p.frame_tiles > 1)
-        p.pd_part[static_cast<int64_t>(p.f_tile + static_cast<int>(blockIdx.y)) * p.V + v] = pw;
+        p.pd_part[static_cast<int64_t>(p.f_tile + static_cast<int>(w.ftile())) * p.V + v] = pw;
       else
-        p.pd[v] = pw;
+        w.pd()[v] = pw;
     }
   }
+}
+
+// Work of a block of one acquisition's launch: the last tiles (deepest rows of the grid, the
+// widest apertures: the most pairs) start first, so that the light shallow tiles fill the
+// tail of the launch.
+struct GridWork {
+  const DasParams& p;
+  __device__ __forceinline__ int64_t tile() const { return static_cast<int64_t>(gridDim.x) - 1 - blockIdx.x; }
+  __device__ __forceinline__ unsigned ftile() const { return blockIdx.y; }
+  __device__ __forceinline__ float2* y() const { return p.y; }
+  __device__ __forceinline__ float* pd() const { return p.pd; }
+};
+
+template <int FT, int FPL, int VPG, int NWC, int NBUF, int MAXR, int FLAGS, bool PART = false>
+__global__ void __launch_bounds__((NWC + 1) * 32) __maxnreg__(MAXR) k_das_exact(const DasParams p) {
+  das_exact_block<FT, FPL, VPG, NWC, NBUF, FLAGS, PART>(p, GridWork{p});
+}
+
+// Many acquisitions in one launch: block b works on items[b] = (frame tile << 16 | entry of
+// a.p, voxel tile).  The entries' tables and tilings travel as kernel parameters (read through
+// the constant cache, like a single acquisition's); the bound output buffers are read from
+// the instance table, so that a captured launch follows a later bind.
+struct ItemWork {
+  const MultiArgs& a;
+  const int2* items;
+  __device__ __forceinline__ int2 item() const { return items[blockIdx.x]; }
+  __device__ __forceinline__ int entry() const { return item().x & 0xffff; }
+  __device__ __forceinline__ int64_t tile() const { return item().y; }
+  __device__ __forceinline__ unsigned ftile() const { return static_cast<unsigned>(item().x) >> 16; }
+  __device__ __forceinline__ float2* y() const { return a.insts[a.inst[entry()]].p.y; }
+  __device__ __forceinline__ float* pd() const { return a.insts[a.inst[entry()]].p.pd; }
+};
+
+template <int FT, int FPL, int VPG, int NWC, int NBUF, int MAXR, int FLAGS>
+__global__ void __launch_bounds__((NWC + 1) * 32) __maxnreg__(MAXR)
+    k_das_exact_multi(const __grid_constant__ MultiArgs a, const int2* items) {
+  const ItemWork w{a, items};
+  das_exact_block<FT, FPL, VPG, NWC, NBUF, FLAGS, true>(a.p[w.entry()], w);
 }
 
 }  // namespace
@@ -449,6 +492,26 @@ cudaError_t launch_das_parts(const DasParams& p, Variant v, int tiles, cudaStrea
     case V_SX16_F4V1W7: return go(k_das_exact<16, 4, 1, 7, 8, 64, kEarly, true>, 7);
     case V_SX8_F8V1W4: return go(k_das_exact<8, 8, 1, 4, 8, 64, kEarly, true>, 4);
     case V_SX8_F4V1W7: return go(k_das_exact<8, 4, 1, 7, 8, 64, kEarly, true>, 7);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+cudaError_t launch_das_multi(const MultiArgs& a, Variant v, const int2* items, int n_items, cudaStream_t s) {
+  size_t sm = 0;
+  for (int k = 0; k < a.n; ++k) sm = std::max(sm, exact_smem_bytes(v, a.p[k].rows_cap, a.p[k].T));
+  auto go = [&](auto* kernel, int nwc) -> cudaError_t {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sm));
+    if (e != cudaSuccess) return e;
+    kernel<<<static_cast<unsigned>(n_items), (nwc + 1) * 32, sm, s>>>(a, items);
+    return cudaGetLastError();
+  };
+  switch (v) {
+    case V_SX32_F8V1W7T14E: case V_SX32_F8V1W7_T8X7E: return go(k_das_exact_multi<32, 8, 1, 7, 8, 64, kEarly>, 7);
+    case V_SX16_F8V1W7: return go(k_das_exact_multi<16, 8, 1, 7, 8, 64, kEarly>, 7);
+    case V_SX16_F8V1W4: return go(k_das_exact_multi<16, 8, 1, 4, 8, 64, kEarly>, 4);
+    case V_SX16_F4V1W7: return go(k_das_exact_multi<16, 4, 1, 7, 8, 64, kEarly>, 7);
+    case V_SX8_F8V1W4: return go(k_das_exact_multi<8, 8, 1, 4, 8, 64, kEarly>, 4);
+    case V_SX8_F4V1W7: return go(k_das_exact_multi<8, 4, 1, 7, 8, 64, kEarly>, 7);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -156,6 +156,14 @@ struct FrameSplit {
   int tiles() const { return full + (tail ? 1 : 0); }
   int padded() const { return 32 * full + tail; }
 };
+struct RepackPart {             // one launch: equal frame tiles on one exact-frame shape
+  Variant v = V_COUNT;
+  int tiles = 0;
+  DasParams base{};
+  size_t at = 0;                // byte offset of its first tile in the workspace
+  float4* d_tbox = nullptr;
+  float2* d_txr = nullptr;
+};
 inline FrameSplit split_frames(int F) {
   const int rest = F % 32;
   FrameSplit f{F / 32, rest == 0 ? 0 : rest <= 8 ? 8 : 16};
@@ -195,10 +203,14 @@ cudaError_t launch_das_staged(const DasParams& p, Variant v, cudaStream_t s);
 // Staged variants whose frame count is a compile-time constant (k_das_exact.cu).
 size_t exact_smem_bytes(Variant v, int rows_cap, int T);
 // Rows of N = T C S samples in any storage type into the tiles of split_frames(F) at dst.
-cudaError_t launch_iq_repack(const void* src, int src_dtype, float* dst, int64_t N, int F, cudaStream_t s);
+// The source is read from *src_slot (device memory) when that is given.
+cudaError_t launch_iq_repack(const void* src, const void* const* src_slot, int src_dtype, float* dst, int64_t N, int F,
+                             cudaStream_t s);
 // Exact-frame kernel over `tiles` repacked frame tiles of variant_shape(v).frame_tile frames.
 cudaError_t launch_das_parts(const DasParams& p, Variant v, int tiles, cudaStream_t s);
-cudaError_t launch_pd_reduce(const float* part, float* pd, int64_t V, int tiles, cudaStream_t s);
+// pd, or *pd_slot (device memory; may hold NULL) when that is given.
+cudaError_t launch_pd_reduce(const float* part, float* pd, float* const* pd_slot, int64_t V, int tiles,
+                             cudaStream_t s);
 cudaError_t launch_das_exact(const DasParams& p, Variant v, cudaStream_t s);
 // Plan-time term table (k_das_table.cu): which staged variants have a table form, the
 // per-(tile, element) windows of every transmit (rows 0 = pair not used) and their
@@ -221,11 +233,26 @@ struct alignas(16) BatchInstance {
   int mode;             // kBatchFrames, kBatchChannels or kBatchStaged
   int frame_lanes;
 };
+// Repacked instances of a batch: per exact-frame shape one launch over (instance, tile) items.
+constexpr int kMultiMax = 64;       // entries of one launch (kernel parameters are limited to 32 KB)
+struct MultiArgs {
+  DasParams p[kMultiMax];           // iq: the entry's repacked tiles; y and pd unused
+  const BatchInstance* insts;       // device table with the bound buffers
+  int inst[kMultiMax];              // entry -> instance
+  int n;
+};
+static_assert(sizeof(MultiArgs) <= 32000, "kernel parameters");
+cudaError_t launch_das_multi(const MultiArgs& a, Variant v, const int2* items, int n_items, cudaStream_t s);
+
 int batch_blocks_per_sm(int iq_dtype, size_t slot_bytes);
 size_t batch_smem_bytes(size_t slot_bytes);
 cudaError_t launch_batch(int iq_dtype, const BatchInstance* insts, const int2* items, int n_items, int* counter,
                          int grid, size_t slot_bytes, cudaStream_t s);
 const DasParams* plan_params(mach_plan p);
+// A plan for a batch: as mach_das_plan without a workspace pool.  plan_repack: the launches
+// over its repacked tiles (0 when it beamforms directly), and the workspace they need.
+mach_status make_batch_plan(const mach_das_desc* d, void* stream, mach_plan* out);
+int plan_repack(mach_plan p, const RepackPart** parts, size_t* ws_bytes, size_t* pd_at);
 int plan_iq_dtype(mach_plan p);
 void pick_tile_shape(int n, int nx, int ny, int nz, bool list, int tile[3]);
 

@@ -37,15 +37,7 @@ struct mach_plan_s {
   int64_t table_bytes = 0;
   // repacked route (see repack_plan): the exact-frame launches over repacked frame tiles, and
   // the pool that each run takes its workspace from
-  struct Part {
-    Variant v = V_COUNT;
-    int tiles = 0;              // frame tiles of the launch
-    DasParams base{};
-    size_t at = 0;              // byte offset of its first tile in the workspace
-    float4* d_tbox = nullptr;
-    float2* d_txr = nullptr;
-  };
-  Part parts[2];
+  RepackPart parts[2];
   int n_parts = 0;
   size_t ws_bytes = 0;          // workspace of one run: repacked IQ, partial Power Doppler sums
   size_t pd_at = 0;
@@ -449,7 +441,7 @@ static mach_status build_term_table(mach_plan_s* p, DasParams& b, cudaStream_t s
 // the device's memory, a capturing stream, or a failed workspace allocation takes the direct
 // kernel.
 static mach_status repack_plan(mach_plan_s* p, const DasParams& b, bool list, cudaStream_t s,
-                               size_t total_mem) {
+                               size_t total_mem, bool own_pool) {
   const VariantShape& direct = variant_shape(p->variant);
   if (direct.exact_frames || direct.channel_lanes) return MACH_OK;
   const int64_t N = static_cast<int64_t>(b.T) * b.C * b.S;
@@ -486,7 +478,7 @@ static mach_status repack_plan(mach_plan_s* p, const DasParams& b, bool list, cu
   };
   if (dev_alloc(reinterpret_cast<void**>(&d_stats), 2 * sizeof(int), &scratch) != MACH_OK) return done(MACH_OK);
   for (int k = 0; k < n; ++k) {
-    mach_plan_s::Part& q = p->parts[k];
+    RepackPart& q = p->parts[k];
     const VariantShape& sh = variant_shape(want[k].v);
     DasParams t = b;
     if (configure_tiles(t, want[k].v, list, b.V, sh.frame_tile) != MACH_OK) return done(MACH_OK);
@@ -514,6 +506,13 @@ static mach_status repack_plan(mach_plan_s* p, const DasParams& b, bool list, cu
     q.base = t;
     q.at = k == 0 ? 0 : static_cast<size_t>(N) * 8 * 32 * fs.full;
   }
+  p->pd_at = iq_bytes;
+  p->ws_bytes = iq_bytes + pd_bytes;
+  if (!own_pool) {
+    p->device_bytes += bytes;
+    p->n_parts = n;
+    return done(MACH_OK);
+  }
   // a pool of the plan's own: each run takes its workspace in stream order, so that calls on
   // several streams never share one; one workspace is kept between runs, the others go back
   cudaMemPoolProps props{};
@@ -525,8 +524,6 @@ static mach_status repack_plan(mach_plan_s* p, const DasParams& b, bool list, cu
     p->pool = nullptr;
     return done(MACH_OK);
   }
-  p->pd_at = iq_bytes;
-  p->ws_bytes = iq_bytes + pd_bytes;
   uint64_t keep = (p->ws_bytes >> 25 << 25) + (64u << 20);   // the pool maps memory in blocks
   if (cudaMemPoolSetAttribute(p->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) cudaGetLastError();
   void* first = nullptr;   // mapped now rather than in the first run
@@ -542,7 +539,7 @@ static mach_status repack_plan(mach_plan_s* p, const DasParams& b, bool list, cu
   return done(MACH_OK);
 }
 
-mach_status mach_das_plan(const mach_das_desc* d, void* stream, mach_plan* out) {
+static mach_status make_plan(const mach_das_desc* d, void* stream, bool own_pool, mach_plan* out) {
   if (!out) return MACH_ERR_INVALID_ARG;
   *out = nullptr;
   mach_status st = validate(d);
@@ -768,7 +765,7 @@ mach_status mach_das_plan(const mach_das_desc* d, void* stream, mach_plan* out) 
     if (!variant_shape(var).staged || !table_supported(var)) return fail(MACH_ERR_UNSUPPORTED);
     if ((st = build_term_table(p, b, s)) != MACH_OK) return fail(st);
   }
-  if (!forced && !d->term_table && (st = repack_plan(p, b, list, s, total_b)) != MACH_OK) return fail(st);
+  if (!forced && !d->term_table && (st = repack_plan(p, b, list, s, total_b, own_pool)) != MACH_OK) return fail(st);
   if (cudaStreamSynchronize(s) != cudaSuccess) return fail(MACH_ERR_CUDA);
   cudaFree(d_raw);
   cudaFree(d_u);
@@ -779,6 +776,10 @@ mach_status mach_das_plan(const mach_das_desc* d, void* stream, mach_plan* out) 
   p->base = b;
   *out = p;
   return MACH_OK;
+}
+
+mach_status mach_das_plan(const mach_das_desc* d, void* stream, mach_plan* out) {
+  return make_plan(d, stream, true, out);
 }
 
 mach_status mach_plan_destroy(mach_plan p) {
@@ -803,7 +804,7 @@ static bool run_repacked(mach_plan p, const void* iq, float* pd, void* y, cudaSt
   }
   const DasParams& b = p->base;
   const int64_t N = static_cast<int64_t>(b.T) * b.C * b.S;
-  cudaError_t e = launch_iq_repack(iq, p->d.iq_dtype, reinterpret_cast<float*>(ws), N, b.F, s);
+  cudaError_t e = launch_iq_repack(iq, nullptr, p->d.iq_dtype, reinterpret_cast<float*>(ws), N, b.F, s);
   float* part = reinterpret_cast<float*>(ws + p->pd_at);
   for (int k = 0; k < p->n_parts && e == cudaSuccess; ++k) {
     DasParams q = p->parts[k].base;
@@ -814,7 +815,7 @@ static bool run_repacked(mach_plan p, const void* iq, float* pd, void* y, cudaSt
     e = launch_das_parts(q, p->parts[k].v, p->parts[k].tiles, s);
   }
   const int tiles = p->parts[0].base.frame_tiles;
-  if (e == cudaSuccess && pd && tiles > 1) e = launch_pd_reduce(part, pd, b.V, tiles, s);
+  if (e == cudaSuccess && pd && tiles > 1) e = launch_pd_reduce(part, pd, nullptr, b.V, tiles, s);
   const cudaError_t f = cudaFreeAsync(ws, s);
   *err = e != cudaSuccess ? e : f;
   return true;
@@ -827,7 +828,7 @@ static mach_status run(mach_plan p, const void* iq, float* pd, void* y, void* st
       (reinterpret_cast<uintptr_t>(pd) & 3u))
     return MACH_ERR_INVALID_ARG;
   cudaError_t re = cudaSuccess;
-  if (p->n_parts && run_repacked(p, iq, pd, y, static_cast<cudaStream_t>(stream), &re))
+  if (p->pool && run_repacked(p, iq, pd, y, static_cast<cudaStream_t>(stream), &re))
     return re == cudaSuccess ? MACH_OK : MACH_ERR_CUDA;
   DasParams q = p->base;
   q.iq = iq;
@@ -881,7 +882,7 @@ mach_status mach_plan_get_info(mach_plan p, mach_plan_info* info) {
   std::memset(info, 0, sizeof(*info));
   const VariantShape& s = variant_shape(p->variant);
   std::strncpy(info->variant, s.name, sizeof(info->variant) - 1);
-  if (p->n_parts) {   // the frame tiles that runs repack the ensemble into
+  if (p->pool) {   // the frame tiles that runs repack the ensemble into
     const size_t n = std::strlen(info->variant);
     std::snprintf(info->variant + n, sizeof(info->variant) - n, p->n_parts == 2 ? "+x%d+x%d" : "+x%d",
                   p->parts[0].base.F, p->parts[1].base.F);
@@ -961,6 +962,15 @@ namespace mach {
 // Host steps shared with the allocation-free entry point (noalloc.cu): the same
 // validation, choice among the non-staged kernels, voxel tiling and phase constants
 // that a plan uses.
+mach_status make_batch_plan(const mach_das_desc* d, void* stream, mach_plan* out) {
+  return make_plan(d, stream, false, out);
+}
+int plan_repack(mach_plan p, const RepackPart** parts, size_t* ws_bytes, size_t* pd_at) {
+  *parts = p->parts;
+  *ws_bytes = p->ws_bytes;
+  *pd_at = p->pd_at;
+  return p->n_parts;
+}
 mach_status host_validate(const mach_das_desc* d) { return validate(d); }
 Variant host_unstaged_variant(int iq_dtype, int F) { return unstaged(pick_variant(iq_dtype, F)); }
 mach_status host_configure_tiles(DasParams& b, Variant v, bool list, int64_t V, int F) {

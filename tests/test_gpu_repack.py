@@ -83,3 +83,36 @@ def test_repacked_runs_share_a_plan_across_streams():
         torch.cuda.synchronize()
     for a, b in zip(got, want):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("dt", ["c64", "f16x2", "bf16x2"])
+def test_batch_of_repacked_instances(dt):
+    """A batch mixing every frame-tile shape (and channel lanes) in 2D and 3D; a captured run
+    follows a later bind, also one that leaves out an instance's Power Doppler."""
+    frames = [2, 5, 8, 13, 16, 20, 32, 33, 41, 49, 64, 25]
+    acqs = [dense(F, dt, 2 + i % 2, 1 + i % 3) for i, F in enumerate(frames)]
+    sets = [[stored(a, 100 * k + i)[0] for i, a in enumerate(acqs)] for k in range(2)]
+    def out():
+        return ([torch.zeros((a.n_vox, a.n_frames), dtype=torch.complex64, device="cuda") for a in acqs],
+                [torch.zeros(a.n_vox, dtype=torch.float32, device="cuda") for a in acqs])
+    with m.Batch([m.plan_kwargs(a) for a in acqs]) as b:
+        y0, pd0 = out()
+        b.bind(sets[0], y0, pd0)
+        b.run()
+        g = torch.cuda.CUDAGraph()
+        torch.cuda.synchronize()
+        with torch.cuda.graph(g):
+            b.run()
+        y1, pd1 = out()
+        b.bind(sets[1], y1, pd1[:-4] + [None] + pd1[-3:])
+        g.replay()
+        torch.cuda.synchronize()
+    assert not pd1[-4].any()
+    for xs, ys, pds in ((sets[0], y0, pd0), (sets[1], y1, pd1)):
+        for i, (a, x, y, pd) in enumerate(zip(acqs, xs, ys, pds)):
+            idx = np.arange(0, a.n_vox, 13)
+            y_ref, pd_ref = oracle.das(a, synth.iqmod.from_storage(x.cpu()), idx)
+            assert nrmse_db(y.cpu().numpy()[idx], y_ref) <= -100, i
+            if pds is pd1 and i == len(acqs) - 4:
+                continue
+            assert nrmse_db(pd.cpu().numpy()[idx].astype(np.float64), pd_ref) <= -100, i
