@@ -627,6 +627,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_conv3d_tcx(const __grid_constan
   }
 }
 
+#include "conv_wgrad.cuh"
+
 // bfloat16 weights in the tensor-core layout of both directions:
 //   forward  wpk [Ci/16][27][2][Co][8]:  (kc, t, g, co, j) = W[t][16kc + 8g + j][co]
 //   flipped  wpkt[Co/16][27][2][Ci][8]:  (kc, t, g, ci, j) = W[t][ci][16kc + 8g + j]
@@ -842,6 +844,54 @@ cudaError_t launch_conv_tc(const void* x, const void* wpk, const float* bias, vo
   if (e != cudaSuccess) return e;
   const int64_t grid = p.tiles < static_cast<int64_t>(sms) * per_sm ? p.tiles : static_cast<int64_t>(sms) * per_sm;
   kern<<<static_cast<unsigned>(grid), kThreads, smem, s>>>(map, p);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_conv_wgrad(const void* x, const void* dy, float* dw, int n, int d, int h, int w, int ci, int co,
+                              cudaStream_t s) {
+  PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
+  if (!enc) return cudaErrorNotSupported;
+  CUtensorMap maps[2];
+  for (int k = 0; k < 2; ++k) {   // input halo bricks, output-gradient tiles
+    const int c = k ? co : ci;
+    const cuuint64_t dims[5] = {static_cast<cuuint64_t>(c), static_cast<cuuint64_t>(w), static_cast<cuuint64_t>(h),
+                                static_cast<cuuint64_t>(d), static_cast<cuuint64_t>(n)};
+    const cuuint64_t row = 2ull * c;
+    const cuuint64_t strides[4] = {row, row * w, row * w * h, row * w * h * d};
+    const cuuint32_t box[5] = {8, static_cast<cuuint32_t>(k ? kTX : kHX), static_cast<cuuint32_t>(k ? kTY : kHY),
+                               static_cast<cuuint32_t>(k ? kWgTZ : kWgTZ + 2), 1};
+    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    if (enc(&maps[k], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(k ? dy : x), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+      return cudaErrorNotSupported;
+  }
+  WgradParams p{};
+  p.dw = dw;
+  p.Ci = ci;
+  p.Co = co;
+  p.tiles_x = (w + kTX - 1) / kTX;
+  p.tiles_y = (h + kTY - 1) / kTY;
+  p.tiles_z = (d + kWgTZ - 1) / kWgTZ;
+  p.tiles = static_cast<int64_t>(p.tiles_x) * p.tiles_y * p.tiles_z * n;
+  p.wait_limit = g_wait_limit ? g_wait_limit : kDefaultWait;
+  p.debug_stall = g_debug_stall;
+  int per_sm = 0, sms = 0;
+  cudaError_t e = kernel_setup(reinterpret_cast<const void*>(k_conv3d_wgrad_tma), kWgSmem, 512, &per_sm, &sms);
+  if (e != cudaSuccess) return e;
+  // One block per SM at a time, three waves of them: the tensor cores' sums lose accuracy in
+  // proportion to the voxels a warp sums in one go, and three waves keep them below those of
+  // the earlier kernel (relative error of dW at 32 -> 32, 8 x 64^3, for 1 / 2 / 3 / 4 waves
+  // 17 / 8.8 / 5.5 / 4.3e-6; earlier kernel 8.3e-6) at the same speed (252 / 257 / 260 / 265 us).
+  // Channel blocks are the fastest grid axis, so that those reading the same voxels run together.
+  const int64_t blocks = static_cast<int64_t>(ci / 16) * (co / 16);
+  int64_t splits = 3LL * sms / blocks;
+  splits = splits < 1 ? 1 : splits;
+  splits = splits < p.tiles ? splits : p.tiles;
+  p.per_block = (p.tiles + splits - 1) / splits;
+  splits = (p.tiles + p.per_block - 1) / p.per_block;
+  const dim3 grid(static_cast<unsigned>(blocks), static_cast<unsigned>(splits));
+  k_conv3d_wgrad_tma<<<grid, (kWgMma + 1) * 32, kWgSmem, s>>>(maps[0], maps[1], p);
   return cudaGetLastError();
 }
 

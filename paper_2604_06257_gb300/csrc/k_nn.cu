@@ -9,10 +9,6 @@
 //    tap at a time through a double-buffered cp.async pipeline; bias, leaky ReLU and the
 //    output conversion are fused into the epilogue.  With `flip` the taps are mirrored,
 //    which turns it into the data gradient (given the transposed weights [27][Cout][Cin]).
-//  * k_conv3d_wgrad: weight gradient dW[t][ci][co] = sum_v X[v + off(t)][ci] dY[v][co]:
-//    per block all 27 taps of one (16 input, CT output channel) block over a run of voxel
-//    tiles, halo and gradient tiles staged once per tile, partial sums added with float32
-//    atomics.
 //  * elementwise kernels: leaky-ReLU backward, 2x average pooling and nearest upsampling
 //    (and their adjoints), channel-slice copies (concatenation), bias gradient, Adam,
 //    and the network boundary (RMS normalisation / packing, loss, output).
@@ -167,124 +163,6 @@ __global__ void __launch_bounds__(128) k_conv3d(const bf16* __restrict__ X, cons
       }
       if (Y) *reinterpret_cast<__nv_bfloat162*>(Y + row * Co + col) = __floats2bfloat162_rn(v0, v1);
       if (Yf) *reinterpret_cast<float2*>(Yf + row * Co + col) = make_float2(v0, v1);
-    }
-  }
-}
-
-// Weight gradient, all 27 taps per block.  A block owns one 16-channel input block, one
-// CT-channel output block and a run of 8 x 16 x 1 voxel tiles.  Per tile it stages the
-// input halo brick (10 x 18 x 3 voxels x 16 channels, zero outside the volume) and the
-// output-gradient tile (128 voxels x CT channels, zero outside) in shared memory once,
-// and every warp accumulates its taps (warp w: taps w, w + 8, w + 16, w + 24) as
-// mma.sync products X_t^T (16 x 16 voxels) x dY (16 voxels x CT) over the tile's voxels.
-// Partial sums are added to dW with float32 atomics at the end.
-constexpr int kWTaps = 4;              // taps per warp (8 warps cover 27)
-constexpr int kHRows = 10 * 18 * 3;    // halo rows of one 8-channel group
-
-template <int CT>
-__global__ void __launch_bounds__(256) k_conv3d_wgrad(const bf16* __restrict__ X, const bf16* __restrict__ dY,
-                                                      float* __restrict__ dW, int N, int D, int H, int W, int Ci,
-                                                      int Co, int64_t tiles, int tiles_x, int tiles_y,
-                                                      int64_t tiles_per_block) {
-  constexpr int kHaloB = 2 * kHRows * 16;
-  constexpr int kGB = (CT / 8) * 128 * 16;
-  constexpr int kStage = kHaloB + kGB;
-  extern __shared__ __align__(128) uint8_t wsm[];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int cb = blockIdx.y, ob = blockIdx.z;
-  const int64_t t_begin = static_cast<int64_t>(blockIdx.x) * tiles_per_block;
-  const int64_t t_end = t_begin + tiles_per_block < tiles ? t_begin + tiles_per_block : tiles;
-
-  auto load = [&](int stage, int64_t tile) {
-    const int tx = static_cast<int>(tile % tiles_x);
-    int64_t r0 = tile / tiles_x;
-    const int ty = static_cast<int>(r0 % tiles_y);
-    r0 /= tiles_y;
-    const int z = static_cast<int>(r0 % D), n = static_cast<int>(r0 / D);
-    const int x0 = tx * 8, y0 = ty * 16;
-    uint8_t* base = wsm + stage * kStage;
-    for (int c = tid; c < 2 * kHRows + (CT / 8) * 128; c += 256) {
-      if (c < 2 * kHRows) {
-        const int g = c / kHRows, r = c % kHRows;
-        const int hz = r / 180, hr = r % 180, hy = hr / 10, hx = hr % 10;
-        const int x = x0 - 1 + hx, y = y0 - 1 + hy, zz = z - 1 + hz;
-        const bool in = x >= 0 && x < W && y >= 0 && y < H && zz >= 0 && zz < D;
-        const bf16* src = in ? X + ((((static_cast<int64_t>(n) * D + zz) * H + y) * W + x) * Ci + cb * 16 + g * 8) : X;
-        cp16(base + (g * kHRows + r) * 16, src, in ? 16 : 0);
-      } else {
-        const int c2 = c - 2 * kHRows;
-        const int cg = c2 / 128, k = c2 % 128;
-        const int x = x0 + (k & 7), y = y0 + (k >> 3);
-        const bool in = x < W && y < H;
-        const bf16* src = in ? dY + ((((static_cast<int64_t>(n) * D + z) * H + y) * W + x) * Co + ob * CT + cg * 8) : dY;
-        cp16(base + kHaloB + (cg * 128 + k) * 16, src, in ? 16 : 0);
-      }
-    }
-    cp_commit();
-  };
-
-  float acc[kWTaps][CT / 8][4];
-#pragma unroll
-  for (int i = 0; i < kWTaps; ++i)
-#pragma unroll
-    for (int j = 0; j < CT / 8; ++j) acc[i][j][0] = acc[i][j][1] = acc[i][j][2] = acc[i][j][3] = 0.f;
-
-  if (t_begin < t_end) load(0, t_begin);
-  for (int64_t tile = t_begin; tile < t_end; ++tile) {
-    const int st = static_cast<int>((tile - t_begin) & 1);
-    if (tile + 1 < t_end) {
-      load(st ^ 1, tile + 1);
-      cp_wait<1>();
-    } else {
-      cp_wait<0>();
-    }
-    __syncthreads();
-    const uint8_t* base = wsm + st * kStage;
-    const uint8_t* halo = base;
-    const uint8_t* gt = base + kHaloB;
-#pragma unroll 2
-    for (int ks = 0; ks < 8; ++ks) {   // 16 voxels (two x-rows of the tile) per K step
-      uint32_t bfr[CT / 16][4];
-#pragma unroll
-      for (int j = 0; j < CT / 16; ++j)
-        ldm_x4_t(bfr[j], gt + ((2 * j + (lane >> 4)) * 128 + ks * 16 + (lane & 15)) * 16);
-      const int mat = lane >> 3;
-      const int kv = ks * 16 + (mat >> 1) * 8 + (lane & 7);   // voxel of this lane's row address
-      const int mx = kv & 7, my = kv >> 3;
-#pragma unroll
-      for (int i = 0; i < kWTaps; ++i) {
-        const int t = warp + 8 * i;
-        if (t < 27) {   // warp-uniform
-          int dz, dy, dx;
-          tap_offset(t, dz, dy, dx);
-          const int row = (dz + 1) * 180 + (my + dy + 1) * 10 + (mx + dx + 1);
-          uint32_t af[4];
-          ldm_x4_t(af, halo + ((mat & 1) * kHRows + row) * 16);
-#pragma unroll
-          for (int j = 0; j < CT / 16; ++j) {
-            mma_bf16(acc[i][2 * j], af, bfr[j][0], bfr[j][1]);
-            mma_bf16(acc[i][2 * j + 1], af, bfr[j][2], bfr[j][3]);
-          }
-        }
-      }
-    }
-    __syncthreads();
-  }
-  if (t_begin >= t_end) return;
-#pragma unroll
-  for (int i = 0; i < kWTaps; ++i) {
-    const int t = warp + 8 * i;
-    if (t >= 27) continue;
-#pragma unroll
-    for (int j = 0; j < CT / 8; ++j) {
-      const int co = ob * CT + 8 * j + 2 * (lane & 3);
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int ci = cb * 16 + (lane >> 2) + 8 * h;
-        float* dst = dW + (static_cast<int64_t>(t) * Ci + ci) * Co + co;
-        atomicAdd(dst, acc[i][j][2 * h]);
-        atomicAdd(dst + 1, acc[i][j][2 * h + 1]);
-      }
     }
   }
 }
@@ -687,24 +565,6 @@ inline unsigned nblocks(int64_t n, int b = 256) { return static_cast<unsigned>((
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 inline mach_status last_status() { return cudaGetLastError() == cudaSuccess ? MACH_OK : MACH_ERR_CUDA; }
 
-template <int CT>
-cudaError_t go_wgrad(const bf16* x, const bf16* dy, float* dw, int n, int d, int h, int w, int ci, int co,
-                     cudaStream_t s) {
-  const int tiles_x = (w + 7) / 8, tiles_y = (h + 15) / 16;
-  const int64_t tiles = static_cast<int64_t>(tiles_x) * tiles_y * d * n;
-  const int64_t chan_blocks = static_cast<int64_t>(ci / 16) * (co / CT);
-  // about four blocks per SM in total, split over runs of tiles
-  int64_t splits = (152LL * 4 + chan_blocks - 1) / chan_blocks;
-  splits = splits < tiles ? splits : tiles;
-  const int64_t per = (tiles + splits - 1) / splits;
-  splits = (tiles + per - 1) / per;
-  const int smem = 2 * (2 * kHRows * 16 + (CT / 8) * 128 * 16);
-  cudaError_t e = cudaFuncSetAttribute(k_conv3d_wgrad<CT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  const dim3 grid(static_cast<unsigned>(splits), static_cast<unsigned>(ci / 16), static_cast<unsigned>(co / CT));
-  k_conv3d_wgrad<CT><<<grid, 256, smem, s>>>(x, dy, dw, n, d, h, w, ci, co, tiles, tiles_x, tiles_y, per);
-  return cudaGetLastError();
-}
 }  // namespace
 
 extern "C" {
@@ -737,12 +597,12 @@ mach_status mach_nn_conv3d_wgrad(const void* x, const void* dy, float* dw, int32
   if (!x || !dy || !dw || n < 1 || nz < 1 || ny < 1 || nx < 1) return MACH_ERR_INVALID_ARG;
   if (ci < 16 || ci % 16 || co < 16 || co % 16) return MACH_ERR_INVALID_ARG;
   if (!aligned16(x) || !aligned16(dy)) return MACH_ERR_INVALID_ARG;
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const bf16* X = static_cast<const bf16*>(x);
-  const bf16* G = static_cast<const bf16*>(dy);
   if (ci / 16 > 65535 || co / 16 > 65535) return MACH_ERR_UNSUPPORTED;
-  const cudaError_t e = co % 32 == 0 ? go_wgrad<32>(X, G, dw, n, nz, ny, nx, ci, co, s)
-                                     : go_wgrad<16>(X, G, dw, n, nz, ny, nx, ci, co, s);
+  const cudaError_t e = launch_conv_wgrad(x, dy, dw, n, nz, ny, nx, ci, co, static_cast<cudaStream_t>(stream));
+  if (e == cudaErrorNotSupported) {
+    cudaGetLastError();
+    return MACH_ERR_UNSUPPORTED;
+  }
   return e == cudaSuccess ? MACH_OK : MACH_ERR_CUDA;
 }
 

@@ -31,6 +31,9 @@ cudaError_t launch_output(const float* o, const float* xf, const float* sums, fl
 bool conv_tc_supported(int ci, int co);
 cudaError_t launch_conv_tc(const void* x, const void* wpk, const float* bias, void* y, float* yf, int n, int d,
                            int h, int w, int ci, int co, int flip, int act, cudaStream_t s);
+// weight gradient (conv_wgrad.cuh); cudaErrorNotSupported when no tensor map describes the tensors
+cudaError_t launch_conv_wgrad(const void* x, const void* dy, float* dw, int n, int d, int h, int w, int ci, int co,
+                              cudaStream_t s);
 cudaError_t launch_pack_weights(const float* w, void* wpk, void* wpkt, int ci, int co, cudaStream_t s);
 
 // bfloat16 copies of float32 weights [27][ci][co]: wb (same layout) and wbt ([27][co][ci])
