@@ -31,6 +31,7 @@
 
 #include "async_copy.cuh"
 #include "mach_nn.h"
+#include "nn_device.cuh"
 #include "nn_internal.h"
 
 namespace mach_nn {
@@ -65,6 +66,8 @@ struct ConvTcParams {
   float* yf;            // [N][D][H][W][Co] or nullptr
   int N, D, H, W, Ci, Co;
   int flip, act;
+  const bf16* mask;     // [N][D][H][W][Co] or nullptr: leaky-ReLU derivative at these activations, applied to y
+  int yf_ch;            // channels of yf's rows: 2 (the first two), else Co
   int tz;               // z planes per tile (1 or 2): one M = 128 MMA per plane and tap
   int resident;         // all weights loaded once per CTA (else 9-tap blocks through a ring)
   int tiles_x, tiles_y, tiles_z;
@@ -83,6 +86,13 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
          (static_cast<uint64_t>(sbo >> 4) << 32) | (1ull << 46);
 }
 
+// The same for rows of 32 bytes (16 channels) stored with the 32-byte swizzle: 8-row groups
+// 256 bytes apart, one K = 16 step per row, start addresses on 256-byte boundaries.
+__device__ __forceinline__ uint64_t smem_desc_sw32(uint32_t addr) {
+  return static_cast<uint64_t>((addr & 0x3FFFFu) >> 4) | (1ull << 16) | (static_cast<uint64_t>(256u >> 4) << 32) |
+         (1ull << 46) | (6ull << 61);
+}
+
 // instruction descriptor, kind::f16: D float32, A and B bfloat16, both K-major, M = 128
 __host__ __device__ constexpr uint32_t instr_desc(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(n >> 3) << 17) | ((128u >> 4) << 24);
@@ -98,6 +108,11 @@ __device__ __forceinline__ bool wait_spin(uint64_t* bar, uint32_t parity, uint32
   return false;
 }
 
+// The same by a convergent warp (the vote keeps it so).
+__device__ __forceinline__ bool wait_warp(uint64_t* bar, uint32_t parity, uint32_t limit) {
+  return __all_sync(0xffffffffu, wait_spin(bar, parity, limit));
+}
+
 __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, int c3,
                                             int c4, uint64_t* bar) {
   asm volatile(
@@ -107,18 +122,32 @@ __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* map
       : "memory");
 }
 
-__device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+// MMAs and commits are issued by one elected lane while the whole warp walks the loops around
+// them: the warp stays convergent, so the descriptors live in uniform registers (inside a
+// one-lane branch each had to be moved there for every MMA: x-folded 48 -> 16 at 8 x 128^3 1003 -> 845 us, 32 -> 16 713 -> 588 us).
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t lead;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(lead));
+  return lead;
+}
+
+__device__ __forceinline__ void mma_f16(uint32_t lead, uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
+                                        uint32_t acc) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc)
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+      "l"(a), "l"(b), "r"(idesc), "r"(acc), "r"(lead)
       : "memory");
 }
 
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-               : "memory");
+__device__ __forceinline__ void mma_commit(uint32_t lead, uint64_t* bar) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(smem_u32(bar)),
+      "r"(lead)
+      : "memory");
 }
+
 
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -270,74 +299,73 @@ __global__ void __launch_bounds__(kThreads, 3) k_conv3d_tc(const __grid_constant
         }
       }
     }
-  } else if (warp == 1) {
-    if (lane == 0) {   // ---------------------------------------------- MMAs
-      const uint32_t idesc = instr_desc(p.Co);
-      bool ok = !p.resident || wait_spin(&fullB[0], 0, limit);
-      if (!ok) give_up();
-      uint32_t a_use = 0, b_use = 0, acc_use = 0;
-      for (int64_t tile = blockIdx.x; ok && tile < p.tiles && !*abort_flag; tile += gridDim.x) {
-        const uint32_t buf = acc_use & 1u, ku = acc_use >> 1;
-        if (ku >= 1 && !wait_spin(&tempty[buf], (ku - 1) & 1u, limit)) {
-          give_up();
+  } else if (warp == 1) {   // -------------------------------------------- MMAs
+    const uint32_t lead = elect_one();
+    const uint32_t idesc = instr_desc(p.Co);
+    bool ok = !p.resident || wait_warp(&fullB[0], 0, limit);
+    if (!ok) if (lane == 0) give_up();
+    uint32_t a_use = 0, b_use = 0, acc_use = 0;
+    for (int64_t tile = blockIdx.x; ok && tile < p.tiles && !__any_sync(0xffffffffu, *abort_flag); tile += gridDim.x) {
+      const uint32_t buf = acc_use & 1u, ku = acc_use >> 1;
+      if (ku >= 1 && !wait_warp(&tempty[buf], (ku - 1) & 1u, limit)) {
+        if (lane == 0) give_up();
+        break;
+      }
+      fence_after();
+      const uint32_t d0 = tmem + buf * (p.tmem_cols >> 1);
+      for (int kc = 0; kc < NC && ok; ++kc) {
+        const uint32_t sa = a_use & 1u, ka = a_use >> 1;
+        if (!wait_warp(&fullA[sa], ka & 1u, limit)) {
+          if (lane == 0) give_up();
+          ok = false;
           break;
         }
-        fence_after();
-        const uint32_t d0 = tmem + buf * (p.tmem_cols >> 1);
-        for (int kc = 0; kc < NC && ok; ++kc) {
-          const uint32_t sa = a_use & 1u, ka = a_use >> 1;
-          if (!wait_spin(&fullA[sa], ka & 1u, limit)) {
-            give_up();
-            ok = false;
-            break;
+        // descriptors: the taps differ only by start address (16-byte units in the low
+        // field), so every MMA costs two additions; the 27 taps unroll at compile time
+        const uint64_t ad0 = smem_desc(smem_u32(sA + sa * a_stage), p.group_pitch, kHX * 16);
+#pragma unroll
+        for (int tb = 0; tb < 3; ++tb) {
+          uint32_t w_base;
+          uint32_t sb = 0;
+          if (p.resident) {
+            w_base = smem_u32(sW) + (static_cast<uint32_t>(kc) * 27 + tb * 9) * tap_bytes;
+          } else {
+            sb = b_use % kNB;
+            if (!wait_warp(&fullB[sb], (b_use / kNB) & 1u, limit)) {
+              if (lane == 0) give_up();
+              ok = false;
+              break;
+            }
+            w_base = smem_u32(sW + sb * 9 * tap_bytes);
           }
-          // descriptors: the taps differ only by start address (16-byte units in the low
-          // field), so every MMA costs two additions; the 27 taps unroll at compile time
-          const uint64_t ad0 = smem_desc(smem_u32(sA + sa * a_stage), p.group_pitch, kHX * 16);
+          const uint64_t bd0 = smem_desc(w_base, static_cast<uint32_t>(p.Co) * 16u, 128u);
 #pragma unroll
-          for (int tb = 0; tb < 3; ++tb) {
-            uint32_t w_base;
-            uint32_t sb = 0;
-            if (p.resident) {
-              w_base = smem_u32(sW) + (static_cast<uint32_t>(kc) * 27 + tb * 9) * tap_bytes;
-            } else {
-              sb = b_use % kNB;
-              if (!wait_spin(&fullB[sb], (b_use / kNB) & 1u, limit)) {
-                give_up();
-                ok = false;
-                break;
-              }
-              w_base = smem_u32(sW + sb * 9 * tap_bytes);
-            }
-            const uint64_t bd0 = smem_desc(w_base, static_cast<uint32_t>(p.Co) * 16u, 128u);
+          for (int tt = 0; tt < 9; ++tt) {
+            const int t = tb * 9 + tt;
+            const int sg = FLIP ? -1 : 1;
+            const int dz = sg * (t / 9 - 1), dy = sg * ((t / 3) % 3 - 1), dx = sg * (t % 3 - 1);
+            const uint32_t row = static_cast<uint32_t>((dz + 1) * (kHX * kHY) + (dy + 1) * kHX + (dx + 1));
+            const uint64_t bd = bd0 + static_cast<uint64_t>(tt) * (tap_bytes >> 4);
+            const uint32_t acc = (kc > 0 || t > 0) ? 1u : 0u;
 #pragma unroll
-            for (int tt = 0; tt < 9; ++tt) {
-              const int t = tb * 9 + tt;
-              const int sg = FLIP ? -1 : 1;
-              const int dz = sg * (t / 9 - 1), dy = sg * ((t / 3) % 3 - 1), dx = sg * (t % 3 - 1);
-              const uint32_t row = static_cast<uint32_t>((dz + 1) * (kHX * kHY) + (dy + 1) * kHX + (dx + 1));
-              const uint64_t bd = bd0 + static_cast<uint64_t>(tt) * (tap_bytes >> 4);
-              const uint32_t acc = (kc > 0 || t > 0) ? 1u : 0u;
-#pragma unroll
-              for (int zz = 0; zz < TZ; ++zz)
-                mma_f16(d0 + static_cast<uint32_t>(zz * p.Co), ad0 + row + static_cast<uint32_t>(zz * kHX * kHY),
-                        bd, idesc, acc);
-            }
-            if (!p.resident) {
-              mma_commit(&emptyB[sb]);
-              ++b_use;
-            }
+            for (int zz = 0; zz < TZ; ++zz)
+              mma_f16(lead, d0 + static_cast<uint32_t>(zz * p.Co), ad0 + row + static_cast<uint32_t>(zz * kHX * kHY),
+                      bd, idesc, acc);
           }
-          if (!ok) break;
-          mma_commit(&emptyA[sa]);
-          ++a_use;
+          if (!p.resident) {
+            mma_commit(lead, &emptyB[sb]);
+            ++b_use;
+          }
         }
         if (!ok) break;
-        mma_commit(&tfull[buf]);
-        ++acc_use;
+        mma_commit(lead, &emptyA[sa]);
+        ++a_use;
       }
-      mma_commit(fin);
+      if (!ok) break;
+      mma_commit(lead, &tfull[buf]);
+      ++acc_use;
     }
+    mma_commit(lead, fin);
   } else {   // ---------------------------------------------------------- epilogue
     const int q = warp & 3;            // tensor-memory lanes 32q .. 32q + 31
     const int row = 32 * q + lane;     // GEMM row within a plane
@@ -362,6 +390,11 @@ __global__ void __launch_bounds__(kThreads, 3) k_conv3d_tc(const __grid_constant
                                (static_cast<uint32_t>(32 * q) << 16);
         for (int c0 = 0; c0 < p.Co; c0 += 16) {
           uint32_t r[16];
+          uint4 m0 = make_uint4(0u, 0u, 0u, 0u), m1 = m0;
+          if (p.mask && inside) {
+            m0 = __ldg(reinterpret_cast<const uint4*>(p.mask + v * p.Co + c0));
+            m1 = __ldg(reinterpret_cast<const uint4*>(p.mask + v * p.Co + c0) + 1);
+          }
           tmem_ld16(taddr + static_cast<uint32_t>(c0), r);
           if (inside) {
             float f[16];
@@ -379,10 +412,17 @@ __global__ void __launch_bounds__(kThreads, 3) k_conv3d_tc(const __grid_constant
                 h[i] = *reinterpret_cast<const uint32_t*>(&b2);
               }
               uint4* dst = reinterpret_cast<uint4*>(p.y + v * p.Co + c0);
-              dst[0] = make_uint4(h[0], h[1], h[2], h[3]);
-              dst[1] = make_uint4(h[4], h[5], h[6], h[7]);
+              uint4 q0 = make_uint4(h[0], h[1], h[2], h[3]), q1 = make_uint4(h[4], h[5], h[6], h[7]);
+              if (p.mask) {
+                q0 = lrelu_grad8(q0, m0);
+                q1 = lrelu_grad8(q1, m1);
+              }
+              dst[0] = q0;
+              dst[1] = q1;
             }
-            if (p.yf) {
+            if (p.yf && p.yf_ch == 2) {
+              if (c0 == 0) *reinterpret_cast<float2*>(p.yf + 2 * v) = make_float2(f[0], f[1]);
+            } else if (p.yf) {
               float4* dst = reinterpret_cast<float4*>(p.yf + v * p.Co + c0);
 #pragma unroll
               for (int i = 0; i < 4; ++i) dst[i] = make_float4(f[4 * i], f[4 * i + 1], f[4 * i + 2], f[4 * i + 3]);
@@ -417,22 +457,28 @@ __global__ void __launch_bounds__(kThreads, 3) k_conv3d_tc(const __grid_constant
 // warp shuffles (rows are x-major, so x +- 1 is lane +- 1).  A tile is 16 (x) x 8 (y) x TZ (z)
 // rows, consecutive tiles 14 apart in x.  The weights are rearranged once per CTA into
 // per-(kc, dz, dy) blocks [g][j * 16 + co][8] (B operand: N = 48 rows 16 bytes apart, the
-// two 8-channel groups 768 bytes apart) and stay resident.
+// two 8-channel groups 768 bytes apart) and stay resident.  The A brick is loaded as rows of
+// 16 channels with the 32-byte swizzle (one TMA element per voxel; no faster than two 8-channel
+// groups, but one load).
 constexpr int kXR = 16;                 // GEMM rows along x per tile
 constexpr int kXO = kXR - 2;            // outputs along x per tile
 constexpr int kYT = 8;                  // y rows per tile: kXR x kYT = 128
 constexpr int kXN = 48;                 // three x taps x 16 output channels
 constexpr uint32_t kFoldBlock = 2u * kXN * 16u;   // one (dz, dy) pair x 16 input channels
 constexpr int kFoldMaxNC = 6;           // input-channel steps whose weights stay resident
+// Eight epilogue warps: two groups of four (tensor-memory lanes 0 ... 127), each draining every
+// other plane.  One group's drain of a plane (three tensor-memory loads, 32 shuffles, the
+// stores) is a serial chain longer than the plane's nine MMAs once their issue is cheap:
+// 16 -> 16 at 8 x 128^3 426 us with one group, 332 us with two (48 -> 16: 845 / 840 us).
+constexpr int kFoldThreads = 64 + 8 * 32;
 
 template <bool FLIP, int TZ>
-__global__ void __launch_bounds__(kThreads, 2) k_conv3d_tcx(const __grid_constant__ CUtensorMap xmap,
+__global__ void __launch_bounds__(kFoldThreads, TZ == 4 ? 1 : 2) k_conv3d_tcx(const __grid_constant__ CUtensorMap xmap,
                                                             const ConvTcParams p) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   uint8_t* sm = smem_raw + (((raw + 1023u) & ~1023u) - raw);
-  const uint32_t a_stage = 2 * p.group_pitch;
-  constexpr uint32_t halo_bytes = static_cast<uint32_t>(kXR * (kYT + 2) * (TZ + 2) * 16);
+  constexpr uint32_t a_stage = static_cast<uint32_t>(kXR * (kYT + 2) * (TZ + 2) * 32);   // one halo brick
   const int NC = p.Ci / 16;
   const uint32_t w_bytes = static_cast<uint32_t>(NC) * 9u * kFoldBlock;
   const uint32_t S = static_cast<uint32_t>(p.a_stages);
@@ -468,7 +514,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_conv3d_tcx(const __grid_constan
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&tfull[i], 1);
-      mbar_init(&tempty[i], 128);
+      mbar_init(&tempty[i], kFoldThreads - 64);
     }
     mbar_init(fin, 1);
     *abort_flag = 0;
@@ -502,62 +548,60 @@ __global__ void __launch_bounds__(kThreads, 2) k_conv3d_tcx(const __grid_constan
             give_up();
             break;
           }
-          mbar_arrive_expect_tx(&fullA[sa], 2 * halo_bytes);
-          for (int g = 0; g < 2; ++g)
-            tma_load_5d(smem_u32(sA + sa * a_stage + g * p.group_pitch), &xmap, kc * 16 + g * 8, tc.x0, tc.y0 - 1,
-                        tc.z0 - 1, tc.n, &fullA[sa]);
+          mbar_arrive_expect_tx(&fullA[sa], a_stage);
+          tma_load_5d(smem_u32(sA + sa * a_stage), &xmap, kc * 16, tc.x0, tc.y0 - 1, tc.z0 - 1, tc.n, &fullA[sa]);
           ++a_use;
         }
       }
     }
-  } else if (warp == 1) {
-    if (lane == 0) {   // ---------------------------------------------- MMAs
-      constexpr uint32_t idesc = instr_desc(kXN);
-      bool ok = true;
-      uint32_t a_use = 0, acc_use = 0;
-      for (int64_t tile = blockIdx.x; tile < p.tiles && !*abort_flag; tile += gridDim.x) {
-        const uint32_t buf = acc_use & 1u, ku = acc_use >> 1;
-        if (ku >= 1 && !wait_spin(&tempty[buf], (ku - 1) & 1u, limit)) {
-          give_up();
+  } else if (warp == 1) {   // -------------------------------------------- MMAs
+    const uint32_t lead = elect_one();
+    constexpr uint32_t idesc = instr_desc(kXN);
+    bool ok = true;
+    uint32_t a_use = 0, acc_use = 0;
+    for (int64_t tile = blockIdx.x; tile < p.tiles && !__any_sync(0xffffffffu, *abort_flag); tile += gridDim.x) {
+      const uint32_t buf = acc_use & 1u, ku = acc_use >> 1;
+      if (ku >= 1 && !wait_warp(&tempty[buf], (ku - 1) & 1u, limit)) {
+        if (lane == 0) give_up();
+        break;
+      }
+      fence_after();
+      const uint32_t d0 = tmem + buf * (p.tmem_cols >> 1);
+      for (int kc = 0; kc < NC && ok; ++kc) {
+        const uint32_t sa = a_use % S, ka = a_use / S;
+        if (!wait_warp(&fullA[sa], ka & 1u, limit)) {
+          if (lane == 0) give_up();
+          ok = false;
           break;
         }
-        fence_after();
-        const uint32_t d0 = tmem + buf * (p.tmem_cols >> 1);
-        for (int kc = 0; kc < NC && ok; ++kc) {
-          const uint32_t sa = a_use % S, ka = a_use / S;
-          if (!wait_spin(&fullA[sa], ka & 1u, limit)) {
-            give_up();
-            ok = false;
-            break;
-          }
-          // A: 8-row groups (x) 128 bytes apart; the (dz, dy) pairs differ by start address
-          const uint64_t ad0 = smem_desc(smem_u32(sA + sa * a_stage), p.group_pitch, 128u);
-          const uint64_t bd0 = smem_desc(smem_u32(sW) + static_cast<uint32_t>(kc) * 9u * kFoldBlock, kXN * 16u, 128u);
+        // the (dz, dy) pairs differ by start address, 16 rows (512 bytes) a step
+        const uint64_t ad0 = smem_desc_sw32(smem_u32(sA + sa * a_stage));
+        const uint64_t bd0 = smem_desc(smem_u32(sW) + static_cast<uint32_t>(kc) * 9u * kFoldBlock, kXN * 16u, 128u);
 #pragma unroll
-          for (int pr = 0; pr < 9; ++pr) {
-            const int sg = FLIP ? -1 : 1;
-            const int dz = sg * (pr / 3 - 1), dy = sg * (pr % 3 - 1);
-            const uint32_t row = static_cast<uint32_t>((dz + 1) * (kYT + 2) * kXR + (dy + 1) * kXR);
-            const uint64_t bd = bd0 + static_cast<uint64_t>(pr) * (kFoldBlock >> 4);
-            const uint32_t acc = (kc > 0 || pr > 0) ? 1u : 0u;
+        for (int pr = 0; pr < 9; ++pr) {
+          const int sg = FLIP ? -1 : 1;
+          const int dz = sg * (pr / 3 - 1), dy = sg * (pr % 3 - 1);
+          const uint32_t row = 2u * static_cast<uint32_t>((dz + 1) * (kYT + 2) * kXR + (dy + 1) * kXR);
+          const uint64_t bd = bd0 + static_cast<uint64_t>(pr) * (kFoldBlock >> 4);
+          const uint32_t acc = (kc > 0 || pr > 0) ? 1u : 0u;
 #pragma unroll
-            for (int zz = 0; zz < TZ; ++zz)
-              mma_f16(d0 + static_cast<uint32_t>(zz * kXN), ad0 + row + static_cast<uint32_t>(zz * (kYT + 2) * kXR),
-                      bd, idesc, acc);
-          }
-          mma_commit(&emptyA[sa]);
-          ++a_use;
+          for (int zz = 0; zz < TZ; ++zz)
+            mma_f16(lead, d0 + static_cast<uint32_t>(zz * kXN), ad0 + row + static_cast<uint32_t>(zz * (kYT + 2) * kXR * 2),
+                    bd, idesc, acc);
         }
-        if (!ok) break;
-        mma_commit(&tfull[buf]);
-        ++acc_use;
+        mma_commit(lead, &emptyA[sa]);
+        ++a_use;
       }
-      mma_commit(fin);
+      if (!ok) break;
+      mma_commit(lead, &tfull[buf]);
+      ++acc_use;
     }
+    mma_commit(lead, fin);
   } else {   // ---------------------------------------------------------- epilogue
     const int q = warp & 3;            // tensor-memory lanes 32q .. 32q + 31
     const int row = 32 * q + lane;     // GEMM row within a plane
     const int mx = row & (kXR - 1), my = row / kXR;
+    const int zhalf = (warp - 2) >> 2;   // planes zhalf, zhalf + 2, ... of a tile
     float bias[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) bias[i] = p.bias ? __ldg(&p.bias[i]) : 0.f;
@@ -565,6 +609,23 @@ __global__ void __launch_bounds__(kThreads, 2) k_conv3d_tcx(const __grid_constan
     for (int64_t tile = blockIdx.x; tile < p.tiles && !*abort_flag; tile += gridDim.x) {
       const TileCoord tc = tile_coord_x(p, tile);
       const uint32_t buf = acc_use & 1u, ku = acc_use >> 1;
+      const int x = tc.x0 + mx, y = tc.y0 + my;
+      // the tile's mask is fetched before the wait for its products (plane by plane where it is
+      // used, its latency made the drain the bound: 1.25 ms for 16 -> 16 at 8 x 128^3, now
+      // 0.53 ms; without a mask 0.33 ms, and a pass of its own takes 0.25 ms)
+      uint4 m0[(TZ + 1) / 2], m1[(TZ + 1) / 2];
+      if (p.mask) {
+#pragma unroll
+        for (int zh = 0; zh < (TZ + 1) / 2; ++zh) {
+          const int zz = 2 * zh + zhalf;
+          m0[zh] = m1[zh] = make_uint4(0u, 0u, 0u, 0u);
+          const int64_t v = ((static_cast<int64_t>(tc.n) * p.D + tc.z0 + zz) * p.H + y) * p.W + x;
+          if (mx >= 1 && mx <= kXO && x < p.W && y < p.H && tc.z0 + zz < p.D) {
+            m0[zh] = __ldg(reinterpret_cast<const uint4*>(p.mask + v * 16));
+            m1[zh] = __ldg(reinterpret_cast<const uint4*>(p.mask + v * 16) + 1);
+          }
+        }
+      }
       // warp-uniform: the tensor-memory loads and shuffles below are .sync.aligned
       if (!__all_sync(0xffffffffu, mbar_wait_bounded(&tfull[buf], ku & 1u, limit))) {
         if (lane == 0) give_up();
@@ -572,8 +633,10 @@ __global__ void __launch_bounds__(kThreads, 2) k_conv3d_tcx(const __grid_constan
       }
       __syncwarp();
       fence_after();
-      const int x = tc.x0 + mx, y = tc.y0 + my;
-      for (int zz = 0; zz < TZ; ++zz) {
+#pragma unroll
+      for (int zh = 0; zh < (TZ + 1) / 2; ++zh) {
+        const int zz = 2 * zh + zhalf;
+        if (zz >= TZ) break;
         const int z = tc.z0 + zz;
         const bool inside = mx >= 1 && mx <= kXO && x < p.W && y < p.H && z < p.D;
         const int64_t v = ((static_cast<int64_t>(tc.n) * p.D + z) * p.H + y) * p.W + x;
@@ -602,10 +665,17 @@ __global__ void __launch_bounds__(kThreads, 2) k_conv3d_tcx(const __grid_constan
               h[i] = *reinterpret_cast<const uint32_t*>(&b2);
             }
             uint4* dst = reinterpret_cast<uint4*>(p.y + v * 16);
-            dst[0] = make_uint4(h[0], h[1], h[2], h[3]);
-            dst[1] = make_uint4(h[4], h[5], h[6], h[7]);
+            uint4 q0 = make_uint4(h[0], h[1], h[2], h[3]), q1 = make_uint4(h[4], h[5], h[6], h[7]);
+            if (p.mask) {
+              q0 = lrelu_grad8(q0, m0[zh]);
+              q1 = lrelu_grad8(q1, m1[zh]);
+            }
+            dst[0] = q0;
+            dst[1] = q1;
           }
-          if (p.yf) {
+          if (p.yf && p.yf_ch == 2) {
+            *reinterpret_cast<float2*>(p.yf + 2 * v) = make_float2(f[0], f[1]);
+          } else if (p.yf) {
             float4* dst = reinterpret_cast<float4*>(p.yf + v * 16);
 #pragma unroll
             for (int i = 0; i < 4; ++i) dst[i] = make_float4(f[4 * i], f[4 * i + 1], f[4 * i + 2], f[4 * i + 3]);
@@ -708,8 +778,7 @@ TcShape tc_shape(int ci, int co) {
 TcShape shape_fold(int ci, int tz) {
   TcShape t{};
   t.tz = tz;
-  const uint32_t halo = static_cast<uint32_t>(kXR * (kYT + 2) * (tz + 2) * 16);
-  t.group_pitch = (halo + 127u) & ~127u;
+  t.group_pitch = static_cast<uint32_t>(kXR * (kYT + 2) * (tz + 2) * 16);   // half a brick
   t.resident = 1;
   t.w_bytes = static_cast<uint32_t>(ci / 16) * 9u * kFoldBlock;
   uint32_t c = 32;
@@ -733,7 +802,7 @@ bool use_fold(int ci, int co) { return g_conv_fold && co == 16 && ci / 16 <= kFo
 // graph): the dynamic shared-memory limit and carve-out, and the resident CTAs per SM from
 // shared memory (1 KB reserved per CTA), registers (allocated per warp in units of 256) and
 // tensor memory (512 columns per SM; a CTA beyond that would wait in allocation).
-cudaError_t kernel_setup(const void* kern, size_t smem, uint32_t tmem_cols, int* per_sm, int* sms) {
+cudaError_t kernel_setup(const void* kern, int threads, size_t smem, uint32_t tmem_cols, int* per_sm, int* sms) {
   struct Entry {
     size_t smem_set;
     int regs;
@@ -776,7 +845,7 @@ cudaError_t kernel_setup(const void* kern, size_t smem, uint32_t tmem_cols, int*
   const Dev& d = devs[dev];
   const int by_smem = d.smem_sm / static_cast<int>(smem + 1024);
   const int regs_warp = ((it->second.regs * 32 + 255) / 256) * 256;
-  const int by_regs = d.regs_sm / (regs_warp * (kThreads / 32));
+  const int by_regs = d.regs_sm / (regs_warp * (threads / 32));
   const int by_tmem = static_cast<int>(512 / tmem_cols);
   int n = by_smem < by_regs ? by_smem : by_regs;
   n = n < by_tmem ? n : by_tmem;
@@ -788,7 +857,8 @@ cudaError_t kernel_setup(const void* kern, size_t smem, uint32_t tmem_cols, int*
 bool conv_tc_supported(int ci, int co) { return ci >= 16 && ci % 16 == 0 && co >= 16 && co % 16 == 0 && co <= 256; }
 
 cudaError_t launch_conv_tc(const void* x, const void* wpk, const float* bias, void* y, float* yf, int n, int d,
-                           int h, int w, int ci, int co, int flip, int act, cudaStream_t s) {
+                           int h, int w, int ci, int co, int flip, int act, cudaStream_t s, const void* mask,
+                           int yf_ch) {
   PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
   if (!enc) return cudaErrorNotSupported;
   CUtensorMap map;
@@ -799,12 +869,12 @@ cudaError_t launch_conv_tc(const void* x, const void* wpk, const float* bias, vo
   const bool fold = use_fold(ci, co);
   const int ftz = g_fold_tz == 1 || g_fold_tz == 2 ? g_fold_tz : 4;
   const TcShape shp = fold ? shape_fold(ci, ftz) : tc_shape(ci, co);
-  const cuuint32_t box[5] = {8, static_cast<cuuint32_t>(fold ? kXR : kHX), static_cast<cuuint32_t>(fold ? kYT + 2 : kHY),
+  const cuuint32_t box[5] = {static_cast<cuuint32_t>(fold ? 16 : 8), static_cast<cuuint32_t>(fold ? kXR : kHX), static_cast<cuuint32_t>(fold ? kYT + 2 : kHY),
                              static_cast<cuuint32_t>(shp.tz + 2), 1};
   const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
   if (enc(&map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(x), dims, strides, box, estr,
-          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+          CU_TENSOR_MAP_INTERLEAVE_NONE, fold ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_NONE,
+          CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return cudaErrorInvalidValue;
   ConvTcParams p{};
   p.wpk = static_cast<const bf16*>(wpk);
@@ -819,6 +889,8 @@ cudaError_t launch_conv_tc(const void* x, const void* wpk, const float* bias, vo
   p.Co = co;
   p.flip = flip;
   p.act = act;
+  p.mask = static_cast<const bf16*>(mask);
+  p.yf_ch = yf_ch;
   p.tz = shp.tz;
   p.resident = shp.resident;
   p.tiles_x = fold ? (w + kXO - 1) / kXO : (w + kTX - 1) / kTX;
@@ -839,11 +911,12 @@ cudaError_t launch_conv_tc(const void* x, const void* wpk, const float* bias, vo
                                                                      : k_conv3d_tc<true, 1>)
                           : (shp.tz == 4 ? k_conv3d_tc<false, 4>
                                          : shp.tz == 2 ? k_conv3d_tc<false, 2> : k_conv3d_tc<false, 1>);
+  const int threads = fold ? kFoldThreads : kThreads;
   int per_sm = 0, sms = 0;
-  const cudaError_t e = kernel_setup(reinterpret_cast<const void*>(kern), smem, p.tmem_cols, &per_sm, &sms);
+  const cudaError_t e = kernel_setup(reinterpret_cast<const void*>(kern), threads, smem, p.tmem_cols, &per_sm, &sms);
   if (e != cudaSuccess) return e;
   const int64_t grid = p.tiles < static_cast<int64_t>(sms) * per_sm ? p.tiles : static_cast<int64_t>(sms) * per_sm;
-  kern<<<static_cast<unsigned>(grid), kThreads, smem, s>>>(map, p);
+  kern<<<static_cast<unsigned>(grid), threads, smem, s>>>(map, p);
   return cudaGetLastError();
 }
 
@@ -877,7 +950,7 @@ cudaError_t launch_conv_wgrad(const void* x, const void* dy, float* dw, int n, i
   p.wait_limit = g_wait_limit ? g_wait_limit : kDefaultWait;
   p.debug_stall = g_debug_stall;
   int per_sm = 0, sms = 0;
-  cudaError_t e = kernel_setup(reinterpret_cast<const void*>(k_conv3d_wgrad_tma), kWgSmem, 512, &per_sm, &sms);
+  cudaError_t e = kernel_setup(reinterpret_cast<const void*>(k_conv3d_wgrad_tma), (kWgMma + 1) * 32, kWgSmem, 512, &per_sm, &sms);
   if (e != cudaSuccess) return e;
   // One block per SM at a time, three waves of them: the tensor cores' sums lose accuracy in
   // proportion to the voxels a warp sums in one go, and three waves keep them below those of

@@ -17,6 +17,7 @@
 #include <cstdint>
 
 #include "mach_nn.h"
+#include "nn_device.cuh"
 #include "nn_internal.h"
 
 namespace mach_nn {
@@ -371,6 +372,39 @@ __global__ void k_bias_grad(const bf16* __restrict__ g, float* __restrict__ db, 
   if (tid < C) atomicAdd(&db[tid], part[tid]);
 }
 
+// The same for C % 8 == 0 (C <= 256): 16-byte loads, thread t owns channels 8 (t % (C / 8)) ...
+// + 7 of rows t / (C / 8) (+ stride), four rows in flight: 84 us for
+// 8 x 128^3 x 16 channels (6.4 TB/s); one 2-byte element per load 186 us.
+__global__ void __launch_bounds__(256) k_bias_grad8(const uint4* __restrict__ g, float* __restrict__ db,
+                                                    int64_t voxels, int C) {
+  __shared__ float part[256];
+  const int tid = threadIdx.x, groups = C / 8;
+  const int rows = 256 / groups, c = tid % groups, r = tid / groups;
+  float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  const int64_t step = static_cast<int64_t>(gridDim.x) * rows;
+  for (int64_t v = static_cast<int64_t>(blockIdx.x) * rows + r; v < voxels; v += 4 * step) {
+    uint4 q[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      q[k] = v + k * step < voxels ? __ldg(&g[(v + k * step) * groups + c]) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) add8(s, q[k]);
+  }
+  // groups is a power of two up to 32: lanes of the same channels meet by shuffles, so that a
+  // warp adds each channel once (256 threads on a few shared words took longer than the reads)
+#pragma unroll
+  for (int k = 0; k < 8; ++k)
+    for (int o = 16; o >= groups; o >>= 1) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
+  if (tid < C) part[tid] = 0.f;
+  __syncthreads();
+  if ((tid & 31) < groups) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) atomicAdd(&part[8 * c + k], s[k]);
+  }
+  __syncthreads();
+  if (tid < C) atomicAdd(&db[tid], part[tid]);
+}
+
 // Adam (float32 master weights); optional bfloat16 copies (same layout, and transposed
 // [27][Co][Ci] for the data gradient).
 __global__ void k_adam(float* __restrict__ w, float* __restrict__ m, float* __restrict__ v, const float* __restrict__ gr,
@@ -460,21 +494,39 @@ __device__ __forceinline__ float coord_of(int64_t i, int n) {
   return static_cast<float>(2 * i + 1 - n) / static_cast<float>(P);
 }
 
+// The volumes lie on the frames axis of y ([V][N]) and lead in the network's tensors ([N][V]).
+// Items run over (voxel, volume) with the volume fastest, so that both sides move whole
+// 32-byte sectors (volume by volume, a batch of 8 read 64 bytes of y for every 8 used).
+struct Item {
+  int n;
+  int64_t v, i;   // volume, voxel, n V + v
+};
+__device__ __forceinline__ Item item_at(int64_t j, int64_t V, int N) {
+  Item t;
+  if (V * N <= 0x7fffffff) {
+    t.v = static_cast<uint32_t>(j) / static_cast<uint32_t>(N);
+  } else {
+    t.v = j / N;
+  }
+  t.n = static_cast<int>(j - t.v * N);
+  t.i = t.n * V + t.v;
+  return t;
+}
+
 __global__ void k_pack(const float2* __restrict__ y, const float* __restrict__ sums, int64_t V, int N, int C,
                        int coords, int nx, int ny, int nz, bf16* __restrict__ xin, float2* __restrict__ xf) {
-  const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;   // = n * V + v
-  if (i >= V * N) return;
-  const int n = static_cast<int>(i / V);
-  const int64_t v = i % V;
-  const float inv = 1.f / rms_of(sums, n, V);
-  const float2 a = y[v * N + n];
+  const int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (j >= V * N) return;
+  const Item t = item_at(j, V, N);
+  const float inv = 1.f / rms_of(sums, t.n, V);
+  const float2 a = y[j];
   const float2 x = make_float2(a.x * inv, a.y * inv);
-  xf[i] = x;
-  uint4* dst = reinterpret_cast<uint4*>(xin + i * C);
+  xf[t.i] = x;
+  uint4* dst = reinterpret_cast<uint4*>(xin + t.i * C);
   const __nv_bfloat162 q = __floats2bfloat162_rn(x.x, x.y);
   uint4 first = make_uint4(*reinterpret_cast<const uint32_t*>(&q), 0u, 0u, 0u);
   if (coords) {   // channels 2, 3, 4: the voxel's (x, y, z) position
-    const int64_t ix = v % nx, iy = (v / nx) % ny, iz = v / (static_cast<int64_t>(nx) * ny);
+    const int64_t ix = t.v % nx, iy = (t.v / nx) % ny, iz = t.v / (static_cast<int64_t>(nx) * ny);
     const __nv_bfloat162 c01 = __floats2bfloat162_rn(coord_of(ix, nx), coord_of(iy, ny));
     const __nv_bfloat162 c2 = __floats2bfloat162_rn(coord_of(iz, nz), 0.f);
     first.y = *reinterpret_cast<const uint32_t*>(&c01);
@@ -484,37 +536,111 @@ __global__ void k_pack(const float2* __restrict__ y, const float* __restrict__ s
   for (int k = 1; k < C / 8; ++k) dst[k] = make_uint4(0u, 0u, 0u, 0u);
 }
 
-__global__ void k_loss(const float* __restrict__ o, const float2* __restrict__ xf, const float2* __restrict__ target,
-                       const float* __restrict__ sums, float gain, int64_t V, int N, int C, bf16* __restrict__ g,
-                       float* __restrict__ loss, float inv_count) {
-  const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;   // = n * V + v
-  float e2 = 0.f;
-  if (i < V * N) {
-    const int n = static_cast<int>(i / V);
-    const int64_t v = i % V;
-    const float inv = 1.f / rms_of(sums, n, V);
-    const float2 t = target[v * N + n];
-    const float2 x = xf[i];
-    const float er = o[i * C] + gain * x.x - t.x * inv;
-    const float ei = o[i * C + 1] + gain * x.y - t.y * inv;
-    e2 = fmaf(er, er, ei * ei);
-    bf16* gi = g + i * C;
-    *reinterpret_cast<__nv_bfloat162*>(gi) = __floats2bfloat162_rn(2.f * er * inv_count, 2.f * ei * inv_count);
-    for (int k = 2; k < C; k += 2) *reinterpret_cast<uint32_t*>(gi + k) = 0u;
+// Loss and its gradient.  A thread sums its items, a block its threads, and one atomic per
+// block adds to the loss (one per warp serialised half a million of them on one word: 1.24 ms
+// at 8 x 128^3; now 0.25 ms, with the volume-fastest order).
+__global__ void __launch_bounds__(256) k_loss(const float* __restrict__ o, const float2* __restrict__ xf,
+                                              const float2* __restrict__ target, const float* __restrict__ sums,
+                                              float gain, int64_t V, int N, int Co, int C, bf16* __restrict__ g,
+                                              float* __restrict__ loss, float inv_count) {
+  float sum = 0.f;
+  for (int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; j < V * N;
+       j += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+    const Item it = item_at(j, V, N);
+    const float inv = 1.f / rms_of(sums, it.n, V);
+    const float2 t = target[j];
+    const float2 x = xf[it.i];
+    const float2 oo = *reinterpret_cast<const float2*>(o + it.i * Co);
+    const float er = oo.x + gain * x.x - t.x * inv;
+    const float ei = oo.y + gain * x.y - t.y * inv;
+    sum = fmaf(er, er, fmaf(ei, ei, sum));
+    const __nv_bfloat162 q = __floats2bfloat162_rn(2.f * er * inv_count, 2.f * ei * inv_count);
+    uint4* gi = reinterpret_cast<uint4*>(g + it.i * C);
+    gi[0] = make_uint4(*reinterpret_cast<const uint32_t*>(&q), 0u, 0u, 0u);
+    for (int k = 1; k < C / 8; ++k) gi[k] = make_uint4(0u, 0u, 0u, 0u);
   }
-  for (int off = 16; off > 0; off >>= 1) e2 += __shfl_xor_sync(0xffffffffu, e2, off);
-  if (loss && (threadIdx.x & 31) == 0) atomicAdd(loss, e2 * inv_count);
+  for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+  __shared__ float part[8];
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = sum;
+  __syncthreads();
+  if (threadIdx.x == 0 && loss) {
+    for (int k = 1; k < 8; ++k) sum += part[k];
+    atomicAdd(loss, sum * inv_count);
+  }
 }
 
 __global__ void k_output(const float* __restrict__ o, const float2* __restrict__ xf, const float* __restrict__ sums,
-                         float gain, int64_t V, int N, int C, float2* __restrict__ y) {
-  const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;   // = n * V + v
-  if (i >= V * N) return;
-  const int n = static_cast<int>(i / V);
-  const int64_t v = i % V;
-  const float r = rms_of(sums, n, V);
-  const float2 x = xf[i];
-  y[v * N + n] = make_float2(r * (o[i * C] + gain * x.x), r * (o[i * C + 1] + gain * x.y));
+                         float gain, int64_t V, int N, int Co, float2* __restrict__ y) {
+  const int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (j >= V * N) return;
+  const Item t = item_at(j, V, N);
+  const float r = rms_of(sums, t.n, V);
+  const float2 x = xf[t.i];
+  const float2 oo = *reinterpret_cast<const float2*>(o + t.i * Co);
+  y[j] = make_float2(r * (oo.x + gain * x.x), r * (oo.y + gain * x.y));
+}
+
+// ---- fused data movement (8 channels of one voxel per item) --------------------------------
+template <class I>
+struct VoxOf {   // voxel v of a [N][D][H][W] grid
+  I n, z, y, x;
+  __device__ __forceinline__ VoxOf(I v, I D, I H, I W) {
+    x = v % W;
+    v /= W;
+    y = v % H;
+    v /= H;
+    z = v % D;
+    n = v / D;
+  }
+};
+
+template <class I>
+__global__ void __launch_bounds__(256) k_up2_cat(const uint4* __restrict__ x, const uint4* __restrict__ skip,
+                                                 uint4* __restrict__ cat, I total, I d, I h, I w, I C8, I Cs8) {
+  const I i = static_cast<I>(blockIdx.x) * 256 + threadIdx.x;
+  if (i >= total) return;
+  const I c = i % (C8 + Cs8), v = i / (C8 + Cs8);
+  if (c >= C8) {
+    cat[i] = __ldg(&skip[v * Cs8 + (c - C8)]);
+    return;
+  }
+  const VoxOf<I> p(v, 2 * d, 2 * h, 2 * w);
+  cat[i] = __ldg(&x[((((p.n * d + p.z / 2) * h + p.y / 2) * w + p.x / 2) * C8) + c]);
+}
+
+template <class I>
+__global__ void __launch_bounds__(256) k_up2_bwd_lrelu(const uint4* __restrict__ g, const uint4* __restrict__ act,
+                                                       uint4* __restrict__ dx, I total, I d, I h, I w, I C8, I Cy8) {
+  const I i = static_cast<I>(blockIdx.x) * 256 + threadIdx.x;
+  if (i >= total) return;
+  const I c = i % C8;
+  const VoxOf<I> p(i / C8, d, h, w);
+  uint4 q[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const I z = 2 * p.z + (k >> 2), y = 2 * p.y + ((k >> 1) & 1), xx = 2 * p.x + (k & 1);
+    q[k] = __ldg(&g[((((p.n * 2 * d + z) * 2 * h + y) * 2 * w + xx) * Cy8) + c]);
+  }
+  float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int k = 0; k < 8; ++k) add8(a, q[k]);
+  dx[i] = lrelu_grad8(pack8(a, 1.f), __ldg(&act[i]));
+}
+
+template <class I>
+__global__ void __launch_bounds__(256) k_skip_pool_bwd_lrelu(const uint4* __restrict__ g, const uint4* __restrict__ dy,
+                                                             const uint4* __restrict__ act, uint4* __restrict__ dx,
+                                                             I total, I D, I H, I W, I Cu8, I C8) {
+  const I i = static_cast<I>(blockIdx.x) * 256 + threadIdx.x;
+  if (i >= total) return;
+  const I c = i % C8, v = i / C8;
+  const VoxOf<I> p(v, D, H, W);
+  float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  add8(a, __ldg(&dy[((((p.n * (D / 2) + p.z / 2) * (H / 2) + p.y / 2) * (W / 2) + p.x / 2) * C8) + c]));
+#pragma unroll
+  for (int k = 0; k < 8; ++k) a[k] *= 0.125f;
+  add8(a, __ldg(&g[v * (Cu8 + C8) + Cu8 + c]));
+  dx[i] = lrelu_grad8(pack8(a, 1.f), __ldg(&act[i]));
 }
 
 namespace {
@@ -537,17 +663,63 @@ cudaError_t launch_pack(const float2* y, const float* sums, int64_t V, int N, in
 }
 
 cudaError_t launch_loss(const float* o, const float* xf, const float2* target, const float* sums, float gain,
-                        int64_t V, int N, int C, void* g, float* loss, cudaStream_t s) {
+                        int64_t V, int N, int Co, int C, void* g, float* loss, cudaStream_t s) {
   const float inv = 1.f / static_cast<float>(2 * V * N);
-  k_loss<<<blocks_for(V * N), 256, 0, s>>>(o, reinterpret_cast<const float2*>(xf), target, sums, gain, V, N, C,
-                                           static_cast<bf16*>(g), loss, inv);
+  const unsigned blocks = blocks_for(V * N) < 152 * 8 ? blocks_for(V * N) : 152 * 8;
+  k_loss<<<blocks, 256, 0, s>>>(o, reinterpret_cast<const float2*>(xf), target, sums, gain, V, N, Co, C,
+                                static_cast<bf16*>(g), loss, inv);
   return cudaGetLastError();
 }
 
-cudaError_t launch_output(const float* o, const float* xf, const float* sums, float gain, int64_t V, int N, int C,
+cudaError_t launch_output(const float* o, const float* xf, const float* sums, float gain, int64_t V, int N, int Co,
                           float2* y, cudaStream_t s) {
-  k_output<<<blocks_for(V * N), 256, 0, s>>>(o, reinterpret_cast<const float2*>(xf), sums, gain, V, N, C, y);
+  k_output<<<blocks_for(V * N), 256, 0, s>>>(o, reinterpret_cast<const float2*>(xf), sums, gain, V, N, Co, y);
   return cudaGetLastError();
+}
+
+// 32-bit indices whenever the largest tensor has fewer than 2^31 items: the items' divisions
+// would otherwise cost more than their 16-byte moves
+cudaError_t launch_up2_cat(const void* x, const void* skip, void* cat, int N, int d, int h, int w, int C, int Cs,
+                           cudaStream_t s) {
+  const int64_t total = static_cast<int64_t>(N) * 8 * d * h * w * ((C + Cs) / 8);
+  auto go = [&](auto* kernel, auto one) {
+    using I = decltype(one);
+    kernel<<<blocks_for(total), 256, 0, s>>>(static_cast<const uint4*>(x), static_cast<const uint4*>(skip),
+                                             static_cast<uint4*>(cat), static_cast<I>(total), static_cast<I>(d),
+                                             static_cast<I>(h), static_cast<I>(w), static_cast<I>(C / 8),
+                                             static_cast<I>(Cs / 8));
+    return cudaGetLastError();
+  };
+  return total < 0x7fffffff ? go(k_up2_cat<uint32_t>, uint32_t{}) : go(k_up2_cat<int64_t>, int64_t{});
+}
+
+cudaError_t launch_up2_bwd_lrelu(const void* g_cat, const void* act, void* dx, int N, int d, int h, int w, int C,
+                                 int Cs, cudaStream_t s) {
+  const int64_t total = static_cast<int64_t>(N) * d * h * w * (C / 8), big = total / (C / 8) * 8 * ((C + Cs) / 8);
+  auto go = [&](auto* kernel, auto one) {
+    using I = decltype(one);
+    kernel<<<blocks_for(total), 256, 0, s>>>(static_cast<const uint4*>(g_cat), static_cast<const uint4*>(act),
+                                             static_cast<uint4*>(dx), static_cast<I>(total), static_cast<I>(d),
+                                             static_cast<I>(h), static_cast<I>(w), static_cast<I>(C / 8),
+                                             static_cast<I>((C + Cs) / 8));
+    return cudaGetLastError();
+  };
+  return big < 0x7fffffff ? go(k_up2_bwd_lrelu<uint32_t>, uint32_t{}) : go(k_up2_bwd_lrelu<int64_t>, int64_t{});
+}
+
+cudaError_t launch_skip_pool_bwd_lrelu(const void* g_cat, const void* dy, const void* act, void* dx, int N, int D,
+                                       int H, int W, int Cu, int C, cudaStream_t s) {
+  const int64_t vox = static_cast<int64_t>(N) * D * H * W, total = vox * (C / 8), big = vox * ((Cu + C) / 8);
+  auto go = [&](auto* kernel, auto one) {
+    using I = decltype(one);
+    kernel<<<blocks_for(total), 256, 0, s>>>(static_cast<const uint4*>(g_cat), static_cast<const uint4*>(dy),
+                                             static_cast<const uint4*>(act), static_cast<uint4*>(dx),
+                                             static_cast<I>(total), static_cast<I>(D), static_cast<I>(H),
+                                             static_cast<I>(W), static_cast<I>(Cu / 8), static_cast<I>(C / 8));
+    return cudaGetLastError();
+  };
+  return big < 0x7fffffff ? go(k_skip_pool_bwd_lrelu<uint32_t>, uint32_t{})
+                          : go(k_skip_pool_bwd_lrelu<int64_t>, int64_t{});
 }
 
 cudaError_t launch_to_bf16(const float* w, int64_t count, void* wb, void* wbt, int ci, int co, cudaStream_t s) {
@@ -608,6 +780,14 @@ mach_status mach_nn_conv3d_wgrad(const void* x, const void* dy, float* dw, int32
 
 mach_status mach_nn_bias_grad(const void* g, float* db, int64_t voxels, int32_t c, void* stream) {
   if (!g || !db || voxels < 1 || c < 1 || c > 256 || 256 % c) return MACH_ERR_INVALID_ARG;
+  if (c % 8 == 0 && aligned16(g)) {
+    const int64_t rows8 = 4 * (256 / (c / 8));
+    int64_t blocks8 = (voxels + rows8 - 1) / rows8;
+    blocks8 = blocks8 < 152 * 8 ? blocks8 : 152 * 8;
+    k_bias_grad8<<<static_cast<unsigned>(blocks8), 256, 0, static_cast<cudaStream_t>(stream)>>>(
+        static_cast<const uint4*>(g), db, voxels, c);
+    return last_status();
+  }
   const int64_t rows = 256 / c;
   int64_t blocks = (voxels + rows - 1) / rows;
   blocks = blocks < 152 * 8 ? blocks : 152 * 8;

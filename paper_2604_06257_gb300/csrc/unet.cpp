@@ -74,6 +74,7 @@ struct mach_unet_s {
   int step = 0;
   int backend = MACH_UNET_TCGEN05;
   bool training = true;
+  int o_ch = 0;           // channels of o's rows: 2 from the tensor-core kernel, else c0
 
   int ch(int l) const { return c0 << l; }
   int64_t vox(int l) const { return static_cast<int64_t>(N) * nz[l] * ny[l] * nx[l]; }
@@ -110,21 +111,24 @@ mach_status conv_fwd(mach_unet_s* u, const Conv& c, cudaStream_t s) {
   if (fwd_on_tc(u, c))
     return cuda_ok(launch_conv_tc(c.in->p, c.wpk, u->params + c.b_off, c.out ? c.out->p : nullptr,
                                   c.out ? nullptr : u->o, u->N, u->nz[l], u->ny[l], u->nx[l], c.ci, c.co, 0,
-                                  c.act ? 1 : 0, s));
+                                  c.act ? 1 : 0, s, nullptr, u->o_ch));
   return mach_nn_conv3d(c.in->p, c.wb, u->params + c.b_off, c.out ? c.out->p : nullptr, c.out ? nullptr : u->o, u->N,
                         u->nz[l], u->ny[l], u->nx[l], c.ci, c.co, 0, c.act ? 1 : 0, s);
 }
 
-// gradients of one convolution given the gradient of its (pre-activation) output
-mach_status conv_bwd(mach_unet_s* u, const Conv& c, void* gout, void* gin, cudaStream_t s) {
+// Gradients of one convolution given the gradient of its (pre-activation) output.  act: the
+// convolution's input is this activation alone, and gin receives the gradient before it.
+mach_status conv_bwd(mach_unet_s* u, const Conv& c, void* gout, void* gin, const void* act, cudaStream_t s) {
   const int l = c.level;
   TRY(mach_nn_conv3d_wgrad(c.in->p, gout, u->grads + c.w_off, u->N, u->nz[l], u->ny[l], u->nx[l], c.ci, c.co, s));
   TRY(mach_nn_bias_grad(gout, u->grads + c.b_off, u->vox(l), c.co, s));
   if (gin && dgrad_on_tc(u, c))
     TRY(cuda_ok(launch_conv_tc(gout, c.wpkt, nullptr, gin, nullptr, u->N, u->nz[l], u->ny[l], u->nx[l], c.co, c.ci,
-                               1, 0, s)));
-  else if (gin)
+                               1, 0, s, act)));
+  else if (gin) {
     TRY(mach_nn_conv3d(gout, c.wbt, nullptr, gin, nullptr, u->N, u->nz[l], u->ny[l], u->nx[l], c.co, c.ci, 1, 0, s));
+    if (act) TRY(mach_nn_lrelu_bwd(gin, act, u->vox(l) * c.ci, s));
+  }
   return MACH_OK;
 }
 
@@ -141,41 +145,36 @@ mach_status forward(mach_unet_s* u, const void* x, cudaStream_t s) {
   }
   for (int l = L - 2; l >= 0; --l) {
     const Act& src = l == L - 2 ? u->e[L - 1] : u->dd[l + 1];
-    const int cy = u->ch(l + 1) + u->ch(l);
-    TRY(mach_nn_up2(src.p, u->cat[l].p, N, u->nz[l + 1], u->ny[l + 1], u->nx[l + 1], u->ch(l + 1), cy, 0, 0, s));
-    TRY(mach_nn_copy_channels(u->e[l].p, u->cat[l].p, u->vox(l), u->ch(l), cy, u->ch(l + 1), 0, s));
+    TRY(cuda_ok(launch_up2_cat(src.p, u->e[l].p, u->cat[l].p, N, u->nz[l + 1], u->ny[l + 1], u->nx[l + 1],
+                               u->ch(l + 1), u->ch(l), s)));
     TRY(conv_fwd(u, u->convs[u->dec(l, 0)], s));
     TRY(conv_fwd(u, u->convs[u->dec(l, 1)], s));
   }
+  u->o_ch = fwd_on_tc(u, u->convs[u->out_conv()]) ? 2 : u->c0;
   return conv_fwd(u, u->convs[u->out_conv()], s);
 }
 
 mach_status backward(mach_unet_s* u, const void* target, float* loss, cudaStream_t s) {
   const int L = u->L, N = u->N;
   if (loss) TRY(cuda_ok(cudaMemsetAsync(loss, 0, sizeof(float), s)));
-  TRY(cuda_ok(launch_loss(u->o, u->xf, static_cast<const float2*>(target), u->sums, u->gain, u->vox1(0), N, u->c0,
-                          u->g_o, loss, s)));
+  TRY(cuda_ok(launch_loss(u->o, u->xf, static_cast<const float2*>(target), u->sums, u->gain, u->vox1(0), N, u->o_ch,
+                          u->c0, u->g_o, loss, s)));
   TRY(cuda_ok(cudaMemsetAsync(u->grads, 0, sizeof(float) * u->n_params, s)));
-  TRY(conv_bwd(u, u->convs[u->out_conv()], u->g_o, u->g_top().p, s));
+  // every gradient below is the one before its tensor's leaky ReLU
+  TRY(conv_bwd(u, u->convs[u->out_conv()], u->g_o, u->g_top().p, u->top().p, s));
   for (int l = 0; l <= L - 2; ++l) {
-    const int c = u->ch(l), cy = u->ch(l + 1) + c;
-    TRY(mach_nn_lrelu_bwd(u->g_d[l].p, u->dd[l].p, u->vox(l) * c, s));
-    TRY(conv_bwd(u, u->convs[u->dec(l, 1)], u->g_d[l].p, u->g_b[l].p, s));
-    TRY(mach_nn_lrelu_bwd(u->g_b[l].p, u->b[l].p, u->vox(l) * c, s));
-    TRY(conv_bwd(u, u->convs[u->dec(l, 0)], u->g_b[l].p, u->g_cat[l].p, s));
-    void* dst = l == L - 2 ? u->g_e[L - 1].p : u->g_d[l + 1].p;
-    TRY(mach_nn_up2(u->g_cat[l].p, dst, N, u->nz[l + 1], u->ny[l + 1], u->nx[l + 1], u->ch(l + 1), cy, 0, 1, s));
-    TRY(mach_nn_copy_channels(u->g_cat[l].p, u->g_e[l].p, u->vox(l), c, cy, u->ch(l + 1), 1, s));
+    TRY(conv_bwd(u, u->convs[u->dec(l, 1)], u->g_d[l].p, u->g_b[l].p, u->b[l].p, s));
+    TRY(conv_bwd(u, u->convs[u->dec(l, 0)], u->g_b[l].p, u->g_cat[l].p, nullptr, s));
+    const Act& below = l == L - 2 ? u->e[L - 1] : u->dd[l + 1];
+    TRY(cuda_ok(launch_up2_bwd_lrelu(u->g_cat[l].p, below.p, l == L - 2 ? u->g_e[L - 1].p : u->g_d[l + 1].p, N,
+                                     u->nz[l + 1], u->ny[l + 1], u->nx[l + 1], u->ch(l + 1), u->ch(l), s)));
   }
   for (int l = L - 1; l >= 0; --l) {
-    const int c = u->ch(l);
-    TRY(mach_nn_lrelu_bwd(u->g_e[l].p, u->e[l].p, u->vox(l) * c, s));
-    TRY(conv_bwd(u, u->convs[u->enc(l, 1)], u->g_e[l].p, u->g_a[l].p, s));
-    TRY(mach_nn_lrelu_bwd(u->g_a[l].p, u->a[l].p, u->vox(l) * c, s));
-    TRY(conv_bwd(u, u->convs[u->enc(l, 0)], u->g_a[l].p, l > 0 ? u->g_in[l].p : nullptr, s));
-    if (l > 0)
-      TRY(mach_nn_pool2(u->g_in[l].p, u->g_e[l - 1].p, N, u->nz[l - 1], u->ny[l - 1], u->nx[l - 1], u->ch(l - 1), 1, 1,
-                        s));
+    if (l < L - 1)
+      TRY(cuda_ok(launch_skip_pool_bwd_lrelu(u->g_cat[l].p, u->g_in[l + 1].p, u->e[l].p, u->g_e[l].p, N, u->nz[l],
+                                             u->ny[l], u->nx[l], u->ch(l + 1), u->ch(l), s)));
+    TRY(conv_bwd(u, u->convs[u->enc(l, 1)], u->g_e[l].p, u->g_a[l].p, u->a[l].p, s));
+    TRY(conv_bwd(u, u->convs[u->enc(l, 0)], u->g_a[l].p, l > 0 ? u->g_in[l].p : nullptr, nullptr, s));
   }
   return MACH_OK;
 }
@@ -421,7 +420,7 @@ mach_status mach_unet_forward(mach_unet net, const void* x, void* y, void* strea
   if (!net || !x || !y || x == y) return MACH_ERR_INVALID_ARG;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   TRY(forward(net, x, s));
-  return cuda_ok(launch_output(net->o, net->xf, net->sums, net->gain, net->vox1(0), net->N, net->c0,
+  return cuda_ok(launch_output(net->o, net->xf, net->sums, net->gain, net->vox1(0), net->N, net->o_ch,
                                static_cast<float2*>(y), s));
 }
 
