@@ -161,8 +161,8 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-// Three tensor-memory loads of 16 columns each, one wait for all of them.
-__device__ __forceinline__ void tmem_ld16x3(uint32_t taddr, uint32_t (&a)[16], uint32_t (&b)[16],
+// Three tensor-memory loads of 16 columns, `apart` columns from one to the next, one wait for all of them.
+__device__ __forceinline__ void tmem_ld16x3(uint32_t taddr, uint32_t apart, uint32_t (&a)[16], uint32_t (&b)[16],
                                             uint32_t (&c)[16]) {
 #define MACH_TMEM_LD16(dst, addr)                                                                               \
   asm volatile(                                                                                                \
@@ -172,8 +172,8 @@ __device__ __forceinline__ void tmem_ld16x3(uint32_t taddr, uint32_t (&a)[16], u
         "=r"(dst[14]), "=r"(dst[15])                                                                           \
       : "r"(addr))
   MACH_TMEM_LD16(a, taddr);
-  MACH_TMEM_LD16(b, taddr + 16);
-  MACH_TMEM_LD16(c, taddr + 32);
+  MACH_TMEM_LD16(b, taddr + apart);
+  MACH_TMEM_LD16(c, taddr + 2 * apart);
 #undef MACH_TMEM_LD16
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
@@ -447,40 +447,41 @@ __global__ void __launch_bounds__(kThreads, 3) k_conv3d_tc(const __grid_constant
 }
 
 // ---------------------------------------------------------------------------------------
-// x-folded variant for 16 output channels.  With N = 16 each MMA reads a 4 KB A operand for
+// x-folded variant for 16 and 32 output channels.  With N = 16 each MMA reads a 4 KB A operand for
 // 16 columns of work, and the shared-memory operand reads, not the tensor core, set the
-// pace.  Folding the three x taps of a (dz, dy) pair into N gives one N = 48 MMA per pair:
-//   P_j[x'] = sum_ci W[dz, dy, j - 1][ci] X[x' + .., ci]   (j = 0, 1, 2 -> columns 16 j .. 16 j + 15)
+// pace.  Folding the three x taps of a (dz, dy) pair into N gives one N = 3 Co MMA per pair:
+//   P_j[x'] = sum_ci W[dz, dy, j - 1][ci] X[x' + .., ci]   (j = 0, 1, 2 -> columns Co j .. Co j + Co - 1)
 //   Y[x]    = P_0[x - s] + P_1[x] + P_2[x + s]             (s = 1, or -1 with flip)
 // so a tile's GEMM rows are 16 consecutive x positions (no x halo in the A brick) of which
 // the 14 inner ones are outputs; the epilogue shifts the outer column blocks by one row with
 // warp shuffles (rows are x-major, so x +- 1 is lane +- 1).  A tile is 16 (x) x 8 (y) x TZ (z)
 // rows, consecutive tiles 14 apart in x.  The weights are rearranged once per CTA into
-// per-(kc, dz, dy) blocks [g][j * 16 + co][8] (B operand: N = 48 rows 16 bytes apart, the
-// two 8-channel groups 768 bytes apart) and stay resident.  The A brick is loaded as rows of
+// per-(kc, dz, dy) blocks [g][j * Co + co][8] (B operand: N = 3 Co rows 16 bytes apart, the
+// two 8-channel groups 48 Co bytes apart) and stay resident.  The A brick is loaded as rows of
 // 16 channels with the 32-byte swizzle (one TMA element per voxel; no faster than two 8-channel
 // groups, but one load).
 constexpr int kXR = 16;                 // GEMM rows along x per tile
 constexpr int kXO = kXR - 2;            // outputs along x per tile
 constexpr int kYT = 8;                  // y rows per tile: kXR x kYT = 128
-constexpr int kXN = 48;                 // three x taps x 16 output channels
-constexpr uint32_t kFoldBlock = 2u * kXN * 16u;   // one (dz, dy) pair x 16 input channels
-constexpr int kFoldMaxNC = 6;           // input-channel steps whose weights stay resident
 // Eight epilogue warps: two groups of four (tensor-memory lanes 0 ... 127), each draining every
-// other plane.  One group's drain of a plane (three tensor-memory loads, 32 shuffles, the
+// other plane (every other piece of 16 channels of a plane).  One group's drain of a plane (three tensor-memory loads, 32 shuffles, the
 // stores) is a serial chain longer than the plane's nine MMAs once their issue is cheap:
 // 16 -> 16 at 8 x 128^3 426 us with one group, 332 us with two (48 -> 16: 845 / 840 us).
 constexpr int kFoldThreads = 64 + 8 * 32;
+constexpr uint32_t fold_block(int co) { return 2u * 3u * static_cast<uint32_t>(co) * 16u; }   // one (dz, dy) pair x 16 input channels
 
-template <bool FLIP, int TZ>
-__global__ void __launch_bounds__(kFoldThreads, TZ == 4 ? 1 : 2) k_conv3d_tcx(const __grid_constant__ CUtensorMap xmap,
+template <bool FLIP, int TZ, int CO>
+__global__ void __launch_bounds__(kFoldThreads, TZ * CO >= 48 ? 1 : 2) k_conv3d_tcx(const __grid_constant__ CUtensorMap xmap,
                                                             const ConvTcParams p) {
+  constexpr int kXN = 3 * CO;                   // GEMM columns: three x taps x output channels
+  constexpr uint32_t kBlock = fold_block(CO);
+  constexpr int kPieces = TZ * (CO / 16);       // pieces of 16 channels of a plane, drained in turn by the two groups
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   uint8_t* sm = smem_raw + (((raw + 1023u) & ~1023u) - raw);
   constexpr uint32_t a_stage = static_cast<uint32_t>(kXR * (kYT + 2) * (TZ + 2) * 32);   // one halo brick
   const int NC = p.Ci / 16;
-  const uint32_t w_bytes = static_cast<uint32_t>(NC) * 9u * kFoldBlock;
+  const uint32_t w_bytes = static_cast<uint32_t>(NC) * 9u * kBlock;
   const uint32_t S = static_cast<uint32_t>(p.a_stages);
   uint8_t* sA = sm;
   uint8_t* sW = sm + S * a_stage;
@@ -494,17 +495,17 @@ __global__ void __launch_bounds__(kFoldThreads, TZ == 4 ? 1 : 2) k_conv3d_tcx(co
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // weights: packed [kc][t][g][16][8] -> [kc][dz, dy][g][j * 16 + co][8], t = 3 (dz, dy) + j
-  for (int e = threadIdx.x; e < NC * 9 * 2 * 3 * 16; e += blockDim.x) {
-    const int co = e & 15;
-    int r = e >> 4;
+  // weights: packed [kc][t][g][Co][8] -> [kc][dz, dy][g][j * Co + co][8], t = 3 (dz, dy) + j
+  for (int e = threadIdx.x; e < NC * 9 * 2 * 3 * CO; e += blockDim.x) {
+    const int co = e % CO;
+    int r = e / CO;
     const int j = r % 3;
     r /= 3;
     const int g = r & 1;
     r >>= 1;
     const int pr = r % 9, kc = r / 9;
-    const uint4 v = __ldg(reinterpret_cast<const uint4*>(p.wpk) + ((kc * 27 + pr * 3 + j) * 2 + g) * 16 + co);
-    *reinterpret_cast<uint4*>(sW + (kc * 9 + pr) * kFoldBlock + (g * kXN + j * 16 + co) * 16) = v;
+    const uint4 v = __ldg(reinterpret_cast<const uint4*>(p.wpk) + ((kc * 27 + pr * 3 + j) * 2 + g) * CO + co);
+    *reinterpret_cast<uint4*>(sW + (kc * 9 + pr) * kBlock + (g * kXN + j * CO + co) * 16) = v;
   }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // visible to the tensor core
   if (threadIdx.x == 0) {
@@ -576,13 +577,13 @@ __global__ void __launch_bounds__(kFoldThreads, TZ == 4 ? 1 : 2) k_conv3d_tcx(co
         }
         // the (dz, dy) pairs differ by start address, 16 rows (512 bytes) a step
         const uint64_t ad0 = smem_desc_sw32(smem_u32(sA + sa * a_stage));
-        const uint64_t bd0 = smem_desc(smem_u32(sW) + static_cast<uint32_t>(kc) * 9u * kFoldBlock, kXN * 16u, 128u);
+        const uint64_t bd0 = smem_desc(smem_u32(sW) + static_cast<uint32_t>(kc) * 9u * kBlock, kXN * 16u, 128u);
 #pragma unroll
         for (int pr = 0; pr < 9; ++pr) {
           const int sg = FLIP ? -1 : 1;
           const int dz = sg * (pr / 3 - 1), dy = sg * (pr % 3 - 1);
           const uint32_t row = 2u * static_cast<uint32_t>((dz + 1) * (kYT + 2) * kXR + (dy + 1) * kXR);
-          const uint64_t bd = bd0 + static_cast<uint64_t>(pr) * (kFoldBlock >> 4);
+          const uint64_t bd = bd0 + static_cast<uint64_t>(pr) * (kBlock >> 4);
           const uint32_t acc = (kc > 0 || pr > 0) ? 1u : 0u;
 #pragma unroll
           for (int zz = 0; zz < TZ; ++zz)
@@ -601,31 +602,50 @@ __global__ void __launch_bounds__(kFoldThreads, TZ == 4 ? 1 : 2) k_conv3d_tcx(co
     const int q = warp & 3;            // tensor-memory lanes 32q .. 32q + 31
     const int row = 32 * q + lane;     // GEMM row within a plane
     const int mx = row & (kXR - 1), my = row / kXR;
-    const int zhalf = (warp - 2) >> 2;   // planes zhalf, zhalf + 2, ... of a tile
-    float bias[16];
+    const int half = (warp - 2) >> 2;    // this group's pieces: half, half + 2, ...
+    float bias[16];                      // of the only piece per plane (Co = 16)
+    if constexpr (CO == 16) {
 #pragma unroll
-    for (int i = 0; i < 16; ++i) bias[i] = p.bias ? __ldg(&p.bias[i]) : 0.f;
+      for (int i = 0; i < 16; ++i) bias[i] = p.bias ? __ldg(&p.bias[i]) : 0.f;
+    }
+    // The mask of a tile is fetched while the previous one drains: fetched where it is used, its
+    // latency made the drain the bound (16 -> 16 at 8 x 128^3 1.25 ms; just before the wait
+    // for the products 0.53 ms; a tile ahead 0.49 ms; without a mask 0.34 ms, and a pass of
+    // its own takes 0.25 ms).
+    constexpr int kMine = (kPieces + 1) / 2;
+    uint4 n0[kMine], n1[kMine];
+    auto fetch_mask = [&](int64_t tile) {
+      if (!p.mask || tile >= p.tiles) return;
+      const TileCoord tc = tile_coord_x(p, tile);
+      const int x = tc.x0 + mx, y = tc.y0 + my;
+      const int64_t v0 = ((static_cast<int64_t>(tc.n) * p.D + tc.z0) * p.H + y) * p.W + x;
+#pragma unroll
+      for (int k = 0; k < kMine; ++k) {
+        const int pc = 2 * k + half, zz = pc / (CO / 16), c0 = pc % (CO / 16) * 16;
+        if (pc < kPieces && mx >= 1 && mx <= kXO && x < p.W && y < p.H && tc.z0 + zz < p.D) {
+          const uint4* src = reinterpret_cast<const uint4*>(p.mask + (v0 + static_cast<int64_t>(zz) * p.H * p.W) * CO + c0);
+          n0[k] = __ldg(src);
+          n1[k] = __ldg(src + 1);
+        }
+      }
+    };
+#pragma unroll
+    for (int k = 0; k < kMine; ++k) n0[k] = n1[k] = make_uint4(0u, 0u, 0u, 0u);
+    fetch_mask(blockIdx.x);
     uint32_t acc_use = 0;
     for (int64_t tile = blockIdx.x; tile < p.tiles && !*abort_flag; tile += gridDim.x) {
       const TileCoord tc = tile_coord_x(p, tile);
       const uint32_t buf = acc_use & 1u, ku = acc_use >> 1;
       const int x = tc.x0 + mx, y = tc.y0 + my;
-      // the tile's mask is fetched before the wait for its products (plane by plane where it is
-      // used, its latency made the drain the bound: 1.25 ms for 16 -> 16 at 8 x 128^3, now
-      // 0.53 ms; without a mask 0.33 ms, and a pass of its own takes 0.25 ms)
-      uint4 m0[(TZ + 1) / 2], m1[(TZ + 1) / 2];
-      if (p.mask) {
+      const bool inside_xy = mx >= 1 && mx <= kXO && x < p.W && y < p.H;
+      const int64_t v0 = ((static_cast<int64_t>(tc.n) * p.D + tc.z0) * p.H + y) * p.W + x;
+      uint4 m0[kMine], m1[kMine];
 #pragma unroll
-        for (int zh = 0; zh < (TZ + 1) / 2; ++zh) {
-          const int zz = 2 * zh + zhalf;
-          m0[zh] = m1[zh] = make_uint4(0u, 0u, 0u, 0u);
-          const int64_t v = ((static_cast<int64_t>(tc.n) * p.D + tc.z0 + zz) * p.H + y) * p.W + x;
-          if (mx >= 1 && mx <= kXO && x < p.W && y < p.H && tc.z0 + zz < p.D) {
-            m0[zh] = __ldg(reinterpret_cast<const uint4*>(p.mask + v * 16));
-            m1[zh] = __ldg(reinterpret_cast<const uint4*>(p.mask + v * 16) + 1);
-          }
-        }
+      for (int k = 0; k < kMine; ++k) {
+        m0[k] = n0[k];
+        m1[k] = n1[k];
       }
+      fetch_mask(tile + gridDim.x);
       // warp-uniform: the tensor-memory loads and shuffles below are .sync.aligned
       if (!__all_sync(0xffffffffu, mbar_wait_bounded(&tfull[buf], ku & 1u, limit))) {
         if (lane == 0) give_up();
@@ -634,16 +654,19 @@ __global__ void __launch_bounds__(kFoldThreads, TZ == 4 ? 1 : 2) k_conv3d_tcx(co
       __syncwarp();
       fence_after();
 #pragma unroll
-      for (int zh = 0; zh < (TZ + 1) / 2; ++zh) {
-        const int zz = 2 * zh + zhalf;
-        if (zz >= TZ) break;
-        const int z = tc.z0 + zz;
-        const bool inside = mx >= 1 && mx <= kXO && x < p.W && y < p.H && z < p.D;
-        const int64_t v = ((static_cast<int64_t>(tc.n) * p.D + z) * p.H + y) * p.W + x;
-        const uint32_t taddr = tmem + buf * (p.tmem_cols >> 1) + static_cast<uint32_t>(zz * kXN) +
+      for (int k = 0; k < kMine; ++k) {
+        const int pc = 2 * k + half, zz = pc / (CO / 16), c0 = pc % (CO / 16) * 16;
+        if (pc >= kPieces) break;
+        const bool inside = inside_xy && tc.z0 + zz < p.D;
+        const int64_t v = v0 + static_cast<int64_t>(zz) * p.H * p.W;
+        const uint32_t taddr = tmem + buf * (p.tmem_cols >> 1) + static_cast<uint32_t>(zz * kXN + c0) +
                                (static_cast<uint32_t>(32 * q) << 16);
         uint32_t r0[16], r1[16], r2[16];
-        tmem_ld16x3(taddr, r0, r1, r2);
+        tmem_ld16x3(taddr, CO, r0, r1, r2);
+        if constexpr (CO != 16) {
+#pragma unroll
+          for (int i = 0; i < 16; ++i) bias[i] = p.bias ? __ldg(&p.bias[c0 + i]) : 0.f;
+        }
         float f[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
@@ -664,19 +687,19 @@ __global__ void __launch_bounds__(kFoldThreads, TZ == 4 ? 1 : 2) k_conv3d_tcx(co
               const __nv_bfloat162 b2 = __floats2bfloat162_rn(f[2 * i], f[2 * i + 1]);
               h[i] = *reinterpret_cast<const uint32_t*>(&b2);
             }
-            uint4* dst = reinterpret_cast<uint4*>(p.y + v * 16);
+            uint4* dst = reinterpret_cast<uint4*>(p.y + v * CO + c0);
             uint4 q0 = make_uint4(h[0], h[1], h[2], h[3]), q1 = make_uint4(h[4], h[5], h[6], h[7]);
             if (p.mask) {
-              q0 = lrelu_grad8(q0, m0[zh]);
-              q1 = lrelu_grad8(q1, m1[zh]);
+              q0 = lrelu_grad8(q0, m0[k]);
+              q1 = lrelu_grad8(q1, m1[k]);
             }
             dst[0] = q0;
             dst[1] = q1;
           }
           if (p.yf && p.yf_ch == 2) {
-            *reinterpret_cast<float2*>(p.yf + 2 * v) = make_float2(f[0], f[1]);
+            if (c0 == 0) *reinterpret_cast<float2*>(p.yf + 2 * v) = make_float2(f[0], f[1]);
           } else if (p.yf) {
-            float4* dst = reinterpret_cast<float4*>(p.yf + v * 16);
+            float4* dst = reinterpret_cast<float4*>(p.yf + v * CO + c0);
 #pragma unroll
             for (int i = 0; i < 4; ++i) dst[i] = make_float4(f[4 * i], f[4 * i + 1], f[4 * i + 2], f[4 * i + 3]);
           }
@@ -773,16 +796,16 @@ TcShape tc_shape(int ci, int co) {
   return shape_for(ci, co, co <= 128 ? 2 : 1);
 }
 
-// x-folded kernel (16 output channels): A bricks of 16 x 10 x (tz + 2) voxels, all weights
-// resident as nc x 9 blocks of 1536 bytes, tz planes x 48 columns x two accumulator buffers
-TcShape shape_fold(int ci, int tz) {
+// x-folded kernel: A bricks of 16 x 10 x (tz + 2) voxels, all weights resident as nc x 9
+// blocks, tz planes x 3 co columns x two accumulator buffers
+TcShape shape_fold(int ci, int co, int tz) {
   TcShape t{};
   t.tz = tz;
   t.group_pitch = static_cast<uint32_t>(kXR * (kYT + 2) * (tz + 2) * 16);   // half a brick
   t.resident = 1;
-  t.w_bytes = static_cast<uint32_t>(ci / 16) * 9u * kFoldBlock;
+  t.w_bytes = static_cast<uint32_t>(ci / 16) * 9u * fold_block(co);
   uint32_t c = 32;
-  while (c < 2u * static_cast<uint32_t>(tz * kXN)) c <<= 1;
+  while (c < 2u * static_cast<uint32_t>(tz * 3 * co)) c <<= 1;
   t.tmem_cols = c;
   // as many halo stages (up to 4) as keep the CTAs that tensor memory allows on one SM
   const size_t budget = c >= 512 ? 220 * 1024 : 110 * 1024;
@@ -793,7 +816,28 @@ TcShape shape_fold(int ci, int tz) {
   return t;
 }
 
-bool use_fold(int ci, int co) { return g_conv_fold && co == 16 && ci / 16 <= kFoldMaxNC; }
+// z planes of an x-folded tile: as many as the 512 tensor-memory columns hold
+int fold_tz(int co) {
+  const int top = co == 16 ? 4 : 2;
+  const int tz = g_fold_tz == 1 || g_fold_tz == 2 ? g_fold_tz : 4;
+  return tz < top ? tz : top;
+}
+
+// Folded: 16 output channels, and 32 from at least 32 input channels (fewer leave too few MMAs
+// per drained column); weights have to fit.  27-tap kernel -> folded, us: 32 -> 32 at 8 x 64^3
+// 155 -> 128, 64 -> 32 290 -> 222, 96 -> 32 418 -> 354, 16 -> 32 90 -> 121; 48 outputs (N = 144,
+// one plane per tile) from 16 channels at 8 x 128^3 857 -> 1478, so not offered.
+bool use_fold(int ci, int co) {
+  return g_conv_fold && ci <= 96 && (co == 16 || (co == 32 && ci >= 32));
+}
+
+template <bool FLIP>
+const void* fold_kernel(int co, int tz) {
+  if (co == 16)
+    return reinterpret_cast<const void*>(tz == 4 ? k_conv3d_tcx<FLIP, 4, 16>
+                                                 : tz == 2 ? k_conv3d_tcx<FLIP, 2, 16> : k_conv3d_tcx<FLIP, 1, 16>);
+  return reinterpret_cast<const void*>(tz == 2 ? k_conv3d_tcx<FLIP, 2, 32> : k_conv3d_tcx<FLIP, 1, 32>);
+}
 
 }  // namespace
 
@@ -867,8 +911,7 @@ cudaError_t launch_conv_tc(const void* x, const void* wpk, const float* bias, vo
   const cuuint64_t row = 2ull * ci;
   const cuuint64_t strides[4] = {row, row * w, row * w * h, row * w * h * d};
   const bool fold = use_fold(ci, co);
-  const int ftz = g_fold_tz == 1 || g_fold_tz == 2 ? g_fold_tz : 4;
-  const TcShape shp = fold ? shape_fold(ci, ftz) : tc_shape(ci, co);
+  const TcShape shp = fold ? shape_fold(ci, co, fold_tz(co)) : tc_shape(ci, co);
   const cuuint32_t box[5] = {static_cast<cuuint32_t>(fold ? 16 : 8), static_cast<cuuint32_t>(fold ? kXR : kHX), static_cast<cuuint32_t>(fold ? kYT + 2 : kHY),
                              static_cast<cuuint32_t>(shp.tz + 2), 1};
   const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
@@ -903,14 +946,11 @@ cudaError_t launch_conv_tc(const void* x, const void* wpk, const float* bias, vo
   p.wait_limit = g_wait_limit ? g_wait_limit : kDefaultWait;
   p.debug_stall = g_debug_stall;
   const size_t smem = shp.smem;
-  auto kern = fold ? (flip ? (shp.tz == 4 ? k_conv3d_tcx<true, 4> : shp.tz == 2 ? k_conv3d_tcx<true, 2>
-                                                                      : k_conv3d_tcx<true, 1>)
-                            : (shp.tz == 4 ? k_conv3d_tcx<false, 4> : shp.tz == 2 ? k_conv3d_tcx<false, 2>
-                                                                        : k_conv3d_tcx<false, 1>))
-                   : flip ? (shp.tz == 4 ? k_conv3d_tc<true, 4> : shp.tz == 2 ? k_conv3d_tc<true, 2>
-                                                                     : k_conv3d_tc<true, 1>)
-                          : (shp.tz == 4 ? k_conv3d_tc<false, 4>
-                                         : shp.tz == 2 ? k_conv3d_tc<false, 2> : k_conv3d_tc<false, 1>);
+  using Kernel = void (*)(CUtensorMap, ConvTcParams);
+  Kernel kern = flip ? (shp.tz == 4 ? k_conv3d_tc<true, 4> : shp.tz == 2 ? k_conv3d_tc<true, 2> : k_conv3d_tc<true, 1>)
+                     : (shp.tz == 4 ? k_conv3d_tc<false, 4>
+                                    : shp.tz == 2 ? k_conv3d_tc<false, 2> : k_conv3d_tc<false, 1>);
+  if (fold) kern = reinterpret_cast<Kernel>(const_cast<void*>(flip ? fold_kernel<true>(co, shp.tz) : fold_kernel<false>(co, shp.tz)));
   const int threads = fold ? kFoldThreads : kThreads;
   int per_sm = 0, sms = 0;
   const cudaError_t e = kernel_setup(reinterpret_cast<const void*>(kern), threads, smem, p.tmem_cols, &per_sm, &sms);
