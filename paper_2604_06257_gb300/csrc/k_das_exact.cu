@@ -103,9 +103,11 @@ template <int FL, int FPL>
 __device__ __forceinline__ int chunk_swizzle(int g) {
   return FPL == 8 ? (FL == 4 ? (g & 1) : FL <= 2 ? ((g >> 1) & 1) : 0) : 0;
 }
-template <int FT>
+template <int FT, int FPL>
+constexpr bool kHalves = FT == 16 || (FT == 8 && FPL == 8);   // at 4 frames per lane in rows of 8 it gains nothing
+template <int FT, int FPL>
 __device__ __forceinline__ int half_swap(int g) {
-  return FT <= 16 ? (g & 1) : 0;
+  return kHalves<FT, FPL> ? (g & 1) : 0;
 }
 
 // Accumulators of one lane: VPG voxel slots x FPL frames, as packed pairs.
@@ -132,7 +134,7 @@ __device__ __noinline__ Acc<VPG, FPL> outside_pair(const DasParams& p, Acc<VPG, 
                                                    unsigned order) {
   constexpr int RB = FT * 8, IMO = FT * 4, FL = FT / FPL;
   // chunk and half orders, the frame tile above them
-  const int swz = FT <= 16 || PART ? order & 1 : order, hs = FT <= 16 ? (order >> 1) & 1 : 0;
+  const int swz = kHalves<FT, FPL> || PART ? order & 1 : order, hs = kHalves<FT, FPL> ? (order >> 1) & 1 : 0;
   const unsigned char* gsrc = tile_iq<PART>(p, order >> 2) + ((static_cast<size_t>(m.t) * p.C + m.c) * p.S + m.lo) * RB + jl * 16;
 #pragma unroll
   for (int k = 0; k < VPG; ++k) {
@@ -216,8 +218,8 @@ __device__ __forceinline__ void das_exact_block(const DasParams& p, const W& w) 
   const int sub = lane / WV;
   const int q = lane % WV;
   const int swz = chunk_swizzle<FL, FPL>(g);
-  const int hs = half_swap<FT>(g);
-  const float im_sign = half_swap<FT>(q / VPG) ? -1.0f : 1.0f;   // of the group that reads this lane's terms
+  const int hs = half_swap<FT, FPL>(g);
+  const float im_sign = half_swap<FT, FPL>(q / VPG) ? -1.0f : 1.0f;   // of the group that reads this lane's terms
   float* txc = txc_all + warp * (p.T * 32);
   const int64_t v_term = tile_voxel_blocked(p, tile, warp * WV + q);
   const float4 vpos = v_term >= 0 ? p.vox[v_term] : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -271,7 +273,7 @@ __device__ __forceinline__ void das_exact_block(const DasParams& p, const W& w) 
     const int row = active ? i0 - mm.lo : 0;
     const bool outside = active && (row < 0 || row + 1 >= mm.rows);
     float4 tw = tap_weights(rec);
-    if constexpr (FT <= 16) {   // exact
+    if constexpr (kHalves<FT, FPL>) {   // exact
       tw.y *= im_sign;
       tw.w *= im_sign;
     }
@@ -308,7 +310,7 @@ __device__ __forceinline__ void das_exact_block(const DasParams& p, const W& w) 
           for (int c = 0; c < FPL / 4; ++c) {
             // chunk c lies (c ^ swz - swz) FL * 16 bytes from chunk 0's lane address
             const uint32_t b = a + ((c ^ swz) - swz) * FL * 16;
-            if constexpr (FT <= 16) {
+            if constexpr (kHalves<FT, FPL>) {
               const uint32_t z = b + im_at;
               mac4(&acc.a[k][4 * c], cw, lds128(b), lds128(z), lds128(b + RB), lds128(z + RB));
             } else {
@@ -318,7 +320,7 @@ __device__ __forceinline__ void das_exact_block(const DasParams& p, const W& w) 
         }
       } else {
         acc = outside_pair<FT, FPL, VPG, G, PART>(p, acc, meta[slot], smem + slot * slot_bytes + jl * 16, cw_at, of_at,
-                                            jl, FT <= 16 || PART ? swz | hs << 1 | w.ftile() << 2 : swz);
+                                            jl, kHalves<FT, FPL> || PART ? swz | hs << 1 | w.ftile() << 2 : swz);
       }
       if constexpr ((FLAGS & kEarly) != 0) {   // every lane has read the slot: release it
         __syncwarp();
