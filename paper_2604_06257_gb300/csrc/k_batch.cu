@@ -20,13 +20,13 @@
 //  - frame lanes (F <= 16 or a multiple of 4, and the fallback when an instance's windows
 //    exceed the ring): FL lanes share a voxel (FL = 2, 4, 8 or 16 at run time), each lane
 //    holds 4 frames of 4 voxels (2 voxels for FL = 2), taps read through L1;
-//  - channel lanes (F <= 4): 8 lanes share a voxel and split its elements; partial sums
-//    meet in a shuffle tree.
+//  - channel lanes (F <= 4): a voxel's elements are split over the 8 warps (das_slices.cuh).
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <cstdint>
 
+#include "das_slices.cuh"
 #include "das_staged.cuh"
 
 namespace mach {
@@ -137,62 +137,6 @@ __device__ __forceinline__ void batch_frames_tile(const DasParams& p, int FL, in
   }
 }
 
-template <class IQ>
-__device__ __forceinline__ void batch_channels_tile(const DasParams& p, int64_t tile) {
-  constexpr int CL = 8, G = 32 / CL, FMAX = 4;
-  const int lane = threadIdx.x & 31;
-  const int warp = threadIdx.x >> 5;
-  const int g = lane / CL, jl = lane % CL;
-  const int64_t v = tile_voxel(p, tile, warp * G + g);
-  const IQ* __restrict__ iq = static_cast<const IQ*>(p.iq);
-  float2 acc[FMAX];
-#pragma unroll
-  for (int f = 0; f < FMAX; ++f) acc[f] = make_float2(0.f, 0.f);
-  if (v >= 0) {
-    const float4 vpos = p.vox[v];
-    for (int c = jl; c < p.C; c += CL) {
-      const TermGeo geo = term_geometry(vpos, __ldg(&p.elem[c]), p);
-      if (geo.a < 0.f) continue;
-      for (int t = 0; t < p.T; ++t) {
-        const float4 r = term_record(__ldg(&p.tx[static_cast<size_t>(t) * p.V + v]), geo, p);
-        const int i0 = __float_as_int(r.w);
-        if (i0 < 0) continue;
-        const float4 cw = tap_weights(r);
-        const float c0r = cw.x, c0i = cw.y, c1r = cw.z, c1i = cw.w;
-        const IQ* row0 = iq + ((static_cast<size_t>(t) * p.C + c) * p.S + i0) * p.F;
-#pragma unroll
-        for (int f = 0; f < FMAX; ++f) {
-          if (f < p.F) {
-            float2 x0[1], x1[1];
-            load_vec<IQ, 1, false>(row0 + f, x0);
-            load_vec<IQ, 1, false>(row0 + p.F + f, x1);
-            mac1(acc[f], c0r, c0i, c1r, c1i, x0[0], x1[0]);
-          }
-        }
-      }
-    }
-  }
-#pragma unroll
-  for (int f = 0; f < FMAX; ++f) {
-#pragma unroll
-    for (int o = CL / 2; o > 0; o >>= 1) {
-      acc[f].x += __shfl_xor_sync(0xffffffffu, acc[f].x, o);
-      acc[f].y += __shfl_xor_sync(0xffffffffu, acc[f].y, o);
-    }
-  }
-  if (jl == 0 && v >= 0) {
-    float pw = 0.f;
-#pragma unroll
-    for (int f = 0; f < FMAX; ++f) {
-      if (f < p.F) {
-        pw = fmaf(acc[f].x, acc[f].x, fmaf(acc[f].y, acc[f].y, pw));
-        if (p.y) p.y[v * p.F + f] = acc[f];
-      }
-    }
-    if (p.pd) p.pd[v] = pw;
-  }
-}
-
 // ---- staged path ---------------------------------------------------------------------------
 
 // Shared memory of a batch block: [ring][per-warp scratch][slot metadata][barriers].  The
@@ -218,6 +162,8 @@ struct BatchSlotMeta {
   int skip;             // elements (complex samples) before row lo in the slot
   int pad_[3];
 };
+static_assert(kSlices == kBatchWarps && kSlices * 4 * kSliceVox * sizeof(float2) <= kBatchWarps * kBatchTx * 32 * 16,
+              "the slices' sums fit the scratch");
 static_assert(sizeof(BatchSlotMeta) == 48, "slot metadata (BatchLayout reserves 48 bytes per slot)");
 
 // Producer of one staged item: like produce_windows, for rows of any length.  A window is
@@ -499,7 +445,14 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 2)
       }
       __syncthreads();   // the ring is drained before the next item re-initialises it
     } else if (mode == kBatchChannels) {
-      batch_channels_tile<IQ>(p, w.y);
+      // the scratch of all warps as one array: 8 slices x F x 32 sums
+      float2* part = reinterpret_cast<float2*>(smem + L.scratch_off());
+      switch (p.F) {
+        case 1: das_slices_tile<IQ, 1>(p, w.y, part); break;
+        case 2: das_slices_tile<IQ, 2>(p, w.y, part); break;
+        case 3: das_slices_tile<IQ, 3>(p, w.y, part); break;
+        default: das_slices_tile<IQ, 4>(p, w.y, part); break;
+      }
     } else if (fl == 2) {
       if (p.F % 4 == 0) batch_frames_tile<IQ, 4, 1, 2>(p, fl, w.y, reinterpret_cast<float4*>(scratch));
       else if (p.F % 2 == 0) batch_frames_tile<IQ, 2, 2, 2>(p, fl, w.y, reinterpret_cast<float4*>(scratch));

@@ -12,14 +12,16 @@
 // (the paper's delay reuse across frames, Sec. 4.4).  The gather per term is one
 // coalesced row segment of FL x FPL frames per tap.
 //
-// "Channel lanes" kernels (F <= 4): CL lanes share one voxel, lane j takes elements
-// j, j + CL, ...; each lane evaluates its own terms, and the partial sums are combined by
-// a shuffle tree (pairwise, so rounding grows with log CL).
+// "Channel lanes" kernels (F <= 4): CL slices of the elements share one voxel, slice j takes
+// elements j, j + CL, ..., and the partial sums meet in a pairwise tree (rounding grows with
+// log CL).  With CL = 8 the slices are the warps of a block (das_slices.cuh); CL = 16 and 32
+// are lanes.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <cstdint>
 
+#include "das_slices.cuh"
 #include "das_term.cuh"
 #include "tap_mac.cuh"
 #include "mach_internal.h"
@@ -145,7 +147,14 @@ __global__ void __launch_bounds__(NWARP * 32) k_das_frames(const DasParams p) {
   }
 }
 
-// ---- channel-lane kernel (short ensembles) --------------------------------------------
+// ---- channel-lane kernels (short ensembles) -------------------------------------------
+template <class IQ, int F>
+__global__ void __launch_bounds__(kSlices * 32) k_das_slices(const DasParams p) {
+  __shared__ float2 part[kSlices * F * kSliceVox];
+  // deepest tiles (widest apertures, most terms) first: light tiles fill the launch's tail
+  das_slices_tile<IQ, F>(p, static_cast<int64_t>(gridDim.x) - 1 - blockIdx.x, part);
+}
+
 template <class IQ, int CL, int FMAX, int NWARP>
 __global__ void __launch_bounds__(NWARP * 32) k_das_channels(const DasParams p) {
   constexpr int G = 32 / CL;
@@ -293,6 +302,17 @@ cudaError_t go(K kernel, const DasParams& p, size_t smem, cudaStream_t s) {
   kernel<<<grid, kWarps * 32, smem, s>>>(p);
   return cudaGetLastError();
 }
+template <class IQ>
+cudaError_t go_slices(const DasParams& p, cudaStream_t s) {
+  static_assert(kWarps == kSlices, "a block's warps are the slices");
+  switch (p.F) {
+    case 1: return go(k_das_slices<IQ, 1>, p, 0, s);
+    case 2: return go(k_das_slices<IQ, 2>, p, 0, s);
+    case 3: return go(k_das_slices<IQ, 3>, p, 0, s);
+    case 4: return go(k_das_slices<IQ, 4>, p, 0, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
 }  // namespace
 
 const VariantShape& variant_shape(Variant v) { return kShapes[v]; }
@@ -306,18 +326,18 @@ cudaError_t launch_das(const DasParams& p, Variant v, cudaStream_t s) {
   cudaError_t e;
   switch (kShapes[v].staged ? V_COUNT : v) {
     case V_COUNT: e = launch_das_staged(p, v, s); break;
-    case V_CH_C64: e = go(k_das_channels<float2, 8, 4, kWarps>, p, sm, s); break;
+    case V_CH_C64: e = go_slices<float2>(p, s); break;
     case V_CH_C64_L16: e = go(k_das_channels<float2, 16, 4, kWarps>, p, sm, s); break;
     case V_CH_C64_L32: e = go(k_das_channels<float2, 32, 4, kWarps>, p, sm, s); break;
     case V_F16_C64: e = go(k_das_frames<float2, 2, 1, 8, 8, kWarps>, p, sm, s); break;
     case V_F32_C64: e = go(k_das_frames<float2, 2, 2, 8, 8, kWarps>, p, sm, s); break;
     case V_F64_C64: e = go(k_das_frames<float2, 2, 2, 16, 8, kWarps>, p, sm, s); break;
     case V_S32_C64: e = go(k_das_frames<float2, 1, 1, 32, 16, kWarps>, p, sm, s); break;
-    case V_CH_H16: e = go(k_das_channels<__half2, 8, 4, kWarps>, p, sm, s); break;
+    case V_CH_H16: e = go_slices<__half2>(p, s); break;
     case V_F32_H16: e = go(k_das_frames<__half2, 4, 1, 8, 8, kWarps>, p, sm, s); break;
     case V_F64_H16: e = go(k_das_frames<__half2, 4, 1, 16, 8, kWarps>, p, sm, s); break;
     case V_S32_H16: e = go(k_das_frames<__half2, 1, 1, 32, 16, kWarps>, p, sm, s); break;
-    case V_CH_B16: e = go(k_das_channels<__nv_bfloat162, 8, 4, kWarps>, p, sm, s); break;
+    case V_CH_B16: e = go_slices<__nv_bfloat162>(p, s); break;
     case V_F32_B16: e = go(k_das_frames<__nv_bfloat162, 4, 1, 8, 8, kWarps>, p, sm, s); break;
     case V_F64_B16: e = go(k_das_frames<__nv_bfloat162, 4, 1, 16, 8, kWarps>, p, sm, s); break;
     case V_S32_B16: e = go(k_das_frames<__nv_bfloat162, 1, 1, 32, 16, kWarps>, p, sm, s); break;
