@@ -157,8 +157,18 @@ __device__ __noinline__ Acc<VPG, FPL> outside_pair(const DasParams& p, Acc<VPG, 
 // slots per lane group; NWC consumer warps + 1 producer warp; NBUF ring slots; MAXR
 // registers per thread.
 // FLAGS bit 0: consumers suspended in hardware while waiting for a window; bit 1: a warp
-// releases each ring slot right after its last read instead of at the end of the round.
-constexpr int kSleep = 1, kEarly = 2;
+// releases each ring slot right after its last read instead of at the end of the round;
+// bit 2: every kept term is known to lie in its staged window (windows_hold), so no term has to
+// look for its taps elsewhere.
+constexpr int kSleep = 1, kEarly = 2, kInside = 4;
+
+// A window spans the delays between a tile's nearest and farthest points plus two rows on each
+// side (pair_window).  The bounds and a term's own delay are float32 sums of at most a few
+// roundings of values below S, so for S <= 2^18 (an ulp of 1/64 row or less) they cannot
+// disagree by two rows (kWindowsHold; repacked ensembles are not longer).  The check and the
+// out-of-line path behind it cost registers: 94 x 94 x 178 voxels, 32 frames 91.4 -> 89.7 ms
+// without them.
+bool windows_hold(const DasParams& p) { return p.S <= kWindowsHold; }
 
 //
 // PART: the launch covers frames p.f_first ... of an ensemble of p.f_total frames that the
@@ -271,7 +281,8 @@ __device__ __forceinline__ void das_exact_block(const DasParams& p, const W& w) 
     const int i0 = __float_as_int(rec.w);
     const bool active = i0 >= 0;
     const int row = active ? i0 - mm.lo : 0;
-    const bool outside = active && (row < 0 || row + 1 >= mm.rows);
+    bool outside = false;
+    if constexpr ((FLAGS & kInside) == 0) outside = active && (row < 0 || row + 1 >= mm.rows);
     float4 tw = tap_weights(rec);
     if constexpr (kHalves<FT, FPL>) {   // exact
       tw.y *= im_sign;
@@ -280,7 +291,8 @@ __device__ __forceinline__ void das_exact_block(const DasParams& p, const W& w) 
     sts128(coef_w + store_at * 16, tw);
     sts32(offs_w + store_at * 4, row * RB);
     const unsigned act = __ballot_sync(0xffffffffu, active);
-    const unsigned outm = __ballot_sync(0xffffffffu, outside);
+    unsigned outm = 0u;
+    if constexpr ((FLAGS & kInside) == 0) outm = __ballot_sync(0xffffffffu, outside);
     const unsigned ended = __ballot_sync(0xffffffffu, mm.c < 0);
     __syncwarp();
 #pragma unroll
@@ -300,7 +312,7 @@ __device__ __forceinline__ void das_exact_block(const DasParams& p, const W& w) 
       const uint32_t win = lane_tap + slot * slot_bytes;
       const uint32_t cw_at = coef_w + (i * WV + g) * 16;
       const uint32_t of_at = offs_w + (i * WV + g) * 4;
-      if (!(outm & gm)) {
+      if ((FLAGS & kInside) || !(outm & gm)) {
         // every kept term lies in the staged window: branch-free over the voxels
 #pragma unroll
         for (int k = 0; k < VPG; ++k) {
@@ -454,18 +466,21 @@ cudaError_t launch_das_exact(const DasParams& p, Variant v, cudaStream_t s) {
     case V_SX32_F8V1W15T24S: return go_staged(k_das_exact<32, 8, 1, 15, 8, 64, kSleep>, 15, p, sm, s);
     case V_SX32_F8V1W7T14: return go_staged(k_das_exact<32, 8, 1, 7, 8, 64, 0>, 7, p, sm, s);
     case V_SX32_F8V1W7T14E: case V_SX32_F8V1W7_T8X7E:
-      return go_staged(k_das_exact<32, 8, 1, 7, 8, 64, kEarly>, 7, p, sm, s);
+      return windows_hold(p) ? go_staged(k_das_exact<32, 8, 1, 7, 8, 64, kEarly | kInside>, 7, p, sm, s)
+                             : go_staged(k_das_exact<32, 8, 1, 7, 8, 64, kEarly>, 7, p, sm, s);
     case V_SX32_F4V2W7T14: return go_staged(k_das_exact<32, 4, 2, 7, 8, 64, 0>, 7, p, sm, s);
     case V_SX32_F8V1W15T30R12: return go_staged(k_das_exact<32, 8, 1, 15, 12, 64, 0>, 15, p, sm, s);
     case V_SX32_F8V1W15T30R12E: return go_staged(k_das_exact<32, 8, 1, 15, 12, 64, kEarly>, 15, p, sm, s);
     case V_SX64_C64P: case V_SX64_C64P_T16: case V_SX64_C64P_T8X8:
-      return go_staged(k_das_exact<64, 4, 4, 8, 8, 72, 0>, 8, p, sm, s);
+      return windows_hold(p) ? go_staged(k_das_exact<64, 4, 4, 8, 8, 72, kInside>, 8, p, sm, s)
+                             : go_staged(k_das_exact<64, 4, 4, 8, 8, 72, 0>, 8, p, sm, s);
     case V_SX64_C64P_T16E: return go_staged(k_das_exact<64, 4, 4, 8, 8, 72, kEarly>, 8, p, sm, s);
     case V_SX64_C64PS: return go_staged(k_das_exact<64, 4, 4, 8, 8, 72, kSleep>, 8, p, sm, s);
     case V_SX64_C64PE: return go_staged(k_das_exact<64, 4, 4, 8, 8, 72, kEarly>, 8, p, sm, s);
     case V_SX64_F8V2: return go_staged(k_das_exact<64, 8, 2, 8, 8, 72, 0>, 8, p, sm, s);
     case V_SX16_F4V2W7: case V_SX16_F4V2W7_T8X14:
-      return go_staged(k_das_exact<16, 4, 2, 7, 8, 64, kEarly>, 7, p, sm, s);
+      return windows_hold(p) ? go_staged(k_das_exact<16, 4, 2, 7, 8, 64, kEarly | kInside>, 7, p, sm, s)
+                             : go_staged(k_das_exact<16, 4, 2, 7, 8, 64, kEarly>, 7, p, sm, s);
     case V_SX16_F8V1W7: return go_staged(k_das_exact<16, 8, 1, 7, 8, 64, kEarly>, 7, p, sm, s);
     case V_SX16_F8V1W4: return go_staged(k_das_exact<16, 8, 1, 4, 8, 64, kEarly>, 4, p, sm, s);
     case V_SX8_F8V1W4: return go_staged(k_das_exact<8, 8, 1, 4, 8, 64, kEarly>, 4, p, sm, s);
@@ -488,12 +503,12 @@ cudaError_t launch_das_parts(const DasParams& p, Variant v, int tiles, cudaStrea
     return cudaGetLastError();
   };
   switch (v) {
-    case V_SX32_F8V1W7T14E: case V_SX32_F8V1W7_T8X7E: return go(k_das_exact<32, 8, 1, 7, 8, 64, kEarly, true>, 7);
-    case V_SX16_F8V1W7: return go(k_das_exact<16, 8, 1, 7, 8, 64, kEarly, true>, 7);
-    case V_SX16_F8V1W4: return go(k_das_exact<16, 8, 1, 4, 8, 64, kEarly, true>, 4);
-    case V_SX16_F4V1W7: return go(k_das_exact<16, 4, 1, 7, 8, 64, kEarly, true>, 7);
-    case V_SX8_F8V1W4: return go(k_das_exact<8, 8, 1, 4, 8, 64, kEarly, true>, 4);
-    case V_SX8_F4V1W7: return go(k_das_exact<8, 4, 1, 7, 8, 64, kEarly, true>, 7);
+    case V_SX32_F8V1W7T14E: case V_SX32_F8V1W7_T8X7E: return go(k_das_exact<32, 8, 1, 7, 8, 64, kEarly | kInside, true>, 7);
+    case V_SX16_F8V1W7: return go(k_das_exact<16, 8, 1, 7, 8, 64, kEarly | kInside, true>, 7);
+    case V_SX16_F8V1W4: return go(k_das_exact<16, 8, 1, 4, 8, 64, kEarly | kInside, true>, 4);
+    case V_SX16_F4V1W7: return go(k_das_exact<16, 4, 1, 7, 8, 64, kEarly | kInside, true>, 7);
+    case V_SX8_F8V1W4: return go(k_das_exact<8, 8, 1, 4, 8, 64, kEarly | kInside, true>, 4);
+    case V_SX8_F4V1W7: return go(k_das_exact<8, 4, 1, 7, 8, 64, kEarly | kInside, true>, 7);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -508,12 +523,12 @@ cudaError_t launch_das_multi(const MultiArgs& a, Variant v, const int2* items, i
     return cudaGetLastError();
   };
   switch (v) {
-    case V_SX32_F8V1W7T14E: case V_SX32_F8V1W7_T8X7E: return go(k_das_exact_multi<32, 8, 1, 7, 8, 64, kEarly>, 7);
-    case V_SX16_F8V1W7: return go(k_das_exact_multi<16, 8, 1, 7, 8, 64, kEarly>, 7);
-    case V_SX16_F8V1W4: return go(k_das_exact_multi<16, 8, 1, 4, 8, 64, kEarly>, 4);
-    case V_SX16_F4V1W7: return go(k_das_exact_multi<16, 4, 1, 7, 8, 64, kEarly>, 7);
-    case V_SX8_F8V1W4: return go(k_das_exact_multi<8, 8, 1, 4, 8, 64, kEarly>, 4);
-    case V_SX8_F4V1W7: return go(k_das_exact_multi<8, 4, 1, 7, 8, 64, kEarly>, 7);
+    case V_SX32_F8V1W7T14E: case V_SX32_F8V1W7_T8X7E: return go(k_das_exact_multi<32, 8, 1, 7, 8, 64, kEarly | kInside>, 7);
+    case V_SX16_F8V1W7: return go(k_das_exact_multi<16, 8, 1, 7, 8, 64, kEarly | kInside>, 7);
+    case V_SX16_F8V1W4: return go(k_das_exact_multi<16, 8, 1, 4, 8, 64, kEarly | kInside>, 4);
+    case V_SX16_F4V1W7: return go(k_das_exact_multi<16, 4, 1, 7, 8, 64, kEarly | kInside>, 7);
+    case V_SX8_F8V1W4: return go(k_das_exact_multi<8, 8, 1, 4, 8, 64, kEarly | kInside>, 4);
+    case V_SX8_F4V1W7: return go(k_das_exact_multi<8, 4, 1, 7, 8, 64, kEarly | kInside>, 7);
     default: return cudaErrorInvalidValue;
   }
 }

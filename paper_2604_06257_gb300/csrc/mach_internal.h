@@ -156,6 +156,7 @@ struct FrameSplit {
   int tiles() const { return full + (tail ? 1 : 0); }
   int padded() const { return 32 * full + tail; }
 };
+constexpr int kWindowsHold = 1 << 18;   // samples up to which a term cannot leave its staged window
 struct RepackPart {             // one launch: equal frame tiles on one exact-frame shape
   Variant v = V_COUNT;
   int tiles = 0;

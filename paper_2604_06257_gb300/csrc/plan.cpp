@@ -449,7 +449,7 @@ static mach_status repack_plan(mach_plan_s* p, const DasParams& b, bool list, cu
   const FrameSplit fs = split_frames(b.F);
   const size_t iq_bytes = static_cast<size_t>(N) * 8 * fs.padded();
   const size_t pd_bytes = fs.tiles() > 1 ? sizeof(float) * static_cast<size_t>(b.V) * fs.tiles() : 0;
-  if (iq_bytes + pd_bytes > total_mem / 16) return MACH_OK;
+  if (iq_bytes + pd_bytes > total_mem / 16 || b.S > kWindowsHold) return MACH_OK;
   if (fs.full > 65535) return MACH_OK;   // grid y limit
   const bool grid3d = !list && b.ny > 1;
   struct Want { Variant v; int tiles; } want[2];
