@@ -33,7 +33,8 @@ struct mach_batch_s {
   // per exact-frame shape and kMultiMax entries)
   struct Repacked {
     int inst, dtype, F, tiles;
-    int64_t N, V;
+    int64_t TC, V;
+    int S, range[2];                     // samples per row, those that windows touch
     size_t at;                           // its bytes in the workspace below
     size_t pd_at;
   };
@@ -122,7 +123,8 @@ mach_status plan_repacked(mach_batch_s* b, cudaStream_t s) {
   for (const auto& q : b->repacked) {
     const RepackPart* parts = nullptr;
     size_t ws_i = 0, pd_i = 0;
-    const int np = plan_repack(b->plans[q.inst], &parts, &ws_i, &pd_i);
+    int range[2];
+    const int np = plan_repack(b->plans[q.inst], &parts, &ws_i, &pd_i, range);
     for (int k = 0; k < np; ++k) {
       // 2D and 3D shapes of 32 frames are one kernel
       const Variant v = parts[k].v == V_SX32_F8V1W7_T8X7E ? V_SX32_F8V1W7T14E : parts[k].v;
@@ -230,11 +232,12 @@ mach_status mach_batch_plan(const mach_das_desc* descs, int32_t n, const mach_ti
     // repacked tiles
     const RepackPart* parts = nullptr;
     size_t ws_i = 0, pd_i = 0;
-    if (!shapes && plan_repack(b->plans[i], &parts, &ws_i, &pd_i) && ws_total + ws_i <= total_mem / 16) {
+    int range[2];
+    if (!shapes && plan_repack(b->plans[i], &parts, &ws_i, &pd_i, range) && ws_total + ws_i <= total_mem / 16) {
       is_repacked[i] = 1;
       const DasParams& q = *plan_params(b->plans[i]);
-      b->repacked.push_back({i, dt, q.F, parts[0].base.frame_tiles, static_cast<int64_t>(q.T) * q.C * q.S, q.V,
-                             ws_total, pd_i});
+      b->repacked.push_back({i, dt, q.F, parts[0].base.frame_tiles, static_cast<int64_t>(q.T) * q.C, q.V, q.S,
+                             {range[0], range[1]}, ws_total, pd_i});
       ws_total += (ws_i + 255) / 256 * 256;
     }
     mach_tile_shape sh = shapes ? shapes[i] : default_shape(descs[i].n_frames);
@@ -414,7 +417,8 @@ mach_status mach_batch_run(mach_batch b, void* stream) {
   // the repacked tiles first: their launches hold the longest blocks
   for (const auto& q : b->repacked) {
     if (e != cudaSuccess) break;
-    e = launch_iq_repack(nullptr, &b->d_insts[q.inst].p.iq, q.dtype, reinterpret_cast<float*>(b->ws + q.at), q.N, q.F, s);
+    e = launch_iq_repack(nullptr, &b->d_insts[q.inst].p.iq, q.dtype, reinterpret_cast<float*>(b->ws + q.at), q.TC, q.S,
+                         q.range[0], q.range[1], q.F, s);
   }
   for (const auto& m : b->multi) {
     if (e != cudaSuccess) break;

@@ -255,25 +255,32 @@ constexpr int kRepackItems = 4;   // items in flight per thread
 template <int DT, int VEC>
 __global__ void __launch_bounds__(256) k_iq_repack(const void* __restrict__ src,
                                                    const void* const* __restrict__ src_slot,
-                                                   float* __restrict__ dst, int64_t N, int F, int full,
-                                                   int tail, int rows_per_block) {
+                                                   float* __restrict__ dst, int64_t TC, int S, int s0, int span,
+                                                   int F, int full, int tail, int rows_per_block) {
   const int quads = (32 * full + tail) / 4;
   if (src_slot) src = *src_slot;
-  const int64_t n0 = static_cast<int64_t>(blockIdx.x) * rows_per_block;
-  const int items = static_cast<int>(min(static_cast<int64_t>(rows_per_block), N - n0)) * quads;
+  const int64_t N = TC * S;
+  const int64_t r0 = static_cast<int64_t>(blockIdx.x) * rows_per_block;   // the block's first row of the range
+  const int64_t tc0 = r0 / span;
+  const int at0 = static_cast<int>(r0 - tc0 * span);
+  const int items = static_cast<int>(min(static_cast<int64_t>(rows_per_block), TC * span - r0)) * quads;
+  auto row_of = [&](int i) {   // sample row of item i
+    const int at = at0 + i / quads, k = at / span;
+    return (tc0 + k) * S + s0 + (at - k * span);
+  };
   for (int base = threadIdx.x; base < items; base += 256 * kRepackItems) {
     float4 re[kRepackItems], im[kRepackItems];
 #pragma unroll
     for (int k = 0; k < kRepackItems; ++k) {
       const int i = base + 256 * k;
       re[k] = im[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (i < items) load_quad<DT, VEC>(src, n0 + i / quads, 4 * (i % quads), F, re[k], im[k]);
+      if (i < items) load_quad<DT, VEC>(src, row_of(i), 4 * (i % quads), F, re[k], im[k]);
     }
 #pragma unroll
     for (int k = 0; k < kRepackItems; ++k) {
       const int i = base + 256 * k;
       if (i >= items) break;
-      const int64_t n = n0 + i / quads;
+      const int64_t n = row_of(i);
       const int f = 4 * (i % quads);
       const int ft = f < 32 * full ? 32 : tail;              // frames of the item's tile
       float* row = dst + (f < 32 * full ? (f / 32) * N * 64 : full * N * 64) + n * (2 * ft);
@@ -284,15 +291,16 @@ __global__ void __launch_bounds__(256) k_iq_repack(const void* __restrict__ src,
   }
 }
 
-cudaError_t launch_iq_repack(const void* src, const void* const* src_slot, int src_dtype, float* dst, int64_t N, int F,
-                             cudaStream_t s) {
+cudaError_t launch_iq_repack(const void* src, const void* const* src_slot, int src_dtype, float* dst, int64_t TC, int S,
+                             int s0, int s1, int F, cudaStream_t s) {
+  if (s1 <= s0) return cudaSuccess;   // no window: nothing is read
   const FrameSplit fs = split_frames(F);
   const int quads = fs.padded() / 4;
   const int rows = std::max(1, 256 * kRepackItems * 2 / quads);
-  const unsigned grid = static_cast<unsigned>((N + rows - 1) / rows);
+  const unsigned grid = static_cast<unsigned>((TC * (s1 - s0) + rows - 1) / rows);
   const int vec = F % 4 == 0 ? 4 : (F % 2 == 0 ? 2 : 1);
   auto go = [&](auto* kernel) {
-    kernel<<<grid, 256, 0, s>>>(src, src_slot, dst, N, F, fs.full, fs.tail, rows);
+    kernel<<<grid, 256, 0, s>>>(src, src_slot, dst, TC, S, s0, s1 - s0, F, fs.full, fs.tail, rows);
     return cudaGetLastError();
   };
   switch (src_dtype) {

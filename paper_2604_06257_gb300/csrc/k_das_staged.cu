@@ -5,6 +5,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
+#include <climits>
 #include <cstdint>
 
 #include "das_staged.cuh"
@@ -70,27 +71,34 @@ __global__ void __launch_bounds__(256) k_tile_bounds(DasParams p, int per_cta, f
 }
 
 // Largest window over all (tile, transmit, element) and the number of pairs needing a
-// copy: out[0] = max rows, out[1] = pairs (saturating).
+// copy: out[0] = max rows, out[1] = pairs (saturating).  range (optional): the samples any
+// window touches, range[0] = first, range[1] = one past the last.
 __global__ void __launch_bounds__(256) k_window_stats(DasParams p, const float4* tbox, const float2* txr,
-                                                      int64_t tiles, int* out) {
+                                                      int64_t tiles, int* out, int* range) {
   const int64_t id = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (id >= tiles * p.C) return;
   const int64_t tile = id / p.C;
   const int c = static_cast<int>(id % p.C);
   const float4 e = p.elem[c];
-  int best = 0, n = 0;
+  int best = 0, n = 0, first = INT_MAX, last = 0;
   for (int t = 0; t < p.T; ++t) {
     int lo, rows;
     if (pair_window(tbox[2 * tile], tbox[2 * tile + 1], txr[tile * p.T + t], e, p, lo, rows)) {
       best = max(best, rows);
+      first = min(first, lo);
+      last = max(last, lo + rows);
       ++n;
     }
   }
   if (best) atomicMax(out, best);
   if (n) atomicAdd(out + 1, n);
+  if (range && n) {
+    atomicMin(range, first);
+    atomicMax(range + 1, last);
+  }
 }
 
-cudaError_t launch_tile_bounds(const DasParams& p, float4* tbox, float2* txr, int* d_out, cudaStream_t s) {
+cudaError_t launch_tile_bounds(const DasParams& p, float4* tbox, float2* txr, int* d_out, cudaStream_t s, int* d_range) {
   const int64_t tiles = static_cast<int64_t>(p.tiles_x) * p.tiles_y * p.tiles_z;
   const int per_cta = p.tile_x * p.tile_y * p.tile_z;
   k_tile_bounds<<<static_cast<unsigned>(tiles), 256, 0, s>>>(p, per_cta, tbox, txr);
@@ -98,7 +106,7 @@ cudaError_t launch_tile_bounds(const DasParams& p, float4* tbox, float2* txr, in
   if (e != cudaSuccess) return e;
   if ((e = cudaMemsetAsync(d_out, 0, 2 * sizeof(int), s)) != cudaSuccess) return e;
   const int64_t n = tiles * p.C;
-  k_window_stats<<<static_cast<unsigned>((n + 255) / 256), 256, 0, s>>>(p, tbox, txr, tiles, d_out);
+  k_window_stats<<<static_cast<unsigned>((n + 255) / 256), 256, 0, s>>>(p, tbox, txr, tiles, d_out, d_range);
   return cudaGetLastError();
 }
 

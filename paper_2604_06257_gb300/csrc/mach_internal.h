@@ -197,16 +197,19 @@ cudaError_t launch_iq_convert(const float2* src, int src_order, void* dst, int d
 cudaError_t launch_das(const DasParams& p, Variant v, cudaStream_t s);
 // Per-tile bounds for the staged variants; returns the largest window (rows) and the
 // number of (tile, transmit, element) triples that need a copy.
+// d_range (two ints the caller sets to a large value and 0, optional) receives the sample
+// range [first, last) that the windows touch.
 cudaError_t launch_tile_bounds(const DasParams& p, float4* tbox, float2* txr, int* d_rows_pairs,
-                               cudaStream_t s);
+                               cudaStream_t s, int* d_range = nullptr);
 size_t staged_smem_bytes(Variant v, int rows_cap, int F, int T, bool table);
 cudaError_t launch_das_staged(const DasParams& p, Variant v, cudaStream_t s);
 // Staged variants whose frame count is a compile-time constant (k_das_exact.cu).
 size_t exact_smem_bytes(Variant v, int rows_cap, int T);
-// Rows of N = T C S samples in any storage type into the tiles of split_frames(F) at dst.
-// The source is read from *src_slot (device memory) when that is given.
-cudaError_t launch_iq_repack(const void* src, const void* const* src_slot, int src_dtype, float* dst, int64_t N, int F,
-                             cudaStream_t s);
+// Samples [s0, s1) of TC rows of S samples in any storage type into the tiles of
+// split_frames(F) at dst; the other samples' places are left as they are (no window touches
+// them).  The source is read from *src_slot (device memory) when that is given.
+cudaError_t launch_iq_repack(const void* src, const void* const* src_slot, int src_dtype, float* dst, int64_t TC, int S,
+                             int s0, int s1, int F, cudaStream_t s);
 // Exact-frame kernel over `tiles` repacked frame tiles of variant_shape(v).frame_tile frames.
 cudaError_t launch_das_parts(const DasParams& p, Variant v, int tiles, cudaStream_t s);
 // pd, or *pd_slot (device memory; may hold NULL) when that is given.
@@ -253,7 +256,7 @@ const DasParams* plan_params(mach_plan p);
 // A plan for a batch: as mach_das_plan without a workspace pool.  plan_repack: the launches
 // over its repacked tiles (0 when it beamforms directly), and the workspace they need.
 mach_status make_batch_plan(const mach_das_desc* d, void* stream, mach_plan* out);
-int plan_repack(mach_plan p, const RepackPart** parts, size_t* ws_bytes, size_t* pd_at);
+int plan_repack(mach_plan p, const RepackPart** parts, size_t* ws_bytes, size_t* pd_at, int range[2]);
 int plan_iq_dtype(mach_plan p);
 void pick_tile_shape(int n, int nx, int ny, int nz, bool list, int tile[3]);
 

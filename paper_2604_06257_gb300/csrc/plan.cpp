@@ -41,6 +41,7 @@ struct mach_plan_s {
   int n_parts = 0;
   size_t ws_bytes = 0;          // workspace of one run: repacked IQ, partial Power Doppler sums
   size_t pd_at = 0;
+  int range[2] = {0, 0};        // samples that the parts' windows touch
   cudaMemPool_t pool = nullptr;
 };
 
@@ -476,7 +477,10 @@ static mach_status repack_plan(mach_plan_s* p, const DasParams& b, bool list, cu
       }
     return e;
   };
-  if (dev_alloc(reinterpret_cast<void**>(&d_stats), 2 * sizeof(int), &scratch) != MACH_OK) return done(MACH_OK);
+  if (dev_alloc(reinterpret_cast<void**>(&d_stats), 4 * sizeof(int), &scratch) != MACH_OK) return done(MACH_OK);
+  const int unset[2] = {INT32_MAX, 0};
+  if (cudaMemcpyAsync(d_stats + 2, unset, sizeof(unset), cudaMemcpyHostToDevice, s) != cudaSuccess)
+    return done(MACH_ERR_CUDA);
   for (int k = 0; k < n; ++k) {
     RepackPart& q = p->parts[k];
     const VariantShape& sh = variant_shape(want[k].v);
@@ -490,8 +494,8 @@ static mach_status repack_plan(mach_plan_s* p, const DasParams& b, bool list, cu
     t.frame_tiles = fs.tiles();
     t.tbox = q.d_tbox;
     t.txr = q.d_txr;
-    int stats[2] = {0, 0};
-    if (launch_tile_bounds(t, q.d_tbox, q.d_txr, d_stats, s) != cudaSuccess ||
+    int stats[4] = {0, 0, 0, 0};   // largest window, windows, sample range so far
+    if (launch_tile_bounds(t, q.d_tbox, q.d_txr, d_stats, s, d_stats + 2) != cudaSuccess ||
         cudaMemcpyAsync(stats, d_stats, sizeof(stats), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
       return done(MACH_ERR_CUDA);
@@ -504,6 +508,8 @@ static mach_status repack_plan(mach_plan_s* p, const DasParams& b, bool list, cu
     q.v = want[k].v;
     q.tiles = want[k].tiles;
     q.base = t;
+    p->range[0] = stats[2];
+    p->range[1] = stats[3];
     q.at = k == 0 ? 0 : static_cast<size_t>(N) * 8 * 32 * fs.full;
   }
   p->pd_at = iq_bytes;
@@ -803,8 +809,8 @@ static bool run_repacked(mach_plan p, const void* iq, float* pd, void* y, cudaSt
     return false;
   }
   const DasParams& b = p->base;
-  const int64_t N = static_cast<int64_t>(b.T) * b.C * b.S;
-  cudaError_t e = launch_iq_repack(iq, nullptr, p->d.iq_dtype, reinterpret_cast<float*>(ws), N, b.F, s);
+  cudaError_t e = launch_iq_repack(iq, nullptr, p->d.iq_dtype, reinterpret_cast<float*>(ws),
+                                   static_cast<int64_t>(b.T) * b.C, b.S, p->range[0], p->range[1], b.F, s);
   float* part = reinterpret_cast<float*>(ws + p->pd_at);
   for (int k = 0; k < p->n_parts && e == cudaSuccess; ++k) {
     DasParams q = p->parts[k].base;
@@ -965,7 +971,9 @@ namespace mach {
 mach_status make_batch_plan(const mach_das_desc* d, void* stream, mach_plan* out) {
   return make_plan(d, stream, false, out);
 }
-int plan_repack(mach_plan p, const RepackPart** parts, size_t* ws_bytes, size_t* pd_at) {
+int plan_repack(mach_plan p, const RepackPart** parts, size_t* ws_bytes, size_t* pd_at, int range[2]) {
+  range[0] = p->range[0];
+  range[1] = p->range[1];
   *parts = p->parts;
   *ws_bytes = p->ws_bytes;
   *pd_at = p->pd_at;
