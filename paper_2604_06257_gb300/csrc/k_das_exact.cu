@@ -1,6 +1,8 @@
 // k_das_exact.cu -- the staged delay-and-sum kernel for split complex64 rows when the
-// ensemble fills the frame tile exactly (F = 32 or F = 64), with receive delays evaluated
-// on the fly (Sec. 4.3's hybrid delays) and reused across the frames (Sec. 4.4).
+// ensemble fills the frame tile exactly (F = 8, 16, 32 or 64), with receive delays evaluated
+// on the fly (Sec. 4.3's hybrid delays) and reused across the frames (Sec. 4.4); the same for
+// the frame tiles of repacked ensembles, of one acquisition (launch_das_parts) or of many in
+// one launch (launch_das_multi).
 //
 // Same work, order and arithmetic as k_das_staged<C64Planar, ...> (das_staged.cuh): the
 // same producer warp stages each usable (element, transmit) pair's sample window into a
