@@ -403,7 +403,7 @@ def das_leg(acq, iq_c64, dt, steps, warmup, flush, stream, cpu_check=True, err_v
 
 
 def ragged_leg(args, flush, steps=3):
-    """The 64-instance ragged batch (float16 IQ) in one persistent launch replayed from a
+    """The 64-instance ragged batch (float16 IQ), one batch run replayed from a
     CUDA graph, default tile shapes."""
     import torch
     import synth
@@ -440,7 +440,7 @@ def ragged_leg(args, flush, steps=3):
     del iqs
     return {"value": points / t, "unit": UNIT, "ms_per_step": t * 1e3, "steps": steps,
             "config": {"workload": f"{len(acqs)} seeded instances (seed 4, 2D and 3D, 1-48 frames, 1-15 transmits, "
-                                   "float16 IQ), one persistent launch replayed from a CUDA graph, default tile shapes",
+                                   "float16 IQ), one batch run replayed from a CUDA graph, default tile shapes",
                        "points_per_step": points}, "batch": info}
 
 
@@ -727,7 +727,7 @@ def run_ours(args):
 
 def run_ragged(args):
     """64 seeded instances (2D and 3D, 1-48 frames, 1-15 transmits, float16 IQ) in one
-    persistent launch: default shapes, autotuned shapes, and the same instances beamformed
+    batch run: default shapes, autotuned shapes, and the same instances beamformed
     one plan after another."""
     import torch
     import synth

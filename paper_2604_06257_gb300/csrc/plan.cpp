@@ -434,9 +434,11 @@ static mach_status build_term_table(mach_plan_s* p, DasParams& b, cudaStream_t s
 // exact-frame kernels.
 // What it buys (251 x 251 px, 128 elements, 2048 samples, V / S = 31, cold L2; direct kernel
 // -> repacking and exact-frame kernels, us): complex64 5 frames 304 -> 71, 8: 214 -> 71,
-// 16: 214 -> 86, 25: 314 -> 122, 32: 154 -> 123, 40: 273 -> 192, 64: 378 -> 234,
-// 200: 1193 -> 731; float16 25: 322 -> 124, 32: 162 -> 125, 64: 257 -> 235.  The odd counts
-// gain most: the direct kernels read them one frame at a time.
+// 16: 214 -> 86, 25: 314 -> 122, 32: 154 -> 116, 40: 273 -> 192, 64: 378 -> 234,
+// 200: 1193 -> 731; float16 25: 322 -> 124, 32: 162 -> 125, 64: 257 -> 235.  (All but
+// complex64 at 32 frames with every sample rewritten; only those that windows touch are now,
+// which took 25 frames from 123 to 111 between other work.)  The odd counts gain most: the
+// direct kernels read them one frame at a time.
 // The repacking costs one pass over the IQ whatever the grid, the gain grows with the voxels
 // that read each sample, V / S; hence the bounds below.  A workspace above a sixteenth of
 // the device's memory, a capturing stream, or a failed workspace allocation takes the direct
