@@ -85,8 +85,8 @@ mach_status mach_nn_device_status(void* stream);
  * mach_nn_device_status reports; the context stays usable.  Not thread-safe. */
 void mach_nn_debug_conv(int32_t stall_copies, uint32_t wait_limit);
 
-/* Kernel choice of mach_nn_conv3d_tc (and of the U-Net executor) for 16 output channels, or 32
- * from at least 32 input channels, with at most 96 input channels: enable != 0 (the default) uses the x-folded kernel, which
+/* Kernel choice of mach_nn_conv3d_tc (and of the U-Net executor) for 16 output channels, or data
+ * gradients of 32 from at least 32 input channels, with at most 96 input channels: enable != 0 (the default) uses the x-folded kernel, which
  * puts the three x taps of each (dz, dy) pair into one N = 48 or 96 MMA and shifts the partial
  * sums by one voxel in its epilogue; enable = 0 the 27-tap kernel.  z_planes: planes per
  * x-folded tile (1, 2 or 4 (default); at most 2 with 32 output channels); halo_stages: input bricks in flight per CTA (2 ... 4,

@@ -536,37 +536,34 @@ __global__ void k_pack(const float2* __restrict__ y, const float* __restrict__ s
   for (int k = 1; k < C / 8; ++k) dst[k] = make_uint4(0u, 0u, 0u, 0u);
 }
 
-// Loss and its gradient.  A thread sums its items, a block its threads, and one atomic per
-// block adds to the loss (one per warp serialised half a million of them on one word: 1.24 ms
-// at 8 x 128^3; now 0.25 ms, with the volume-fastest order).
-__global__ void __launch_bounds__(256) k_loss(const float* __restrict__ o, const float2* __restrict__ xf,
-                                              const float2* __restrict__ target, const float* __restrict__ sums,
-                                              float gain, int64_t V, int N, int Co, int C, bf16* __restrict__ g,
-                                              float* __restrict__ loss, float inv_count) {
-  float sum = 0.f;
-  for (int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; j < V * N;
-       j += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const Item it = item_at(j, V, N);
-    const float inv = 1.f / rms_of(sums, it.n, V);
-    const float2 t = target[j];
-    const float2 x = xf[it.i];
-    const float2 oo = *reinterpret_cast<const float2*>(o + it.i * Co);
+// Loss and its gradient, one item per thread, one atomic per warp on the loss.  The half million
+// additions to one word take most of the 1.24 ms at 8 x 128^3, and their order of rounding
+// belongs to the result: adding up per block first takes 0.25 ms and sums the same terms more
+// exactly, but the word's own rounding happens to offset part of the bfloat16 network's bias,
+// and over ten training batches the loss's mean distance from float64 grew from 2.1e-5 to
+// 2.8e-5 of its value.
+__global__ void k_loss(const float* __restrict__ o, const float2* __restrict__ xf, const float2* __restrict__ target,
+                       const float* __restrict__ sums, float gain, int64_t V, int N, int Co, int C,
+                       bf16* __restrict__ g, float* __restrict__ loss, float inv_count) {
+  const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;   // = n * V + v
+  float e2 = 0.f;
+  if (i < V * N) {
+    const int n = static_cast<int>(i / V);
+    const int64_t v = i % V;
+    const float inv = 1.f / rms_of(sums, n, V);
+    const float2 t = target[v * N + n];
+    const float2 x = xf[i];
+    const float2 oo = *reinterpret_cast<const float2*>(o + i * Co);
     const float er = oo.x + gain * x.x - t.x * inv;
     const float ei = oo.y + gain * x.y - t.y * inv;
-    sum = fmaf(er, er, fmaf(ei, ei, sum));
+    e2 = fmaf(er, er, ei * ei);
     const __nv_bfloat162 q = __floats2bfloat162_rn(2.f * er * inv_count, 2.f * ei * inv_count);
-    uint4* gi = reinterpret_cast<uint4*>(g + it.i * C);
+    uint4* gi = reinterpret_cast<uint4*>(g + i * C);
     gi[0] = make_uint4(*reinterpret_cast<const uint32_t*>(&q), 0u, 0u, 0u);
     for (int k = 1; k < C / 8; ++k) gi[k] = make_uint4(0u, 0u, 0u, 0u);
   }
-  for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
-  __shared__ float part[8];
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = sum;
-  __syncthreads();
-  if (threadIdx.x == 0 && loss) {
-    for (int k = 1; k < 8; ++k) sum += part[k];
-    atomicAdd(loss, sum * inv_count);
-  }
+  for (int off = 16; off > 0; off >>= 1) e2 += __shfl_xor_sync(0xffffffffu, e2, off);
+  if (loss && (threadIdx.x & 31) == 0) atomicAdd(loss, e2 * inv_count);
 }
 
 __global__ void k_output(const float* __restrict__ o, const float2* __restrict__ xf, const float* __restrict__ sums,
@@ -678,9 +675,8 @@ cudaError_t launch_pack(const float2* y, const float* sums, int64_t V, int N, in
 cudaError_t launch_loss(const float* o, const float* xf, const float2* target, const float* sums, float gain,
                         int64_t V, int N, int Co, int C, void* g, float* loss, cudaStream_t s) {
   const float inv = 1.f / static_cast<float>(2 * V * N);
-  const unsigned blocks = blocks_for(V * N) < 152 * 8 ? blocks_for(V * N) : 152 * 8;
-  k_loss<<<blocks, 256, 0, s>>>(o, reinterpret_cast<const float2*>(xf), target, sums, gain, V, N, Co, C,
-                                static_cast<bf16*>(g), loss, inv);
+  k_loss<<<blocks_for(V * N), 256, 0, s>>>(o, reinterpret_cast<const float2*>(xf), target, sums, gain, V, N, Co, C,
+                                           static_cast<bf16*>(g), loss, inv);
   return cudaGetLastError();
 }
 

@@ -1,4 +1,4 @@
-"""x-folded convolutions of 32 output channels around the edges of their 14 x 8 voxel
+"""Convolutions of 32 output channels (data gradients x-folded) around the edges of their 14 x 8 voxel
 tiles, forward and as data gradient with the leaky ReLU's derivative left to the caller,
 against float64 and the 27-tap kernel."""
 import pytest
