@@ -42,6 +42,8 @@ struct ExactLayout {
   __host__ __device__ size_t meta_off() const { return tx_off() + (tx_bytes + 15) / 16 * 16; }
   __host__ __device__ size_t bar_off() const { return meta_off() + NBUF * 32; }
   __host__ __device__ size_t total() const { return bar_off() + 2 * NBUF * 8; }
+  // repacked tiles: two more rows, of zeros
+  __host__ __device__ size_t zero_off() const { return (total() + 127) / 128 * 128; }
 };
 
 __device__ __forceinline__ float4 lds128(uint32_t a) {
@@ -174,9 +176,12 @@ bool windows_hold(const DasParams& p) { return p.S <= kWindowsHold; }
 
 //
 // PART: the launch covers frames p.f_first ... of an ensemble of p.f_total frames that the
-// frame tiles need not fill: a tile's rows (zero beyond the last
+// frame tiles need not fill.  A tile's rows (zero beyond the last
 // frame) start p.iq_tile_bytes after the previous tile's, frames past the last one are not
 // written, and Power Doppler leaves as one partial sum per tile when there are several.
+// Dropped terms read two rows of zeros instead of the window's first two, so that an infinite
+// or NaN sample reaches only the voxels whose kept terms touch it, as with the direct kernels
+// that repacked ensembles would otherwise take.
 //
 // das_exact_block is one block's work.  W says what that is: voxel tile, frame tile and
 // outputs, read where they are needed (a value kept across the hot loop costs registers that
@@ -210,6 +215,10 @@ __device__ __forceinline__ void das_exact_block(const DasParams& p, const W& w) 
       mbar_init(&empty[b], NWC);
     }
     mbar_init_fence();
+  }
+  if constexpr (PART) {
+    for (int i = threadIdx.x; i < 2 * RB / 16; i += (NWC + 1) * 32)
+      sts128(smem_u32(smem) + static_cast<uint32_t>(L.zero_off()) + i * 16, make_float4(0.f, 0.f, 0.f, 0.f));
   }
   __syncthreads();
 
@@ -291,7 +300,11 @@ __device__ __forceinline__ void das_exact_block(const DasParams& p, const W& w) 
       tw.w *= im_sign;
     }
     sts128(coef_w + store_at * 16, tw);
-    sts32(offs_w + store_at * 4, row * RB);
+    int off = row * RB;
+    if constexpr (PART) {
+      if (!active) off = static_cast<int>(L.zero_off()) - my_slot * static_cast<int>(slot_bytes);
+    }
+    sts32(offs_w + store_at * 4, off);
     const unsigned act = __ballot_sync(0xffffffffu, active);
     unsigned outm = 0u;
     if constexpr ((FLAGS & kInside) == 0) outm = __ballot_sync(0xffffffffu, outside);
@@ -443,6 +456,12 @@ __global__ void __launch_bounds__((NWC + 1) * 32) __maxnreg__(MAXR)
 
 }  // namespace
 
+size_t repacked_smem_bytes(Variant v, int rows_cap, int T) {
+  const VariantShape& sh = variant_shape(v);
+  const int rb = sh.frame_tile * 8;
+  return ExactLayout<8>(rows_cap, rb, T, sh.warps).zero_off() + 2 * rb;   // every such shape has 8 slots
+}
+
 size_t exact_smem_bytes(Variant v, int rows_cap, int T) {
   const VariantShape& sh = variant_shape(v);
   const int rb = sh.frame_tile * 8;
@@ -496,7 +515,7 @@ cudaError_t launch_das_exact(const DasParams& p, Variant v, cudaStream_t s) {
 // launch per run of equal frame tiles.
 cudaError_t launch_das_parts(const DasParams& p, Variant v, int tiles, cudaStream_t s) {
   DasParams q = p;
-  const size_t sm = exact_smem_bytes(v, p.rows_cap, p.T);
+  const size_t sm = repacked_smem_bytes(v, p.rows_cap, p.T);
   auto go = [&](auto* kernel, int nwc) -> cudaError_t {
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sm));
     if (e != cudaSuccess) return e;
@@ -517,7 +536,7 @@ cudaError_t launch_das_parts(const DasParams& p, Variant v, int tiles, cudaStrea
 
 cudaError_t launch_das_multi(const MultiArgs& a, Variant v, const int2* items, int n_items, cudaStream_t s) {
   size_t sm = 0;
-  for (int k = 0; k < a.n; ++k) sm = std::max(sm, exact_smem_bytes(v, a.p[k].rows_cap, a.p[k].T));
+  for (int k = 0; k < a.n; ++k) sm = std::max(sm, repacked_smem_bytes(v, a.p[k].rows_cap, a.p[k].T));
   auto go = [&](auto* kernel, int nwc) -> cudaError_t {
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sm));
     if (e != cudaSuccess) return e;

@@ -205,6 +205,7 @@ size_t staged_smem_bytes(Variant v, int rows_cap, int F, int T, bool table);
 cudaError_t launch_das_staged(const DasParams& p, Variant v, cudaStream_t s);
 // Staged variants whose frame count is a compile-time constant (k_das_exact.cu).
 size_t exact_smem_bytes(Variant v, int rows_cap, int T);
+size_t repacked_smem_bytes(Variant v, int rows_cap, int T);   // of the launches over repacked tiles
 // Samples [s0, s1) of TC rows of S samples in any storage type into the tiles of
 // split_frames(F) at dst; the other samples' places are left as they are (no window touches
 // them).  The source is read from *src_slot (device memory) when that is given.

@@ -502,7 +502,7 @@ static mach_status repack_plan(mach_plan_s* p, const DasParams& b, bool list, cu
         cudaStreamSynchronize(s) != cudaSuccess)
       return done(MACH_ERR_CUDA);
     t.rows_cap = std::max(2, stats[0]);
-    if (exact_smem_bytes(want[k].v, t.rows_cap, b.T) > kStagedSmemCap) return done(MACH_OK);
+    if (repacked_smem_bytes(want[k].v, t.rows_cap, b.T) > kStagedSmemCap) return done(MACH_OK);
     t.f_first = k == 0 ? 0 : 32 * fs.full;
     t.f_total = b.F;
     t.f_tile = k == 0 ? 0 : fs.full;

@@ -116,3 +116,28 @@ def test_batch_of_repacked_instances(dt):
             if pds is pd1 and i == len(acqs) - 4:
                 continue
             assert nrmse_db(pd.cpu().numpy()[idx].astype(np.float64), pd_ref) <= -100, i
+
+
+@pytest.mark.parametrize("F,direct", [(7, "frames_c64_scalar_ft32"), (25, "frames_c64_scalar_ft32"), (12, "frames_c64_ft16"),
+                                      (70, "frames_c64_ft64")])
+def test_nan_and_inf_samples_reach_only_kept_terms(F, direct):
+    """The same frames of the same voxels are not finite as with the kernel that skips dropped
+    terms."""
+    acq = dense(F, "c64", 2, 2)
+    x, _ = stored(acq, F)
+    for k, bad in ((0, float("nan")), (11, float("inf")), (23, -float("inf"))):
+        x[k % 2, k, 60 + k, (3 * k) % F] = bad
+        x[1 - k % 2, k, 40, (5 * k) % F] = bad
+    with m.Plan(**m.plan_kwargs(acq)) as p:
+        assert "+x" in p.info()["variant"]
+        y = p.run(x)
+    m.mach_debug_force_variant(direct)
+    try:
+        with m.Plan(**m.plan_kwargs(acq)) as p:
+            ref = p.run(x)
+    finally:
+        m.mach_debug_force_variant(None)
+    torch.cuda.synchronize()
+    ok = torch.isfinite(torch.view_as_real(ref)).all(-1)
+    assert bool(ok.any()) and not bool(ok.all())
+    assert torch.equal(torch.isfinite(torch.view_as_real(y)).all(-1), ok)
