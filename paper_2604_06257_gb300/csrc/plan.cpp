@@ -542,7 +542,7 @@ static mach_status repack_plan(mach_plan_s* p, const DasParams& b, bool list, cu
     p->pool = nullptr;
     return done(MACH_OK);
   }
-  p->device_bytes += bytes;
+  p->device_bytes += bytes + static_cast<int64_t>(p->ws_bytes);   // the pool keeps one workspace
   p->n_parts = n;
   return done(MACH_OK);
 }
