@@ -286,7 +286,7 @@ mach_status mach_batch_plan(const mach_das_desc* descs, int32_t n, const mach_ti
       void *tb = nullptr, *tr = nullptr, *st = nullptr;
       if (cudaMalloc(&tb, sizeof(float4) * 2 * tiles) != cudaSuccess ||
           cudaMalloc(&tr, sizeof(float2) * p.T * tiles) != cudaSuccess ||
-          cudaMalloc(&st, 2 * sizeof(int)) != cudaSuccess) {
+          cudaMalloc(&st, kBoundStats * sizeof(int)) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(tb);
         cudaFree(tr);
@@ -300,7 +300,7 @@ mach_status mach_batch_plan(const mach_das_desc* descs, int32_t n, const mach_ti
       p.tbox = static_cast<float4*>(tb);
       p.txr = static_cast<float2*>(tr);
       p.txr_stride = p.T;
-      int stats[2] = {0, 0};
+      int stats[kBoundStats] = {};
       if (launch_tile_bounds(p, static_cast<float4*>(tb), static_cast<float2*>(tr), static_cast<int*>(st), s) != cudaSuccess ||
           cudaMemcpyAsync(stats, st, sizeof(stats), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
           cudaStreamSynchronize(s) != cudaSuccess) {

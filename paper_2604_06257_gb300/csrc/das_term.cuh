@@ -111,9 +111,11 @@ __device__ __forceinline__ int64_t tile_voxel_blocked(const DasParams& p, int64_
 // the receive delay over the box lies between the distances from e to the nearest and
 // farthest points of the box.  Returns false when no voxel of the tile can have a kept
 // term (aperture or range rule), so the pair is skipped.  Two rows of margin on each
-// side absorb float rounding of the bounds.
+// side absorb float rounding of the bounds while the delays are below kReachHolds samples;
+// `reach` (optional) receives the largest one that enters a used pair's terms.
 __device__ __forceinline__ bool pair_window(const float4 blo, const float4 bhi, const float2 txr,
-                                            const float4 e, const DasParams& p, int& lo, int& rows) {
+                                            const float4 e, const DasParams& p, int& lo, int& rows,
+                                            float* reach = nullptr) {
   const float ax = blo.x - e.x, bx = bhi.x - e.x;
   const float ay = blo.y - e.y, by = bhi.y - e.y;
   const float az = blo.z - e.z, bz = bhi.z - e.z;
@@ -133,6 +135,7 @@ __device__ __forceinline__ bool pair_window(const float4 blo, const float4 bhi, 
   if (h < l + 1) return false;
   lo = l;
   rows = h - l + 1;
+  if (reach) *reach = fmaxf(rmax, fmaxf(fabsf(txr.x), fabsf(txr.y)));
   return true;
 }
 

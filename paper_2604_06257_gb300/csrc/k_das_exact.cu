@@ -120,26 +120,18 @@ struct Acc {
   float2 a[VPG][FPL];
 };
 
-// IQ of the block's frame tile (PART: one of several in p.iq, see das_exact_block).
-template <bool PART>
-__device__ __forceinline__ const unsigned char* tile_iq(const DasParams& p, unsigned ftile) {
-  const unsigned char* iq = static_cast<const unsigned char*>(p.iq);
-  if constexpr (PART) iq += ftile * p.iq_tile_bytes;
-  return iq;
-}
-
-// The terms of one pair when some kept term falls outside the staged window (not
-// expected: the windows carry a margin): such terms read their taps from global memory.
+// The terms of one pair when some kept term falls outside the staged window (delays beyond
+// those that windows_hold covers): such terms read their taps from global memory.
 // Out of line, with the accumulators passed and returned by value, so that neither its
 // registers nor an address of the accumulators burden the hot loop.
-template <int FT, int FPL, int VPG, int G, bool PART>
+template <int FT, int FPL, int VPG, int G>
 __device__ __noinline__ Acc<VPG, FPL> outside_pair(const DasParams& p, Acc<VPG, FPL> acc, const SlotMeta m,
                                                    const unsigned char* wsrc, uint32_t cw_at, uint32_t of_at, int jl,
-                                                   unsigned order) {
+                                                   int order) {
   constexpr int RB = FT * 8, IMO = FT * 4, FL = FT / FPL;
-  // chunk and half orders, the frame tile above them
-  const int swz = kHalves<FT, FPL> || PART ? order & 1 : order, hs = kHalves<FT, FPL> ? (order >> 1) & 1 : 0;
-  const unsigned char* gsrc = tile_iq<PART>(p, order >> 2) + ((static_cast<size_t>(m.t) * p.C + m.c) * p.S + m.lo) * RB + jl * 16;
+  const int swz = kHalves<FT, FPL> ? order & 1 : order, hs = kHalves<FT, FPL> ? order >> 1 : 0;   // chunk and half orders
+  const unsigned char* gsrc =
+      static_cast<const unsigned char*>(p.iq) + ((static_cast<size_t>(m.t) * p.C + m.c) * p.S + m.lo) * RB + jl * 16;
 #pragma unroll
   for (int k = 0; k < VPG; ++k) {
     const float4 cw = lds128(cw_at + k * G * 16);
@@ -165,15 +157,9 @@ __device__ __noinline__ Acc<VPG, FPL> outside_pair(const DasParams& p, Acc<VPG, 
 // bit 2: every kept term is known to lie in its staged window (windows_hold), so no term has to
 // look for its taps elsewhere.
 constexpr int kSleep = 1, kEarly = 2, kInside = 4;
-
-// A window spans the delays between a tile's nearest and farthest points plus two rows on each
-// side (pair_window).  The bounds and a term's own delay are float32 sums of at most a few
-// roundings of values below S, so for S <= 2^18 (an ulp of 1/64 row or less) they cannot
-// disagree by two rows (kWindowsHold; repacked ensembles are not longer).  The check and the
+// The plan decides that from the delays it has (DasParams::inside); the check and the
 // out-of-line path behind it cost registers: 94 x 94 x 178 voxels, 32 frames 91.4 -> 89.7 ms
-// without them.
-bool windows_hold(const DasParams& p) { return p.S <= kWindowsHold; }
-
+// without them.  Ensembles for which it does not hold are not repacked.
 //
 // PART: the launch covers frames p.f_first ... of an ensemble of p.f_total frames that the
 // frame tiles need not fill.  A tile's rows (zero beyond the last
@@ -197,6 +183,7 @@ __device__ __forceinline__ void das_exact_block(const DasParams& p, const W& w) 
   static_assert(FPL == 4 || FPL == 8, "4 or 8 frames per lane");
   static_assert(WV * PB == 32, "a round must fill the warp");
   static_assert(NBUF >= PB && NBUF % PB == 0, "a round must fit in the ring");
+  static_assert(!PART || (FLAGS & kInside) != 0, "outside_pair reads p.iq as one frame tile");
   extern __shared__ __align__(128) unsigned char smem[];
   const ExactLayout<NBUF> L(p.rows_cap, RB, p.T, NWC);
   SlotMeta* meta = reinterpret_cast<SlotMeta*>(smem + L.meta_off());
@@ -224,7 +211,9 @@ __device__ __forceinline__ void das_exact_block(const DasParams& p, const W& w) 
 
   if (warp == NWC) {   // producer
     int r = 0;
-    const bool ok = produce_windows<NBUF>(p, tile_iq<PART>(p, w.ftile()), tile, lane, smem, L.slot_bytes, 8, meta, full, empty, r);
+    const unsigned char* iq = static_cast<const unsigned char*>(p.iq);
+    if constexpr (PART) iq += w.ftile() * p.iq_tile_bytes;
+    const bool ok = produce_windows<NBUF>(p, iq, tile, lane, smem, L.slot_bytes, 8, meta, full, empty, r);
     if (lane == 0) finish_producer<NBUF, PB>(p, ok, r, meta, full, empty);
     return;
   }
@@ -346,8 +335,8 @@ __device__ __forceinline__ void das_exact_block(const DasParams& p, const W& w) 
           }
         }
       } else {
-        acc = outside_pair<FT, FPL, VPG, G, PART>(p, acc, meta[slot], smem + slot * slot_bytes + jl * 16, cw_at, of_at,
-                                            jl, kHalves<FT, FPL> || PART ? swz | hs << 1 | w.ftile() << 2 : swz);
+        acc = outside_pair<FT, FPL, VPG, G>(p, acc, meta[slot], smem + slot * slot_bytes + jl * 16, cw_at, of_at,
+                                            jl, kHalves<FT, FPL> ? swz | hs << 1 : swz);
       }
       if constexpr ((FLAGS & kEarly) != 0) {   // every lane has read the slot: release it
         __syncwarp();
@@ -487,21 +476,21 @@ cudaError_t launch_das_exact(const DasParams& p, Variant v, cudaStream_t s) {
     case V_SX32_F8V1W15T24S: return go_staged(k_das_exact<32, 8, 1, 15, 8, 64, kSleep>, 15, p, sm, s);
     case V_SX32_F8V1W7T14: return go_staged(k_das_exact<32, 8, 1, 7, 8, 64, 0>, 7, p, sm, s);
     case V_SX32_F8V1W7T14E: case V_SX32_F8V1W7_T8X7E:
-      return windows_hold(p) ? go_staged(k_das_exact<32, 8, 1, 7, 8, 64, kEarly | kInside>, 7, p, sm, s)
-                             : go_staged(k_das_exact<32, 8, 1, 7, 8, 64, kEarly>, 7, p, sm, s);
+      return p.inside ? go_staged(k_das_exact<32, 8, 1, 7, 8, 64, kEarly | kInside>, 7, p, sm, s)
+                      : go_staged(k_das_exact<32, 8, 1, 7, 8, 64, kEarly>, 7, p, sm, s);
     case V_SX32_F4V2W7T14: return go_staged(k_das_exact<32, 4, 2, 7, 8, 64, 0>, 7, p, sm, s);
     case V_SX32_F8V1W15T30R12: return go_staged(k_das_exact<32, 8, 1, 15, 12, 64, 0>, 15, p, sm, s);
     case V_SX32_F8V1W15T30R12E: return go_staged(k_das_exact<32, 8, 1, 15, 12, 64, kEarly>, 15, p, sm, s);
     case V_SX64_C64P: case V_SX64_C64P_T16: case V_SX64_C64P_T8X8:
-      return windows_hold(p) ? go_staged(k_das_exact<64, 4, 4, 8, 8, 72, kInside>, 8, p, sm, s)
-                             : go_staged(k_das_exact<64, 4, 4, 8, 8, 72, 0>, 8, p, sm, s);
+      return p.inside ? go_staged(k_das_exact<64, 4, 4, 8, 8, 72, kInside>, 8, p, sm, s)
+                      : go_staged(k_das_exact<64, 4, 4, 8, 8, 72, 0>, 8, p, sm, s);
     case V_SX64_C64P_T16E: return go_staged(k_das_exact<64, 4, 4, 8, 8, 72, kEarly>, 8, p, sm, s);
     case V_SX64_C64PS: return go_staged(k_das_exact<64, 4, 4, 8, 8, 72, kSleep>, 8, p, sm, s);
     case V_SX64_C64PE: return go_staged(k_das_exact<64, 4, 4, 8, 8, 72, kEarly>, 8, p, sm, s);
     case V_SX64_F8V2: return go_staged(k_das_exact<64, 8, 2, 8, 8, 72, 0>, 8, p, sm, s);
     case V_SX16_F4V2W7: case V_SX16_F4V2W7_T8X14:
-      return windows_hold(p) ? go_staged(k_das_exact<16, 4, 2, 7, 8, 64, kEarly | kInside>, 7, p, sm, s)
-                             : go_staged(k_das_exact<16, 4, 2, 7, 8, 64, kEarly>, 7, p, sm, s);
+      return p.inside ? go_staged(k_das_exact<16, 4, 2, 7, 8, 64, kEarly | kInside>, 7, p, sm, s)
+                      : go_staged(k_das_exact<16, 4, 2, 7, 8, 64, kEarly>, 7, p, sm, s);
     case V_SX16_F8V1W7: return go_staged(k_das_exact<16, 8, 1, 7, 8, 64, kEarly>, 7, p, sm, s);
     case V_SX16_F8V1W4: return go_staged(k_das_exact<16, 8, 1, 4, 8, 64, kEarly>, 4, p, sm, s);
     case V_SX8_F8V1W4: return go_staged(k_das_exact<8, 8, 1, 4, 8, 64, kEarly>, 4, p, sm, s);

@@ -70,9 +70,10 @@ __global__ void __launch_bounds__(256) k_tile_bounds(DasParams p, int per_cta, f
   }
 }
 
-// Largest window over all (tile, transmit, element) and the number of pairs needing a
-// copy: out[0] = max rows, out[1] = pairs (saturating).  range (optional): the samples any
-// window touches, range[0] = first, range[1] = one past the last.
+// Largest window over all (tile, transmit, element), the number of pairs needing a copy and
+// the largest delay behind any window: out[0] = max rows, out[1] = pairs (saturating), out[2] =
+// samples as the bits of a non-negative float.  range (optional): the samples any window
+// touches, range[0] = first, range[1] = one past the last.
 __global__ void __launch_bounds__(256) k_window_stats(DasParams p, const float4* tbox, const float2* txr,
                                                       int64_t tiles, int* out, int* range) {
   const int64_t id = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -81,10 +82,13 @@ __global__ void __launch_bounds__(256) k_window_stats(DasParams p, const float4*
   const int c = static_cast<int>(id % p.C);
   const float4 e = p.elem[c];
   int best = 0, n = 0, first = INT_MAX, last = 0;
+  float far = 0.f;
   for (int t = 0; t < p.T; ++t) {
     int lo, rows;
-    if (pair_window(tbox[2 * tile], tbox[2 * tile + 1], txr[tile * p.T + t], e, p, lo, rows)) {
+    float reach;
+    if (pair_window(tbox[2 * tile], tbox[2 * tile + 1], txr[tile * p.T + t], e, p, lo, rows, &reach)) {
       best = max(best, rows);
+      far = fmaxf(far, reach);
       first = min(first, lo);
       last = max(last, lo + rows);
       ++n;
@@ -92,6 +96,7 @@ __global__ void __launch_bounds__(256) k_window_stats(DasParams p, const float4*
   }
   if (best) atomicMax(out, best);
   if (n) atomicAdd(out + 1, n);
+  if (n) atomicMax(out + 2, __float_as_int(far));
   if (range && n) {
     atomicMin(range, first);
     atomicMax(range + 1, last);
@@ -104,7 +109,7 @@ cudaError_t launch_tile_bounds(const DasParams& p, float4* tbox, float2* txr, in
   k_tile_bounds<<<static_cast<unsigned>(tiles), 256, 0, s>>>(p, per_cta, tbox, txr);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  if ((e = cudaMemsetAsync(d_out, 0, 2 * sizeof(int), s)) != cudaSuccess) return e;
+  if ((e = cudaMemsetAsync(d_out, 0, kBoundStats * sizeof(int), s)) != cudaSuccess) return e;
   const int64_t n = tiles * p.C;
   k_window_stats<<<static_cast<unsigned>((n + 255) / 256), 256, 0, s>>>(p, tbox, txr, tiles, d_out, d_range);
   return cudaGetLastError();

@@ -143,6 +143,7 @@ struct DasParams {
   // repacked ensembles only (F is then the frame tile, frame_tiles the tiles of all launches)
   int f_first, f_total;       // first frame of the launch, frames of the ensemble
   int f_tile;                 // frame tiles of the launches before this one
+  int inside;                 // exact-frame kernels: every kept term lies in its staged window (windows_hold)
   size_t iq_tile_bytes;       // repacked bytes of one frame tile
 };
 
@@ -156,7 +157,16 @@ struct FrameSplit {
   int tiles() const { return full + (tail ? 1 : 0); }
   int padded() const { return 32 * full + tail; }
 };
-constexpr int kWindowsHold = 1 << 18;   // samples up to which a term cannot leave its staged window
+// Whether a kept term provably lies in its staged window.  A window spans the delays between a
+// tile's nearest and farthest points plus two rows on each side (pair_window).  Its bounds and
+// a term's own delay s = s_tx + rx add the same two quantities, rx each time as a float32
+// root of a sum of three squares in some order, which differ by at most 4.5 units of 2^-24
+// relative to the larger one: below 2^20 samples by 0.3 rows.  Both sums round once more by at
+// most 2^-7 rows, s being below S <= 2^18.  (s below S does not bound s_tx and rx: with a large
+// t0, or transmit delays of the user's, they cancel; from 2^25 samples on the bounds do miss terms.)
+constexpr int kWindowsHold = 1 << 18;       // samples per row
+constexpr float kReachHolds = 1048576.f;    // samples of receive or transmit delay, 2^20
+inline bool windows_hold(int S, float reach) { return S <= kWindowsHold && reach <= kReachHolds; }
 struct RepackPart {             // one launch: equal frame tiles on one exact-frame shape
   Variant v = V_COUNT;
   int tiles = 0;
@@ -195,11 +205,13 @@ cudaError_t launch_tables(const TableParams& tp, cudaStream_t s);
 cudaError_t launch_iq_convert(const float2* src, int src_order, void* dst, int dst_dtype, int64_t T, int64_t C,
                               int64_t S, int64_t F, cudaStream_t s);
 cudaError_t launch_das(const DasParams& p, Variant v, cudaStream_t s);
-// Per-tile bounds for the staged variants; returns the largest window (rows) and the
-// number of (tile, transmit, element) triples that need a copy.
+// Per-tile bounds for the staged variants; d_stats (kBoundStats ints) receives the largest
+// window (rows), the number of (tile, transmit, element) triples that need a copy, and the
+// largest delay of those (bits of a float; see windows_hold).
 // d_range (two ints the caller sets to a large value and 0, optional) receives the sample
 // range [first, last) that the windows touch.
-cudaError_t launch_tile_bounds(const DasParams& p, float4* tbox, float2* txr, int* d_rows_pairs,
+constexpr int kBoundStats = 3;
+cudaError_t launch_tile_bounds(const DasParams& p, float4* tbox, float2* txr, int* d_stats,
                                cudaStream_t s, int* d_range = nullptr);
 size_t staged_smem_bytes(Variant v, int rows_cap, int F, int T, bool table);
 cudaError_t launch_das_staged(const DasParams& p, Variant v, cudaStream_t s);

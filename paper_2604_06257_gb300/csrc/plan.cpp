@@ -68,6 +68,12 @@ mach_status dev_alloc(void** p, size_t bytes, int64_t* total) {
   return MACH_OK;
 }
 
+float float_of(int bits) {
+  float f;
+  std::memcpy(&f, &bits, sizeof(f));
+  return f;
+}
+
 bool finite3(const float* p, int64_t n) {
   for (int64_t i = 0; i < 3 * n; ++i)
     if (!std::isfinite(p[i])) return false;
@@ -479,9 +485,10 @@ static mach_status repack_plan(mach_plan_s* p, const DasParams& b, bool list, cu
       }
     return e;
   };
-  if (dev_alloc(reinterpret_cast<void**>(&d_stats), 4 * sizeof(int), &scratch) != MACH_OK) return done(MACH_OK);
+  if (dev_alloc(reinterpret_cast<void**>(&d_stats), (kBoundStats + 2) * sizeof(int), &scratch) != MACH_OK)
+    return done(MACH_OK);
   const int unset[2] = {INT32_MAX, 0};
-  if (cudaMemcpyAsync(d_stats + 2, unset, sizeof(unset), cudaMemcpyHostToDevice, s) != cudaSuccess)
+  if (cudaMemcpyAsync(d_stats + kBoundStats, unset, sizeof(unset), cudaMemcpyHostToDevice, s) != cudaSuccess)
     return done(MACH_ERR_CUDA);
   for (int k = 0; k < n; ++k) {
     RepackPart& q = p->parts[k];
@@ -496,12 +503,13 @@ static mach_status repack_plan(mach_plan_s* p, const DasParams& b, bool list, cu
     t.frame_tiles = fs.tiles();
     t.tbox = q.d_tbox;
     t.txr = q.d_txr;
-    int stats[4] = {0, 0, 0, 0};   // largest window, windows, sample range so far
-    if (launch_tile_bounds(t, q.d_tbox, q.d_txr, d_stats, s, d_stats + 2) != cudaSuccess ||
+    int stats[kBoundStats + 2] = {};   // bounds, sample range so far
+    if (launch_tile_bounds(t, q.d_tbox, q.d_txr, d_stats, s, d_stats + kBoundStats) != cudaSuccess ||
         cudaMemcpyAsync(stats, d_stats, sizeof(stats), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
       return done(MACH_ERR_CUDA);
     t.rows_cap = std::max(2, stats[0]);
+    if (!windows_hold(b.S, float_of(stats[2]))) return done(MACH_OK);   // its kernels have no other way
     if (repacked_smem_bytes(want[k].v, t.rows_cap, b.T) > kStagedSmemCap) return done(MACH_OK);
     t.f_first = k == 0 ? 0 : 32 * fs.full;
     t.f_total = b.F;
@@ -510,8 +518,8 @@ static mach_status repack_plan(mach_plan_s* p, const DasParams& b, bool list, cu
     q.v = want[k].v;
     q.tiles = want[k].tiles;
     q.base = t;
-    p->range[0] = stats[2];
-    p->range[1] = stats[3];
+    p->range[0] = stats[kBoundStats];
+    p->range[1] = stats[kBoundStats + 1];
     q.at = k == 0 ? 0 : static_cast<size_t>(N) * 8 * 32 * fs.full;
   }
   p->pd_at = iq_bytes;
@@ -725,7 +733,8 @@ static mach_status make_plan(const mach_das_desc* d, void* stream, bool own_pool
       return fail(st);
     if ((st = dev_alloc(reinterpret_cast<void**>(&p->d_txr), sizeof(float2) * T * tiles_max, &p->device_bytes)) != MACH_OK)
       return fail(st);
-    if ((st = dev_alloc(reinterpret_cast<void**>(&d_stats), 2 * sizeof(int), &scratch_bytes)) != MACH_OK) return fail(st);
+    if ((st = dev_alloc(reinterpret_cast<void**>(&d_stats), kBoundStats * sizeof(int), &scratch_bytes)) != MACH_OK)
+      return fail(st);
     b.tbox = p->d_tbox;
     b.txr = p->d_txr;
     bool fits = false;
@@ -736,13 +745,14 @@ static mach_status make_plan(const mach_das_desc* d, void* stream, bool own_pool
         if ((st = configure_tiles(b, var, list, V, F)) != MACH_OK) return fail(st);
       }
       if (launch_tile_bounds(b, p->d_tbox, p->d_txr, d_stats, s) != cudaSuccess) return fail(MACH_ERR_CUDA);
-      int stats[2] = {0, 0};
+      int stats[kBoundStats] = {};
       if (cudaMemcpyAsync(stats, d_stats, sizeof(stats), cudaMemcpyDeviceToHost, s) != cudaSuccess)
         return fail(MACH_ERR_CUDA);
       if (cudaStreamSynchronize(s) != cudaSuccess) return fail(MACH_ERR_CUDA);
       p->rows_cap = std::max(2, stats[0]);
       p->copy_pairs = stats[1];
       b.rows_cap = p->rows_cap;
+      b.inside = windows_hold(S, float_of(stats[2]));
       fits = staged_smem_bytes(var, p->rows_cap, F, T, tab) <= kStagedSmemCap;
     }
     if (!fits) {
