@@ -25,6 +25,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <cstdint>
+#include <type_traits>
 
 #include "das_slices.cuh"
 #include "das_staged.cuh"
@@ -166,11 +167,22 @@ static_assert(kSlices == kBatchWarps && kSlices * 4 * kSliceVox * sizeof(float2)
               "the slices' sums fit the scratch");
 static_assert(sizeof(BatchSlotMeta) == 48, "slot metadata (BatchLayout reserves 48 bytes per slot)");
 
+// The block's ring lives as long as the block: its barriers are initialised once and every
+// staged item goes on where the last one ended (an mbarrier may not be initialised again
+// while it is valid).  Uses are counted modulo two turns of the ring, which keeps slot and parity: use
+// k takes slot k % kBatchRing, its copy completes phase (k / kBatchRing) & 1 of that slot's
+// "full" barrier, and it may start once the "empty" phase before has completed (on a fresh
+// barrier the phase before the first counts as completed).
+constexpr int kRingWrap = 2 * kBatchRing;
+__device__ __forceinline__ int ring_slot(int k) { return k % kBatchRing; }
+__device__ __forceinline__ uint32_t ring_full(int k) { return (k / kBatchRing) & 1; }
+__device__ __forceinline__ uint32_t ring_empty(int k) { return ((k / kBatchRing) & 1) ^ 1; }
+
 // Producer of one staged item: like produce_windows, for rows of any length.  A window is
 // rows x F complex samples starting at byte `start` of the IQ array; the bulk copy covers
 // [start rounded down to 16 bytes, end rounded up to 16 bytes), clamped so that it never
 // reads past the array (a window whose end would be clamped loses its last rows: terms
-// there read global memory).
+// there read global memory).  r counts the ring's uses.
 template <class IQ>
 __device__ __forceinline__ bool batch_produce(const DasParams& p, int64_t tile, int lane, unsigned char* ring,
                                               size_t slot_bytes, BatchSlotMeta* meta, uint64_t* full, uint64_t* empty,
@@ -207,8 +219,8 @@ __device__ __forceinline__ bool batch_produce(const DasParams& p, int64_t tile, 
       ej.z = __shfl_sync(0xffffffffu, e.z, j);
       ej.w = 0.f;
       if (lane == 0) {
-        const int slot = r % kBatchRing;
-        if (r >= kBatchRing && !mbar_wait_bounded(&empty[slot], ((r / kBatchRing) - 1) & 1, p.wait_limit)) {
+        const int slot = ring_slot(r);
+        if (!mbar_wait_bounded(&empty[slot], ring_empty(r), p.wait_limit)) {
           atomicOr(p.err, 1);
           ok = false;
         } else {
@@ -242,11 +254,11 @@ __device__ __forceinline__ bool batch_produce(const DasParams& p, int64_t tile, 
 // Consumers of one staged item (generic staged consumer of das_staged.cuh with the
 // instance's parameters in shared memory and a per-slot row offset).  FL lanes per voxel,
 // 4 frames per lane: VEC = 4 consecutive frames (F % 4 == 0) or VEC = 1 with NV = 4 frames
-// FL apart.
+// FL apart.  r0: the ring's first use by this item, then by the next.  False when a wait gave up.
 template <class IQ, int VEC, int NV, int FL>
-__device__ __forceinline__ void batch_consume(const DasParams& p, int64_t tile, int warp, int lane,
+__device__ __forceinline__ bool batch_consume(const DasParams& p, int64_t tile, int warp, int lane,
                                               const unsigned char* ring, size_t slot_bytes, float4* terms, float* txc,
-                                              const BatchSlotMeta* meta, uint64_t* full, uint64_t* empty) {
+                                              const BatchSlotMeta* meta, uint64_t* full, uint64_t* empty, int& r0) {
   constexpr int VPG = 4;
   constexpr int G = 32 / FL;
   constexpr int WV = G * VPG;
@@ -278,9 +290,10 @@ __device__ __forceinline__ void batch_consume(const DasParams& p, int64_t tile, 
   geo.rx = 0.f;
   geo.a = -1.f;
   bool ok = true, done = false;
-  for (int r = 0; !done; r += PB) {
-    const int mine = r + sub, my_slot = mine % kBatchRing;
-    const bool got = mbar_wait_bounded(&full[my_slot], (mine / kBatchRing) & 1, p.wait_limit);
+  int r = r0;
+  for (; !done; r += PB) {
+    const int mine = r + sub, my_slot = ring_slot(mine);
+    const bool got = mbar_wait_bounded(&full[my_slot], ring_full(mine), p.wait_limit);
     if (__any_sync(0xffffffffu, !got)) {
       if (lane == 0) atomicOr(p.err, 1);
       ok = false;
@@ -317,7 +330,7 @@ __device__ __forceinline__ void batch_consume(const DasParams& p, int64_t tile, 
         break;
       }
       if (!(act & gm)) continue;
-      const int slot = (r + i) % kBatchRing;
+      const int slot = ring_slot(r + i);
       const int lo = meta[slot].lo, rows = meta[slot].rows;
       const E* win = ringE + slot * slot_elems + meta[slot].skip * IqStore<IQ>::eps;
       const float4* tp = terms + i * WV;
@@ -351,9 +364,10 @@ __device__ __forceinline__ void batch_consume(const DasParams& p, int64_t tile, 
       }
     }
     __syncwarp();
-    if (lane < PB) mbar_arrive(&empty[(r + lane) % kBatchRing]);
+    if (lane < PB) mbar_arrive(&empty[ring_slot(r + lane)]);
   }
-  if (!ok) return;
+  if (!ok) return false;
+  r0 = r % kRingWrap;   // the markers fill the last round
 #pragma unroll
   for (int k = 0; k < VPG; ++k) {
     const int64_t v = tile_voxel(p, tile, warp * WV + g * VPG + k);
@@ -374,6 +388,7 @@ __device__ __forceinline__ void batch_consume(const DasParams& p, int64_t tile, 
     for (int o = FL / 2; o > 0; o >>= 1) pw += __shfl_xor_sync(0xffffffffu, pw, o);
     if (jl == 0 && v >= 0 && p.pd) p.pd[v] = pw;
   }
+  return true;
 }
 
 // counter[0]: next work item; counter[1]: blocks that have finished.
@@ -389,6 +404,14 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 2)
   uint64_t* empty = full + kBatchRing;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   unsigned char* scratch = smem + L.scratch_off() + warp * (L.scratch_bytes / kBatchWarps);
+  if (threadIdx.x == 0) {
+    for (int b = 0; b < kBatchRing; ++b) {
+      mbar_init(&full[b], 1);
+      mbar_init(&empty[b], kBatchConsumers);
+    }
+    mbar_init_fence();
+  }
+  int ring_at = 0;   // the ring's next use (visible barriers: the loop's first __syncthreads)
   for (;;) {
     if (threadIdx.x == 0) s_item = atomicAdd(&counter[0], 1);
     __syncthreads();
@@ -400,50 +423,60 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 2)
     const DasParams p = B.p;
     const int mode = B.mode, fl = B.frame_lanes;
     if (mode == kBatchStaged) {
-      if (threadIdx.x == 0) {   // a fresh ring for this item
-        for (int b = 0; b < kBatchRing; ++b) {
-          mbar_init(&full[b], 1);
-          mbar_init(&empty[b], kBatchConsumers);
-        }
-        mbar_init_fence();
-      }
-      __syncthreads();
+      bool ok = true;
+      int copied = ring_at, used = ring_at;   // one past the item's copies, and past its markers
       if (warp == kBatchConsumers) {
-        int r = 0;
-        const bool ok = batch_produce<IQ>(p, w.y, lane, smem, slot_bytes, meta, full, empty, r);
-        if (lane == 0) {   // end markers (one per pair a consumer round holds), or drain
-          const int PB = fl == 16 ? 4 : 2;
-          if (ok) {
-            for (int k = 0; k < PB; ++k) {
-              const int rr = r + k, slot = rr % kBatchRing;
-              if (rr >= kBatchRing && !mbar_wait_bounded(&empty[slot], ((rr / kBatchRing) - 1) & 1, p.wait_limit)) {
-                atomicOr(p.err, 1);
-                break;
-              }
-              meta[slot].c = -1;
-              mbar_arrive(&full[slot]);
+        ok = batch_produce<IQ>(p, w.y, lane, smem, slot_bytes, meta, full, empty, copied);
+        // end markers (of no element) up to a whole round of the consumers, one at least
+        const int PB = fl == 16 ? 4 : 2;
+        const int ends = PB - (copied - ring_at) % PB;
+        used = copied;
+        if (lane == 0 && ok) {
+          for (int k = 0; k < ends; ++k) {
+            const int slot = ring_slot(used);
+            if (!mbar_wait_bounded(&empty[slot], ring_empty(used), p.wait_limit)) {
+              atomicOr(p.err, 1);
+              ok = false;
+              break;
             }
-          } else {
-            for (int k = max(0, r - kBatchRing); k < r; ++k)
-              mbar_wait_bounded(&full[k % kBatchRing], (k / kBatchRing) & 1, p.wait_limit);
+            meta[slot].c = -1;
+            mbar_arrive(&full[slot]);
+            ++used;
           }
         }
       } else {
         float4* terms = reinterpret_cast<float4*>(scratch);
         float* txc = reinterpret_cast<float*>(scratch + 32 * 16);
+        auto consume = [&](auto vec, auto nv, auto lanes) {
+          ok = batch_consume<IQ, decltype(vec)::value, decltype(nv)::value, decltype(lanes)::value>(
+              p, w.y, warp, lane, smem, slot_bytes, terms, txc, meta, full, empty, used);
+        };
+        using I1 = std::integral_constant<int, 1>;
+        using I2 = std::integral_constant<int, 2>;
+        using I4 = std::integral_constant<int, 4>;
+        using I8 = std::integral_constant<int, 8>;
+        using I16 = std::integral_constant<int, 16>;
         // 16-byte vectors when F % 4 == 0, 8-byte pairs for the other even F, else single samples
         const int vec = p.F % 4 == 0 ? 4 : (p.F % 2 == 0 ? 2 : 1);
         if (fl == 16) {
-          if (vec == 4) batch_consume<IQ, 4, 1, 16>(p, w.y, warp, lane, smem, slot_bytes, terms, txc, meta, full, empty);
-          else if (vec == 2) batch_consume<IQ, 2, 2, 16>(p, w.y, warp, lane, smem, slot_bytes, terms, txc, meta, full, empty);
-          else batch_consume<IQ, 1, 4, 16>(p, w.y, warp, lane, smem, slot_bytes, terms, txc, meta, full, empty);
+          if (vec == 4) consume(I4{}, I1{}, I16{});
+          else if (vec == 2) consume(I2{}, I2{}, I16{});
+          else consume(I1{}, I4{}, I16{});
         } else {
-          if (vec == 4) batch_consume<IQ, 4, 1, 8>(p, w.y, warp, lane, smem, slot_bytes, terms, txc, meta, full, empty);
-          else if (vec == 2) batch_consume<IQ, 2, 2, 8>(p, w.y, warp, lane, smem, slot_bytes, terms, txc, meta, full, empty);
-          else batch_consume<IQ, 1, 4, 8>(p, w.y, warp, lane, smem, slot_bytes, terms, txc, meta, full, empty);
+          if (vec == 4) consume(I4{}, I1{}, I8{});
+          else if (vec == 2) consume(I2{}, I2{}, I8{});
+          else consume(I1{}, I4{}, I8{});
         }
       }
-      __syncthreads();   // the ring is drained before the next item re-initialises it
+      if (__syncthreads_or(!ok)) {
+        // A wait gave up, and the warps no longer agree on the ring: this block takes no more
+        // items.  The copies whose slots no marker took over land before it leaves.
+        if (warp == kBatchConsumers && lane == 0)
+          for (int k = max(ring_at, used - kBatchRing); k < copied; ++k)
+            mbar_wait_bounded(&full[ring_slot(k)], ring_full(k), p.wait_limit);
+        break;
+      }
+      ring_at = __shfl_sync(0xffffffffu, used, 0) % kRingWrap;
     } else if (mode == kBatchChannels) {
       // the scratch of all warps as one array: 8 slices x F x 32 sums
       float2* part = reinterpret_cast<float2*>(smem + L.scratch_off());

@@ -1,5 +1,7 @@
 """Ragged batches: many instances in one persistent launch, against the FP64 oracle and
 against single-instance plans; graph capture; the autotuner's choices."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -194,3 +196,61 @@ def test_ragged_batch_full_scale_bench_instances():
         assert ep <= -60, (a.name, ep)
         worst_y, worst_pd = max(worst_y, ey), max(worst_pd, ep)
     print(f"64 instances at full scale: worst frames NRMSE {worst_y:.1f} dB, worst Power Doppler {worst_pd:.1f} dB")
+
+
+def staged_batch():
+    """Twelve instances of several staged items per block each, of both lane mappings, every load width
+    and (last) the other two modes between them."""
+    frames = [25, 18, 28, 33, 34, 36, 25, 49, 20, 50, 3, 12]
+    base = synth.make_acquisition("doppler2d", "small")
+    mid = len(base.elem_pos) // 2
+    acqs = [base.replace(grid_dims=(112, 1, 96 + 4 * (i % 3)), grid_origin=(-5.6e-3, 0.0, 5e-3), grid_step=(1e-4, 0.0, 1e-4),
+                         elem_pos=base.elem_pos[mid - 15 - i:mid + 15], tx_angles=np.zeros((1 + i % 2, 2)), n_samples=460,
+                         n_frames=F) for i, F in enumerate(frames)]
+    shapes = [(2, 8 if F <= 32 else 16, None) if F > 16 else (1, 0, None) if F <= 4 else (0, 4, None) for F in frames]
+    iqs = [synth.random_iq(a, 200 + i, device="cuda") for i, a in enumerate(acqs)]
+    return acqs, shapes, iqs
+
+
+def test_blocks_that_take_several_staged_items():
+    acqs, shapes, iqs = staged_batch()
+    ys = [torch.zeros((a.n_vox, a.n_frames), dtype=torch.complex64, device="cuda") for a in acqs]
+    with m.Batch([m.plan_kwargs(a) for a in acqs], shapes=shapes) as b:
+        info = b.info()
+        # a block cannot keep to one staged item
+        tiles = [np.prod([-(-n // t) for n, t in zip(a.grid_dims, s[2])]) for a, s in zip(acqs, info["shapes"]) if s[0] == 2]
+        assert sum(tiles) > 3 * info["blocks"], (tiles, info["blocks"])
+        b.bind(iqs, ys, None)
+        for _ in range(2):
+            b.run()
+        torch.cuda.synchronize()
+    for a, iq, y in zip(acqs, iqs, ys):
+        idx = np.arange(0, a.n_vox, 11)
+        y_ref, _ = oracle.das(a, iq.cpu(), idx)
+        assert nrmse_db(y.cpu().numpy()[idx], y_ref) <= -100, a.n_frames
+
+
+def test_staged_items_whose_copies_stall_end_the_launch():
+    """Every wait runs out; the blocks give up one item each and leave, and the next batch is right."""
+    acqs, shapes, iqs = staged_batch()
+    kws = [m.plan_kwargs(a) for a in acqs]
+    ys = [torch.zeros((a.n_vox, a.n_frames), dtype=torch.complex64, device="cuda") for a in acqs]
+    m.mach_debug_set_wait_limit(2000)
+    m.mach_debug_stall_producer(True)
+    try:
+        with m.Batch(kws, shapes=shapes) as b:
+            b.bind(iqs, ys, None)
+            t0 = time.perf_counter()
+            b.run()
+            torch.cuda.synchronize()
+            # a few waits of 2000 polls; one timeout per item would take several times that
+            assert time.perf_counter() - t0 < 1.0
+    finally:
+        m.mach_debug_stall_producer(False)
+        m.mach_debug_set_wait_limit(0)
+    with m.Batch(kws, shapes=shapes) as b:
+        b.bind(iqs, ys, None)
+        b.run()
+        torch.cuda.synchronize()
+    y_ref, _ = oracle.das(acqs[0], iqs[0].cpu(), np.arange(0, acqs[0].n_vox, 11))
+    assert nrmse_db(ys[0].cpu().numpy()[::11], y_ref) <= -100
