@@ -30,8 +30,9 @@
  *    error before launching leaves the outputs untouched.  CUDA errors map to
  *    MACH_ERR_CUDA.  No C++ exception crosses this boundary.
  *  - Workspaces: ensembles that no kernel reads directly in their storage type and frame
- *    count are rewritten into whole frame tiles on every run (grids of at least 6 or 16
- *    voxels per sample; mach_plan_info.variant then names the tiles, e.g. "+x32+x8").  Each
+ *    count are rewritten into whole frame tiles on every run where that was measured faster
+ *    (dense grids of at least 6 or 16 voxels per sample and enough work; mach_plan_info.variant
+ *    then names the tiles, e.g. "+x32+x8").  Each
  *    run takes its workspace, 8 bytes per sample and padded frame, in stream order from a
  *    memory pool that the plan owns (at most a sixteenth of the device memory per run; one
  *    workspace is kept between runs and released with the plan).  Runs on a capturing
@@ -347,10 +348,13 @@ void mach_debug_fail_alloc_after(int32_t n);
  *  - force the kernel variant named `name` (mach_plan_info.variant) for later plans, or
  *    restore the automatic choice with NULL / "".  INVALID_ARG for an unknown name;
  *    mach_das_plan returns UNSUPPORTED if the forced variant cannot serve the plan.
+ *  - rewrite ensembles into frame tiles (see Workspaces) wherever the kernels can, not only
+ *    where it is faster.
  *  - set the polls per bounded device wait (0 restores the default).
  *  - make the staged producer announce its copies without issuing them, so that the
  *    consumers' waits run out (exercises MACH_ERR_TIMEOUT without a fault). */
 mach_status mach_debug_force_variant(const char *name);
+void mach_debug_force_repack(int32_t on);
 void mach_debug_set_wait_limit(uint32_t polls);
 void mach_debug_stall_producer(int32_t on);
 

@@ -30,7 +30,7 @@ ORDER = {"tcsf": 0, "ftcs": 1}
 EXPORTS = ("mach_das_plan", "mach_das_run", "mach_power_doppler", "mach_plan_destroy",
            "mach_status_string", "mach_plan_get_info", "mach_plan_tx_table", "mach_das_terms",
            "mach_version", "mach_debug_fail_alloc_after", "mach_plan_device_status",
-           "mach_debug_force_variant", "mach_debug_set_wait_limit", "mach_debug_stall_producer",
+           "mach_debug_force_variant", "mach_debug_force_repack", "mach_debug_set_wait_limit", "mach_debug_stall_producer",
            "mach_das_run_noalloc", "mach_iq_convert", "mach_batch_plan", "mach_batch_bind",
            "mach_batch_run", "mach_batch_get_info", "mach_batch_destroy", "mach_das_run_per_tx",
            "mach_rf_to_iq", "mach_power_doppler_host_stream")
@@ -117,6 +117,8 @@ def lib():
         L.mach_plan_device_status.restype = C.c_int
         L.mach_debug_force_variant.argtypes = [C.c_char_p]
         L.mach_debug_force_variant.restype = C.c_int
+        L.mach_debug_force_repack.argtypes = [i32]
+        L.mach_debug_force_repack.restype = None
         L.mach_debug_set_wait_limit.argtypes = [C.c_uint32]
         L.mach_debug_set_wait_limit.restype = None
         L.mach_debug_stall_producer.argtypes = [i32]
@@ -158,6 +160,10 @@ def mach_debug_force_variant(name) -> None:
     st = lib().mach_debug_force_variant(None if not name else name.encode())
     if st != MACH_OK:
         raise MachError(st, "mach_debug_force_variant")
+
+
+def mach_debug_force_repack(on: bool) -> None:
+    lib().mach_debug_force_repack(1 if on else 0)
 
 
 def mach_debug_set_wait_limit(polls: int) -> None:

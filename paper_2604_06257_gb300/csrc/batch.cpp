@@ -286,7 +286,7 @@ mach_status mach_batch_plan(const mach_das_desc* descs, int32_t n, const mach_ti
       void *tb = nullptr, *tr = nullptr, *st = nullptr;
       if (cudaMalloc(&tb, sizeof(float4) * 2 * tiles) != cudaSuccess ||
           cudaMalloc(&tr, sizeof(float2) * p.T * tiles) != cudaSuccess ||
-          cudaMalloc(&st, kBoundStats * sizeof(int)) != cudaSuccess) {
+          cudaMalloc(&st, sizeof(BoundStats)) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(tb);
         cudaFree(tr);
@@ -300,14 +300,14 @@ mach_status mach_batch_plan(const mach_das_desc* descs, int32_t n, const mach_ti
       p.tbox = static_cast<float4*>(tb);
       p.txr = static_cast<float2*>(tr);
       p.txr_stride = p.T;
-      int stats[kBoundStats] = {};
-      if (launch_tile_bounds(p, static_cast<float4*>(tb), static_cast<float2*>(tr), static_cast<int*>(st), s) != cudaSuccess ||
-          cudaMemcpyAsync(stats, st, sizeof(stats), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+      BoundStats stats{};
+      if (launch_tile_bounds(p, static_cast<float4*>(tb), static_cast<float2*>(tr), static_cast<BoundStats*>(st), s) != cudaSuccess ||
+          cudaMemcpyAsync(&stats, st, sizeof(stats), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
           cudaStreamSynchronize(s) != cudaSuccess) {
         release(b);
         return MACH_ERR_CUDA;
       }
-      p.rows_cap = std::max(2, stats[0]);
+      p.rows_cap = std::max(2, stats.rows);
       const size_t sample = (dt == MACH_IQ_F16X2 || dt == MACH_IQ_BF16X2) ? 4 : 8;
       const size_t need = (static_cast<size_t>(p.rows_cap) * p.F * sample + 32 + 127) / 128 * 128;
       if (need <= kBatchSlotCap) {

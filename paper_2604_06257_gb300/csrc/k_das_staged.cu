@@ -5,7 +5,6 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
-#include <climits>
 #include <cstdint>
 
 #include "das_staged.cuh"
@@ -70,18 +69,15 @@ __global__ void __launch_bounds__(256) k_tile_bounds(DasParams p, int per_cta, f
   }
 }
 
-// Largest window over all (tile, transmit, element), the number of pairs needing a copy and
-// the largest delay behind any window: out[0] = max rows, out[1] = pairs (saturating), out[2] =
-// samples as the bits of a non-negative float.  range (optional): the samples any window
-// touches, range[0] = first, range[1] = one past the last.
+// What the windows over all (tile, transmit, element) need (see BoundStats).
 __global__ void __launch_bounds__(256) k_window_stats(DasParams p, const float4* tbox, const float2* txr,
-                                                      int64_t tiles, int* out, int* range) {
+                                                      int64_t tiles, BoundStats* out) {
   const int64_t id = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (id >= tiles * p.C) return;
   const int64_t tile = id / p.C;
   const int c = static_cast<int>(id % p.C);
   const float4 e = p.elem[c];
-  int best = 0, n = 0, first = INT_MAX, last = 0;
+  int best = 0, n = 0, first = p.S, last = 0;
   float far = 0.f;
   for (int t = 0; t < p.T; ++t) {
     int lo, rows;
@@ -94,24 +90,23 @@ __global__ void __launch_bounds__(256) k_window_stats(DasParams p, const float4*
       ++n;
     }
   }
-  if (best) atomicMax(out, best);
-  if (n) atomicAdd(out + 1, n);
-  if (n) atomicMax(out + 2, __float_as_int(far));
-  if (range && n) {
-    atomicMin(range, first);
-    atomicMax(range + 1, last);
-  }
+  if (n == 0) return;
+  atomicMax(&out->rows, best);
+  atomicMax(&out->reach_bits, __float_as_int(far));
+  atomicAdd(&out->pairs, static_cast<unsigned long long>(n));
+  atomicMax(&out->from_end, p.S - first);
+  atomicMax(&out->last, last);
 }
 
-cudaError_t launch_tile_bounds(const DasParams& p, float4* tbox, float2* txr, int* d_out, cudaStream_t s, int* d_range) {
+cudaError_t launch_tile_bounds(const DasParams& p, float4* tbox, float2* txr, BoundStats* d_out, cudaStream_t s) {
   const int64_t tiles = static_cast<int64_t>(p.tiles_x) * p.tiles_y * p.tiles_z;
   const int per_cta = p.tile_x * p.tile_y * p.tile_z;
   k_tile_bounds<<<static_cast<unsigned>(tiles), 256, 0, s>>>(p, per_cta, tbox, txr);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  if ((e = cudaMemsetAsync(d_out, 0, kBoundStats * sizeof(int), s)) != cudaSuccess) return e;
+  if ((e = cudaMemsetAsync(d_out, 0, sizeof(BoundStats), s)) != cudaSuccess) return e;
   const int64_t n = tiles * p.C;
-  k_window_stats<<<static_cast<unsigned>((n + 255) / 256), 256, 0, s>>>(p, tbox, txr, tiles, d_out, d_range);
+  k_window_stats<<<static_cast<unsigned>((n + 255) / 256), 256, 0, s>>>(p, tbox, txr, tiles, d_out);
   return cudaGetLastError();
 }
 

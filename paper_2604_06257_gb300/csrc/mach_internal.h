@@ -205,14 +205,14 @@ cudaError_t launch_tables(const TableParams& tp, cudaStream_t s);
 cudaError_t launch_iq_convert(const float2* src, int src_order, void* dst, int dst_dtype, int64_t T, int64_t C,
                               int64_t S, int64_t F, cudaStream_t s);
 cudaError_t launch_das(const DasParams& p, Variant v, cudaStream_t s);
-// Per-tile bounds for the staged variants; d_stats (kBoundStats ints) receives the largest
-// window (rows), the number of (tile, transmit, element) triples that need a copy, and the
-// largest delay of those (bits of a float; see windows_hold).
-// d_range (two ints the caller sets to a large value and 0, optional) receives the sample
-// range [first, last) that the windows touch.
-constexpr int kBoundStats = 3;
-cudaError_t launch_tile_bounds(const DasParams& p, float4* tbox, float2* txr, int* d_stats,
-                               cudaStream_t s, int* d_range = nullptr);
+// Per-tile bounds for the staged variants, and what their windows need.
+struct BoundStats {
+  int rows;                    // the largest window
+  int reach_bits;              // the largest delay behind a window (a non-negative float's bits; see windows_hold)
+  unsigned long long pairs;    // (tile, transmit, element) triples that need a copy
+  int from_end, last;          // samples that windows touch: [S - from_end, last)
+};
+cudaError_t launch_tile_bounds(const DasParams& p, float4* tbox, float2* txr, BoundStats* d_stats, cudaStream_t s);
 size_t staged_smem_bytes(Variant v, int rows_cap, int F, int T, bool table);
 cudaError_t launch_das_staged(const DasParams& p, Variant v, cudaStream_t s);
 // Staged variants whose frame count is a compile-time constant (k_das_exact.cu).

@@ -49,6 +49,7 @@ namespace {
 
 int g_fail_alloc_countdown = 0;   // test hook: > 0 -> the n-th allocation fails
 int g_force_variant = -1;         // test hook: variant index, or -1 for automatic choice
+bool g_force_repack = false;      // test hook: repack whenever the kernels can
 uint32_t g_wait_limit = 0;        // test hook: polls per bounded wait (0 = default)
 int g_stall = 0;                  // test hook: staged producer never issues its copies
 constexpr uint32_t kDefaultWaitLimit = 1u << 24;   // ~ seconds of polling
@@ -445,10 +446,41 @@ static mach_status build_term_table(mach_plan_s* p, DasParams& b, cudaStream_t s
 // complex64 at 32 frames with every sample rewritten; only those that windows touch are now,
 // which took 25 frames from 123 to 111 between other work.)  The odd counts gain most: the
 // direct kernels read them one frame at a time.
-// The repacking costs one pass over the IQ whatever the grid, the gain grows with the voxels
-// that read each sample, V / S; hence the bounds below.  A workspace above a sixteenth of
-// the device's memory, a capturing stream, or a failed workspace allocation takes the direct
-// kernel.
+// The repacking costs a few launches and one pass over the IQ, the gain grows with the voxels
+// that read each sample: hence the bounds on V / S, and repack_pays.  A workspace above a
+// sixteenth of the device's memory, a capturing stream, or a failed workspace allocation takes
+// the direct kernel.
+
+// Whether repacking pays over the direct kernel, from what the repacked launches would do: points
+// (voxels x windows x padded frames) and their share of the whole grid's, and the direct
+// kernel's tiles.  Measured as the direct kernel's time over the repacked run's, cold L2: 2D
+// grids of 48^2 ... 384^2 px with 64 ... 192 elements, 3D of 20^3 ... 64^3 voxels with 256 and
+// 576, 1 ... 9 transmits, F-numbers 1 ... 6 and no aperture, all storage types.
+//  * L1 kernels (5 to 16 frames, odd and long ensembles): 1.05 ... 5.5 wherever V >= 6 S.
+//  * Staged kernels of 32 frames, which read split or interleaved rows as they are: complex64
+//    0.81 ... 1.7 below 1e7 points (half of them below 1.04), 0.96 ... 1.2 at a share below 0.2,
+//    else 1.01 ... 2.15; 16-bit pairs, whose rows are half as long, 0.62 ... 1.8 below 4e7 points,
+//    0.89 ... 0.97 at a share of 1/9, else 1.04 ... 2.1.
+//  * Staged kernels of 64 frames (33 to 64): a tile holds 8 x 4 or 16 x 4 voxels for all frames, and
+//    two frame tiles double the term evaluations: 0.40 ... 1.5, slower in more than half of the
+//    grids.  From three waves of two blocks per SM and a share of 0.3 on, where the direct
+//    kernel's tail is short and its terms many: 0.99 ... 1.5.  (A 64-frame ring of two pairs,
+//    taken for long windows: 0.87 ... 2.4, from 2e7 points on 0.97 ... 2.4.)
+//  * Batches: every instance's pass is a launch of its own (about 8 us in which the other
+//    instances wait), against the lane mappings of the persistent kernel: six equal instances
+//    0.45 ... 1.3 below 5e6 points each, 24 of them 0.85 ... 1.4 from 2e7 to 5e7, 0.98 ... 2.9 above.
+static bool repack_pays(Variant direct, bool batch, double points, double share, int64_t tiles) {
+  if (batch) return points >= 5e7;
+  switch (direct) {
+    case V_ST32_C64_V4W7: case V_ST32_C64P_V4W7: return points >= 1e7 && share >= 0.2;
+    case V_ST32_H16_V4: case V_ST32_B16_V4: return points >= 4e7 && share >= 0.125;
+    case V_ST64_C64: return points >= 2e7;
+    case V_ST64_C64_V4: case V_ST64_C64P_V4: case V_ST64_H16_V4: case V_ST64_B16_V4: case V_ST64_H16:
+      return tiles >= 3 * 2 * 152 && share >= 0.3;
+    default: return true;
+  }
+}
+
 static mach_status repack_plan(mach_plan_s* p, const DasParams& b, bool list, cudaStream_t s,
                                size_t total_mem, bool own_pool) {
   const VariantShape& direct = variant_shape(p->variant);
@@ -471,7 +503,7 @@ static mach_status repack_plan(mach_plan_s* p, const DasParams& b, bool list, cu
   //    8 frames: 4 per lane, 7 warps 64 | 115 | 2947 us; 8 per lane, 4 warps 91 | 138 | 2672 us
   if (fs.tail == 8) want[n++] = {grid3d ? V_SX8_F8V1W4 : V_SX8_F4V1W7, 1};
   if (fs.tail == 16) want[n++] = {grid3d ? V_SX16_F8V1W4 : b.T == 1 ? V_SX16_F8V1W7 : V_SX16_F4V1W7, 1};
-  int* d_stats = nullptr;
+  BoundStats* d_stats = nullptr;
   int64_t scratch = 0, bytes = 0;
   // every way out but the last one leaves the plan on its direct kernel
   auto done = [&](mach_status e) {
@@ -485,11 +517,7 @@ static mach_status repack_plan(mach_plan_s* p, const DasParams& b, bool list, cu
       }
     return e;
   };
-  if (dev_alloc(reinterpret_cast<void**>(&d_stats), (kBoundStats + 2) * sizeof(int), &scratch) != MACH_OK)
-    return done(MACH_OK);
-  const int unset[2] = {INT32_MAX, 0};
-  if (cudaMemcpyAsync(d_stats + kBoundStats, unset, sizeof(unset), cudaMemcpyHostToDevice, s) != cudaSuccess)
-    return done(MACH_ERR_CUDA);
+  if (dev_alloc(reinterpret_cast<void**>(&d_stats), 2 * sizeof(BoundStats), &scratch) != MACH_OK) return done(MACH_OK);
   for (int k = 0; k < n; ++k) {
     RepackPart& q = p->parts[k];
     const VariantShape& sh = variant_shape(want[k].v);
@@ -503,14 +531,6 @@ static mach_status repack_plan(mach_plan_s* p, const DasParams& b, bool list, cu
     t.frame_tiles = fs.tiles();
     t.tbox = q.d_tbox;
     t.txr = q.d_txr;
-    int stats[kBoundStats + 2] = {};   // bounds, sample range so far
-    if (launch_tile_bounds(t, q.d_tbox, q.d_txr, d_stats, s, d_stats + kBoundStats) != cudaSuccess ||
-        cudaMemcpyAsync(stats, d_stats, sizeof(stats), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess)
-      return done(MACH_ERR_CUDA);
-    t.rows_cap = std::max(2, stats[0]);
-    if (!windows_hold(b.S, float_of(stats[2]))) return done(MACH_OK);   // its kernels have no other way
-    if (repacked_smem_bytes(want[k].v, t.rows_cap, b.T) > kStagedSmemCap) return done(MACH_OK);
     t.f_first = k == 0 ? 0 : 32 * fs.full;
     t.f_total = b.F;
     t.f_tile = k == 0 ? 0 : fs.full;
@@ -518,10 +538,30 @@ static mach_status repack_plan(mach_plan_s* p, const DasParams& b, bool list, cu
     q.v = want[k].v;
     q.tiles = want[k].tiles;
     q.base = t;
-    p->range[0] = stats[kBoundStats];
-    p->range[1] = stats[kBoundStats + 1];
     q.at = k == 0 ? 0 : static_cast<size_t>(N) * 8 * 32 * fs.full;
+    if (launch_tile_bounds(t, q.d_tbox, q.d_txr, d_stats + k, s) != cudaSuccess) return done(MACH_ERR_CUDA);
   }
+  BoundStats stats[2] = {};
+  if (cudaMemcpyAsync(stats, d_stats, n * sizeof(BoundStats), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+      cudaStreamSynchronize(s) != cudaSuccess)
+    return done(MACH_ERR_CUDA);
+  double points = 0.0;
+  int lo = b.S, hi = 0;
+  for (int k = 0; k < n; ++k) {
+    DasParams& t = p->parts[k].base;
+    t.rows_cap = std::max(2, stats[k].rows);
+    if (!windows_hold(b.S, float_of(stats[k].reach_bits))) return done(MACH_OK);   // its kernels have no other way
+    if (repacked_smem_bytes(want[k].v, t.rows_cap, b.T) > kStagedSmemCap) return done(MACH_OK);
+    lo = std::min(lo, b.S - stats[k].from_end);
+    hi = std::max(hi, stats[k].last);
+    points += static_cast<double>(stats[k].pairs) * (t.tile_x * t.tile_y * t.tile_z) * t.F * want[k].tiles;
+  }
+  p->range[0] = lo;
+  p->range[1] = hi;
+  const double all = static_cast<double>(b.V) * b.C * b.T * fs.padded();
+  if (!g_force_repack && !repack_pays(p->variant, !own_pool, points, points / all,
+                                      static_cast<int64_t>(b.tiles_x) * b.tiles_y * b.tiles_z))
+    return done(MACH_OK);
   p->pd_at = iq_bytes;
   p->ws_bytes = iq_bytes + pd_bytes;
   if (!own_pool) {
@@ -642,7 +682,7 @@ static mach_status make_plan(const mach_das_desc* d, void* stream, bool own_pool
 
   float* d_raw = nullptr;
   double* d_u = nullptr;
-  int* d_stats = nullptr;
+  BoundStats* d_stats = nullptr;
   int64_t scratch_bytes = 0;
   auto fail = [&](mach_status e) {
     cudaFree(d_raw);
@@ -733,7 +773,7 @@ static mach_status make_plan(const mach_das_desc* d, void* stream, bool own_pool
       return fail(st);
     if ((st = dev_alloc(reinterpret_cast<void**>(&p->d_txr), sizeof(float2) * T * tiles_max, &p->device_bytes)) != MACH_OK)
       return fail(st);
-    if ((st = dev_alloc(reinterpret_cast<void**>(&d_stats), kBoundStats * sizeof(int), &scratch_bytes)) != MACH_OK)
+    if ((st = dev_alloc(reinterpret_cast<void**>(&d_stats), sizeof(BoundStats), &scratch_bytes)) != MACH_OK)
       return fail(st);
     b.tbox = p->d_tbox;
     b.txr = p->d_txr;
@@ -745,14 +785,14 @@ static mach_status make_plan(const mach_das_desc* d, void* stream, bool own_pool
         if ((st = configure_tiles(b, var, list, V, F)) != MACH_OK) return fail(st);
       }
       if (launch_tile_bounds(b, p->d_tbox, p->d_txr, d_stats, s) != cudaSuccess) return fail(MACH_ERR_CUDA);
-      int stats[kBoundStats] = {};
-      if (cudaMemcpyAsync(stats, d_stats, sizeof(stats), cudaMemcpyDeviceToHost, s) != cudaSuccess)
+      BoundStats stats{};
+      if (cudaMemcpyAsync(&stats, d_stats, sizeof(stats), cudaMemcpyDeviceToHost, s) != cudaSuccess)
         return fail(MACH_ERR_CUDA);
       if (cudaStreamSynchronize(s) != cudaSuccess) return fail(MACH_ERR_CUDA);
-      p->rows_cap = std::max(2, stats[0]);
-      p->copy_pairs = stats[1];
+      p->rows_cap = std::max(2, stats.rows);
+      p->copy_pairs = static_cast<int64_t>(stats.pairs);
       b.rows_cap = p->rows_cap;
-      b.inside = windows_hold(S, float_of(stats[2]));
+      b.inside = windows_hold(S, float_of(stats.reach_bits));
       fits = staged_smem_bytes(var, p->rows_cap, F, T, tab) <= kStagedSmemCap;
     }
     if (!fits) {
@@ -951,6 +991,8 @@ mach_status mach_debug_force_variant(const char* name) {
     }
   return MACH_ERR_INVALID_ARG;
 }
+
+void mach_debug_force_repack(int32_t on) { g_force_repack = on != 0; }
 
 void mach_debug_set_wait_limit(uint32_t polls) { g_wait_limit = polls; }
 

@@ -12,6 +12,14 @@ from metrics import nrmse_db
 
 pytestmark = pytest.mark.gpu
 
+
+@pytest.fixture(scope="module", autouse=True)
+def repack_small_grids():
+    """These grids are too small for repacking to pay; test_gpu_repack_rule.py has the rule."""
+    m.mach_debug_force_repack(True)
+    yield
+    m.mach_debug_force_repack(False)
+
 CASES = [(F, dt) for F in (5, 8, 9, 16, 17, 25, 31, 32, 33, 40, 41, 49, 64, 65, 100)
          for dt in ("c64", "f16x2", "bf16x2", "c64split")
          if dt != "c64split" or (F % 4 == 0 and F not in (8, 16, 32, 64))]

@@ -12,6 +12,13 @@ from metrics import nrmse_db
 
 pytestmark = pytest.mark.gpu
 
+
+@pytest.fixture(scope="module", autouse=True)
+def repack_wherever_the_kernels_can():
+    m.mach_debug_force_repack(True)
+    yield
+    m.mach_debug_force_repack(False)
+
 S, REACH = 200, 2.0 ** 26            # samples a record, samples of receive delay
 EDGE = 24                            # more rows than 4.5 units of 2^-24 of REACH
 
