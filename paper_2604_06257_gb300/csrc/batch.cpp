@@ -63,10 +63,6 @@ void release(mach_batch_s* b) {
   delete b;
 }
 
-// Largest ring slot the staged path uses: eight slots plus the per-warp scratch then leave
-// room for two blocks per SM.
-constexpr size_t kBatchSlotCap = 11 * 1024;
-
 int voxels_per_block(const mach_tile_shape& s) {
   if (s.mode == kBatchChannels) return 32;
   if (s.mode == kBatchStaged) return 7 * 4 * (32 / s.frame_lanes);   // 7 consumer warps + a producer warp

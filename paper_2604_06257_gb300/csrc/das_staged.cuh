@@ -401,7 +401,7 @@ constexpr int kRing = 4;    // ring slots (8 when a round holds 4 pairs)
 
 template <class K>
 cudaError_t go_staged(K kernel, int nwc, const DasParams& p, size_t smem, cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kStagedSmemCap));
   if (e != cudaSuccess) return e;
   const int64_t tiles = static_cast<int64_t>(p.tiles_x) * p.tiles_y * p.tiles_z;
   kernel<<<dim3(static_cast<unsigned>(tiles), static_cast<unsigned>(p.frame_tiles)), (nwc + 1) * 32, smem, s>>>(p);

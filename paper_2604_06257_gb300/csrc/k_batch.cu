@@ -509,10 +509,16 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 2)
 }
 
 template <class IQ>
+static cudaError_t raise_limit() {   // see kBatchSlotCap
+  return cudaFuncSetAttribute(k_das_batch<IQ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              static_cast<int>(BatchLayout(kBatchSlotCap).total()));
+}
+
+template <class IQ>
 static cudaError_t go_batch(const BatchInstance* insts, const int2* items, int n_items, int* counter, int grid,
                             size_t slot_bytes, cudaStream_t s) {
   const size_t smem = BatchLayout(slot_bytes).total();
-  cudaError_t e = cudaFuncSetAttribute(k_das_batch<IQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  const cudaError_t e = raise_limit<IQ>();
   if (e != cudaSuccess) return e;
   k_das_batch<IQ><<<grid, kBatchWarps * 32, smem, s>>>(insts, items, n_items, counter, slot_bytes);
   return cudaGetLastError();
@@ -526,16 +532,15 @@ int batch_blocks_per_sm(int iq_dtype, size_t slot_bytes) {
   cudaError_t e;
   switch (iq_dtype) {
     case MACH_IQ_F16X2:
-      cudaFuncSetAttribute(k_das_batch<__half2>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+      raise_limit<__half2>();
       e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_das_batch<__half2>, kBatchWarps * 32, smem);
       break;
     case MACH_IQ_BF16X2:
-      cudaFuncSetAttribute(k_das_batch<__nv_bfloat162>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(smem));
+      raise_limit<__nv_bfloat162>();
       e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_das_batch<__nv_bfloat162>, kBatchWarps * 32, smem);
       break;
     default:
-      cudaFuncSetAttribute(k_das_batch<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+      raise_limit<float2>();
       e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_das_batch<float2>, kBatchWarps * 32, smem);
       break;
   }

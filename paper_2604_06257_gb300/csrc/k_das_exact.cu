@@ -506,7 +506,8 @@ cudaError_t launch_das_parts(const DasParams& p, Variant v, int tiles, cudaStrea
   DasParams q = p;
   const size_t sm = repacked_smem_bytes(v, p.rows_cap, p.T);
   auto go = [&](auto* kernel, int nwc) -> cudaError_t {
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sm));
+    const cudaError_t e =
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kStagedSmemCap));
     if (e != cudaSuccess) return e;
     const int64_t blocks = static_cast<int64_t>(p.tiles_x) * p.tiles_y * p.tiles_z;
     kernel<<<dim3(static_cast<unsigned>(blocks), static_cast<unsigned>(tiles)), (nwc + 1) * 32, sm, s>>>(q);
@@ -527,7 +528,8 @@ cudaError_t launch_das_multi(const MultiArgs& a, Variant v, const int2* items, i
   size_t sm = 0;
   for (int k = 0; k < a.n; ++k) sm = std::max(sm, repacked_smem_bytes(v, a.p[k].rows_cap, a.p[k].T));
   auto go = [&](auto* kernel, int nwc) -> cudaError_t {
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sm));
+    const cudaError_t e =
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kStagedSmemCap));
     if (e != cudaSuccess) return e;
     kernel<<<static_cast<unsigned>(n_items), (nwc + 1) * 32, sm, s>>>(a, items);
     return cudaGetLastError();

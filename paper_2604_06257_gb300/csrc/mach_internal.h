@@ -213,6 +213,13 @@ struct BoundStats {
   int from_end, last;          // samples that windows touch: [S - from_end, last)
 };
 cudaError_t launch_tile_bounds(const DasParams& p, float4* tbox, float2* txr, BoundStats* d_stats, cudaStream_t s);
+// Largest shared memory of a staged kernel's block: room for two blocks per SM.  Launches raise
+// a kernel's limit to this, the same value for all of them: other threads' launches of
+// that kernel, with another plan's size, must not find a limit below theirs.
+constexpr size_t kStagedSmemCap = 110 * 1024;
+// Largest ring slot of the batch kernel: eight slots plus the per-warp scratch then leave room
+// for two blocks per SM.  Its limit is that of this slot, likewise.
+constexpr size_t kBatchSlotCap = 11 * 1024;
 size_t staged_smem_bytes(Variant v, int rows_cap, int F, int T, bool table);
 cudaError_t launch_das_staged(const DasParams& p, Variant v, cudaStream_t s);
 // Staged variants whose frame count is a compile-time constant (k_das_exact.cu).

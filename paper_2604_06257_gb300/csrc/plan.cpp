@@ -53,7 +53,6 @@ bool g_force_repack = false;      // test hook: repack whenever the kernels can
 uint32_t g_wait_limit = 0;        // test hook: polls per bounded wait (0 = default)
 int g_stall = 0;                  // test hook: staged producer never issues its copies
 constexpr uint32_t kDefaultWaitLimit = 1u << 24;   // ~ seconds of polling
-constexpr size_t kStagedSmemCap = 110 * 1024;       // leaves room for two blocks per SM
 
 mach_status dev_alloc(void** p, size_t bytes, int64_t* total) {
   *p = nullptr;
