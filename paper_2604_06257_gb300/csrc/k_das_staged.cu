@@ -69,33 +69,48 @@ __global__ void __launch_bounds__(256) k_tile_bounds(DasParams p, int per_cta, f
   }
 }
 
-// What the windows over all (tile, transmit, element) need (see BoundStats).
+// What the windows over all (tile, transmit, element) need (see BoundStats).  One thread per
+// (tile, element); a block adds up its threads' figures before it touches the five words that
+// all blocks share (a thread's own atomics there took most of a large plan's bounds).
 __global__ void __launch_bounds__(256) k_window_stats(DasParams p, const float4* tbox, const float2* txr,
                                                       int64_t tiles, BoundStats* out) {
+  __shared__ int sum[5];   // rows, reach, S - first, last, pairs
+  if (threadIdx.x < 5) sum[threadIdx.x] = 0;
+  __syncthreads();
   const int64_t id = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (id >= tiles * p.C) return;
-  const int64_t tile = id / p.C;
-  const int c = static_cast<int>(id % p.C);
-  const float4 e = p.elem[c];
-  int best = 0, n = 0, first = p.S, last = 0;
+  int best = 0, n = 0, from_end = 0, last = 0;
   float far = 0.f;
-  for (int t = 0; t < p.T; ++t) {
-    int lo, rows;
-    float reach;
-    if (pair_window(tbox[2 * tile], tbox[2 * tile + 1], txr[tile * p.T + t], e, p, lo, rows, &reach)) {
-      best = max(best, rows);
-      far = fmaxf(far, reach);
-      first = min(first, lo);
-      last = max(last, lo + rows);
-      ++n;
+  if (id < tiles * p.C) {
+    const int64_t tile = id / p.C;
+    const int c = static_cast<int>(id % p.C);
+    const float4 e = p.elem[c];
+    for (int t = 0; t < p.T; ++t) {
+      int lo, rows;
+      float reach;
+      if (pair_window(tbox[2 * tile], tbox[2 * tile + 1], txr[tile * p.T + t], e, p, lo, rows, &reach)) {
+        best = max(best, rows);
+        far = fmaxf(far, reach);
+        from_end = max(from_end, p.S - lo);
+        last = max(last, lo + rows);
+        ++n;
+      }
     }
   }
-  if (n == 0) return;
-  atomicMax(&out->rows, best);
-  atomicMax(&out->reach_bits, __float_as_int(far));
-  atomicAdd(&out->pairs, static_cast<unsigned long long>(n));
-  atomicMax(&out->from_end, p.S - first);
-  atomicMax(&out->last, last);
+  const int v[4] = {best, __float_as_int(far), from_end, last};   // none below zero
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int m = __reduce_max_sync(0xffffffffu, v[k]);
+    if ((threadIdx.x & 31) == 0) atomicMax(&sum[k], m);
+  }
+  const int pairs = __reduce_add_sync(0xffffffffu, n);
+  if ((threadIdx.x & 31) == 0) atomicAdd(&sum[4], pairs);
+  __syncthreads();
+  if (threadIdx.x != 0 || sum[4] == 0) return;
+  atomicMax(&out->rows, sum[0]);
+  atomicMax(&out->reach_bits, sum[1]);
+  atomicMax(&out->from_end, sum[2]);
+  atomicMax(&out->last, sum[3]);
+  atomicAdd(&out->pairs, static_cast<unsigned long long>(sum[4]));
 }
 
 cudaError_t launch_tile_bounds(const DasParams& p, float4* tbox, float2* txr, BoundStats* d_out, cudaStream_t s) {
