@@ -341,8 +341,11 @@ mach_status mach_das_run_noalloc(const mach_das_desc *d, const void *iq_dev, voi
 const char *mach_version(void);
 
 /* Test hook: make the n-th device allocation from now fail (n >= 1); n <= 0 disarms.
- * Lets tests exercise the MACH_ERR_OOM clean-up path without exhausting memory. */
+ * Lets tests exercise the MACH_ERR_OOM clean-up path without exhausting memory.  Counts the
+ * allocations of plans and batches, and the workspace of each repacked run.
+ * mach_debug_allocs_to_failure: n less the allocations since (0: failed, or disarmed). */
 void mach_debug_fail_alloc_after(int32_t n);
+int32_t mach_debug_allocs_to_failure(void);
 
 /* Test hooks (process-wide, not thread-safe; read when a plan is created):
  *  - force the kernel variant named `name` (mach_plan_info.variant) for later plans, or

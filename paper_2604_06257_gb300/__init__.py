@@ -29,7 +29,7 @@ ORDER = {"tcsf": 0, "ftcs": 1}
 
 EXPORTS = ("mach_das_plan", "mach_das_run", "mach_power_doppler", "mach_plan_destroy",
            "mach_status_string", "mach_plan_get_info", "mach_plan_tx_table", "mach_das_terms",
-           "mach_version", "mach_debug_fail_alloc_after", "mach_plan_device_status",
+           "mach_version", "mach_debug_fail_alloc_after", "mach_debug_allocs_to_failure", "mach_plan_device_status",
            "mach_debug_force_variant", "mach_debug_force_repack", "mach_debug_set_wait_limit", "mach_debug_stall_producer",
            "mach_das_run_noalloc", "mach_iq_convert", "mach_batch_plan", "mach_batch_bind",
            "mach_batch_run", "mach_batch_get_info", "mach_batch_destroy", "mach_das_run_per_tx",
@@ -113,6 +113,8 @@ def lib():
         L.mach_version.restype = C.c_char_p
         L.mach_debug_fail_alloc_after.argtypes = [i32]
         L.mach_debug_fail_alloc_after.restype = None
+        L.mach_debug_allocs_to_failure.argtypes = []
+        L.mach_debug_allocs_to_failure.restype = i32
         L.mach_plan_device_status.argtypes = [vp, vp]
         L.mach_plan_device_status.restype = C.c_int
         L.mach_debug_force_variant.argtypes = [C.c_char_p]
@@ -154,6 +156,10 @@ def mach_version() -> str:
 
 def mach_debug_fail_alloc_after(n: int) -> None:
     lib().mach_debug_fail_alloc_after(int(n))
+
+
+def mach_debug_allocs_to_failure() -> int:
+    return lib().mach_debug_allocs_to_failure()
 
 
 def mach_debug_force_variant(name) -> None:

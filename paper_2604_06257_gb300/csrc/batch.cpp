@@ -51,12 +51,19 @@ struct mach_batch_s {
 
 namespace {
 
+void drop_repacked(mach_batch_s* b) {
+  for (auto& m : b->multi) cudaFree(m->d_items);
+  cudaFree(b->ws);
+  b->multi.clear();
+  b->repacked.clear();
+  b->ws = nullptr;
+}
+
 void release(mach_batch_s* b) {
   if (!b) return;
   for (mach_plan p : b->plans) mach_plan_destroy(p);
   for (void* q : b->bounds) cudaFree(q);
-  for (auto& m : b->multi) cudaFree(m->d_items);
-  cudaFree(b->ws);
+  drop_repacked(b);
   cudaFree(b->d_insts);
   cudaFree(b->d_items);
   cudaFree(b->d_counter);
@@ -111,7 +118,8 @@ void staged_tile(int n, int nx, int ny, int nz, bool list, int tile[3]) {
 
 // The launches over the repacked instances' frame tiles: instances grouped by exact-frame
 // shape, each group's (frame tile, voxel tile) items longest first; the workspace for all of
-// them, which runs share in stream order as they do the work counter.
+// them, which runs share in stream order as they do the work counter.  OOM, UNSUPPORTED: the
+// instances can still take their lane mappings.
 mach_status plan_repacked(mach_batch_s* b, cudaStream_t s) {
   struct Item { int entry, ftile; int64_t tile; double cost; };
   struct Group { std::vector<Item> items; mach_batch_s::Multi* m = nullptr; };
@@ -153,10 +161,10 @@ mach_status plan_repacked(mach_batch_s* b, cudaStream_t s) {
     for (size_t k = 0; k < h.size(); ++k)
       h[k] = make_int2(g.items[k].entry | g.items[k].ftile << 16, static_cast<int>(g.items[k].tile));
     g.m->n_items = static_cast<int>(h.size());
-    if (cudaMalloc(&g.m->d_items, sizeof(int2) * h.size()) != cudaSuccess) {
-      cudaGetLastError();
-      return MACH_ERR_OOM;
-    }
+    int64_t bytes = 0;
+    if (const mach_status st = dev_alloc(reinterpret_cast<void**>(&g.m->d_items), sizeof(int2) * h.size(), &bytes);
+        st != MACH_OK)
+      return st;
     if (cudaMemcpyAsync(g.m->d_items, h.data(), sizeof(int2) * h.size(), cudaMemcpyHostToDevice, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
       return MACH_ERR_CUDA;
@@ -280,15 +288,16 @@ mach_status mach_batch_plan(const mach_das_desc* descs, int32_t n, const mach_ti
       // windows exceed the ring slot take the frame-lane path instead
       const int64_t tiles = static_cast<int64_t>(p.tiles_x) * p.tiles_y * p.tiles_z;
       void *tb = nullptr, *tr = nullptr, *st = nullptr;
-      if (cudaMalloc(&tb, sizeof(float4) * 2 * tiles) != cudaSuccess ||
-          cudaMalloc(&tr, sizeof(float2) * p.T * tiles) != cudaSuccess ||
-          cudaMalloc(&st, sizeof(BoundStats)) != cudaSuccess) {
-        cudaGetLastError();
+      int64_t bytes = 0;
+      mach_status ms = dev_alloc(&tb, sizeof(float4) * 2 * tiles, &bytes);
+      if (ms == MACH_OK) ms = dev_alloc(&tr, sizeof(float2) * p.T * tiles, &bytes);
+      if (ms == MACH_OK) ms = dev_alloc(&st, sizeof(BoundStats), &bytes);
+      if (ms != MACH_OK) {
         cudaFree(tb);
         cudaFree(tr);
         cudaFree(st);
         release(b);
-        return MACH_ERR_OOM;
+        return ms;
       }
       b->bounds.push_back(tb);
       b->bounds.push_back(tr);
@@ -333,18 +342,19 @@ mach_status mach_batch_plan(const mach_das_desc* descs, int32_t n, const mach_ti
     for (int64_t t = tiles - 1; t >= 0; --t) items.push_back({i, t, cost});
     b->points += static_cast<int64_t>(p.V) * p.C * p.T * p.F;
   }
+  int64_t bytes = 0;
   if (!b->repacked.empty()) {
-    if (cudaMalloc(&b->ws, ws_total) == cudaSuccess) {
-      if (const mach_status st = plan_repacked(b, s); st != MACH_OK) {
-        release(b);
-        return st;
-      }
+    mach_status st = dev_alloc(reinterpret_cast<void**>(&b->ws), ws_total, &bytes);
+    if (st == MACH_OK) st = plan_repacked(b, s);
+    if (st == MACH_ERR_CUDA) {
+      release(b);
+      return st;
+    }
+    if (st == MACH_OK) {
       items.erase(std::remove_if(items.begin(), items.end(), [&](const Item& t) { return is_repacked[t.inst]; }),
                   items.end());
-    } else {   // no memory for the workspace: every instance on its lane mapping
-      cudaGetLastError();
-      b->ws = nullptr;
-      b->repacked.clear();
+    } else {   // no memory for the workspace or its lists: every instance on its lane mapping
+      drop_repacked(b);
     }
   }
   if (items.size() > static_cast<size_t>(INT32_MAX)) {
@@ -355,12 +365,12 @@ mach_status mach_batch_plan(const mach_das_desc* descs, int32_t n, const mach_ti
   std::vector<int2> hitems(items.size());
   for (size_t k = 0; k < items.size(); ++k) hitems[k] = make_int2(items[k].inst, static_cast<int>(items[k].tile));
   b->n_items = static_cast<int>(items.size());
-  if (cudaMalloc(&b->d_insts, sizeof(BatchInstance) * n) != cudaSuccess ||
-      cudaMalloc(&b->d_items, sizeof(int2) * std::max<size_t>(1, hitems.size())) != cudaSuccess ||
-      cudaMalloc(&b->d_counter, 2 * sizeof(int)) != cudaSuccess) {
-    cudaGetLastError();
+  mach_status ms = dev_alloc(reinterpret_cast<void**>(&b->d_insts), sizeof(BatchInstance) * n, &bytes);
+  if (ms == MACH_OK) ms = dev_alloc(reinterpret_cast<void**>(&b->d_items), sizeof(int2) * hitems.size(), &bytes);
+  if (ms == MACH_OK) ms = dev_alloc(reinterpret_cast<void**>(&b->d_counter), 2 * sizeof(int), &bytes);
+  if (ms != MACH_OK) {
     release(b);
-    return MACH_ERR_OOM;
+    return ms;
   }
   for (auto& m : b->multi) m->args.insts = b->d_insts;
   if ((!hitems.empty() && cudaMemcpyAsync(b->d_items, hitems.data(), sizeof(int2) * hitems.size(),

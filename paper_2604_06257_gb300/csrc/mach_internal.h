@@ -273,6 +273,10 @@ size_t batch_smem_bytes(size_t slot_bytes);
 cudaError_t launch_batch(int iq_dtype, const BatchInstance* insts, const int2* items, int n_items, int* counter,
                          int grid, size_t slot_bytes, cudaStream_t s);
 const DasParams* plan_params(mach_plan p);
+// Device memory, counted in *total; OOM also when the allocation test hook says so
+// (alloc_denied, for memory that comes by other calls).
+mach_status dev_alloc(void** p, size_t bytes, int64_t* total);
+bool alloc_denied();
 // A plan for a batch: as mach_das_plan without a workspace pool.  plan_repack: the launches
 // over its repacked tiles (0 when it beamforms directly), and the workspace they need.
 mach_status make_batch_plan(const mach_das_desc* d, void* stream, mach_plan* out);

@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdint>
 #include <cstdio>
@@ -47,26 +48,12 @@ struct mach_plan_s {
 
 namespace {
 
-int g_fail_alloc_countdown = 0;   // test hook: > 0 -> the n-th allocation fails
+std::atomic<int> g_fail_alloc_countdown{0};   // test hook: > 0 -> the n-th allocation fails
 int g_force_variant = -1;         // test hook: variant index, or -1 for automatic choice
 bool g_force_repack = false;      // test hook: repack whenever the kernels can
 uint32_t g_wait_limit = 0;        // test hook: polls per bounded wait (0 = default)
 int g_stall = 0;                  // test hook: staged producer never issues its copies
 constexpr uint32_t kDefaultWaitLimit = 1u << 24;   // ~ seconds of polling
-
-mach_status dev_alloc(void** p, size_t bytes, int64_t* total) {
-  *p = nullptr;
-  if (g_fail_alloc_countdown > 0 && --g_fail_alloc_countdown == 0) return MACH_ERR_OOM;
-  if (bytes == 0) bytes = 16;
-  const cudaError_t e = cudaMalloc(p, bytes);
-  if (e == cudaErrorMemoryAllocation) {
-    cudaGetLastError();
-    return MACH_ERR_OOM;
-  }
-  if (e != cudaSuccess) return MACH_ERR_CUDA;
-  *total += static_cast<int64_t>(bytes);
-  return MACH_OK;
-}
 
 float float_of(int bits) {
   float f;
@@ -312,6 +299,8 @@ const char* mach_status_string(mach_status s) {
 const char* mach_version(void) { return "mach-gb300 0.1.0 sm_103a"; }
 
 void mach_debug_fail_alloc_after(int32_t n) { g_fail_alloc_countdown = n > 0 ? n : 0; }
+
+int32_t mach_debug_allocs_to_failure(void) { return g_fail_alloc_countdown.load(); }
 
 // Tile geometry of a variant: voxel box per block and the number of blocks.
 static mach_status configure_tiles(DasParams& b, Variant var, bool list, int64_t V, int F) {
@@ -582,7 +571,7 @@ static mach_status repack_plan(mach_plan_s* p, const DasParams& b, bool list, cu
   uint64_t keep = (p->ws_bytes >> 25 << 25) + (64u << 20);   // the pool maps memory in blocks
   if (cudaMemPoolSetAttribute(p->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) cudaGetLastError();
   void* first = nullptr;   // mapped now rather than in the first run
-  if (cudaMallocFromPoolAsync(&first, p->ws_bytes, p->pool, s) != cudaSuccess ||
+  if (alloc_denied() || cudaMallocFromPoolAsync(&first, p->ws_bytes, p->pool, s) != cudaSuccess ||
       cudaFreeAsync(first, s) != cudaSuccess) {
     cudaGetLastError();
     cudaMemPoolDestroy(p->pool);
@@ -855,7 +844,7 @@ static bool run_repacked(mach_plan p, const void* iq, float* pd, void* y, cudaSt
   }
   if (cap != cudaStreamCaptureStatusNone) return false;
   char* ws = nullptr;
-  if (cudaMallocFromPoolAsync(reinterpret_cast<void**>(&ws), p->ws_bytes, p->pool, s) != cudaSuccess) {
+  if (alloc_denied() || cudaMallocFromPoolAsync(reinterpret_cast<void**>(&ws), p->ws_bytes, p->pool, s) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
@@ -1018,6 +1007,24 @@ mach_status mach_das_terms(mach_plan p, const int64_t* vox_idx_dev, int64_t n, i
 }  // extern "C"
 
 namespace mach {
+bool alloc_denied() {
+  return g_fail_alloc_countdown.load() > 0 && g_fail_alloc_countdown.fetch_sub(1) == 1;
+}
+
+mach_status dev_alloc(void** p, size_t bytes, int64_t* total) {
+  *p = nullptr;
+  if (alloc_denied()) return MACH_ERR_OOM;
+  if (bytes == 0) bytes = 16;
+  const cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    return MACH_ERR_OOM;
+  }
+  if (e != cudaSuccess) return MACH_ERR_CUDA;
+  *total += static_cast<int64_t>(bytes);
+  return MACH_OK;
+}
+
 // Host steps shared with the allocation-free entry point (noalloc.cu): the same
 // validation, choice among the non-staged kernels, voxel tiling and phase constants
 // that a plan uses.
