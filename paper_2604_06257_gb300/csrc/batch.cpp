@@ -26,7 +26,7 @@ struct mach_batch_s {
   int grid = 0;
   int per_sm = 0;
   size_t slot_bytes = 128;               // ring slot of the staged path (largest staged window)
-  std::vector<void*> bounds;             // per staged instance: tile boxes and transmit-delay ranges
+  std::vector<void*> bounds;             // 2 per instance (null: not staged): tile boxes, transmit-delay ranges
   int64_t points = 0;
   bool bound = false;
   // repacked instances: what each needs before the shared launches, and the launches (one
@@ -226,8 +226,10 @@ mach_status mach_batch_plan(const mach_das_desc* descs, int32_t n, const mach_ti
   struct Item { int inst; int64_t tile; double cost; };
   std::vector<Item> items;
   std::vector<char> is_repacked(n, 0);
+  std::vector<size_t> slots(n, 0);         // ring slots that staged instances need
+  b->bounds.assign(2 * static_cast<size_t>(n), nullptr);
   for (int i = 0; i < n; ++i) {
-    mach_status st = make_batch_plan(&descs[i], stream, &b->plans[i]);
+    mach_status st = make_batch_plan(&descs[i], !shapes, stream, &b->plans[i]);
     if (st != MACH_OK) {
       release(b);
       return st;
@@ -299,9 +301,8 @@ mach_status mach_batch_plan(const mach_das_desc* descs, int32_t n, const mach_ti
         release(b);
         return ms;
       }
-      b->bounds.push_back(tb);
-      b->bounds.push_back(tr);
-      b->bounds.push_back(st);
+      b->bounds[2 * i] = tb;
+      b->bounds[2 * i + 1] = tr;
       p.tbox = static_cast<float4*>(tb);
       p.txr = static_cast<float2*>(tr);
       p.txr_stride = p.T;
@@ -309,14 +310,16 @@ mach_status mach_batch_plan(const mach_das_desc* descs, int32_t n, const mach_ti
       if (launch_tile_bounds(p, static_cast<float4*>(tb), static_cast<float2*>(tr), static_cast<BoundStats*>(st), s) != cudaSuccess ||
           cudaMemcpyAsync(&stats, st, sizeof(stats), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
           cudaStreamSynchronize(s) != cudaSuccess) {
+        cudaFree(st);
         release(b);
         return MACH_ERR_CUDA;
       }
+      cudaFree(st);
       p.rows_cap = std::max(2, stats.rows);
       const size_t sample = (dt == MACH_IQ_F16X2 || dt == MACH_IQ_BF16X2) ? 4 : 8;
       const size_t need = (static_cast<size_t>(p.rows_cap) * p.F * sample + 32 + 127) / 128 * 128;
       if (need <= kBatchSlotCap) {
-        b->slot_bytes = std::max(b->slot_bytes, need);
+        slots[i] = need;
       } else if (shapes) {
         release(b);
         return MACH_ERR_UNSUPPORTED;
@@ -353,10 +356,21 @@ mach_status mach_batch_plan(const mach_das_desc* descs, int32_t n, const mach_ti
     if (st == MACH_OK) {
       items.erase(std::remove_if(items.begin(), items.end(), [&](const Item& t) { return is_repacked[t.inst]; }),
                   items.end());
+      for (int i = 0; i < n; ++i) {   // what the lane mappings of repacked instances would have needed
+        if (!is_repacked[i]) continue;
+        slots[i] = 0;
+        b->host_insts[i].p.tbox = nullptr;
+        b->host_insts[i].p.txr = nullptr;
+        for (int k = 0; k < 2; ++k) {
+          cudaFree(b->bounds[2 * i + k]);
+          b->bounds[2 * i + k] = nullptr;
+        }
+      }
     } else {   // no memory for the workspace or its lists: every instance on its lane mapping
       drop_repacked(b);
     }
   }
+  for (const size_t q : slots) b->slot_bytes = std::max(b->slot_bytes, q);
   if (items.size() > static_cast<size_t>(INT32_MAX)) {
     release(b);
     return MACH_ERR_UNSUPPORTED;

@@ -277,9 +277,10 @@ const DasParams* plan_params(mach_plan p);
 // (alloc_denied, for memory that comes by other calls).
 mach_status dev_alloc(void** p, size_t bytes, int64_t* total);
 bool alloc_denied();
-// A plan for a batch: as mach_das_plan without a workspace pool.  plan_repack: the launches
+// A plan for a batch: as mach_das_plan without a workspace pool, or (repack false) without the
+// tables of a repacking plan altogether.  plan_repack: the launches
 // over its repacked tiles (0 when it beamforms directly), and the workspace they need.
-mach_status make_batch_plan(const mach_das_desc* d, void* stream, mach_plan* out);
+mach_status make_batch_plan(const mach_das_desc* d, bool repack, void* stream, mach_plan* out);
 int plan_repack(mach_plan p, const RepackPart** parts, size_t* ws_bytes, size_t* pd_at, int range[2]);
 int plan_iq_dtype(mach_plan p);
 void pick_tile_shape(int n, int nx, int ny, int nz, bool list, int tile[3]);

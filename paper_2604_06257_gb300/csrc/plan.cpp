@@ -469,8 +469,11 @@ static bool repack_pays(Variant direct, bool batch, double points, double share,
   }
 }
 
+// What a plan is for: runs of its own, a batch's repacked launches, a batch's lane mappings.
+enum PlanFor { kForRuns, kForBatch, kForLanes };
+
 static mach_status repack_plan(mach_plan_s* p, const DasParams& b, bool list, cudaStream_t s,
-                               size_t total_mem, bool own_pool) {
+                               size_t total_mem, PlanFor use) {
   const VariantShape& direct = variant_shape(p->variant);
   if (direct.exact_frames || direct.channel_lanes) return MACH_OK;
   const int64_t N = static_cast<int64_t>(b.T) * b.C * b.S;
@@ -547,12 +550,12 @@ static mach_status repack_plan(mach_plan_s* p, const DasParams& b, bool list, cu
   p->range[0] = lo;
   p->range[1] = hi;
   const double all = static_cast<double>(b.V) * b.C * b.T * fs.padded();
-  if (!g_force_repack && !repack_pays(p->variant, !own_pool, points, points / all,
+  if (!g_force_repack && !repack_pays(p->variant, use == kForBatch, points, points / all,
                                       static_cast<int64_t>(b.tiles_x) * b.tiles_y * b.tiles_z))
     return done(MACH_OK);
   p->pd_at = iq_bytes;
   p->ws_bytes = iq_bytes + pd_bytes;
-  if (!own_pool) {
+  if (use == kForBatch) {
     p->device_bytes += bytes;
     p->n_parts = n;
     return done(MACH_OK);
@@ -583,7 +586,7 @@ static mach_status repack_plan(mach_plan_s* p, const DasParams& b, bool list, cu
   return done(MACH_OK);
 }
 
-static mach_status make_plan(const mach_das_desc* d, void* stream, bool own_pool, mach_plan* out) {
+static mach_status make_plan(const mach_das_desc* d, void* stream, PlanFor use, mach_plan* out) {
   if (!out) return MACH_ERR_INVALID_ARG;
   *out = nullptr;
   mach_status st = validate(d);
@@ -811,7 +814,8 @@ static mach_status make_plan(const mach_das_desc* d, void* stream, bool own_pool
     if (!variant_shape(var).staged || !table_supported(var)) return fail(MACH_ERR_UNSUPPORTED);
     if ((st = build_term_table(p, b, s)) != MACH_OK) return fail(st);
   }
-  if (!forced && !d->term_table && (st = repack_plan(p, b, list, s, total_b, own_pool)) != MACH_OK) return fail(st);
+  if (use != kForLanes && !forced && !d->term_table && (st = repack_plan(p, b, list, s, total_b, use)) != MACH_OK)
+    return fail(st);
   if (cudaStreamSynchronize(s) != cudaSuccess) return fail(MACH_ERR_CUDA);
   cudaFree(d_raw);
   cudaFree(d_u);
@@ -825,7 +829,7 @@ static mach_status make_plan(const mach_das_desc* d, void* stream, bool own_pool
 }
 
 mach_status mach_das_plan(const mach_das_desc* d, void* stream, mach_plan* out) {
-  return make_plan(d, stream, true, out);
+  return make_plan(d, stream, kForRuns, out);
 }
 
 mach_status mach_plan_destroy(mach_plan p) {
@@ -1028,8 +1032,8 @@ mach_status dev_alloc(void** p, size_t bytes, int64_t* total) {
 // Host steps shared with the allocation-free entry point (noalloc.cu): the same
 // validation, choice among the non-staged kernels, voxel tiling and phase constants
 // that a plan uses.
-mach_status make_batch_plan(const mach_das_desc* d, void* stream, mach_plan* out) {
-  return make_plan(d, stream, false, out);
+mach_status make_batch_plan(const mach_das_desc* d, bool repack, void* stream, mach_plan* out) {
+  return make_plan(d, stream, repack ? kForBatch : kForLanes, out);
 }
 int plan_repack(mach_plan p, const RepackPart** parts, size_t* ws_bytes, size_t* pd_at, int range[2]) {
   range[0] = p->range[0];

@@ -254,3 +254,28 @@ def test_staged_items_whose_copies_stall_end_the_launch():
         torch.cuda.synchronize()
     y_ref, _ = oracle.das(acqs[0], iqs[0].cpu(), np.arange(0, acqs[0].n_vox, 11))
     assert nrmse_db(ys[0].cpu().numpy()[::11], y_ref) <= -100
+
+
+def test_explicit_shapes_need_no_repacking_tables():
+    """Device allocations of a batch that names its lane mappings: none for frame tiles."""
+    base = synth.make_acquisition("doppler2d", "small")
+    acqs = [base.replace(grid_dims=(67, 1, 61), n_samples=200, n_frames=F) for F in (20, 25)]
+    kws = [m.plan_kwargs(a) for a in acqs]
+
+    def allocations(shapes):
+        m.mach_debug_fail_alloc_after(1000)
+        try:
+            with m.Batch(kws, shapes=shapes) as b:
+                return 1000 - m.mach_debug_allocs_to_failure(), b.info()
+        finally:
+            m.mach_debug_fail_alloc_after(0)
+
+    m.mach_debug_force_repack(True)
+    try:
+        n_default, info = allocations(None)
+        n_lanes, _ = allocations([(s[0], s[1], None) for s in info["shapes"]])
+    finally:
+        m.mach_debug_force_repack(False)
+    # the workspace, one item list (both run in 32-frame tiles) and per instance its statistics,
+    # tile boxes and transmit ranges
+    assert n_default - n_lanes == 2 + 3 * len(acqs)
