@@ -79,12 +79,10 @@ __global__ void __launch_bounds__((kWgMma + 1) * 32, 1)
   if (warp == kWgMma) {   // ------------------------------------------------- copies
     if (lane == 0 && !p.debug_stall) {
       int k = 0;
-      bool ok = true;
       for (int64_t tile = t0; tile < t1; ++tile, ++k) {
         const int st = k % kWgStages;
         if (k >= kWgStages && !wait_spin(&empty[st], ((k / kWgStages) - 1) & 1, p.wait_limit)) {
           atomicOr(&g_conv_tc_err, 1);
-          ok = false;
           break;
         }
         const int tx = static_cast<int>(tile % p.tiles_x);
@@ -101,9 +99,7 @@ __global__ void __launch_bounds__((kWgMma + 1) * 32, 1)
                       &full[st]);
         }
       }
-      if (!ok)   // the copies in flight land before the block leaves
-        for (int j = k - kWgStages; j < k; ++j)
-          if (j >= 0) mbar_wait_bounded(&full[j % kWgStages], (j / kWgStages) & 1, p.wait_limit);
+      await_copies(full, kWgStages, k);
     }
     return;
   }

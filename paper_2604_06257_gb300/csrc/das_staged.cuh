@@ -133,14 +133,17 @@ __device__ __forceinline__ bool produce_windows(const DasParams& p, const unsign
 }
 
 // Lane 0 of the producer after its last pair: one end-of-sequence marker per pair a
-// consumer round can hold; or, when abandoning after a timeout, a bounded wait for the
-// copies already issued, so that none lands after the block has exited.
+// consumer round can hold, unless a wait gave up.  Then it waits for the copies that no marker
+// has followed in their slots (the others are consumed): should the consumers give up,
+// none lands after the block has exited.  Issued copies do land, however short the limit that a
+// test gives the other waits.
 template <int NBUF, int PB>
 __device__ __forceinline__ void finish_producer(const DasParams& p, bool ok, int r, SlotMeta* meta, uint64_t* full,
                                                 uint64_t* empty) {
+  int marks = 0;
   if (ok) {
-    for (int k = 0; k < PB; ++k) {
-      const int rr = r + k, slot = rr % NBUF;
+    for (; marks < PB; ++marks) {
+      const int rr = r + marks, slot = rr % NBUF;
       if (rr >= NBUF && !mbar_wait_bounded(&empty[slot], ((rr / NBUF) - 1) & 1, p.wait_limit)) {
         atomicOr(p.err, 1);
         break;
@@ -148,9 +151,10 @@ __device__ __forceinline__ void finish_producer(const DasParams& p, bool ok, int
       meta[slot].c = -1;
       mbar_arrive(&full[slot]);
     }
-  } else {
-    for (int k = max(0, r - NBUF); k < r; ++k) mbar_wait_bounded(&full[k % NBUF], (k / NBUF) & 1, p.wait_limit);
   }
+  if (p.debug_stall) return;   // none was issued
+  for (int k = max(0, r + marks - NBUF); k < r; ++k)
+    mbar_wait_bounded(&full[k % NBUF], (k / NBUF) & 1, kDefaultWaitLimit);
 }
 
 // MAXR: register cap per thread, chosen so that the intended number of blocks fits per SM.

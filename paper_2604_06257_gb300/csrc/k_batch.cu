@@ -471,9 +471,9 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 2)
       if (__syncthreads_or(!ok)) {
         // A wait gave up, and the warps no longer agree on the ring: this block takes no more
         // items.  The copies whose slots no marker took over land before it leaves.
-        if (warp == kBatchConsumers && lane == 0)
+        if (warp == kBatchConsumers && lane == 0 && !p.debug_stall)
           for (int k = max(ring_at, used - kBatchRing); k < copied; ++k)
-            mbar_wait_bounded(&full[ring_slot(k)], ring_full(k), p.wait_limit);
+            mbar_wait_bounded(&full[ring_slot(k)], ring_full(k), kDefaultWaitLimit);
         break;
       }
       ring_at = __shfl_sync(0xffffffffu, used, 0) % kRingWrap;

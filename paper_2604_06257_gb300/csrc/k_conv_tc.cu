@@ -113,6 +113,14 @@ __device__ __forceinline__ bool wait_warp(uint64_t* bar, uint32_t parity, uint32
   return __all_sync(0xffffffffu, wait_spin(bar, parity, limit));
 }
 
+// The last copies into a ring of `stages` slots, of `issued` in all: a block whose other warps gave
+// up must not leave before they have landed.  (They do, however short the limit that a test
+// gives the other waits.)
+__device__ __forceinline__ void await_copies(uint64_t* full, uint32_t stages, uint32_t issued) {
+  for (uint32_t k = issued > stages ? issued - stages : 0u; k < issued; ++k)
+    mbar_wait_bounded(&full[k % stages], (k / stages) & 1u, kDefaultWait);
+}
+
 __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, int c3,
                                             int c4, uint64_t* bar) {
   asm volatile(
@@ -298,6 +306,8 @@ __global__ void __launch_bounds__(kThreads, 3) k_conv3d_tc(const __grid_constant
           }
         }
       }
+      await_copies(fullA, 2, a_use);
+      await_copies(fullB, kNB, p.resident ? 1u : b_use);
     }
   } else if (warp == 1) {   // -------------------------------------------- MMAs
     const uint32_t lead = elect_one();
@@ -439,7 +449,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_conv3d_tc(const __grid_constant
 
   __syncthreads();
   if (warp == 0) {
-    if (!mbar_wait_bounded(fin, 0, limit)) atomicOr(&g_conv_tc_err, 2);
+    if (!mbar_wait_bounded(fin, 0, kDefaultWait)) atomicOr(&g_conv_tc_err, 2);   // no MMA in flight writes freed columns
     __syncwarp();
     fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(p.tmem_cols) : "memory");
@@ -554,6 +564,7 @@ __global__ void __launch_bounds__(kFoldThreads, TZ * CO >= 48 ? 1 : 2) k_conv3d_
           ++a_use;
         }
       }
+      await_copies(fullA, S, a_use);
     }
   } else if (warp == 1) {   // -------------------------------------------- MMAs
     const uint32_t lead = elect_one();
@@ -713,7 +724,7 @@ __global__ void __launch_bounds__(kFoldThreads, TZ * CO >= 48 ? 1 : 2) k_conv3d_
 
   __syncthreads();
   if (warp == 0) {
-    if (!mbar_wait_bounded(fin, 0, limit)) atomicOr(&g_conv_tc_err, 2);
+    if (!mbar_wait_bounded(fin, 0, kDefaultWait)) atomicOr(&g_conv_tc_err, 2);   // no MMA in flight writes freed columns
     __syncwarp();
     fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(p.tmem_cols) : "memory");

@@ -82,6 +82,8 @@ enum Variant : int32_t {
   V_COUNT
 };
 
+constexpr uint32_t kDefaultWaitLimit = 1u << 24;   // polls of a bounded device wait: seconds
+
 struct VariantShape {
   const char* name;
   int frames_per_lane;   // frames one thread accumulates

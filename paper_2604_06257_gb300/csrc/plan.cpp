@@ -53,7 +53,6 @@ int g_force_variant = -1;         // test hook: variant index, or -1 for automat
 bool g_force_repack = false;      // test hook: repack whenever the kernels can
 uint32_t g_wait_limit = 0;        // test hook: polls per bounded wait (0 = default)
 int g_stall = 0;                  // test hook: staged producer never issues its copies
-constexpr uint32_t kDefaultWaitLimit = 1u << 24;   // ~ seconds of polling
 
 float float_of(int bits) {
   float f;
