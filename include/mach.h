@@ -34,9 +34,11 @@
  *    (dense grids of at least 6 or 16 voxels per sample and enough work; mach_plan_info.variant
  *    then names the tiles, e.g. "+x32+x8").  Each
  *    run takes its workspace, 8 bytes per sample and padded frame, in stream order from a
- *    memory pool that the plan owns (at most a sixteenth of the device memory per run; one
- *    workspace is kept between runs and released with the plan).  Runs on a capturing
- *    stream, or without memory for the workspace, allocate nothing and beamform directly.
+ *    memory pool that the plans of a device share (at most a sixteenth of the device memory
+ *    per run; the largest plan's workspace is kept between runs, counted in the device_bytes of
+ *    every plan, and released with the last one).  Runs on a capturing stream, or without
+ *    memory for the workspace, allocate nothing and beamform directly: the same frames up
+ *    to the order of float32 sums (about 1e-7 of their size), not bit for bit.
  *  - Threads: a plan is read-only after creation.  Calls that share a plan may run on
  *    different streams concurrently, except when mach_plan_info.frame_tiles > 1 and
  *    Power Doppler is requested (those calls share the plan's partial-sum scratch and

@@ -8,7 +8,10 @@
 #include <cstdint>
 #include <cstdio>
 #include <cstring>
+#include <map>
+#include <mutex>
 #include <new>
+#include <set>
 #include <vector>
 
 #include "mach.h"
@@ -37,7 +40,7 @@ struct mach_plan_s {
   float4* d_term_rec = nullptr;
   int64_t table_bytes = 0;
   // repacked route (see repack_plan): the exact-frame launches over repacked frame tiles, and
-  // the pool that each run takes its workspace from
+  // the device's pool that each run takes its workspace from
   RepackPart parts[2];
   int n_parts = 0;
   size_t ws_bytes = 0;          // workspace of one run: repacked IQ, partial Power Doppler sums
@@ -47,6 +50,57 @@ struct mach_plan_s {
 };
 
 namespace {
+
+// The pools that repacked runs take their workspaces from, one per device for all plans: stream
+// order keeps concurrent runs' blocks apart, and what lies idle between runs is one
+// workspace, of the largest plan there is, however many plans there are.  The last plan of a
+// device gives its pool back.
+struct DevicePool {
+  cudaMemPool_t pool = nullptr;
+  std::multiset<size_t> plans;   // workspace bytes of each plan
+};
+std::mutex g_pools_lock;
+std::map<int, DevicePool>& pools() {
+  static auto* p = new std::map<int, DevicePool>;   // never destroyed: plans may outlive statics
+  return *p;
+}
+
+void keep_largest(DevicePool& d) {
+  uint64_t keep = (*d.plans.rbegin() >> 25 << 25) + (64u << 20);   // the pool maps memory in blocks
+  if (cudaMemPoolSetAttribute(d.pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) cudaGetLastError();
+}
+
+cudaMemPool_t take_pool(int device, size_t bytes) {
+  std::lock_guard<std::mutex> hold(g_pools_lock);
+  DevicePool& d = pools()[device];
+  if (!d.pool) {
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = device;
+    if (cudaMemPoolCreate(&d.pool, &props) != cudaSuccess) {
+      cudaGetLastError();
+      d.pool = nullptr;
+      return nullptr;
+    }
+  }
+  d.plans.insert(bytes);
+  keep_largest(d);
+  return d.pool;
+}
+
+void return_pool(int device, size_t bytes) {
+  std::lock_guard<std::mutex> hold(g_pools_lock);
+  DevicePool& d = pools()[device];
+  d.plans.erase(d.plans.find(bytes));
+  if (d.plans.empty()) {
+    cudaMemPoolDestroy(d.pool);
+    d.pool = nullptr;
+    return;
+  }
+  keep_largest(d);
+  if (*d.plans.rbegin() < bytes && cudaMemPoolTrimTo(d.pool, *d.plans.rbegin()) != cudaSuccess) cudaGetLastError();
+}
 
 std::atomic<int> g_fail_alloc_countdown{0};   // test hook: > 0 -> the n-th allocation fails
 int g_force_variant = -1;         // test hook: variant index, or -1 for automatic choice
@@ -275,7 +329,7 @@ void release(mach_plan_s* p) {
     cudaFree(q.d_tbox);
     cudaFree(q.d_txr);
   }
-  if (p->pool) cudaMemPoolDestroy(p->pool);
+  if (p->pool) return_pool(p->device, p->ws_bytes);
   delete p;
 }
 
@@ -559,28 +613,18 @@ static mach_status repack_plan(mach_plan_s* p, const DasParams& b, bool list, cu
     p->n_parts = n;
     return done(MACH_OK);
   }
-  // a pool of the plan's own: each run takes its workspace in stream order, so that calls on
-  // several streams never share one; one workspace is kept between runs, the others go back
-  cudaMemPoolProps props{};
-  props.allocType = cudaMemAllocationTypePinned;
-  props.location.type = cudaMemLocationTypeDevice;
-  props.location.id = p->device;
-  if (cudaMemPoolCreate(&p->pool, &props) != cudaSuccess) {
-    cudaGetLastError();
-    p->pool = nullptr;
-    return done(MACH_OK);
-  }
-  uint64_t keep = (p->ws_bytes >> 25 << 25) + (64u << 20);   // the pool maps memory in blocks
-  if (cudaMemPoolSetAttribute(p->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) cudaGetLastError();
+  // each run takes its workspace in stream order, so that calls on several streams never share one
+  p->pool = take_pool(p->device, p->ws_bytes);
+  if (!p->pool) return done(MACH_OK);
   void* first = nullptr;   // mapped now rather than in the first run
   if (alloc_denied() || cudaMallocFromPoolAsync(&first, p->ws_bytes, p->pool, s) != cudaSuccess ||
       cudaFreeAsync(first, s) != cudaSuccess) {
     cudaGetLastError();
-    cudaMemPoolDestroy(p->pool);
+    return_pool(p->device, p->ws_bytes);
     p->pool = nullptr;
     return done(MACH_OK);
   }
-  p->device_bytes += bytes + static_cast<int64_t>(p->ws_bytes);   // the pool keeps one workspace
+  p->device_bytes += bytes + static_cast<int64_t>(p->ws_bytes);   // kept by the pool, once for all plans
   p->n_parts = n;
   return done(MACH_OK);
 }

@@ -123,3 +123,46 @@ def test_batches_do_without_the_workspace():
     assert without >= 4 and partly >= 3, (without, partly)
     torch.cuda.synchronize()
     assert abs(torch.cuda.mem_get_info()[0] - free0) < (64 << 20)
+
+
+def run_concurrently(plans, acqs):
+    """Runs of two plans at once have a workspace each, also while a third plan goes."""
+    xs = [stored(a, i)[0] for i, a in enumerate(acqs[:2])]
+    want = [p.run(x).clone() for p, x in zip(plans[::2], xs)]
+    got = [torch.zeros_like(w) for w in want]
+    streams = [torch.cuda.Stream() for _ in xs]
+    torch.cuda.synchronize()
+    for _ in range(3):
+        for p, x, y, s in zip(plans[::2], xs, got, streams):
+            m.mach_das_run(p.handle, x, y, stream=s)
+    plans.pop().close()
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for a, b in zip(got, want))
+
+
+def test_idle_plans_share_one_workspace():
+    """Device memory that plans hold between runs: one workspace for all of them, none after the last."""
+    acqs = [dense(F, "c64split", 2, 3) for F in (2048, 2028, 2016)]
+    ws = 3 * 24 * 200 * 8 * 2048
+
+    def held():
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        return free0 - torch.cuda.mem_get_info()[0]
+
+    free0 = 0
+    warm = [m.Plan(**m.plan_kwargs(a)) for a in acqs for _ in range(2)]   # modules load, torch's own blocks come
+    run_concurrently(warm, acqs)
+    for p in warm:
+        p.close()
+    free0 = -held()
+    plans = [m.Plan(**m.plan_kwargs(a)) for a in acqs for _ in range(2)]
+    try:
+        assert all("+x" in p.info()["variant"] and p.info()["device_bytes"] > 0.95 * ws for p in plans)
+        assert held() < 2 * ws
+        run_concurrently(plans, acqs)
+        assert held() < 2 * ws
+    finally:
+        for p in plans:
+            p.close()
+    assert held() < (64 << 20)
