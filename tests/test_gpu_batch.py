@@ -1,4 +1,4 @@
-"""Ragged batches: many instances in one persistent launch, against the FP64 oracle and
+"""Ragged batches: many instances in one batch run, against the FP64 oracle and
 against single-instance plans; graph capture; the autotuner's choices."""
 import time
 

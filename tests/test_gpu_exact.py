@@ -336,3 +336,29 @@ def test_few_frames(F, T, expect):
         assert nrmse_db(y.cpu().numpy(), y_l.cpu().numpy()) < -120
     assert nrmse_db(pd.cpu().numpy().astype(np.float64), pd_l.cpu().numpy().astype(np.float64)) < -120
     print(F, T, info["tile"], info["frame_tiles"], check_oracle(acq, iq, y, pd))
+
+
+@pytest.mark.parametrize("name,F", [("staged_c64p_x16_f8v1w7", 16), ("staged_c64p_x16_f8v1w4", 16), ("staged_c64p_x8_f8v1w4", 8),
+                                    ("staged_c64p_x16_f4v1w7", 16)])
+@pytest.mark.parametrize("T", [1, 3])
+def test_short_ensemble_shapes(name, F, T):
+    """The shapes that repacked tails run in, forced on native split rows, 2D and 3D: the frames of the
+    default kernel of that frame count bit for bit, and within the oracle bars."""
+    acq2, iq2 = small_2d(F, T)
+    acq3 = synth.make_acquisition("ulm3d", "small").replace(n_frames=F)
+    for acq, iq in ((acq2, iq2), (acq3, synth.random_iq(acq3, 60 + F))):
+        a = acq.replace(iq_dtype="c64split")
+        kw = m.plan_kwargs(a)
+        x = synth.iqmod.to_c64split(iq.cuda())
+        with forced(kw, name) as p:
+            assert p.info()["variant"] == name
+            pd, y = p.power_doppler(x, want_y=True)
+            torch.cuda.synchronize()
+            assert p.device_status() == m.MACH_OK
+        with m.Plan(**kw) as p:
+            assert p.info()["variant"] != name
+            pd_d, y_d = p.power_doppler(x, want_y=True)
+            torch.cuda.synchronize()
+        assert torch.equal(y, y_d)
+        assert nrmse_db(pd.cpu().numpy().astype(np.float64), pd_d.cpu().numpy().astype(np.float64)) < -120
+        check_oracle(acq, iq, y, pd)

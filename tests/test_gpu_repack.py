@@ -149,3 +149,67 @@ def test_nan_and_inf_samples_reach_only_kept_terms(F, direct):
     ok = torch.isfinite(torch.view_as_real(ref)).all(-1)
     assert bool(ok.any()) and not bool(ok.all())
     assert torch.equal(torch.isfinite(torch.view_as_real(y)).all(-1), ok)
+
+
+def batch_and_plans(acqs, xs):
+    """(batch frames, single plans' frames, those with the kernels that read the ensembles directly);
+    checks that the batch has other items than its lane mappings would."""
+    ys = [torch.zeros((a.n_vox, a.n_frames), dtype=torch.complex64, device="cuda") for a in acqs]
+    with m.Batch([m.plan_kwargs(a) for a in acqs]) as b:
+        b.bind(xs, ys, None)
+        b.run()
+        torch.cuda.synchronize()
+        info = b.info()
+    with m.Batch([m.plan_kwargs(a) for a in acqs], shapes=[(s[0], s[1], None) for s in info["shapes"]]) as b:
+        assert b.info()["items"] != info["items"]
+    plans, direct = [], []
+    for a, x in zip(acqs, xs):
+        with m.Plan(**m.plan_kwargs(a)) as p:
+            name = p.info()["variant"]
+            plans.append(p.run(x))
+        m.mach_debug_force_variant(name.split("+")[0])
+        try:
+            with m.Plan(**m.plan_kwargs(a)) as p:
+                direct.append(p.run(x))
+        finally:
+            m.mach_debug_force_variant(None)
+        assert ("+x" in name) == (a.n_frames > 4)
+    torch.cuda.synchronize()
+    return ys, plans, direct
+
+
+def test_batch_instances_are_repacked():
+    """Bit for bit the frames of a repacking plan, which differ from those of the direct kernels where
+    several transmits are summed in another order; the 73 instances with a 32-frame tile
+    exceed one launch's entries."""
+    frames = [25, 32, 27, 31] * 18 + [41, 5, 16, 2, 13]
+    acqs = [dense(F, "c64", 2 + (i // 4) % 2, 1 + i % 2) for i, F in enumerate(frames)]
+    xs = [stored(a, i)[0] for i, a in enumerate(acqs)]
+    ys, plans, direct = batch_and_plans(acqs, xs)
+    for a, y, p, d in zip(acqs, ys, plans, direct):
+        assert torch.equal(y, p)
+        assert nrmse_db(y.cpu().numpy(), d.cpu().numpy()) <= -110
+    assert sum(not torch.equal(y, d) for y, d in zip(ys, direct)) >= 10
+
+
+def test_batch_repacks_up_to_its_budget():
+    """Two instances (of the same IQ) whose workspaces together exceed a sixteenth of the device's
+    memory: the first is repacked, the second beamformed by a lane mapping."""
+    total = torch.cuda.mem_get_info()[1]
+    acq = dense(64, "c64", 3, 2)
+    C = int(0.6 * total / 16 / (2 * acq.n_samples * 64 * 8))      # elements that fill 0.6 of it
+    e = np.zeros((C, 3), np.float32)
+    e[:, 0], e[:, 1] = np.linspace(-4e-3, 4e-3, C), np.linspace(-1e-3, 1e-3, C)
+    acq = acq.replace(elem_pos=e)
+    x = torch.view_as_complex(torch.randn((2, C, acq.n_samples, 64, 2), device="cuda"))
+    ys = [torch.zeros((acq.n_vox, 64), dtype=torch.complex64, device="cuda") for _ in range(2)]
+    with m.Batch([m.plan_kwargs(acq)] * 2) as b:
+        b.bind([x, x], ys, None)
+        b.run()
+        torch.cuda.synchronize()
+    with m.Plan(**m.plan_kwargs(acq)) as p:
+        assert "+x32" in p.info()["variant"]
+        y = p.run(x)
+        torch.cuda.synchronize()
+    assert torch.equal(ys[0], y) and not torch.equal(ys[1], y)
+    assert nrmse_db(ys[1].cpu().numpy(), y.cpu().numpy()) <= -100

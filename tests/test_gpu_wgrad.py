@@ -33,7 +33,8 @@ def test_weight_gradient_tile_edges(shape, ci, co):
     nn.mach_nn_conv3d_wgrad(x, g, dw)
     torch.cuda.synchronize()
     ref, mag = reference(x, g)
-    # float32 sums of M products: one rounding a term, and the added 0.5
+    # one rounding of 2^-24 a term at most, and the added 0.5; a chain of roundings is a quarter of a
+    # block's voxels and then the blocks' atomics, for the large shape far below 65536
     M = int(np.prod(shape))
     bound = (min(M, 65536) + 64) * 2.0 ** -24 * mag + 2.0 ** -24
     assert bool(((dw.double() - 0.5 - ref).abs() <= bound).all())
