@@ -6,6 +6,7 @@
 #include <cstring>
 #include <memory>
 #include <new>
+#include <stdexcept>
 #include <vector>
 
 #include "mach.h"
@@ -176,42 +177,10 @@ mach_status plan_repacked(mach_batch_s* b, cudaStream_t s) {
 
 extern "C" {
 
-mach_status mach_batch_plan(const mach_das_desc* descs, int32_t n, const mach_tile_shape* shapes, void* stream,
-                            mach_batch* out) {
-  if (!out) return MACH_ERR_INVALID_ARG;
-  *out = nullptr;
-  if (!descs || n < 1) return MACH_ERR_INVALID_ARG;
+// Everything of a batch into b, which the caller releases if this fails.
+static mach_status plan_batch(const mach_das_desc* descs, int32_t n, const mach_tile_shape* shapes, cudaStream_t s,
+                              mach_batch_s* b) {
   const int dt = descs[0].iq_dtype;
-  for (int i = 0; i < n; ++i) {
-    mach_status st = host_validate(&descs[i]);
-    if (st != MACH_OK) return st;
-    if (descs[i].term_table) return MACH_ERR_UNSUPPORTED;
-    if (descs[i].iq_dtype != dt) return MACH_ERR_INVALID_ARG;
-    if (descs[i].n_frames > 64) return MACH_ERR_UNSUPPORTED;
-    if (shapes) {
-      const mach_tile_shape& s = shapes[i];
-      if (s.mode == kBatchChannels) {
-        if (descs[i].n_frames > 4) return MACH_ERR_INVALID_ARG;
-      } else if (s.mode == kBatchStaged) {
-        if (s.frame_lanes != 8 && s.frame_lanes != 16) return MACH_ERR_INVALID_ARG;
-        if (4 * s.frame_lanes < descs[i].n_frames) return MACH_ERR_INVALID_ARG;
-      } else if (s.mode == kBatchFrames) {
-        if (s.frame_lanes != 2 && s.frame_lanes != 4 && s.frame_lanes != 8 && s.frame_lanes != 16)
-          return MACH_ERR_INVALID_ARG;
-        if (4 * s.frame_lanes < descs[i].n_frames) return MACH_ERR_INVALID_ARG;
-      } else {
-        return MACH_ERR_INVALID_ARG;
-      }
-      const bool zero = s.tile[0] == 0 && s.tile[1] == 0 && s.tile[2] == 0;
-      if (!zero && (s.tile[0] < 1 || s.tile[1] < 1 || s.tile[2] < 1 ||
-                    s.tile[0] * s.tile[1] * s.tile[2] != voxels_per_block(s)))
-        return MACH_ERR_INVALID_ARG;
-    }
-  }
-  if (dt == MACH_IQ_C64_SPLIT) return MACH_ERR_UNSUPPORTED;
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  mach_batch_s* b = new (std::nothrow) mach_batch_s();
-  if (!b) return MACH_ERR_OOM;
   b->n = n;
   b->iq_dtype = dt;
   b->plans.assign(n, nullptr);
@@ -220,7 +189,6 @@ mach_status mach_batch_plan(const mach_das_desc* descs, int32_t n, const mach_ti
   size_t free_mem = 0, total_mem = 0, ws_total = 0;
   if (cudaMemGetInfo(&free_mem, &total_mem) != cudaSuccess) {
     cudaGetLastError();
-    release(b);
     return MACH_ERR_CUDA;
   }
   struct Item { int inst; int64_t tile; double cost; };
@@ -229,11 +197,8 @@ mach_status mach_batch_plan(const mach_das_desc* descs, int32_t n, const mach_ti
   std::vector<size_t> slots(n, 0);         // ring slots that staged instances need
   b->bounds.assign(2 * static_cast<size_t>(n), nullptr);
   for (int i = 0; i < n; ++i) {
-    mach_status st = make_batch_plan(&descs[i], !shapes, stream, &b->plans[i]);
-    if (st != MACH_OK) {
-      release(b);
-      return st;
-    }
+    mach_status st = make_batch_plan(&descs[i], !shapes, s, &b->plans[i]);
+    if (st != MACH_OK) return st;
     // default shapes only: an instance that its plan would repack joins the launches over
     // repacked tiles
     const RepackPart* parts = nullptr;
@@ -269,15 +234,9 @@ mach_status mach_batch_plan(const mach_das_desc* descs, int32_t n, const mach_ti
       return true;
     };
     if (!set_tiles(sh)) {
-      if (sh.mode != kBatchStaged || shapes) {
-        release(b);
-        return MACH_ERR_UNSUPPORTED;
-      }
+      if (sh.mode != kBatchStaged || shapes) return MACH_ERR_UNSUPPORTED;
       sh = frames_shape(descs[i].n_frames);
-      if (!set_tiles(sh)) {
-        release(b);
-        return MACH_ERR_UNSUPPORTED;
-      }
+      if (!set_tiles(sh)) return MACH_ERR_UNSUPPORTED;
     }
     p.frame_tiles = 1;
     p.wb_x = p.wb_y = p.wb_z = 0;
@@ -298,7 +257,6 @@ mach_status mach_batch_plan(const mach_das_desc* descs, int32_t n, const mach_ti
         cudaFree(tb);
         cudaFree(tr);
         cudaFree(st);
-        release(b);
         return ms;
       }
       b->bounds[2 * i] = tb;
@@ -311,7 +269,6 @@ mach_status mach_batch_plan(const mach_das_desc* descs, int32_t n, const mach_ti
           cudaMemcpyAsync(&stats, st, sizeof(stats), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
           cudaStreamSynchronize(s) != cudaSuccess) {
         cudaFree(st);
-        release(b);
         return MACH_ERR_CUDA;
       }
       cudaFree(st);
@@ -321,15 +278,11 @@ mach_status mach_batch_plan(const mach_das_desc* descs, int32_t n, const mach_ti
       if (need <= kBatchSlotCap) {
         slots[i] = need;
       } else if (shapes) {
-        release(b);
         return MACH_ERR_UNSUPPORTED;
       } else {
         sh = frames_shape(descs[i].n_frames);
         sh.tile[0] = sh.tile[1] = sh.tile[2] = 0;
-        if (!set_tiles(sh)) {
-          release(b);
-          return MACH_ERR_UNSUPPORTED;
-        }
+        if (!set_tiles(sh)) return MACH_ERR_UNSUPPORTED;
       }
     }
     b->host_insts[i].p = p;
@@ -349,10 +302,7 @@ mach_status mach_batch_plan(const mach_das_desc* descs, int32_t n, const mach_ti
   if (!b->repacked.empty()) {
     mach_status st = dev_alloc(reinterpret_cast<void**>(&b->ws), ws_total, &bytes);
     if (st == MACH_OK) st = plan_repacked(b, s);
-    if (st == MACH_ERR_CUDA) {
-      release(b);
-      return st;
-    }
+    if (st == MACH_ERR_CUDA) return st;
     if (st == MACH_OK) {
       items.erase(std::remove_if(items.begin(), items.end(), [&](const Item& t) { return is_repacked[t.inst]; }),
                   items.end());
@@ -371,10 +321,7 @@ mach_status mach_batch_plan(const mach_das_desc* descs, int32_t n, const mach_ti
     }
   }
   for (const size_t q : slots) b->slot_bytes = std::max(b->slot_bytes, q);
-  if (items.size() > static_cast<size_t>(INT32_MAX)) {
-    release(b);
-    return MACH_ERR_UNSUPPORTED;
-  }
+  if (items.size() > static_cast<size_t>(INT32_MAX)) return MACH_ERR_UNSUPPORTED;
   std::stable_sort(items.begin(), items.end(), [](const Item& a, const Item& c) { return a.cost > c.cost; });
   std::vector<int2> hitems(items.size());
   for (size_t k = 0; k < items.size(); ++k) hitems[k] = make_int2(items[k].inst, static_cast<int>(items[k].tile));
@@ -382,25 +329,70 @@ mach_status mach_batch_plan(const mach_das_desc* descs, int32_t n, const mach_ti
   mach_status ms = dev_alloc(reinterpret_cast<void**>(&b->d_insts), sizeof(BatchInstance) * n, &bytes);
   if (ms == MACH_OK) ms = dev_alloc(reinterpret_cast<void**>(&b->d_items), sizeof(int2) * hitems.size(), &bytes);
   if (ms == MACH_OK) ms = dev_alloc(reinterpret_cast<void**>(&b->d_counter), 2 * sizeof(int), &bytes);
-  if (ms != MACH_OK) {
-    release(b);
-    return ms;
-  }
+  if (ms != MACH_OK) return ms;
   for (auto& m : b->multi) m->args.insts = b->d_insts;
   if ((!hitems.empty() && cudaMemcpyAsync(b->d_items, hitems.data(), sizeof(int2) * hitems.size(),
                                           cudaMemcpyHostToDevice, s) != cudaSuccess) ||
       cudaMemsetAsync(b->d_counter, 0, 2 * sizeof(int), s) != cudaSuccess ||
       cudaMemcpyAsync(b->d_insts, b->host_insts.data(), sizeof(BatchInstance) * n, cudaMemcpyHostToDevice, s) !=
           cudaSuccess ||
-      cudaStreamSynchronize(s) != cudaSuccess) {
-    release(b);
+      cudaStreamSynchronize(s) != cudaSuccess)
     return MACH_ERR_CUDA;
-  }
   int dev = 0, sms = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   b->per_sm = batch_blocks_per_sm(dt, b->slot_bytes);
   b->grid = std::max(1, std::min(b->n_items, sms * b->per_sm));
+  return MACH_OK;
+}
+
+mach_status mach_batch_plan(const mach_das_desc* descs, int32_t n, const mach_tile_shape* shapes, void* stream,
+                            mach_batch* out) {
+  if (!out) return MACH_ERR_INVALID_ARG;
+  *out = nullptr;
+  if (!descs || n < 1) return MACH_ERR_INVALID_ARG;
+  const int dt = descs[0].iq_dtype;
+  for (int i = 0; i < n; ++i) {
+    mach_status st = host_validate(&descs[i]);
+    if (st != MACH_OK) return st;
+    if (descs[i].term_table) return MACH_ERR_UNSUPPORTED;
+    if (descs[i].iq_dtype != dt) return MACH_ERR_INVALID_ARG;
+    if (descs[i].n_frames > 64) return MACH_ERR_UNSUPPORTED;
+    if (shapes) {
+      const mach_tile_shape& s = shapes[i];
+      if (s.mode == kBatchChannels) {
+        if (descs[i].n_frames > 4) return MACH_ERR_INVALID_ARG;
+      } else if (s.mode == kBatchStaged) {
+        if (s.frame_lanes != 8 && s.frame_lanes != 16) return MACH_ERR_INVALID_ARG;
+        if (4 * s.frame_lanes < descs[i].n_frames) return MACH_ERR_INVALID_ARG;
+      } else if (s.mode == kBatchFrames) {
+        if (s.frame_lanes != 2 && s.frame_lanes != 4 && s.frame_lanes != 8 && s.frame_lanes != 16)
+          return MACH_ERR_INVALID_ARG;
+        if (4 * s.frame_lanes < descs[i].n_frames) return MACH_ERR_INVALID_ARG;
+      } else {
+        return MACH_ERR_INVALID_ARG;
+      }
+      const bool zero = s.tile[0] == 0 && s.tile[1] == 0 && s.tile[2] == 0;
+      if (!zero && (s.tile[0] < 1 || s.tile[1] < 1 || s.tile[2] < 1 ||
+                    s.tile[0] * s.tile[1] * s.tile[2] != voxels_per_block(s)))
+        return MACH_ERR_INVALID_ARG;
+    }
+  }
+  if (dt == MACH_IQ_C64_SPLIT) return MACH_ERR_UNSUPPORTED;
+  mach_batch_s* b = new (std::nothrow) mach_batch_s();
+  if (!b) return MACH_ERR_OOM;
+  mach_status st;
+  try {
+    st = plan_batch(descs, n, shapes, static_cast<cudaStream_t>(stream), b);
+  } catch (const std::bad_alloc&) {   // the host lists grow with the tiles of every instance
+    st = MACH_ERR_OOM;
+  } catch (const std::length_error&) {
+    st = MACH_ERR_OOM;
+  }
+  if (st != MACH_OK) {
+    release(b);
+    return st;
+  }
   *out = b;
   return MACH_OK;
 }

@@ -685,17 +685,6 @@ static mach_status make_plan(const mach_das_desc* d, void* stream, PlanFor use, 
   }
   if (need > free_b) return MACH_ERR_OOM;
 
-  mach_plan_s* p = new (std::nothrow) mach_plan_s();
-  if (!p) return MACH_ERR_OOM;
-  p->d = *d;
-  p->d.elem_pos = nullptr;
-  p->d.vox_pos = nullptr;
-  p->d.tx_angles = nullptr;
-  p->d.tx_table_dev = nullptr;
-  p->d.n_vox = V;
-  p->variant = var;
-  cudaGetDevice(&p->device);
-
   const double k = d->fs / d->c;
   const double t0fs = d->t0 * d->fs;
   std::vector<float4> elem(C);
@@ -713,6 +702,17 @@ static mach_status make_plan(const mach_das_desc* d, void* stream, PlanFor use, 
       u[3 * t + 2] = std::cos(az) * std::cos(el);
     }
   }
+
+  mach_plan_s* p = new (std::nothrow) mach_plan_s();
+  if (!p) return MACH_ERR_OOM;
+  p->d = *d;
+  p->d.elem_pos = nullptr;
+  p->d.vox_pos = nullptr;
+  p->d.tx_angles = nullptr;
+  p->d.tx_table_dev = nullptr;
+  p->d.n_vox = V;
+  p->variant = var;
+  cudaGetDevice(&p->device);
 
   float* d_raw = nullptr;
   double* d_u = nullptr;
@@ -872,7 +872,11 @@ static mach_status make_plan(const mach_das_desc* d, void* stream, PlanFor use, 
 }
 
 mach_status mach_das_plan(const mach_das_desc* d, void* stream, mach_plan* out) {
-  return make_plan(d, stream, kForRuns, out);
+  try {
+    return make_plan(d, stream, kForRuns, out);
+  } catch (const std::bad_alloc&) {   // of the host copies of the elements and transmits
+    return MACH_ERR_OOM;
+  }
 }
 
 mach_status mach_plan_destroy(mach_plan p) {

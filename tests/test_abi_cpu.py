@@ -3,6 +3,7 @@ rejects bad arguments before touching CUDA."""
 import ctypes as C
 import os
 import re
+import sys
 
 import numpy as np
 import pytest
@@ -222,3 +223,34 @@ def test_every_variant_name_the_tests_force_is_known():
         assert e.value.status == m.MACH_ERR_INVALID_ARG
     finally:
         m.mach_debug_force_variant(None)
+
+
+LIMITED = """
+import ctypes as C, resource, sys
+sys.path.insert(0, sys.argv[1])
+import numpy as np
+import paper_2604_06257_gb300 as m
+kw = dict(ndim=2, elem_pos=np.zeros((1, 3), np.float32), tx_angles=np.zeros((1, 2)), fs=1e6, fc=0.0, c=1500.0, t0=0.0,
+          f_number=1.0, apod="boxcar", n_samples=8, n_frames=8, grid_dims=(1, 1, 1), grid_origin=(0.0, 0.0, 0.01),
+          grid_step=(0.0, 0.0, 0.0), iq_dtype="c64")
+n = 500_000
+one, keep = m.make_desc(**kw)
+arr = (m.mach_das_desc * n)()
+size = C.sizeof(one)
+C.memmove(arr, bytes(C.string_at(C.byref(one), size)) * n, size * n)
+lib = m.lib()
+pages = int(open("/proc/self/statm").read().split()[0])
+resource.setrlimit(resource.RLIMIT_AS, (pages * 4096 + (64 << 20),) * 2)
+h = C.c_void_p()
+print("status", lib.mach_batch_plan(C.cast(arr, C.c_void_p), n, None, None, C.byref(h)), h.value)
+"""
+
+
+def test_host_memory_failure_is_a_status_not_an_exception():
+    """A batch whose host lists (hundreds of bytes an instance) do not fit in the address space left
+    to the process: OUT OF MEMORY, and no exception leaves the C interface."""
+    import subprocess
+    r = subprocess.run([sys.executable, "-c", LIMITED, ROOT], capture_output=True, text=True, timeout=300,
+                       env={**os.environ, "CUDA_VISIBLE_DEVICES": ""})
+    assert r.returncode == 0, r.stderr[-2000:]
+    assert r.stdout.split() == ["status", str(m.MACH_ERR_OOM), "None"], r.stdout
