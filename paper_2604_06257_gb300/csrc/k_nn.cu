@@ -495,8 +495,8 @@ __device__ __forceinline__ float coord_of(int64_t i, int n) {
 }
 
 // The volumes lie on the frames axis of y ([V][N]) and lead in the network's tensors ([N][V]).
-// Items run over (voxel, volume) with the volume fastest, so that both sides move whole
-// 32-byte sectors (volume by volume, a batch of 8 read 64 bytes of y for every 8 used).
+// Items run over (voxel, volume) with the volume fastest where whole rows of y are written (volume
+// by volume, a batch of 8 moved 64 bytes of y for every 8 used).
 struct Item {
   int n;
   int64_t v, i;   // volume, voxel, n V + v
@@ -513,13 +513,25 @@ __device__ __forceinline__ Item item_at(int64_t j, int64_t V, int N) {
   return t;
 }
 
-__global__ void k_pack(const float2* __restrict__ y, const float* __restrict__ sums, int64_t V, int N, int C,
-                       int coords, int nx, int ny, int nz, bf16* __restrict__ xin, float2* __restrict__ xf) {
-  const int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (j >= V * N) return;
-  const Item t = item_at(j, V, N);
+// G = 2^lg volumes (1, 2 or 4, N permitting) of 256 / G voxels per block, the volumes fastest: a warp
+// reads a 32-byte sector of y per voxel and writes 64 consecutive bytes of xf per volume; the
+// blocks of the same voxels' other volumes come next.  Batches of 8 / 16 / 64 volumes of 96^3
+// voxels, cold caches: 67 / 133 / 535 us.  One volume per block (each sector of y read four
+// times, from L2 mostly) 71 / 159 / 648, eight 78 / 150 / 632; all volumes of a voxel in
+// consecutive threads 78 / 233 / 3383 (with many volumes a warp writes 8 bytes here and there),
+// volume by volume over the whole grid 75 / 319 / 1290.
+__global__ void __launch_bounds__(256) k_pack(const float2* __restrict__ y, const float* __restrict__ sums, int64_t V,
+                                              int N, int C, int coords, int nx, int ny, int nz, int lg, int chunks,
+                                              bf16* __restrict__ xin, float2* __restrict__ xf) {
+  const int64_t tile = blockIdx.x / static_cast<unsigned>(chunks);
+  const int chunk = static_cast<int>(blockIdx.x - tile * chunks);
+  Item t;
+  t.n = (chunk << lg) + static_cast<int>(threadIdx.x & ((1u << lg) - 1u));
+  t.v = tile * (256 >> lg) + (threadIdx.x >> lg);
+  if (t.n >= N || t.v >= V) return;
+  t.i = t.n * V + t.v;
   const float inv = 1.f / rms_of(sums, t.n, V);
-  const float2 a = y[j];
+  const float2 a = y[t.v * N + t.n];
   const float2 x = make_float2(a.x * inv, a.y * inv);
   xf[t.i] = x;
   uint4* dst = reinterpret_cast<uint4*>(xin + t.i * C);
@@ -667,8 +679,12 @@ cudaError_t launch_vol_sumsq(const float2* y, float* sums, float* part, int64_t 
 
 cudaError_t launch_pack(const float2* y, const float* sums, int64_t V, int N, int C, int coords, int nx, int ny,
                         int nz, void* xin, float* xf, cudaStream_t s) {
-  k_pack<<<blocks_for(V * N), 256, 0, s>>>(y, sums, V, N, C, coords, nx, ny, nz, static_cast<bf16*>(xin),
-                                           reinterpret_cast<float2*>(xf));
+  int lg = 0;
+  while (lg < 2 && (1 << lg) < N) ++lg;
+  const int chunks = (N + (1 << lg) - 1) >> lg;
+  const int64_t blocks = (V + (256 >> lg) - 1) / (256 >> lg) * chunks;
+  k_pack<<<static_cast<unsigned>(blocks), 256, 0, s>>>(y, sums, V, N, C, coords, nx, ny, nz, lg, chunks,
+                                                       static_cast<bf16*>(xin), reinterpret_cast<float2*>(xf));
   return cudaGetLastError();
 }
 
