@@ -130,8 +130,8 @@ __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* map
       : "memory");
 }
 
-// MMAs and commits are issued by one elected lane while the whole warp walks the loops around
-// them: the warp stays convergent, so the descriptors live in uniform registers (inside a
+// In the kernels of at most 64 output channels MMAs and commits are issued by one elected lane while
+// the whole warp walks the loops around them: the warp stays convergent, so the descriptors live in uniform registers (inside a
 // one-lane branch each had to be moved there for every MMA: x-folded 48 -> 16 at 8 x 128^3 1003 -> 845 us, 32 -> 16 713 -> 588 us).
 __device__ __forceinline__ uint32_t elect_one() {
   uint32_t lead;
@@ -216,7 +216,12 @@ __device__ __forceinline__ TileCoord tile_coord_x(const ConvTcParams& p, int64_t
   return c;
 }
 
-template <bool FLIP, int TZ>
+// WARP: the whole issuing warp walks its loops (see elect_one), else lane 0 alone.  The loads of the
+// descriptors that the former saves count while an MMA is short; above 64 output channels its
+// votes after each wait cost more: 128 -> 128 at 64^3 154 us against 145, 64 -> 128 86 against 83,
+// 32 -> 96 47 against 45, 112 -> 80 117 against 114.  At most 64: 64 -> 64 53.4 against 53.5, 192 -> 64
+// 145 against 148, 96 -> 32 at 4 x 33 x 20 x 47 53 against 57.
+template <bool FLIP, int TZ, bool WARP>
 __global__ void __launch_bounds__(kThreads, 3) k_conv3d_tc(const __grid_constant__ CUtensorMap xmap,
                                                            const ConvTcParams p) {
   extern __shared__ uint8_t smem_raw[];
@@ -309,24 +314,34 @@ __global__ void __launch_bounds__(kThreads, 3) k_conv3d_tc(const __grid_constant
       await_copies(fullA, 2, a_use);
       await_copies(fullB, kNB, p.resident ? 1u : b_use);
     }
-  } else if (warp == 1) {   // -------------------------------------------- MMAs
-    const uint32_t lead = elect_one();
+  } else if (warp == 1 && (WARP || lane == 0)) {   // ---------------------- MMAs
+    const uint32_t lead = WARP ? elect_one() : 1u;
     const uint32_t idesc = instr_desc(p.Co);
-    bool ok = !p.resident || wait_warp(&fullB[0], 0, limit);
-    if (!ok) if (lane == 0) give_up();
+    auto wait = [&](uint64_t* bar, uint32_t parity) {
+      if constexpr (WARP) return wait_warp(bar, parity, limit);
+      const bool got = wait_spin(bar, parity, limit);
+      if (!got) give_up();
+      return got;
+    };
+    auto aborted = [&]() {
+      if constexpr (WARP) return __any_sync(0xffffffffu, *abort_flag);
+      else return *abort_flag;
+    };
+    bool ok = !p.resident || wait(&fullB[0], 0);
+    if (!ok) if (WARP && lane == 0) give_up();
     uint32_t a_use = 0, b_use = 0, acc_use = 0;
-    for (int64_t tile = blockIdx.x; ok && tile < p.tiles && !__any_sync(0xffffffffu, *abort_flag); tile += gridDim.x) {
+    for (int64_t tile = blockIdx.x; ok && tile < p.tiles && !aborted(); tile += gridDim.x) {
       const uint32_t buf = acc_use & 1u, ku = acc_use >> 1;
-      if (ku >= 1 && !wait_warp(&tempty[buf], (ku - 1) & 1u, limit)) {
-        if (lane == 0) give_up();
+      if (ku >= 1 && !wait(&tempty[buf], (ku - 1) & 1u)) {
+        if (WARP && lane == 0) give_up();
         break;
       }
       fence_after();
       const uint32_t d0 = tmem + buf * (p.tmem_cols >> 1);
       for (int kc = 0; kc < NC && ok; ++kc) {
         const uint32_t sa = a_use & 1u, ka = a_use >> 1;
-        if (!wait_warp(&fullA[sa], ka & 1u, limit)) {
-          if (lane == 0) give_up();
+        if (!wait(&fullA[sa], ka & 1u)) {
+          if (WARP && lane == 0) give_up();
           ok = false;
           break;
         }
@@ -341,8 +356,8 @@ __global__ void __launch_bounds__(kThreads, 3) k_conv3d_tc(const __grid_constant
             w_base = smem_u32(sW) + (static_cast<uint32_t>(kc) * 27 + tb * 9) * tap_bytes;
           } else {
             sb = b_use % kNB;
-            if (!wait_warp(&fullB[sb], (b_use / kNB) & 1u, limit)) {
-              if (lane == 0) give_up();
+            if (!wait(&fullB[sb], (b_use / kNB) & 1u)) {
+              if (WARP && lane == 0) give_up();
               ok = false;
               break;
             }
@@ -376,7 +391,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_conv3d_tc(const __grid_constant
       ++acc_use;
     }
     mma_commit(lead, fin);
-  } else {   // ---------------------------------------------------------- epilogue
+  } else if (WARP || warp > 1) {   // --------------------------------------- epilogue
     const int q = warp & 3;            // tensor-memory lanes 32q .. 32q + 31
     const int row = 32 * q + lane;     // GEMM row within a plane
     const int mx = row & 7, my = row >> 3;
@@ -846,6 +861,11 @@ bool use_fold(int ci, int co, bool flip) {
 }
 
 using ConvKernel = void (*)(CUtensorMap, ConvTcParams);
+template <bool FLIP>
+ConvKernel tc_kernel(int co, int tz) {   // the planes that tc_shape gives
+  if (co > 64) return tz == 2 ? k_conv3d_tc<FLIP, 2, false> : k_conv3d_tc<FLIP, 1, false>;
+  return tz == 4 ? k_conv3d_tc<FLIP, 4, true> : k_conv3d_tc<FLIP, 2, true>;
+}
 ConvKernel fold_kernel(int co, int tz, bool flip) {
   if (co == 32) return tz == 2 ? k_conv3d_tcx<true, 2, 32> : k_conv3d_tcx<true, 1, 32>;
   if (flip) return tz == 4 ? k_conv3d_tcx<true, 4, 16> : tz == 2 ? k_conv3d_tcx<true, 2, 16> : k_conv3d_tcx<true, 1, 16>;
@@ -959,10 +979,7 @@ cudaError_t launch_conv_tc(const void* x, const void* wpk, const float* bias, vo
   p.wait_limit = g_wait_limit ? g_wait_limit : kDefaultWait;
   p.debug_stall = g_debug_stall;
   const size_t smem = shp.smem;
-  ConvKernel kern = flip ? (shp.tz == 4 ? k_conv3d_tc<true, 4> : shp.tz == 2 ? k_conv3d_tc<true, 2> : k_conv3d_tc<true, 1>)
-                     : (shp.tz == 4 ? k_conv3d_tc<false, 4>
-                                    : shp.tz == 2 ? k_conv3d_tc<false, 2> : k_conv3d_tc<false, 1>);
-  if (fold) kern = fold_kernel(co, shp.tz, flip != 0);
+  const ConvKernel kern = fold ? fold_kernel(co, shp.tz, flip != 0) : flip ? tc_kernel<true>(co, shp.tz) : tc_kernel<false>(co, shp.tz);
   const int threads = fold ? kFoldThreads : kThreads;
   int per_sm = 0, sms = 0;
   const cudaError_t e = kernel_setup(reinterpret_cast<const void*>(kern), threads, smem, p.tmem_cols, &per_sm, &sms);
