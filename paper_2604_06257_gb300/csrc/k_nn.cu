@@ -794,6 +794,9 @@ mach_status mach_nn_bias_grad(const void* g, float* db, int64_t voxels, int32_t 
   if (c % 8 == 0 && aligned16(g)) {
     const int64_t rows8 = 4 * (256 / (c / 8));
     int64_t blocks8 = (voxels + rows8 - 1) / rows8;
+    // Every block ends in c atomics on the same c words: with many channels it takes four rounds of rows
+    // at least (256 channels, 32^3 voxels: 10 us, one round 18.5, 2-byte loads 16).
+    if (c >= 128) blocks8 = (blocks8 + 3) / 4;
     blocks8 = blocks8 < 152 * 8 ? blocks8 : 152 * 8;
     k_bias_grad8<<<static_cast<unsigned>(blocks8), 256, 0, static_cast<cudaStream_t>(stream)>>>(
         static_cast<const uint4*>(g), db, voxels, c);
