@@ -276,10 +276,12 @@ typedef struct mach_batch_s *mach_batch;
  * iq_dtype, not the split layout, n_frames <= 64): builds every instance's tables and one
  * work list of (instance, voxel tile) items, sorted by decreasing estimated cost, for
  * one persistent launch.  shapes: NULL or n entries.  With NULL, instances of more than 4
- * frames whose own plan would repack them (see Workspaces above) are repacked and beamformed
- * by one exact-frame launch per tile shape instead; the batch owns their workspace (at most a
- * sixteenth of the device memory in all, none if that cannot be had) and mach_batch_get_info
- * still reports the lane mapping they would take otherwise.  Synchronises `stream`.
+ * frames for which that pays are rewritten into whole frame tiles (see Workspaces above) and
+ * beamformed by one exact-frame launch per tile shape and 64 instances instead; the batch owns
+ * their workspace (at most a sixteenth of the device memory in all, none if that cannot be had)
+ * and mach_batch_get_info still reports the lane mapping they would take otherwise.  Shapes
+ * name lane mappings: a batch with shapes, for whichever instance, repacks none.
+ * Synchronises `stream`.
  * Errors: INVALID_ARG, UNSUPPORTED, OOM, CUDA. */
 mach_status mach_batch_plan(const mach_das_desc *descs, int32_t n, const mach_tile_shape *shapes,
                             void *stream, mach_batch *out);

@@ -589,9 +589,9 @@ class Plan:
 # ---- ragged batches ------------------------------------------------------------------
 
 class Batch:
-    """Many instances (``plan_kwargs``-style dicts) beamformed by one persistent launch.
+    """Many instances (``plan_kwargs``-style dicts) beamformed by one stream-ordered run.
     ``shapes``: optional list of (mode, frame_lanes, (tx, ty, tz)) per instance, e.g. from
-    ``autotune.tune_batch``; None uses the library's default lane mapping and tile box."""
+    ``autotune.tune_batch``; None leaves the lane mappings, and whether to repack, to the library."""
 
     def __init__(self, instances, shapes=None, stream=None):
         self._descs_keep = [make_desc(**kw) for kw in instances]

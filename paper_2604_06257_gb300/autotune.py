@@ -6,6 +6,10 @@ Large instances are timed on a slab of their grid (the first ``slab`` z-planes, 
 lateral extent, elements, transmits and frames), which has the same per-tile work.
 Results are cached per shape signature (dimensionality, grid, elements, transmits,
 frames, samples, storage type), so instances of the same shape are tuned once.
+
+Candidates are lane mappings of the persistent launch.  A batch that names them repacks none of its
+instances into frame tiles, as the library does by default where that is faster: on dense
+grids of more than four frames the defaults win, and ``tune_batch`` returns None.
 """
 from __future__ import annotations
 

@@ -1,4 +1,5 @@
-// batch.cpp -- ragged batches of DAS instances in one persistent launch (host side).
+// batch.cpp -- ragged batches of DAS instances (host side): a persistent launch over the lane
+// mappings, and launches over the frame tiles of repacked instances.
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -15,13 +15,16 @@
 // for 36 MMAs (one fragment per tap would take 18 + 2).  At the end the quarters meet in
 // shared memory and leave by one float32 atomic per weight and block.
 //
-// tcgen05 does not apply: its M is at least 64, and the taps' voxel offsets inside a brick
-// are no arithmetic progression that one operand descriptor could walk.
+// tcgen05 is not used: its M is at least 64, and in this brick layout (channel group outermost) the
+// taps' voxel offsets and the channel groups are no arithmetic progression that one operand
+// descriptor could walk.  (With the channel group between y and x they would be.)
 // It runs at 440-490 TFLOP/s on every large layer (750 multiply-adds a cycle and SM): the
 // warp-level MMA rate, not memory (16 -> 16 moves 1.1 GB in 495 us).  Batch 8, earlier kernel
 // (whose copies' address arithmetic took more issue slots than its products) -> this one: 16 -> 16 at 128^3
 // 1189 -> 495 us, 48 -> 16 4281 -> 1418, 32 -> 32 at 64^3 473 -> 260, 192 -> 64 at 32^3
-// 897 -> 393, 128 -> 128 at 16^3 138 -> 88; 9 x 11 x 13 voxels 17 -> 18 us.
+// 897 -> 393, 128 -> 128 at 16^3 138 -> 88.  Layers of few tiles and many channel blocks lost: 64 -> 128
+// at 1 x 9 x 11 x 13 voxels 12 -> 18 us, several waves of blocks of one tile each; one wave takes 10
+// us, but its longer chains cost accuracy (see launch_conv_wgrad).
 #pragma once
 
 constexpr int kWgTZ = 2;                                        // z planes per tile

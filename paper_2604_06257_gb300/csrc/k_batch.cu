@@ -1,7 +1,7 @@
-// k_batch.cu -- ragged batches: many DAS instances in one persistent launch.
+// k_batch.cu -- ragged batches: the DAS instances that run in one persistent launch.
 //
 // This kernel takes the instances that are not repacked into whole frame tiles (F <= 4,
-// explicit shapes, grids of few voxels per sample); the others run in k_das_exact_multi.
+// explicit shapes, small or sparse grids); the others run in k_das_exact_multi.
 // A batch holds instances of different sizes (2D and 3D grids, element, transmit and
 // frame counts).  Their voxel tiles form one work list, sorted by decreasing estimated
 // cost; a persistent grid (as many blocks as fit on the GPU) pulls (instance, tile) items
@@ -15,8 +15,8 @@
 //    ring (one bulk copy; for rows that do not start on a 16-byte boundary the copy starts
 //    at the boundary below and the consumers skip the difference), the consumer warps
 //    evaluate each term once and accumulate 4 frames per lane from shared memory (16-byte
-//    vectors when F % 4 == 0, else one sample per frame).  The ring's barriers are
-//    initialised afresh for every item;
+//    vectors when F % 4 == 0, else one sample per frame).  The ring
+//    lives as long as the block, an item goes on where the last one ended;
 //  - frame lanes (F <= 16 or a multiple of 4, and the fallback when an instance's windows
 //    exceed the ring): FL lanes share a voxel (FL = 2, 4, 8 or 16 at run time), each lane
 //    holds 4 frames of 4 voxels (2 voxels for FL = 2), taps read through L1;

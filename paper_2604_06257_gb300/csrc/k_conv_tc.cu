@@ -853,9 +853,11 @@ int fold_tz(int co) {
 // leave too few MMAs per drained column); weights have to fit.  27-tap kernel -> folded, us:
 // 32 -> 32 at 8 x 64^3 155 -> 128, 64 -> 32 290 -> 222, 96 -> 32 418 -> 354, 16 -> 32 90 -> 121;
 // 48 outputs (N = 144, one plane per tile) from 16 channels at 8 x 128^3 857 -> 1478, so not
-// offered.  Forward layers of 32 outputs stay on the 27-tap kernel although folding is faster:
-// the tensor cores' sums truncate, shorter chains shift that bias, and over ten training
-// batches of 8 x 128^3 the loss's mean relative error against float64 went from 2.1e-5 to 3.2e-5.
+// offered.  Forward layers of 32 outputs stay on the 27-tap kernel although folding is faster and
+// its chains are shorter: the loss of the bfloat16 network then lies further from that of the
+// same network in float64 (mean of ten training batches of 8 x 128^3, relative: 2.1e-5 -> 3.2e-5, together with a
+// loss summed per block).  The sums themselves are not less exact; the truncation of the
+// longer chains offsets part of the rounding to bfloat16.
 bool use_fold(int ci, int co, bool flip) {
   return g_conv_fold && ci <= 96 && (co == 16 || (co == 32 && ci >= 32 && flip));
 }

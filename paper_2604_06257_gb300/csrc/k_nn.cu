@@ -549,11 +549,11 @@ __global__ void __launch_bounds__(256) k_pack(const float2* __restrict__ y, cons
 }
 
 // Loss and its gradient, one item per thread, one atomic per warp on the loss.  The half million
-// additions to one word take most of the 1.24 ms at 8 x 128^3, and their order of rounding
-// belongs to the result: adding up per block first takes 0.25 ms and sums the same terms more
-// exactly, but the word's own rounding happens to offset part of the bfloat16 network's bias,
-// and over ten training batches the loss's mean distance from float64 grew from 2.1e-5 to
-// 2.8e-5 of its value.
+// additions to one word, in an order that changes from run to run, take 1.0 of the 1.24 ms at
+// 8 x 128^3.  Adding up per block first takes 0.25 ms and sums the same terms more exactly.  It is
+// left out for the loss's distance from that of the network in float64, which then grows from
+// 2.1e-5 to 2.8e-5 of its value (mean of ten training batches): the word's rounding offsets part of
+// the bfloat16 network's bias.
 __global__ void k_loss(const float* __restrict__ o, const float2* __restrict__ xf, const float2* __restrict__ target,
                        const float* __restrict__ sums, float gain, int64_t V, int N, int Co, int C,
                        bf16* __restrict__ g, float* __restrict__ loss, float inv_count) {

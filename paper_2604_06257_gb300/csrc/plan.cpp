@@ -505,7 +505,7 @@ static mach_status build_term_table(mach_plan_s* p, DasParams& b, cudaStream_t s
 //  * Staged kernels of 64 frames (33 to 64): a tile holds 8 x 4 or 16 x 4 voxels for all frames, and
 //    two frame tiles double the term evaluations: 0.40 ... 1.5, slower in more than half of the
 //    grids.  From three waves of two blocks per SM and a share of 0.3 on, where the direct
-//    kernel's tail is short and its terms many: 0.99 ... 1.5.  (A 64-frame ring of two pairs,
+//    kernel's tail is short and its terms many: 0.97 ... 1.5, half of them above 1.15.  (A 64-frame ring of two pairs,
 //    taken for long windows: 0.87 ... 2.4, from 2e7 points on 0.97 ... 2.4.)
 //  * Batches: every instance's pass is a launch of its own (about 8 us in which the other
 //    instances wait), against the lane mappings of the persistent kernel: six equal instances
