@@ -118,6 +118,47 @@ void staged_tile(int n, int nx, int ny, int nz, bool list, int tile[3]) {
   }
 }
 
+// Which instances are repacked (bytes of `repack`, one per plan).  Repacking an instance takes launches
+// of its own, in which the others wait; the lane mappings share one persistent launch but do more
+// work per term.  Microseconds of either, fitted to batches of 30 equal float16 and complex64
+// instances (2D of 48^2 ... 128^2 px, 3D of 28^3 voxels, 1 and 3 transmits, F-numbers 1 ... 3, 5 to 64
+// frames; lanes within a tenth, repacked runs within a sixth, half of the time):
+//  * lanes: every (voxel, element) and (voxel, element, transmit) is looked at, terms inside the
+//    aperture take the lanes' frame slots; staged windows skip most of the rest;
+//  * repacked: the pass, a reduction when there are several frame tiles, points and terms.
+// The launch of the lane mappings takes 25 us at least.  Both are estimates, so lanes have to be a
+// third cheaper.  Against always repacking (3, 6, 12 and 30 equal instances): 0.7 to 7.8 times the
+// speed, hardly ever below 1; against never repacking 0.54 ... 8, in 90 of 100 above 0.85.  In a mixed batch a
+// persistent launch of a few small instances is all tail (ten float16 instances 3.58 ms, 3.77 with
+// the four small ones on lanes).
+void choose_repacked(const std::vector<mach_plan>& plans, const mach_das_desc* descs, std::vector<char>& repack) {
+  constexpr double kLaunch = 9.0, kReduce = 4.0, kFloor = 25.0, kMargin = 1.3;
+  std::vector<char> cheap(plans.size(), 0);   // lanes would be cheaper
+  double lanes_sum = 0.0, repacked_sum = 0.0;
+  for (size_t i = 0; i < plans.size(); ++i) {
+    RepackNeeds q;
+    if (!plan_repack(plans[i], &q)) continue;
+    repack[i] = 1;
+    const DasParams& p = *plan_params(plans[i]);
+    const FrameSplit fs = split_frames(p.F);
+    const double vc = static_cast<double>(p.V) * p.C, terms = q.points / fs.padded();
+    const double repacked = kLaunch + (fs.tiles() > 1 ? kReduce : 0.0) + q.points / 1.04e6 + terms / 1.78e5;
+    const mach_tile_shape sh = default_shape(descs[i].n_frames);
+    const double lanes =
+        sh.mode == kBatchStaged
+            ? vc * p.T / 5.9e5 + terms * 2 * sh.frame_lanes / 6.0e5
+            : vc / 2.5e5 + vc * p.T / (sh.frame_lanes <= 2 ? 4.0e5 : sh.frame_lanes <= 4 ? 2.1e5 : sh.frame_lanes <= 8 ? 1.6e5 : 1.0e5) +
+                  terms * 4 * sh.frame_lanes / 1.15e6;
+    if (repacked < kMargin * lanes) continue;
+    cheap[i] = 1;
+    lanes_sum += lanes;
+    repacked_sum += repacked;
+  }
+  if (repack_forced() || repacked_sum < kMargin * (kFloor + lanes_sum)) return;
+  for (size_t i = 0; i < plans.size(); ++i)
+    if (cheap[i]) repack[i] = 0;
+}
+
 // The launches over the repacked instances' frame tiles: instances grouped by exact-frame
 // shape, each group's (frame tile, voxel tile) items longest first; the workspace for all of
 // them, which runs share in stream order as they do the work counter.  OOM, UNSUPPORTED: the
@@ -127,10 +168,9 @@ mach_status plan_repacked(mach_batch_s* b, cudaStream_t s) {
   struct Group { std::vector<Item> items; mach_batch_s::Multi* m = nullptr; };
   std::vector<Group> groups;
   for (const auto& q : b->repacked) {
-    const RepackPart* parts = nullptr;
-    size_t ws_i = 0, pd_i = 0;
-    int range[2];
-    const int np = plan_repack(b->plans[q.inst], &parts, &ws_i, &pd_i, range);
+    RepackNeeds needs;
+    const int np = plan_repack(b->plans[q.inst], &needs);
+    const RepackPart* parts = needs.parts;
     for (int k = 0; k < np; ++k) {
       // 2D and 3D shapes of 32 frames are one kernel
       const Variant v = parts[k].v == V_SX32_F8V1W7_T8X7E ? V_SX32_F8V1W7T14E : parts[k].v;
@@ -197,21 +237,24 @@ static mach_status plan_batch(const mach_das_desc* descs, int32_t n, const mach_
   std::vector<char> is_repacked(n, 0);
   std::vector<size_t> slots(n, 0);         // ring slots that staged instances need
   b->bounds.assign(2 * static_cast<size_t>(n), nullptr);
+  for (int i = 0; i < n; ++i)
+    if (const mach_status st = make_batch_plan(&descs[i], !shapes, s, &b->plans[i]); st != MACH_OK) return st;
+  // default shapes only: the instances worth repacking join the launches over repacked tiles
+  if (!shapes) choose_repacked(b->plans, descs, is_repacked);
   for (int i = 0; i < n; ++i) {
-    mach_status st = make_batch_plan(&descs[i], !shapes, s, &b->plans[i]);
-    if (st != MACH_OK) return st;
-    // default shapes only: an instance that its plan would repack joins the launches over
-    // repacked tiles
-    const RepackPart* parts = nullptr;
-    size_t ws_i = 0, pd_i = 0;
-    int range[2];
-    if (!shapes && plan_repack(b->plans[i], &parts, &ws_i, &pd_i, range) && ws_total + ws_i <= total_mem / 16) {
-      is_repacked[i] = 1;
-      const DasParams& q = *plan_params(b->plans[i]);
-      b->repacked.push_back({i, dt, q.F, parts[0].base.frame_tiles, static_cast<int64_t>(q.T) * q.C, q.V, q.S,
-                             {range[0], range[1]}, ws_total, pd_i});
-      ws_total += (ws_i + 255) / 256 * 256;
+    if (!is_repacked[i]) continue;
+    RepackNeeds q;
+    plan_repack(b->plans[i], &q);
+    if (ws_total + q.ws_bytes > total_mem / 16) {
+      is_repacked[i] = 0;
+      continue;
     }
+    const DasParams& p = *plan_params(b->plans[i]);
+    b->repacked.push_back({i, dt, p.F, q.parts[0].base.frame_tiles, static_cast<int64_t>(p.T) * p.C, p.V, p.S,
+                           {q.range[0], q.range[1]}, ws_total, q.pd_at});
+    ws_total += (q.ws_bytes + 255) / 256 * 256;
+  }
+  for (int i = 0; i < n; ++i) {
     mach_tile_shape sh = shapes ? shapes[i] : default_shape(descs[i].n_frames);
     const DasParams base = *plan_params(b->plans[i]);
     DasParams p = base;

@@ -283,7 +283,14 @@ bool alloc_denied();
 // tables of a repacking plan altogether.  plan_repack: the launches
 // over its repacked tiles (0 when it beamforms directly), and the workspace they need.
 mach_status make_batch_plan(const mach_das_desc* d, bool repack, void* stream, mach_plan* out);
-int plan_repack(mach_plan p, const RepackPart** parts, size_t* ws_bytes, size_t* pd_at, int range[2]);
+struct RepackNeeds {
+  const RepackPart* parts;
+  size_t ws_bytes, pd_at;       // workspace, and where the partial Power Doppler sums lie in it
+  int range[2];                 // samples that windows touch
+  double points;                // voxels x windows x padded frames
+};
+int plan_repack(mach_plan p, RepackNeeds* needs);
+bool repack_forced();           // test hook
 int plan_iq_dtype(mach_plan p);
 void pick_tile_shape(int n, int nx, int ny, int nz, bool list, int tile[3]);
 

@@ -46,6 +46,7 @@ struct mach_plan_s {
   size_t ws_bytes = 0;          // workspace of one run: repacked IQ, partial Power Doppler sums
   size_t pd_at = 0;
   int range[2] = {0, 0};        // samples that the parts' windows touch
+  double points = 0.0;          // what the parts beamform: voxels x windows x padded frames
   cudaMemPool_t pool = nullptr;
 };
 
@@ -504,20 +505,18 @@ static mach_status build_term_table(mach_plan_s* p, DasParams& b, cudaStream_t s
 //    0.89 ... 0.97 at a share of 1/9, else 1.04 ... 2.1.
 //  * Staged kernels of 64 frames (33 to 64): a tile holds 8 x 4 or 16 x 4 voxels for all frames, and
 //    two frame tiles double the term evaluations: 0.40 ... 1.5, slower in more than half of the
-//    grids.  From three waves of two blocks per SM and a share of 0.3 on, where the direct
-//    kernel's tail is short and its terms many: 0.97 ... 1.5, half of them above 1.15.  (A 64-frame ring of two pairs,
+//    grids.  From three waves of two blocks per SM and a share of 0.4 on, where the direct
+//    kernel's tail is short and its terms many: 0.98 ... 1.5, half of them above 1.13; at shares of
+//    0.33 to 0.36 from 0.94 on.  (A 64-frame ring of two pairs,
 //    taken for long windows: 0.87 ... 2.4, from 2e7 points on 0.97 ... 2.4.)
-//  * Batches: every instance's pass is a launch of its own (about 8 us in which the other
-//    instances wait), against the lane mappings of the persistent kernel: six equal instances
-//    0.45 ... 1.3 below 5e6 points each, 24 of them 0.85 ... 1.4 from 2e7 to 5e7, 0.98 ... 2.9 above.
-static bool repack_pays(Variant direct, bool batch, double points, double share, int64_t tiles) {
-  if (batch) return points >= 5e7;
+// A batch's instances have other kernels to compare with: batch.cpp decides.
+static bool repack_pays(Variant direct, double points, double share, int64_t tiles) {
   switch (direct) {
     case V_ST32_C64_V4W7: case V_ST32_C64P_V4W7: return points >= 1e7 && share >= 0.2;
     case V_ST32_H16_V4: case V_ST32_B16_V4: return points >= 4e7 && share >= 0.125;
     case V_ST64_C64: return points >= 2e7;
     case V_ST64_C64_V4: case V_ST64_C64P_V4: case V_ST64_H16_V4: case V_ST64_B16_V4: case V_ST64_H16:
-      return tiles >= 3 * 2 * 152 && share >= 0.3;
+      return tiles >= 3 * 2 * 152 && share >= 0.4;
     default: return true;
   }
 }
@@ -603,9 +602,10 @@ static mach_status repack_plan(mach_plan_s* p, const DasParams& b, bool list, cu
   p->range[0] = lo;
   p->range[1] = hi;
   const double all = static_cast<double>(b.V) * b.C * b.T * fs.padded();
-  if (!g_force_repack && !repack_pays(p->variant, use == kForBatch, points, points / all,
-                                      static_cast<int64_t>(b.tiles_x) * b.tiles_y * b.tiles_z))
+  if (!g_force_repack && use != kForBatch &&
+      !repack_pays(p->variant, points, points / all, static_cast<int64_t>(b.tiles_x) * b.tiles_y * b.tiles_z))
     return done(MACH_OK);
+  p->points = points;
   p->pd_at = iq_bytes;
   p->ws_bytes = iq_bytes + pd_bytes;
   if (use == kForBatch) {
@@ -1082,14 +1082,11 @@ mach_status dev_alloc(void** p, size_t bytes, int64_t* total) {
 mach_status make_batch_plan(const mach_das_desc* d, bool repack, void* stream, mach_plan* out) {
   return make_plan(d, stream, repack ? kForBatch : kForLanes, out);
 }
-int plan_repack(mach_plan p, const RepackPart** parts, size_t* ws_bytes, size_t* pd_at, int range[2]) {
-  range[0] = p->range[0];
-  range[1] = p->range[1];
-  *parts = p->parts;
-  *ws_bytes = p->ws_bytes;
-  *pd_at = p->pd_at;
+int plan_repack(mach_plan p, RepackNeeds* needs) {
+  *needs = {p->parts, p->ws_bytes, p->pd_at, {p->range[0], p->range[1]}, p->points};
   return p->n_parts;
 }
+bool repack_forced() { return g_force_repack; }
 mach_status host_validate(const mach_das_desc* d) { return validate(d); }
 Variant host_unstaged_variant(int iq_dtype, int F) { return unstaged(pick_variant(iq_dtype, F)); }
 mach_status host_configure_tiles(DasParams& b, Variant v, bool list, int64_t V, int F) {

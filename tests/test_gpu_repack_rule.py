@@ -68,12 +68,31 @@ def test_either_route_gives_the_same_frames():
     assert nrmse_db(pd_r.cpu().numpy().astype(np.float64), pd.cpu().numpy().astype(np.float64)) <= -110
 
 
-def test_batches_of_small_instances_stay_in_one_launch():
-    """Items of a batch: those of the lane mappings where nothing is repacked."""
-    for acq, repacked in ((grid(64, 25, "f16x2", 1.5, 1, 248), False), (grid(128, 25, "f16x2", 1.0, 3, 585), True)):
-        kws = [m.plan_kwargs(acq)] * 6
+def batch_items(acqs):
+    """Items of the default batch, of its lane mappings, and with everything repacked."""
+    kws = [m.plan_kwargs(a) for a in acqs]
+    with m.Batch(kws) as b:
+        info = b.info()
+    with m.Batch(kws, shapes=[(s[0], s[1], None) for s in info["shapes"]]) as b:
+        lanes = b.info()["items"]
+    m.mach_debug_force_repack(True)
+    try:
         with m.Batch(kws) as b:
-            info = b.info()
-        with m.Batch(kws, shapes=[(s[0], s[1], None) for s in info["shapes"]]) as b:
-            lanes = b.info()["items"]
-        assert (info["items"] != lanes) == repacked, (info, lanes)
+            repacked = b.info()["items"]
+    finally:
+        m.mach_debug_force_repack(False)
+    assert lanes != repacked
+    return info["items"], lanes, repacked
+
+
+def test_batches_of_small_instances_stay_in_one_launch():
+    """Many small instances run in the persistent launch: repacked one after another they took two to eight
+    times as long.  A few, larger ones, and small ones that are dear on lanes are repacked."""
+    small = grid(64, 25, "f16x2", 1.5, 1, 248)
+    large = grid(40, 28, "f16x2", 1.0, 3, 452, 3, 576)
+    for acqs, repacked in (([small], True), ([small] * 12, False), ([small] * 30, False), ([large] * 2, True),
+                           ([grid(128, 25, "f16x2", 1.0, 3, 585)] * 6, True), ([grid(28, 16, "c64", 3.0, 1, 423, 3, 256)] * 12, True)):
+        items, lanes, all_repacked = batch_items(acqs)
+        assert items == (all_repacked if repacked else lanes), len(acqs)
+    items, lanes, all_repacked = batch_items([small] * 12 + [large])
+    assert items not in (lanes, all_repacked)         # the large one alone
