@@ -499,10 +499,10 @@ static mach_status build_term_table(mach_plan_s* p, DasParams& b, cudaStream_t s
 // grids of 48^2 ... 384^2 px with 64 ... 192 elements, 3D of 20^3 ... 64^3 voxels with 256 and
 // 576, 1 ... 9 transmits, F-numbers 1 ... 6 and no aperture, all storage types.
 //  * L1 kernels (5 to 16 frames, odd and long ensembles): 1.05 ... 5.5 wherever V >= 6 S.
-//  * Staged kernels of 32 frames, which read split or interleaved rows as they are: complex64
-//    0.81 ... 1.7 below 1e7 points (half of them below 1.04), 0.96 ... 1.2 at a share below 0.2,
-//    else 1.01 ... 2.15; 16-bit pairs, whose rows are half as long, 0.62 ... 1.8 below 4e7 points,
-//    0.89 ... 0.97 at a share of 1/9, else 1.04 ... 2.1.
+//  * Staged kernels of 32 frames, which read split or interleaved rows as they are: 0.59 ... 1.8 below
+//    1e7 points, four fifths of them slower; from there on 0.64 ... 1.4 at shares of 1/9 and below,
+//    seven tenths of them slower; else 0.81 ... 2.15, nine tenths of them faster, half above 1.23.  (The
+//    slower ones are mostly 2D grids at shares of 0.12 to 0.2, among others of 1.1 to 1.5.)
 //  * Staged kernels of 64 frames (33 to 64): a tile holds 8 x 4 or 16 x 4 voxels for all frames, and
 //    two frame tiles double the term evaluations: 0.40 ... 1.5, slower in more than half of the
 //    grids.  From three waves of two blocks per SM and a share of 0.4 on, where the direct
@@ -512,8 +512,8 @@ static mach_status build_term_table(mach_plan_s* p, DasParams& b, cudaStream_t s
 // A batch's instances have other kernels to compare with: batch.cpp decides.
 static bool repack_pays(Variant direct, double points, double share, int64_t tiles) {
   switch (direct) {
-    case V_ST32_C64_V4W7: case V_ST32_C64P_V4W7: return points >= 1e7 && share >= 0.2;
-    case V_ST32_H16_V4: case V_ST32_B16_V4: return points >= 4e7 && share >= 0.125;
+    case V_ST32_C64_V4W7: case V_ST32_C64P_V4W7: case V_ST32_H16_V4: case V_ST32_B16_V4:
+      return points >= 1e7 && share >= 0.1125;
     case V_ST64_C64: return points >= 2e7;
     case V_ST64_C64_V4: case V_ST64_C64P_V4: case V_ST64_H16_V4: case V_ST64_B16_V4: case V_ST64_H16:
       return tiles >= 3 * 2 * 152 && share >= 0.4;

@@ -34,7 +34,8 @@ DIRECT = [  # repacked, these took 1.1 to 2 times as long
 REPACKED = [
     (48, 5, "c64", 3.0, 1, 135), (48, 33, "c64", 1.0, 1, 135), (64, 12, "c64split", 3.0, 1, 240), (128, 20, "c64", 1.0, 1, 585),
     (128, 28, "c64split", 1.0, 3, 585), (192, 20, "f16x2", 1.0, 3, 784), (256, 40, "c64", 1.0, 3, 983), (256, 64, "f16x2", 1.0, 3, 983),
-    (64, 72, "c64", 1.0, 1, 240)]
+    (64, 72, "c64", 1.0, 1, 240), (144, 20, "f16x2", 1.0, 1, 518, 2, 240), (144, 24, "bf16x2", 1.0, 1, 518, 2, 240),
+    (256, 28, "c64split", 3.0, 3, 983)]
 
 
 @pytest.mark.parametrize("case", DIRECT)
